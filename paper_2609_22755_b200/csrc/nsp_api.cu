@@ -39,6 +39,13 @@ struct nsp_plan {
                                       // cost-1 tail = q tile 0 of every segment runs in the first-tile forward kernel)
   bool deterministic = false;         // plan option: dQ tiles added in key-tile order
   bool rounded_dq = false;            // plan option: dQ terms rounded to a fixed quantum (order-independent sums)
+  // Small batches launch the preprocess and the main kernel chained as well (see launch_chained_if), so that the main
+  // kernel runs beside the first-tile kernel on SMs that one leaves idle and neither pays its launch: 8,192 tokens at
+  // 32q/4kv 615 -> 590 us, four short sequences at 8q/2kv 97 -> 64 us. A large batch fills every SM with either kernel,
+  // and a block that starts on an SM still set up for its predecessor keeps that one's split between L1 and shared
+  // memory: with L1 at 28 KB instead of 60 KB the main kernel is 3 % slower (425,984 tokens: 527 -> 550 ms a step) and
+  // the preprocess kernel 25 %. The lines cross between 110 and 300 steps per SM.
+  bool small_bwd = false;
   int32_t max_len = 0;                // longest segment: no preprocess / main / postprocess launch when <= 128
   int32_t* d_front = nullptr;        // [n_bwd / kFrontBlock + 1] start-alignment counters of the backward kernel
   int32_t* d_counters = nullptr;  // [0] forward cursor, [1] backward cursor
@@ -319,6 +326,7 @@ int nsp_plan_tiles(const int32_t* cu_seqlens, const int32_t* hq, const int32_t* 
     return NSP_ERR_UNSUPPORTED;
   }
 
+  int64_t bwd_steps = 0;  // (key tile, q tile, q head) steps of the backward pass
   std::vector<nsp_tile_t> bwd_exec, bwd_first;
   std::vector<SegInfo> pack_segs;
   std::vector<RowInfo> pack_rows;
@@ -378,6 +386,10 @@ int nsp_plan_tiles(const int32_t* cu_seqlens, const int32_t* hq, const int32_t* 
     }
     p->n_first = static_cast<int64_t>(bwd_first.size());
     p->n_fwd_main = nf;
+    for (const SegInfo& sg : p->seg) {
+      const int64_t Mt = (static_cast<int64_t>(sg.len) + bm - 1) / bm;
+      bwd_steps += sg.hq * (Mt * (Mt + 1) / 2);
+    }
     for (const SegInfo& sg : p->seg)
       if (sg.len > 0) p->n_fwd_main -= sg.hq;
     for (const SegInfo& sg : p->seg) p->max_len = std::max(p->max_len, sg.len);
@@ -393,6 +405,7 @@ int nsp_plan_tiles(const int32_t* cu_seqlens, const int32_t* hq, const int32_t* 
     return NSP_ERR_CUDA;
   }
   p->num_sms = prop.multiProcessorCount;
+  p->small_bwd = bwd_steps <= static_cast<int64_t>(kSmallBwdStepsPerSm) * p->num_sms;
   if (prop.major != 10) {
     delete p;
     return NSP_ERR_UNSUPPORTED;
@@ -526,8 +539,6 @@ int nsp_attn_fwd(const nsp_plan_t* plan, const void* q, const void* k, const voi
         !encode_run_map(&maps.o[r], o, run.q_off, run.tokens, run.hq, plan->head_dim))
       return NSP_ERR_CUDA;
   }
-  if (cudaMemsetAsync(plan->d_counters, 0, sizeof(int32_t), st) != cudaSuccess) return NSP_ERR_CUDA;
-  if (cudaMemsetAsync(plan->d_counters + 3, 0, sizeof(int32_t), st) != cudaSuccess) return NSP_ERR_CUDA;
   FwdArgs a;
   a.seg = plan->d_seg;
   a.status = status_word(plan);
@@ -555,7 +566,7 @@ int nsp_attn_fwd(const nsp_plan_t* plan, const void* q, const void* k, const voi
   a.n_items = static_cast<int32_t>(plan->withhold ? plan->n_fwd : plan->n_fwd_main);
   a.counter = plan->d_counters;
   prof_mark(plan, NSP_KERNEL_FWD, 0, st);
-  if (launch_fwd(maps, a, plan->head_dim, plan->num_sms, st) != cudaSuccess) return NSP_ERR_CUDA;
+  if (launch_fwd(maps, a, plan->head_dim, plan->num_sms, !plan->withhold, st) != cudaSuccess) return NSP_ERR_CUDA;
   prof_mark(plan, NSP_KERNEL_FWD, 1, st);
   return NSP_OK;
 }
@@ -614,15 +625,11 @@ int bwd_impl(const nsp_plan_t* plan, const uint8_t* recompute, const void* q, co
       return NSP_ERR_CUDA;
     if (recompute) fmaps.q[r] = maps.q[r], fmaps.k[r] = maps.k[r], fmaps.v[r] = maps.v[r];
   }
-  if (cudaMemsetAsync(plan->d_counters + 1, 0, 2 * sizeof(int32_t), st) != cudaSuccess) return NSP_ERR_CUDA;
-  if (cudaMemsetAsync(plan->d_front, 0, sizeof(int32_t) * (plan->n_bwd / kFrontBlock + 1), st) != cudaSuccess)
-    return NSP_ERR_CUDA;
   if (recompute) {
     // from pageable memory the runtime stages the flags before it returns; a pinned array must stay unchanged until
     // the stream has passed this copy
     if (cudaMemcpyAsync(d_mask, recompute, static_cast<size_t>(plan->n_seg), cudaMemcpyHostToDevice, st) != cudaSuccess)
       return NSP_ERR_CUDA;
-    if (cudaMemsetAsync(plan->d_counters, 0, sizeof(int32_t), st) != cudaSuccess) return NSP_ERR_CUDA;
     FwdArgs fa;
     fa.seg = plan->d_seg;
     fa.items = plan->d_fwd;
@@ -641,7 +648,7 @@ int bwd_impl(const nsp_plan_t* plan, const uint8_t* recompute, const void* q, co
     fa.d_o = static_cast<const __nv_bfloat16*>(d_o);
     fa.delta = delta;
     prof_mark(plan, NSP_KERNEL_FWD, 0, st);
-    if (launch_fwd(fmaps, fa, plan->head_dim, plan->num_sms, st) != cudaSuccess) return NSP_ERR_CUDA;
+    if (launch_fwd(fmaps, fa, plan->head_dim, plan->num_sms, false, st) != cudaSuccess) return NSP_ERR_CUDA;
     prof_mark(plan, NSP_KERNEL_FWD, 1, st);
   }
   // Segments of at most 128 tokens are finished by the first-tile kernel alone; a batch made only of such segments
@@ -657,7 +664,8 @@ int bwd_impl(const nsp_plan_t* plan, const uint8_t* recompute, const void* q, co
     if (launch_bwd_preprocess(plan->d_seg, plan->n_seg, plan->d_row_base, plan->lse_elems, plan->head_dim,
                               static_cast<const __nv_bfloat16*>(o), static_cast<const __nv_bfloat16*>(d_o), delta,
                               dq_acc, recompute ? d_mask : nullptr, recompute ? lse : nullptr,
-                              recompute ? lse_ws : nullptr, st) != cudaSuccess)
+                              recompute ? lse_ws : nullptr, plan->d_front,
+                              static_cast<int>(plan->n_bwd / kFrontBlock + 1), plan->small_bwd, st) != cudaSuccess)
       return NSP_ERR_CUDA;
   }
   prof_mark(plan, NSP_KERNEL_BWD_PRE, 1, st);
@@ -694,7 +702,7 @@ int bwd_impl(const nsp_plan_t* plan, const uint8_t* recompute, const void* q, co
   a.n_items = static_cast<int32_t>(plan->n_bwd);
   a.counter = plan->d_counters + 1;
   prof_mark(plan, NSP_KERNEL_BWD_MAIN, 0, st);
-  if (multi && launch_bwd(maps, a, plan->head_dim, plan->num_sms, st) != cudaSuccess) return NSP_ERR_CUDA;
+  if (multi && launch_bwd(maps, a, plan->head_dim, plan->num_sms, plan->small_bwd, st) != cudaSuccess) return NSP_ERR_CUDA;
   prof_mark(plan, NSP_KERNEL_BWD_MAIN, 1, st);
   prof_mark(plan, NSP_KERNEL_BWD_POST, 0, st);
   if (multi && launch_bwd_postprocess(plan->d_seg, plan->n_seg, plan->d_row_base, plan->lse_elems, plan->head_dim, dq_acc, dq,

@@ -240,6 +240,12 @@ __global__ void __launch_bounds__(kBwdThreads, 1) bwd_kernel(const __grid_consta
     if (warp == 0 && !misaligned) tmem_dealloc(s.tmem_base, kBwdTmemCols);
     return;
   }
+  // Chain: preprocess, first-tile kernel, main kernel, postprocess. The first-tile kernel waits for the preprocess kernel
+  // and only then lets the main kernel start, which therefore finds delta, the zeroed accumulator and the copied LSE
+  // complete (it reads them from L2) and runs beside the first-tile kernel where SMs are free. What the main kernel
+  // needs of the first-tile kernel itself, its part of dK / dV of key tile 0, it waits for in that item's epilogue.
+  if constexpr (FIRST) grid_wait_predecessor();
+  grid_launch_dependents();
   volatile int32_t* abort_flag = &s.abort;
   uint32_t gs = 0;  // steps completed so far by this CTA (every role advances it identically)
   uint32_t gi = 0;  // items completed so far
@@ -258,7 +264,10 @@ __global__ void __launch_bounds__(kBwdThreads, 1) bwd_kernel(const __grid_consta
     for (;;) {
       const int idx = atomicAdd(a.counter, 1);
       x.it = idx;
-      if (idx >= a.n_items) break;
+      if (idx >= a.n_items) {
+        reset_cursor(a.counter, idx, a.n_items, 1);
+        break;
+      }
       const nsp_tile_t item = a.items[idx];
       const SegInfo sg = a.seg[item.seg];
       x.q_off = sg.q_off, x.kv_off = sg.kv_off, x.lse_off = sg.lse_off;
@@ -553,8 +562,8 @@ __global__ void __launch_bounds__(kBwdThreads, 1) bwd_kernel(const __grid_consta
                 }
               }
               NSP_CHECK(at >= 0 && at < a.lse_elems, a.status, c.it, kWhereCheckBwdLse, qi) {
-                lv = a.lse[at] * kLog2e;
-                dv_ = a.delta[at];
+                lv = __ldcg(a.lse + at) * kLog2e;
+                dv_ = __ldcg(a.delta + at);
               }
             }
             s.lse[st][col] = lv;
@@ -975,6 +984,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) bwd_kernel(const __grid_consta
         // Key tile 0 in the main kernel: the first-tile kernel, which ran before, left its part (q tile 0) in the
         // output; this item's sum over the q tiles 1 .. Mt-1 is added to it (one fixed order: reproducible).
         const bool add = !FIRST && c.first;
+        if (add) grid_wait_predecessor();
         if (a.dkv_f32 && (c.n + 1) * kBN <= c.len) {
           // ---- fp32 outputs, full key tile: staged in shared memory (every operand buffer is free now: dK over K
           // and V, dV over the Q ring), swizzled as sub-tiles of 32 columns, and written by TMA tile stores (added,
@@ -1074,6 +1084,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) bwd_kernel(const __grid_consta
     }
   }
 
+  if constexpr (!FIRST) grid_wait_predecessor();
   tc_fence_before_sync();
   __syncthreads();
   if (warp == 0) tmem_dealloc(s.tmem_base, kBwdTmemCols);
@@ -1105,7 +1116,11 @@ __global__ void __launch_bounds__(256) bwd_preprocess_kernel(const SegInfo* __re
                                                              float* __restrict__ delta, float* __restrict__ dq_acc,
                                                              const uint8_t* __restrict__ seg_skip,
                                                              const float* __restrict__ lse_in,
-                                                             float* __restrict__ lse_out) {
+                                                             float* __restrict__ lse_out, int32_t* __restrict__ front,
+                                                             int n_front) {
+  grid_wait_predecessor();
+  grid_launch_dependents();
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n_front; i += gridDim.x * blockDim.x) front[i] = 0;
   constexpr int kLanesPerRow = D / 8, kRowsPerLoad = 32 / kLanesPerRow, kRowsPerPass = 4 * kRowsPerLoad;
   const int lane = threadIdx.x & 31, sub = lane / kLanesPerRow, l = lane % kLanesPerRow;
   const int64_t n_groups = (total_rows + kRowsPerPass - 1) / kRowsPerPass;
@@ -1178,6 +1193,8 @@ __global__ void __launch_bounds__(256) bwd_postprocess_kernel(const SegInfo* __r
                                                               const int64_t* __restrict__ row_base, int64_t total_rows,
                                                               const float* __restrict__ acc, void* __restrict__ dq,
                                                               int dq_f32, float scale) {
+  grid_wait_predecessor();
+  grid_launch_dependents();
   constexpr int kLanesPerRow = D / 8, kRowsPerLoad = 32 / kLanesPerRow, kRowsPerPass = 4 * kRowsPerLoad;
   const int lane = threadIdx.x & 31, sub = lane / kLanesPerRow, l = lane % kLanesPerRow;
   const int64_t n_groups = (total_rows + kRowsPerPass - 1) / kRowsPerPass;
@@ -1219,46 +1236,41 @@ __global__ void __launch_bounds__(256) bwd_postprocess_kernel(const SegInfo* __r
 cudaError_t launch_bwd_preprocess(const SegInfo* d_seg, int n_seg, const int64_t* d_row_base, int64_t total_rows,
                                   int head_dim, const __nv_bfloat16* o, const __nv_bfloat16* d_o, float* delta,
                                   float* dq_acc, const uint8_t* seg_skip, const float* lse_in, float* lse_out,
-                                  cudaStream_t st) {
+                                  int32_t* front, int n_front, bool chained, cudaStream_t st) {
   if (total_rows == 0) return cudaSuccess;
   int64_t blocks = ((total_rows + 7) / 8 * 32 + 255) / 256;  // about one warp per eight rows, grid-stride beyond 16 waves
   if (blocks > 148 * 8 * 16) blocks = 148 * 8 * 16;
-  if (head_dim == 64)
-    bwd_preprocess_kernel<64><<<static_cast<unsigned>(blocks), 256, 0, st>>>(d_seg, n_seg, d_row_base, total_rows, o, d_o,
-                                                                             delta, dq_acc, seg_skip, lse_in, lse_out);
-  else
-    bwd_preprocess_kernel<128><<<static_cast<unsigned>(blocks), 256, 0, st>>>(d_seg, n_seg, d_row_base, total_rows, o, d_o,
-                                                                              delta, dq_acc, seg_skip, lse_in, lse_out);
   count_launches(1);
-  return cudaGetLastError();
+  return launch_chained_if(chained, head_dim == 64 ? bwd_preprocess_kernel<64> : bwd_preprocess_kernel<128>,
+                           static_cast<unsigned>(blocks), 256, 0, st, d_seg, n_seg, d_row_base, total_rows, o, d_o, delta,
+                           dq_acc, seg_skip, lse_in, lse_out, front, n_front);
 }
 
 namespace {
 template <bool FIRST, int DET, int D>
-cudaError_t launch_bwd_t(const BwdMaps& maps, const BwdArgs& args, int num_sms, cudaStream_t st) {
+cudaError_t launch_bwd_t(const BwdMaps& maps, const BwdArgs& args, int num_sms, bool chained, cudaStream_t st) {
   if (args.n_items == 0) return cudaSuccess;
   cudaError_t e = cudaFuncSetAttribute(bwd_kernel<FIRST, DET, D>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        static_cast<int>(sizeof(BwdSmem<FIRST, D>)));
   if (e != cudaSuccess) return e;
   const int grid = args.n_items < num_sms ? args.n_items : num_sms;
-  bwd_kernel<FIRST, DET, D><<<grid, kBwdThreads, sizeof(BwdSmem<FIRST, D>), st>>>(maps, args);
   count_launches(1);
-  return cudaGetLastError();
+  return launch_chained_if(chained, bwd_kernel<FIRST, DET, D>, grid, kBwdThreads, sizeof(BwdSmem<FIRST, D>), st, maps, args);
 }
 }  // namespace
 
-cudaError_t launch_bwd(const BwdMaps& maps, const BwdArgs& args, int head_dim, int num_sms, cudaStream_t st) {
+cudaError_t launch_bwd(const BwdMaps& maps, const BwdArgs& args, int head_dim, int num_sms, bool chained, cudaStream_t st) {
   if (head_dim == 64)
-    return args.dq_turn    ? launch_bwd_t<false, 1, 64>(maps, args, num_sms, st)
-           : args.dq_rounded ? launch_bwd_t<false, 2, 64>(maps, args, num_sms, st)
-                             : launch_bwd_t<false, 0, 64>(maps, args, num_sms, st);
-  return args.dq_turn    ? launch_bwd_t<false, 1, 128>(maps, args, num_sms, st)
-         : args.dq_rounded ? launch_bwd_t<false, 2, 128>(maps, args, num_sms, st)
-                           : launch_bwd_t<false, 0, 128>(maps, args, num_sms, st);
+    return args.dq_turn    ? launch_bwd_t<false, 1, 64>(maps, args, num_sms, chained, st)
+           : args.dq_rounded ? launch_bwd_t<false, 2, 64>(maps, args, num_sms, chained, st)
+                             : launch_bwd_t<false, 0, 64>(maps, args, num_sms, chained, st);
+  return args.dq_turn    ? launch_bwd_t<false, 1, 128>(maps, args, num_sms, chained, st)
+         : args.dq_rounded ? launch_bwd_t<false, 2, 128>(maps, args, num_sms, chained, st)
+                           : launch_bwd_t<false, 0, 128>(maps, args, num_sms, chained, st);
 }
 cudaError_t launch_bwd_first(const BwdMaps& maps, const BwdArgs& args, int head_dim, int num_sms, cudaStream_t st) {
-  return head_dim == 64 ? launch_bwd_t<true, 0, 64>(maps, args, num_sms, st)
-                        : launch_bwd_t<true, 0, 128>(maps, args, num_sms, st);
+  return head_dim == 64 ? launch_bwd_t<true, 0, 64>(maps, args, num_sms, true, st)
+                        : launch_bwd_t<true, 0, 128>(maps, args, num_sms, true, st);
 }
 
 cudaError_t launch_bwd_postprocess(const SegInfo* d_seg, int n_seg, const int64_t* d_row_base, int64_t total_rows,
@@ -1267,14 +1279,10 @@ cudaError_t launch_bwd_postprocess(const SegInfo* d_seg, int n_seg, const int64_
   if (total_rows == 0) return cudaSuccess;
   int64_t blocks = ((total_rows + 7) / 8 * 32 + 255) / 256;
   if (blocks > 148 * 8 * 16) blocks = 148 * 8 * 16;
-  if (head_dim == 64)
-    bwd_postprocess_kernel<64><<<static_cast<unsigned>(blocks), 256, 0, st>>>(d_seg, n_seg, d_row_base, total_rows,
-                                                                              dq_acc, dq, dq_f32, scale);
-  else
-    bwd_postprocess_kernel<128><<<static_cast<unsigned>(blocks), 256, 0, st>>>(d_seg, n_seg, d_row_base, total_rows,
-                                                                               dq_acc, dq, dq_f32, scale);
   count_launches(1);
-  return cudaGetLastError();
+  return launch_chained_if(true, head_dim == 64 ? bwd_postprocess_kernel<64> : bwd_postprocess_kernel<128>,
+                           static_cast<unsigned>(blocks), 256, 0, st, d_seg, n_seg, d_row_base, total_rows, dq_acc, dq, dq_f32,
+                           scale);
 }
 
 }  // namespace nsp

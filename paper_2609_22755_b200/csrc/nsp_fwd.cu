@@ -126,6 +126,9 @@ __global__ void __launch_bounds__(kFwdThreads, 1) fwd_kernel(const __grid_consta
   __syncthreads();
   tc_fence_after_sync();
 
+  // Chained behind the first-tile kernel, whose inputs are this kernel's and whose outputs it does not touch: the two
+  // run side by side where SMs are free, and the wait comes at the end.
+  grid_launch_dependents();
   const uint32_t tmem = s.tmem_base;
   volatile int32_t* abort_flag = &s.abort;
   uint32_t gp = 0;  // pops so far
@@ -156,7 +159,10 @@ __global__ void __launch_bounds__(kFwdThreads, 1) fwd_kernel(const __grid_consta
     for (;;) {
       const int it = atomicAdd(a.counter, 2);
       p.it0 = it;
-      if (it >= a.n_items) break;
+      if (it >= a.n_items) {
+        reset_cursor(a.counter, it, (a.n_items + 1) / 2 * 2, 2);
+        break;
+      }
       bool have_b = it + 1 < a.n_items;
       nsp_tile_t ia = a.items[it];
       nsp_tile_t ib = have_b ? a.items[it + 1] : ia;
@@ -689,6 +695,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1) fwd_kernel(const __grid_consta
     }
   }
 
+  grid_wait_predecessor();
   cta_sync();  // after a timeout the stragglers are not waited for for ever
   if (warp == 0) tmem_dealloc(s.tmem_base, kFwdTmemCols);
 }
@@ -697,24 +704,23 @@ __global__ void __launch_bounds__(kFwdThreads, 1) fwd_kernel(const __grid_consta
 
 namespace {
 template <int D, bool RECOMP>
-cudaError_t launch_fwd_t(const FwdMaps& maps, const FwdArgs& args, int num_sms, cudaStream_t st) {
+cudaError_t launch_fwd_t(const FwdMaps& maps, const FwdArgs& args, int num_sms, bool chained, cudaStream_t st) {
   cudaError_t e = cudaFuncSetAttribute(fwd_kernel<D, RECOMP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        static_cast<int>(sizeof(FwdSmem<D>)));
   if (e != cudaSuccess) return e;
   const int pops = (args.n_items + 1) / 2;
   const int grid = pops < num_sms ? pops : num_sms;
-  fwd_kernel<D, RECOMP><<<grid, kFwdThreads, sizeof(FwdSmem<D>), st>>>(maps, args);
   count_launches(1);
-  return cudaGetLastError();
+  return launch_chained_if(chained, fwd_kernel<D, RECOMP>, grid, kFwdThreads, sizeof(FwdSmem<D>), st, maps, args);
 }
 }  // namespace
 
-cudaError_t launch_fwd(const FwdMaps& maps, const FwdArgs& args, int head_dim, int num_sms, cudaStream_t st) {
+cudaError_t launch_fwd(const FwdMaps& maps, const FwdArgs& args, int head_dim, int num_sms, bool chained, cudaStream_t st) {
   if (args.n_items == 0) return cudaSuccess;
   const bool recomp = args.delta != nullptr || args.seg_mask != nullptr;
   if (head_dim == 64)
-    return recomp ? launch_fwd_t<64, true>(maps, args, num_sms, st) : launch_fwd_t<64, false>(maps, args, num_sms, st);
-  return recomp ? launch_fwd_t<128, true>(maps, args, num_sms, st) : launch_fwd_t<128, false>(maps, args, num_sms, st);
+    return recomp ? launch_fwd_t<64, true>(maps, args, num_sms, chained, st) : launch_fwd_t<64, false>(maps, args, num_sms, chained, st);
+  return recomp ? launch_fwd_t<128, true>(maps, args, num_sms, chained, st) : launch_fwd_t<128, false>(maps, args, num_sms, chained, st);
 }
 
 }  // namespace nsp

@@ -106,6 +106,8 @@ __global__ void __launch_bounds__(kThreads, 1) fwd_first_kernel(const __grid_con
   tc_fence_before_sync();
   __syncthreads();
   tc_fence_after_sync();
+  grid_wait_predecessor();
+  grid_launch_dependents();
   const uint32_t tmem = s.tmem_base;
   volatile int32_t* abort_flag = &s.abort;
 
@@ -122,6 +124,8 @@ __global__ void __launch_bounds__(kThreads, 1) fwd_first_kernel(const __grid_con
       x.len = sg.len, x.hq = sg.hq, x.G = sg.hq / sg.hkv, x.g = item.head, x.run = sg.run, x.tok0 = sg.tok_in_run;
       x.rounds = (x.G + 1) / 2;
       x.rows = sg.rows;
+    } else {
+      reset_cursor(a.counter, idx, a.n_items, 1);
     }
   };
   auto next_item = [&]() -> bool {
@@ -425,9 +429,8 @@ cudaError_t launch_t(const FwdMaps& maps, const FwdArgs& args, int num_sms, cuda
                                        static_cast<int>(sizeof(FwdFirstSmem<D>)));
   if (e != cudaSuccess) return e;
   const int grid = args.n_items < num_sms ? args.n_items : num_sms;
-  fwd_first_kernel<D><<<grid, kThreads, sizeof(FwdFirstSmem<D>), st>>>(maps, args);
   count_launches(1);
-  return cudaGetLastError();
+  return launch_chained_if(true, fwd_first_kernel<D>, grid, kThreads, sizeof(FwdFirstSmem<D>), st, maps, args);
 }
 
 }  // namespace

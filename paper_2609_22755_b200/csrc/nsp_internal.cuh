@@ -1,6 +1,7 @@
 // Internal structures shared by the host API and the kernels of libnsp (never visible across the C ABI).
 #pragma once
 #include <cstdint>
+#include <utility>
 #include <cuda.h>
 #include <cuda_runtime.h>
 #include "../../include/nsp.h"
@@ -10,6 +11,7 @@ namespace nsp {
 constexpr int kHeadDim = NSP_HEAD_DIM;
 constexpr int kBM = 128;  // query rows per tile
 constexpr int kBN = 128;  // key rows per tile
+constexpr int kSmallBwdStepsPerSm = 192;  // see nsp_plan::small_bwd
 constexpr int kFrontBlock = 16;  // backward: consecutive work items whose CTAs start together
 
 // Per-segment table entry (device + host copy).
@@ -135,7 +137,7 @@ struct FwdArgs {
   const SegInfo* seg;
   const nsp_tile_t* items;
   int32_t n_items;
-  int32_t* counter;  // work-list cursor, zeroed before the launch
+  int32_t* counter;  // work-list cursor: zero at the launch, and left at zero (see reset_cursor)
   StatusWord status;
   __nv_bfloat16* o;
   float* lse;
@@ -155,7 +157,7 @@ struct BwdArgs {
   const SegInfo* seg;
   const nsp_tile_t* items;
   int32_t n_items;
-  int32_t* counter;  // work-list cursor, zeroed before the launch
+  int32_t* counter;  // work-list cursor: zero at the launch, and left at zero (see reset_cursor)
   StatusWord status;
   const float* lse;
   const float* delta;
@@ -171,9 +173,34 @@ struct BwdArgs {
   float scale_log2;
   long long wait_limit;  // SM clocks a device-side wait may take before it gives up
   int64_t q_elems, kv_elems, lse_elems;  // tensor sizes (checked build)
-  int32_t* front;    // [n_items / kFrontBlock + 1] arrival counters, zeroed before the launch (see next_item)
+  int32_t* front;    // [n_items / kFrontBlock + 1] arrival counters, zeroed by the preprocess kernel (see next_item)
   const RowInfo* rows;  // row tables of the packs (first-tile kernel)
 };
+
+// A persistent kernel's work-list cursor goes back to zero without a memset between the launches (which would also cut
+// the programmatic dependency between them): every CTA pops until its first failure and never again, so the pop that is
+// `grid` - 1 steps past the first failing position is the last one of the launch. (A launch that gave up after a
+// timeout leaves the cursor as it is; the plan then refuses further work.)
+__device__ __forceinline__ void reset_cursor(int32_t* counter, int pop, int first_failing, int step) {
+  if (pop == first_failing + step * (static_cast<int>(gridDim.x) - 1)) *reinterpret_cast<volatile int32_t*>(counter) = 0;
+}
+
+// <<<grid, threads, smem, st>>>, chained: with programmatic stream serialization (see grid_wait_predecessor).
+template <typename... P, typename... A>
+inline cudaError_t launch_chained_if(bool chained, void (*kernel)(P...), unsigned grid, unsigned threads, size_t smem,
+                                     cudaStream_t st, A&&... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = chained ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
+}
 
 // Host-side launchers implemented next to their kernels.
 cudaError_t launch_plan_build(const SegInfo* d_seg, int n_seg, int bm, int bn, nsp_tile_t* d_fwd, int64_t n_fwd,
@@ -181,19 +208,20 @@ cudaError_t launch_plan_build(const SegInfo* d_seg, int n_seg, int bm, int bn, n
                               size_t sort_tmp_bytes, const int64_t* d_fwd_base, const int64_t* d_bwd_base,
                               cudaStream_t st);
 size_t plan_sort_tmp_bytes(int64_t max_items);
-cudaError_t launch_fwd(const FwdMaps& maps, const FwdArgs& args, int head_dim, int num_sms, cudaStream_t st);
+// chained: launched right behind launch_fwd_first, whose inputs are this kernel's too
+cudaError_t launch_fwd(const FwdMaps& maps, const FwdArgs& args, int head_dim, int num_sms, bool chained, cudaStream_t st);
 // q tile 0 of every segment: items (segment, kv head); args.items / n_items / counter are that list's
 cudaError_t launch_fwd_first(const FwdMaps& maps, const FwdArgs& args, int head_dim, int num_sms, cudaStream_t st);
 // The backward launches, in the order they run: preprocess (delta and zeroed accumulator rows for tokens 128.. of
 // every segment), first-tile kernel (q tile 0 of every segment: its dQ rows, and its part of dK / dV), main kernel,
 // postprocess (tokens 128..). seg_skip (may be null): segments whose delta is left alone; lse_in / lse_out (may be
-// null): LSE copied for the rows whose delta is written.
+// null): LSE copied for the rows whose delta is written. front [n_front]: the main kernel's arrival counters, zeroed.
 cudaError_t launch_bwd_preprocess(const SegInfo* d_seg, int n_seg, const int64_t* d_row_base, int64_t total_rows,
                                   int head_dim, const __nv_bfloat16* o, const __nv_bfloat16* d_o, float* delta,
                                   float* dq_acc, const uint8_t* seg_skip, const float* lse_in, float* lse_out,
-                                  cudaStream_t st);
+                                  int32_t* front, int n_front, bool chained, cudaStream_t st);
 cudaError_t launch_bwd_first(const BwdMaps& maps, const BwdArgs& args, int head_dim, int num_sms, cudaStream_t st);
-cudaError_t launch_bwd(const BwdMaps& maps, const BwdArgs& args, int head_dim, int num_sms, cudaStream_t st);  // args.dq_turn / args.dq_rounded select the reproducible variants
+cudaError_t launch_bwd(const BwdMaps& maps, const BwdArgs& args, int head_dim, int num_sms, bool chained, cudaStream_t st);  // args.dq_turn / args.dq_rounded select the reproducible variants
 cudaError_t launch_bwd_postprocess(const SegInfo* d_seg, int n_seg, const int64_t* d_row_base, int64_t total_rows,
                                    int head_dim, const float* dq_acc, void* dq, int dq_f32, float scale,
                                    cudaStream_t st);

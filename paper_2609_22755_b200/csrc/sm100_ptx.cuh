@@ -89,6 +89,15 @@ __device__ __forceinline__ void tc_fence_after_sync() {
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 }
 
+// ---------------------------------------------------------------- programmatic dependent launch
+// The kernels of a call follow one another with programmatic stream serialization (launch_chained_if): a kernel may start
+// while its predecessor still runs, once every block of the predecessor has called grid_launch_dependents.
+// grid_wait_predecessor returns when the predecessor has completed and its writes are visible. Two rules keep the chain
+// transitive: a kernel calls grid_launch_dependents only when all that its successor uses before the successor's own
+// wait has completed, and no kernel ends before its own grid_wait_predecessor.
+__device__ __forceinline__ void grid_wait_predecessor() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 // ---------------------------------------------------------------- TMA (tiled loads, own-GPU memory, no multicast)
 // 3-D tile load: coordinates (c0 innermost). c0 * elem_size must be a multiple of 16 B.
 __device__ __forceinline__ void tma_load_3d(void* smem_dst, const void* tmap, uint64_t* bar, int32_t c0, int32_t c1,

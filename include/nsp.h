@@ -99,7 +99,8 @@ typedef struct {
  *   backward item (s, g, n), g in [0,hkv[s]), n in [0, ceil(L_s/bn)): cost = (hq[s]/hkv[s]) * (ceil(L_s/bm) - floor(n*bn/bm))
  *   order: cost descending, then seg, tile, head ascending (a total order: the list is unique).
  * cu_seqlens [n_seg+1], hq [n_seg], hkv [n_seg]: host arrays, copied. Zero-length segments and n_seg == 0 are legal.
- * opts may be NULL (= {128,128,1,0}). The lists are built by kernels enqueued on `stream`.
+ * opts may be NULL (= {128,128,1,0}). The lists are built on a stream of the plan's own and are complete when the call
+ * returns; it does not wait for work enqueued on `stream` or any other stream (`stream` is not used).
  * Errors: INVALID_ARG (null, n_seg < 0, cu_seqlens[0] != 0, decreasing cu_seqlens, hq/hkv <= 0, hq % hkv != 0),
  * UNSUPPORTED (head_dim other than 128 or 64, > NSP_MAX_RUNS runs, unsupported tile sizes, >= 65536 segments, > 256 heads,
  * >= 65536 tiles in a segment), ALLOC, CUDA. On error *out_plan is NULL.
@@ -341,8 +342,13 @@ int nsp_plan_kernel_ms(const nsp_plan_t* plan, int kernel_id, float* ms);
 /* Number of kernel launches the library has enqueued so far in this process (all plans). */
 int64_t nsp_launch_count(void);
 
-/* Free the plan (device lists, tables, status word). NULL is a no-op. */
+/* Free the plan (device lists, tables, status word). NULL is a no-op. The memory is kept for later plans, at most 64 MiB
+ * (device and pinned host together) in at most eight blocks per process; what the plan's last calls enqueued may still be
+ * running, and the block is not handed out again before that has finished. Call it outside any stream capture. */
 int nsp_plan_destroy(nsp_plan_t* plan);
+
+/* Give back all memory kept from destroyed plans. */
+int nsp_trim(void);
 
 const char* nsp_status_string(int code);
 

@@ -32,7 +32,7 @@ EXPORTS = [
     "nsp_attn_bwd_static", "nsp_recompute_mark", "nsp_plan_recompute_ws_bytes", "nsp_attn_bwd_recompute",
     "nsp_cost_table", "nsp_route_sp_tree", "nsp_a2a_gather_heads", "nsp_a2a_scatter_heads",
     "nsp_selftest_wait_timeout", "nsp_a2a_gather_heads_to", "nsp_plan_set_wait_limit",
-    "nsp_plan_step_host_ws_bytes", "nsp_attn_step_host",
+    "nsp_plan_step_host_ws_bytes", "nsp_attn_step_host", "nsp_trim",
 ]
 CHECKED_EXPORTS = ["nsp_checked_withhold_load"]  # libnsp_checked.so only
 NSP_COST_BUCKETS = 16
@@ -118,6 +118,8 @@ def lib() -> ctypes.CDLL:
         L.nsp_launch_count.restype = ctypes.c_int64
         L.nsp_plan_destroy.argtypes = [vp]
         L.nsp_plan_destroy.restype = ctypes.c_int
+        L.nsp_trim.argtypes = []
+        L.nsp_trim.restype = ctypes.c_int
         L.nsp_plan_set_profiling.argtypes = [vp, ctypes.c_int]
         L.nsp_plan_set_profiling.restype = ctypes.c_int
         L.nsp_plan_kernel_ms.argtypes = [vp, ctypes.c_int, ctypes.POINTER(ctypes.c_float)]
@@ -134,6 +136,13 @@ def status_string(code: int) -> str:
 
 def launch_count() -> int:
     return int(lib().nsp_launch_count())
+
+
+def nsp_trim():
+    """Give back the memory kept from destroyed plans."""
+    rc = lib().nsp_trim()
+    if rc != NSP_OK:
+        raise NspError(rc, "nsp_trim")
 
 
 def _i32(a):

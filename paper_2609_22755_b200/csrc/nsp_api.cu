@@ -9,6 +9,7 @@
 #include <new>
 #include <vector>
 #include <cuda_bf16.h>
+#include "nsp_arena.h"
 #include "nsp_internal.cuh"
 #include "sm100_ptx.cuh"
 
@@ -25,12 +26,25 @@ struct nsp_plan {
   int64_t q_elems = 0, kv_elems = 0, lse_elems = 0, n_fwd = 0, n_bwd = 0;
   std::vector<SegInfo> seg;
   std::vector<RunInfo> runs;
-  // device state
+  // device state, all of it inside the arena
+  Arena* arena = nullptr;
   SegInfo* d_seg = nullptr;
   int64_t* d_row_base = nullptr;  // [n_seg + 1] first packed (token, head) row of each segment
   nsp_tile_t* d_fwd = nullptr;
   nsp_tile_t* d_bwd = nullptr;
-  nsp_tile_t* d_bwd_exec = nullptr;  // the backward items in the order the kernel walks them (see build_bwd_exec_order)
+  // The backward items in the order the kernel walks them (nsp_plan_get, pass 2). The published work list (pass 1) is
+  // sorted by cost alone; walked in that order, the CTAs that run at the same time hold key tiles of MANY (segment, kv
+  // head) groups, a q tile's fp32 dQ accumulator rows are touched by a few CTAs now and by the others much later, and
+  // they travel to DRAM and back every time (16 segments of 8,192 tokens, 32q/4kv: 193 GB of DRAM traffic for a backward
+  // pass whose tensors total 5 GB, L2 hit rate 21 %, the kernel runs at HBM speed). Walked group by group -- all key
+  // tiles of one (segment, kv head), first key tile (largest cost) first -- the CTAs of a group sweep the q tiles
+  // together and every accumulator row, Q tile and dO tile is fetched once per group. Groups go by segment length
+  // descending (ties: segment, then kv head, ascending): all CTAs then start the longest group at the same moment, which
+  // is what keeps them on the same q tile (started after a tail of shorter groups they enter it scattered and stay
+  // scattered: 131,072 tokens at 16q/1kv next to 131,072 tokens of shorter segments ran 4 % slower that way, a
+  // long-tailed batch 8 %), and the walk ends with the cheapest items of the shortest segments. Same items, same costs:
+  // a permutation of the published list.
+  nsp_tile_t* d_bwd_exec = nullptr;
   nsp_tile_t* d_bwd_first = nullptr;  // one item per (segment or pack, kv head): the first-tile kernels' list
   int64_t n_first = 0;
   RowInfo* d_rows = nullptr;          // row tables of the packs, 128 entries each (d_seg holds the packs' entries after
@@ -121,38 +135,6 @@ bool encode_run_map_f32(CUtensorMap* out, void* base, int64_t elem_off, int64_t 
              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// Order in which the backward kernel walks its work items (nsp_plan_get, pass 2). The published work list (pass 1)
-// is sorted by cost alone; walked in that order, the CTAs that run at the same time hold key tiles of MANY (segment,
-// kv head) groups, a q tile's fp32 dQ accumulator rows are touched by a few CTAs now and by the others much later,
-// and they travel to DRAM and back every time (16 segments of 8,192 tokens, 32q/4kv: 193 GB of DRAM traffic for a
-// backward pass whose tensors total 5 GB, L2 hit rate 21 %, the kernel runs at HBM speed). Walked group by group
-// -- all key tiles of one (segment, kv head), first key tile (largest cost) first -- the CTAs of a group sweep the q
-// tiles together and every accumulator row, Q tile and dO tile is fetched once per group. Groups go by segment
-// length descending (ties: segment, then kv head, ascending): all CTAs then start the longest group at the same
-// moment, which is what keeps them on the same q tile (started after a tail of shorter groups they enter it scattered
-// and stay scattered: 131,072 tokens at 16q/1kv next to 131,072 tokens of shorter segments ran 4 % slower that way, a
-// long-tailed batch 8 %), and the walk ends with the cheapest items of the shortest segments. Same items, same
-// costs: a permutation of the published list.
-std::vector<nsp_tile_t> build_bwd_exec_order(const std::vector<SegInfo>& seg, int bm, int bn) {
-  struct Group { int32_t len, s, g; };
-  std::vector<Group> groups;
-  for (size_t s = 0; s < seg.size(); ++s)
-    if (seg[s].len > 0)
-      for (int g = 0; g < seg[s].hkv; ++g) groups.push_back(Group{seg[s].len, static_cast<int32_t>(s), g});
-  std::stable_sort(groups.begin(), groups.end(), [](const Group& a, const Group& b) { return a.len > b.len; });
-  std::vector<nsp_tile_t> out;
-  for (const Group& gr : groups) {
-    const SegInfo& sg = seg[gr.s];
-    const int64_t Mt = (static_cast<int64_t>(sg.len) + bm - 1) / bm, Nt = (static_cast<int64_t>(sg.len) + bn - 1) / bn;
-    const int G = sg.hq / sg.hkv;
-    for (int64_t n = 0; n < Nt; ++n) {
-      const int64_t cost = G * (Mt - (n * bn) / bm);
-      out.push_back(nsp_tile_t{gr.s, gr.g, static_cast<int32_t>(n), static_cast<int32_t>(cost)});
-    }
-  }
-  return out;
-}
-
 // The plan's failure state: set once a kernel of the plan has recorded a failure. The record sits in mapped pinned
 // host memory, so looking at it costs a host load, not a synchronisation; a failure is seen by the first call made
 // after the failing kernel wrote it.
@@ -187,24 +169,21 @@ inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 void free_plan(nsp_plan* p) {
   if (!p) return;
-  cudaFree(p->d_seg);
-  cudaFree(p->d_row_base);
-  cudaFree(p->d_fwd);
-  cudaFree(p->d_bwd);
-  cudaFree(p->d_bwd_exec);
-  cudaFree(p->d_bwd_first);
-  cudaFree(p->d_rows);
-  cudaFree(p->d_front);
-  cudaFree(p->d_counters);
-  cudaFree(p->d_status);
-  if (p->h_status) cudaFreeHost(p->h_status);
   for (cudaEvent_t e : p->ev)
     if (e) cudaEventDestroy(e);
   for (cudaEvent_t e : p->hev)
     if (e) cudaEventDestroy(e);
   if (p->copy_stream) cudaStreamDestroy(p->copy_stream);
+  arena_release(p->arena);
   delete p;
 }
+
+// Ends every call that enqueues work of a plan, however it returns: see arena_used.
+struct UsesArena {
+  const nsp_plan* plan;
+  cudaStream_t st;
+  ~UsesArena() { arena_used(plan->arena, st); }
+};
 
 // Record the start / stop event of kernel `id` when profiling is on.
 void prof_mark(const nsp_plan* plan, int id, int stop, cudaStream_t st) {
@@ -237,6 +216,7 @@ int64_t nsp_launch_count(void) { return g_launches.load(std::memory_order_relaxe
 
 int nsp_plan_tiles(const int32_t* cu_seqlens, const int32_t* hq, const int32_t* hkv, int32_t n_seg, int32_t head_dim,
                    const nsp_plan_opts* opts, void* stream, nsp_plan_t** out_plan) {
+  (void)stream;
   if (!out_plan) return NSP_ERR_INVALID_ARG;
   *out_plan = nullptr;
   if (n_seg < 0 || (n_seg > 0 && (!cu_seqlens || !hq || !hkv))) return NSP_ERR_INVALID_ARG;
@@ -264,17 +244,19 @@ int nsp_plan_tiles(const int32_t* cu_seqlens, const int32_t* hq, const int32_t* 
   p->rounded_dq = opts && !p->deterministic && (opts->flags & NSP_PLAN_ROUNDED_DQ) != 0;
   p->bm = bm;
   p->bn = bn;
-  std::vector<int64_t> row_base, fwd_base, bwd_base;
+  std::vector<int64_t> row_base;
+  std::vector<int32_t> tile_base;
+  std::vector<PlanKey> keys;
   try {
     p->seg.resize(n_seg);
     row_base.resize(n_seg + 1);
-    fwd_base.resize(n_seg + 1);
-    bwd_base.resize(n_seg + 1);
+    tile_base.resize(n_seg + 1);
+    keys.resize(n_seg);
   } catch (...) {
     delete p;
     return NSP_ERR_ALLOC;
   }
-  int64_t q_off = 0, kv_off = 0, lse_off = 0, nf = 0, nb = 0;
+  int64_t q_off = 0, kv_off = 0, lse_off = 0, nf = 0, nb = 0, tiles = 0;
   for (int s = 0; s < n_seg; ++s) {
     const int64_t L = static_cast<int64_t>(cu_seqlens[s + 1]) - cu_seqlens[s];
     const int64_t Mt = (L + bm - 1) / bm, Nt = (L + bn - 1) / bn;
@@ -304,8 +286,9 @@ int nsp_plan_tiles(const int32_t* cu_seqlens, const int32_t* hq, const int32_t* 
     sg.turn_off = static_cast<int32_t>(nf);  // one turn counter per forward item = (q head, q tile) of the segment
     run.tokens += L;
     row_base[s] = lse_off;
-    fwd_base[s] = nf;
-    bwd_base[s] = nb;
+    tile_base[s] = static_cast<int32_t>(tiles);
+    keys[s] = PlanKey{static_cast<int32_t>(Mt), hq[s], hq[s] / hkv[s], static_cast<int32_t>(L)};
+    tiles += Mt;
     q_off += L * hq[s] * head_dim;
     kv_off += L * hkv[s] * head_dim;
     lse_off += L * hq[s];
@@ -314,8 +297,7 @@ int nsp_plan_tiles(const int32_t* cu_seqlens, const int32_t* hq, const int32_t* 
   }
   for (int s = 0; s < n_seg; ++s) p->seg[s].run_tokens = static_cast<int32_t>(p->runs[p->seg[s].run].tokens);
   row_base[n_seg] = lse_off;
-  fwd_base[n_seg] = nf;
-  bwd_base[n_seg] = nb;
+  tile_base[n_seg] = static_cast<int32_t>(tiles);
   p->q_elems = q_off;
   p->kv_elems = kv_off;
   p->lse_elems = lse_off;
@@ -327,11 +309,10 @@ int nsp_plan_tiles(const int32_t* cu_seqlens, const int32_t* hq, const int32_t* 
   }
 
   int64_t bwd_steps = 0;  // (key tile, q tile, q head) steps of the backward pass
-  std::vector<nsp_tile_t> bwd_exec, bwd_first;
+  std::vector<nsp_tile_t> bwd_first;
   std::vector<SegInfo> pack_segs;
   std::vector<RowInfo> pack_rows;
   try {
-    bwd_exec = build_bwd_exec_order(p->seg, bm, bn);
     // the first-tile kernel's items: key tile 0 of every group, in the same group order; q heads of the group = steps
     // Segments of fewer than 128 tokens that follow one another inside a run (they are contiguous in every tensor)
     // and together hold at most 128 tokens share one first tile: such a pack becomes an entry of its own behind the
@@ -371,17 +352,19 @@ int nsp_plan_tiles(const int32_t* cu_seqlens, const int32_t* hq, const int32_t* 
     }
     p->n_packs = static_cast<int64_t>(pack_segs.size());
     {
-      std::vector<char> listed(pack_segs.size() * 256, 0);  // (pack, kv head) already in the list
-      for (const nsp_tile_t& t : bwd_exec) {
-        if (t.tile != 0) continue;
-        const int32_t G = p->seg[t.seg].hq / p->seg[t.seg].hkv;
-        if (pack_of[t.seg] < 0) {
-          bwd_first.push_back(nsp_tile_t{t.seg, t.head, 0, G});
-        } else {
-          char& seen = listed[static_cast<size_t>(pack_of[t.seg] - n_seg) * 256 + t.head];
-          if (!seen) bwd_first.push_back(nsp_tile_t{pack_of[t.seg], t.head, 0, G});
-          seen = 1;
+      std::vector<int32_t> order;  // segments by length descending: the order of the groups the backward kernel walks
+      for (int s = 0; s < n_seg; ++s)
+        if (p->seg[s].len > 0) order.push_back(s);
+      std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return p->seg[x].len > p->seg[y].len; });
+      std::vector<char> listed(pack_segs.size(), 0);
+      for (const int s : order) {
+        if (pack_of[s] >= 0) {
+          if (listed[pack_of[s] - n_seg]) continue;
+          listed[pack_of[s] - n_seg] = 1;
         }
+        const SegInfo& sg = p->seg[s];
+        for (int g = 0; g < sg.hkv; ++g)
+          bwd_first.push_back(nsp_tile_t{pack_of[s] >= 0 ? pack_of[s] : s, g, 0, sg.hq / sg.hkv});
       }
     }
     p->n_first = static_cast<int64_t>(bwd_first.size());
@@ -399,89 +382,80 @@ int nsp_plan_tiles(const int32_t* cu_seqlens, const int32_t* hq, const int32_t* 
   }
 
   // ---- device side
-  cudaDeviceProp prop;
-  if (cudaGetDevice(&p->device) != cudaSuccess || cudaGetDeviceProperties(&prop, p->device) != cudaSuccess) {
+  int major = 0;
+  if (cudaGetDevice(&p->device) != cudaSuccess ||
+      cudaDeviceGetAttribute(&p->num_sms, cudaDevAttrMultiProcessorCount, p->device) != cudaSuccess ||
+      cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, p->device) != cudaSuccess) {
     delete p;
     return NSP_ERR_CUDA;
   }
-  p->num_sms = prop.multiProcessorCount;
   p->small_bwd = bwd_steps <= static_cast<int64_t>(kSmallBwdStepsPerSm) * p->num_sms;
-  if (prop.major != 10) {
+  if (major != 10) {
     delete p;
     return NSP_ERR_UNSUPPORTED;
   }
-  cudaStream_t st = static_cast<cudaStream_t>(stream);
-  int64_t* d_bases = nullptr;
-  uint64_t* d_keys = nullptr;
-  void* d_tmp = nullptr;
-  const size_t tmp_bytes = plan_sort_tmp_bytes(nf > nb ? nf : nb);
-  bool okc = true;
-  auto A = [&](void** ptr, size_t bytes) {
-    if (okc && cudaMalloc(ptr, bytes ? bytes : 16) != cudaSuccess) okc = false;
+  // Layout of the arena's device block: what the host uploads (counters and status first, all zero), then the lists the
+  // device builds and the start-alignment counters. The pinned host block holds the host's copy of the status record
+  // and, behind it, the image of the upload.
+  size_t at = 0;
+  auto take = [&](size_t bytes) {
+    const size_t here = at;
+    at += align_up(bytes, 256);
+    return here;
   };
-  A(reinterpret_cast<void**>(&p->d_seg), sizeof(SegInfo) * (n_seg + pack_segs.size()));
-  A(reinterpret_cast<void**>(&p->d_rows), sizeof(RowInfo) * pack_rows.size());
-  A(reinterpret_cast<void**>(&p->d_row_base), sizeof(int64_t) * (n_seg + 1));
-  A(reinterpret_cast<void**>(&p->d_fwd), sizeof(nsp_tile_t) * nf);
-  A(reinterpret_cast<void**>(&p->d_bwd), sizeof(nsp_tile_t) * nb);
-  A(reinterpret_cast<void**>(&p->d_bwd_exec), sizeof(nsp_tile_t) * nb);
-  A(reinterpret_cast<void**>(&p->d_bwd_first), sizeof(nsp_tile_t) * p->n_first);
-  A(reinterpret_cast<void**>(&p->d_front), sizeof(int32_t) * (nb / kFrontBlock + 1));
-  A(reinterpret_cast<void**>(&p->d_counters), 4 * sizeof(int32_t));  // [0] forward, [1] backward main, [2] first-tile backward, [3] first-tile forward
-  A(reinterpret_cast<void**>(&p->d_status), 4 * sizeof(int32_t));
-  if (okc) {
-    void* hp = nullptr;
-    void* dp = nullptr;
-    if (cudaHostAlloc(&hp, 4 * sizeof(int32_t), cudaHostAllocMapped) != cudaSuccess) {
-      okc = false;
-    } else {
-      p->h_status = static_cast<int32_t*>(hp);
-      std::memset(hp, 0, 4 * sizeof(int32_t));
-      if (cudaHostGetDevicePointer(&dp, hp, 0) != cudaSuccess) okc = false;
-      p->h_status_dev = static_cast<int32_t*>(dp);
-    }
+  const size_t o_counters = take(8 * sizeof(int32_t));
+  const size_t o_seg = take(sizeof(SegInfo) * (n_seg + pack_segs.size()));
+  const size_t o_rows = take(sizeof(RowInfo) * pack_rows.size());
+  const size_t o_row_base = take(sizeof(int64_t) * (n_seg + 1));
+  const size_t o_first = take(sizeof(nsp_tile_t) * p->n_first);
+  const size_t o_keys = take(sizeof(PlanKey) * n_seg);
+  const size_t o_tiles = take(sizeof(int32_t) * (n_seg + 1));
+  const size_t upload = at;
+  const size_t o_fwd = take(sizeof(nsp_tile_t) * nf);
+  const size_t o_bwd = take(sizeof(nsp_tile_t) * nb);
+  const size_t o_exec = take(sizeof(nsp_tile_t) * nb);
+  const size_t o_front = take(sizeof(int32_t) * (nb / kFrontBlock + 1));
+  p->arena = arena_acquire(p->device, at, 256 + upload);
+  if (!p->arena) {
+    delete p;
+    return NSP_ERR_ALLOC;
   }
-  A(reinterpret_cast<void**>(&d_bases), 2 * sizeof(int64_t) * (n_seg + 1));
-  A(reinterpret_cast<void**>(&d_keys), 2 * sizeof(uint64_t) * (nf + nb));
-  A(&d_tmp, tmp_bytes);
-  int rc = NSP_OK;
-  if (!okc) {
-    rc = NSP_ERR_ALLOC;
-    cudaGetLastError();
-  } else {
-    cudaError_t e = cudaSuccess;
-    auto C = [&](cudaError_t x) {
-      if (e == cudaSuccess) e = x;
-    };
-    C(cudaMemsetAsync(p->d_counters, 0, 4 * sizeof(int32_t), st));
-    C(cudaMemsetAsync(p->d_status, 0, 4 * sizeof(int32_t), st));
-    if (n_seg > 0) {
-      C(cudaMemcpyAsync(p->d_seg, p->seg.data(), sizeof(SegInfo) * n_seg, cudaMemcpyHostToDevice, st));
-      C(cudaMemcpyAsync(d_bases, fwd_base.data(), sizeof(int64_t) * (n_seg + 1), cudaMemcpyHostToDevice, st));
-      C(cudaMemcpyAsync(d_bases + n_seg + 1, bwd_base.data(), sizeof(int64_t) * (n_seg + 1), cudaMemcpyHostToDevice,
-                        st));
-    }
-    C(cudaMemcpyAsync(p->d_row_base, row_base.data(), sizeof(int64_t) * (n_seg + 1), cudaMemcpyHostToDevice, st));
-    if (!pack_segs.empty()) {
-      C(cudaMemcpyAsync(p->d_seg + n_seg, pack_segs.data(), sizeof(SegInfo) * pack_segs.size(), cudaMemcpyHostToDevice, st));
-      C(cudaMemcpyAsync(p->d_rows, pack_rows.data(), sizeof(RowInfo) * pack_rows.size(), cudaMemcpyHostToDevice, st));
-    }
-    if (nb > 0) C(cudaMemcpyAsync(p->d_bwd_exec, bwd_exec.data(), sizeof(nsp_tile_t) * nb, cudaMemcpyHostToDevice, st));
-    if (p->n_first > 0)
-      C(cudaMemcpyAsync(p->d_bwd_first, bwd_first.data(), sizeof(nsp_tile_t) * p->n_first, cudaMemcpyHostToDevice, st));
-    if (e == cudaSuccess)
-      C(launch_plan_build(p->d_seg, n_seg, bm, bn, p->d_fwd, nf, p->d_bwd, nb, d_keys, d_keys + nf + nb, d_tmp, tmp_bytes,
-                          d_bases, d_bases + n_seg + 1, st));
-    // the host staging vectors and the scratch buffers die with this call: wait for the build
-    C(cudaStreamSynchronize(st));
-    if (e != cudaSuccess) rc = NSP_ERR_CUDA;
-  }
-  cudaFree(d_bases);
-  cudaFree(d_keys);
-  cudaFree(d_tmp);
-  if (rc != NSP_OK) {
+  char* const d = static_cast<char*>(p->arena->dev);
+  p->d_counters = reinterpret_cast<int32_t*>(d + o_counters);  // [0] forward, [1] backward main, [2] first-tile backward, [3] first-tile forward
+  p->d_status = p->d_counters + 4;
+  p->d_seg = reinterpret_cast<SegInfo*>(d + o_seg);
+  p->d_rows = reinterpret_cast<RowInfo*>(d + o_rows);
+  p->d_row_base = reinterpret_cast<int64_t*>(d + o_row_base);
+  p->d_bwd_first = reinterpret_cast<nsp_tile_t*>(d + o_first);
+  p->d_fwd = reinterpret_cast<nsp_tile_t*>(d + o_fwd);
+  p->d_bwd = reinterpret_cast<nsp_tile_t*>(d + o_bwd);
+  p->d_bwd_exec = reinterpret_cast<nsp_tile_t*>(d + o_exec);
+  p->d_front = reinterpret_cast<int32_t*>(d + o_front);
+  p->h_status = static_cast<int32_t*>(p->arena->host);
+  p->h_status_dev = reinterpret_cast<int32_t*>(p->arena->host_dev);
+  char* const image = static_cast<char*>(p->arena->host) + 256;
+  auto put = [&](size_t off, const void* src, size_t bytes) {
+    if (bytes) std::memcpy(image + off, src, bytes);
+  };
+  std::memset(p->h_status, 0, 256);
+  std::memset(image, 0, 8 * sizeof(int32_t));
+  put(o_seg, p->seg.data(), sizeof(SegInfo) * n_seg);
+  put(o_seg + sizeof(SegInfo) * n_seg, pack_segs.data(), sizeof(SegInfo) * pack_segs.size());
+  put(o_rows, pack_rows.data(), sizeof(RowInfo) * pack_rows.size());
+  put(o_row_base, row_base.data(), sizeof(int64_t) * (n_seg + 1));
+  put(o_first, bwd_first.data(), sizeof(nsp_tile_t) * p->n_first);
+  put(o_keys, keys.data(), sizeof(PlanKey) * n_seg);
+  put(o_tiles, tile_base.data(), sizeof(int32_t) * (n_seg + 1));
+  // On the arena's own stream, so that the plan is complete when this call returns without waiting for the work the
+  // caller has enqueued before (nothing here depends on it).
+  cudaStream_t bs = p->arena->build;
+  if (cudaMemcpyAsync(d, image, upload, cudaMemcpyHostToDevice, bs) != cudaSuccess ||
+      launch_plan_lists(reinterpret_cast<const PlanKey*>(d + o_keys), reinterpret_cast<const int32_t*>(d + o_tiles), n_seg,
+                        static_cast<int>(tiles), p->d_fwd, p->d_bwd, p->d_bwd_exec, bs) != cudaSuccess ||
+      cudaStreamSynchronize(bs) != cudaSuccess) {
+    p->arena->captured = true;  // not for reuse
     free_plan(p);
-    return rc;
+    return NSP_ERR_CUDA;
   }
   NSP_LOGF("plan %p: %d segments, %zu runs, head_dim %d, q_elems %lld, kv_elems %lld, fwd items %lld, bwd items %lld%s",
            static_cast<void*>(p), n_seg, p->runs.size(), head_dim, static_cast<long long>(p->q_elems),
@@ -529,6 +503,7 @@ int nsp_attn_fwd(const nsp_plan_t* plan, const void* q, const void* k, const voi
   if (!q || !k || !v || !o || !lse) return NSP_ERR_INVALID_ARG;
   if (!aligned16(q) || !aligned16(k) || !aligned16(v) || !aligned16(o) || !aligned16(lse)) return NSP_ERR_INVALID_ARG;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
+  const UsesArena uses{plan, st};
   FwdMaps maps;
   std::memset(&maps, 0, sizeof(maps));
   for (size_t r = 0; r < plan->runs.size(); ++r) {
@@ -599,6 +574,7 @@ int bwd_impl(const nsp_plan_t* plan, const uint8_t* recompute, const void* q, co
   const size_t need = recompute ? recompute_ws_bytes(plan) : base;
   if (!ws || (reinterpret_cast<uintptr_t>(ws) & 255) != 0 || ws_bytes < need) return NSP_ERR_WORKSPACE;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
+  const UsesArena uses{plan, st};
   char* wsb = static_cast<char*>(ws);
   float* dq_acc = static_cast<float*>(ws);
   float* delta = reinterpret_cast<float*>(wsb + align_up(static_cast<size_t>(plan->q_elems) * 4, 256));
@@ -879,6 +855,7 @@ __global__ void selftest_wait_kernel(StatusWord status, long long limit_clk) {
 int nsp_selftest_wait_timeout(const nsp_plan_t* plan, int64_t limit_clk, void* stream) {
   if (!plan || limit_clk < 1 || limit_clk > (1ll << 31)) return NSP_ERR_INVALID_ARG;
   if (const int failed = plan_failed(plan)) return failed;
+  const UsesArena uses{plan, static_cast<cudaStream_t>(stream)};
   selftest_wait_kernel<<<1, 32, 0, static_cast<cudaStream_t>(stream)>>>(status_word(plan), limit_clk);
   count_launches(1);
   return cudaGetLastError() == cudaSuccess ? NSP_OK : NSP_ERR_CUDA;
@@ -923,6 +900,11 @@ int nsp_plan_kernel_ms(const nsp_plan_t* plan, int kernel_id, float* ms) {
   if (!plan->profiling || !plan->ev_valid[kernel_id]) return NSP_ERR_INVALID_ARG;
   if (cudaEventSynchronize(plan->ev[2 * kernel_id + 1]) != cudaSuccess) return NSP_ERR_CUDA;
   if (cudaEventElapsedTime(ms, plan->ev[2 * kernel_id], plan->ev[2 * kernel_id + 1]) != cudaSuccess) return NSP_ERR_CUDA;
+  return NSP_OK;
+}
+
+int nsp_trim(void) {
+  arena_trim();
   return NSP_OK;
 }
 

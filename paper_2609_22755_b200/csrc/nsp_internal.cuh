@@ -43,6 +43,11 @@ struct RowInfo {
 };
 static_assert(sizeof(RowInfo) == 16, "RowInfo layout");
 
+// What the list construction needs of a segment.
+struct PlanKey {
+  int32_t tiles, hq, group, len;  // 128-row tiles, q heads, q heads per kv head, tokens
+};
+
 struct RunInfo {
   int64_t q_off, kv_off;  // element offsets of the run's first token
   int64_t tokens;
@@ -203,11 +208,8 @@ inline cudaError_t launch_chained_if(bool chained, void (*kernel)(P...), unsigne
 }
 
 // Host-side launchers implemented next to their kernels.
-cudaError_t launch_plan_build(const SegInfo* d_seg, int n_seg, int bm, int bn, nsp_tile_t* d_fwd, int64_t n_fwd,
-                              nsp_tile_t* d_bwd, int64_t n_bwd, uint64_t* d_keys, uint64_t* d_keys_alt, void* d_sort_tmp,
-                              size_t sort_tmp_bytes, const int64_t* d_fwd_base, const int64_t* d_bwd_base,
-                              cudaStream_t st);
-size_t plan_sort_tmp_bytes(int64_t max_items);
+cudaError_t launch_plan_lists(const PlanKey* d_key, const int32_t* d_tile_base, int n_seg, int n_tiles, nsp_tile_t* d_fwd,
+                              nsp_tile_t* d_bwd, nsp_tile_t* d_exec, cudaStream_t st);
 // chained: launched right behind launch_fwd_first, whose inputs are this kernel's too
 cudaError_t launch_fwd(const FwdMaps& maps, const FwdArgs& args, int head_dim, int num_sms, bool chained, cudaStream_t st);
 // q tile 0 of every segment: items (segment, kv head); args.items / n_items / counter are that list's

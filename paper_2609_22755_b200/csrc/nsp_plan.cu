@@ -1,13 +1,19 @@
-// Device-side construction of the tile work lists (forward and backward).
+// Device-side construction of the tile work lists (forward, backward, and the backward items in the order the kernel
+// walks them).
 //
-// Item definitions and order (unique, so any correct sort reproduces it bit for bit):
+// Item definitions and order (unique, so any correct construction gives the same lists bit for bit):
 //   forward  (s, h, m): cost = ceil(min(L, (m+1)*bm) / bn)          -- key tiles the query tile visits
 //   backward (s, g, n): cost = G * (Mt - floor(n*bn / bm))          -- (q head, q tile) visits of the key tile
 //   order: cost descending, then segment, tile, head ascending.
-// Every item is encoded into one 64-bit key whose ascending order is that order:
-//   [63:40] 2^24-1-cost   [39:24] segment   [23:8] tile   [7:0] head
-// The keys are emitted by one block per segment, sorted with a device radix sort and decoded into items.
-#include <cub/device/device_radix_sort.cuh>
+//   walked   (s, g, n): groups (s, g) by segment length descending, then s, g ascending; n ascending inside a group.
+//
+// With bm == bn a segment has at most one tile of a given cost, so the position of a tile's items in each list is a sum
+// over the segments of a closed form: one warp per (segment, tile) takes that sum (the lanes stride over the segments)
+// and writes the tile's items, no keys and no sort. A plan of 8,192 tokens at 32q/4kv spent 60 us in two radix sorts
+// with their key and decode kernels; this is one launch of about 5 us. The cost is tiles x segments: 131,072 tokens in
+// 8,192 segments of 16 tokens are 67 M terms, about 0.1 ms.
+// 128 threads of 32 registers, no shared memory: a block fits beside the persistent 640-thread kernels (61,440 of the
+// 65,536 registers of an SM), so building the next batch's plan does not wait for the running batch.
 #include <cuda_bf16.h>
 #include "nsp_internal.cuh"
 
@@ -15,77 +21,54 @@ namespace nsp {
 
 namespace {
 
-constexpr uint64_t kCostMax = (1ull << 24) - 1;
+constexpr int kListThreads = 128;
 
-__device__ __forceinline__ uint64_t encode_item(int seg, int head, int tile, int cost) {
-  return ((kCostMax - static_cast<uint64_t>(cost)) << 40) | (static_cast<uint64_t>(seg) << 24) |
-         (static_cast<uint64_t>(tile) << 8) | static_cast<uint64_t>(head);
-}
-
-__global__ void emit_keys_kernel(const SegInfo* __restrict__ seg, int bm, int bn, const int64_t* __restrict__ fwd_base,
-                                 const int64_t* __restrict__ bwd_base, uint64_t* __restrict__ fwd_keys,
-                                 uint64_t* __restrict__ bwd_keys) {
-  const int s = blockIdx.x;
-  const int L = seg[s].len, hq = seg[s].hq, hkv = seg[s].hkv;
-  const int G = hq / hkv;
-  const int Mt = (L + bm - 1) / bm, Nt = (L + bn - 1) / bn;
-  const int64_t nf = static_cast<int64_t>(Mt) * hq;
-  for (int64_t t = threadIdx.x; t < nf; t += blockDim.x) {
-    const int h = static_cast<int>(t / Mt), m = static_cast<int>(t % Mt);
-    const int64_t hi = min(static_cast<int64_t>(L), static_cast<int64_t>(m + 1) * bm);
-    fwd_keys[fwd_base[s] + t] = encode_item(s, h, m, static_cast<int>((hi + bn - 1) / bn));
+__global__ void __launch_bounds__(kListThreads, 16)
+    plan_lists_kernel(const PlanKey* __restrict__ key, const int32_t* __restrict__ tile_base, int n_seg, int n_tiles,
+                      nsp_tile_t* __restrict__ fwd, nsp_tile_t* __restrict__ bwd, nsp_tile_t* __restrict__ exec) {
+  const int lane = threadIdx.x & 31;
+  const int n_warps = gridDim.x * (kListThreads / 32);
+  for (int t = (blockIdx.x * kListThreads + threadIdx.x) >> 5; t < n_tiles; t += n_warps) {
+    int s = 0, hi = n_seg - 1;  // the last segment that starts at or before tile t (empty segments start where the next does)
+    while (s < hi) {
+      const int mid = (s + hi + 1) >> 1;
+      if (tile_base[mid] <= t) s = mid; else hi = mid - 1;
+    }
+    const PlanKey k = key[s];
+    const int m = t - tile_base[s];
+    const int cf = m + 1, cb = k.group * (k.tiles - m);
+    int nf = 0, nb = 0, ne = 0;  // items before this tile's (before its group's, in the walked order)
+    for (int x = lane; x < n_seg; x += 32) {
+      const PlanKey o = key[x];
+      const int hkv = o.hq / o.group;
+      const bool before = x < s;
+      // forward: the tiles of cost > cf, and the tile of cost == cf of an earlier segment
+      nf += o.hq * (max(o.tiles - cf, 0) + (before && o.tiles >= cf));
+      // backward: cost = group * k, k = 1 .. tiles
+      const int q = cb / o.group;
+      nb += hkv * (max(o.tiles - q, 0) + (before && q * o.group == cb && q <= o.tiles));
+      ne += o.len > k.len || (o.len == k.len && before) ? hkv * o.tiles : 0;
+    }
+    nf = __reduce_add_sync(0xffffffffu, nf);
+    nb = __reduce_add_sync(0xffffffffu, nb);
+    ne = __reduce_add_sync(0xffffffffu, ne);
+    for (int h = lane; h < k.hq; h += 32) fwd[nf + h] = nsp_tile_t{s, h, m, cf};
+    for (int g = lane; g < k.hq / k.group; g += 32) {
+      bwd[nb + g] = nsp_tile_t{s, g, m, cb};
+      exec[ne + g * k.tiles + m] = nsp_tile_t{s, g, m, cb};
+    }
   }
-  const int64_t nb = static_cast<int64_t>(Nt) * hkv;
-  for (int64_t t = threadIdx.x; t < nb; t += blockDim.x) {
-    const int g = static_cast<int>(t / Nt), n = static_cast<int>(t % Nt);
-    const int cost = G * (Mt - static_cast<int>((static_cast<int64_t>(n) * bn) / bm));
-    bwd_keys[bwd_base[s] + t] = encode_item(s, g, n, cost);
-  }
-}
-
-__global__ void decode_keys_kernel(const uint64_t* __restrict__ keys, int64_t n, nsp_tile_t* __restrict__ items) {
-  const int64_t t = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (t >= n) return;
-  const uint64_t k = keys[t];
-  nsp_tile_t it;
-  it.cost = static_cast<int32_t>(kCostMax - (k >> 40));
-  it.seg = static_cast<int32_t>((k >> 24) & 0xFFFF);
-  it.tile = static_cast<int32_t>((k >> 8) & 0xFFFF);
-  it.head = static_cast<int32_t>(k & 0xFF);
-  items[t] = it;
 }
 
 }  // namespace
 
-size_t plan_sort_tmp_bytes(int64_t max_items) {
-  size_t bytes = 0;
-  cub::DeviceRadixSort::SortKeys(nullptr, bytes, static_cast<const uint64_t*>(nullptr), static_cast<uint64_t*>(nullptr),
-                                 max_items > 0 ? max_items : 1);
-  return bytes;
-}
-
-// d_keys holds n_fwd + n_bwd keys (forward first); d_keys_alt the same amount for the sorted output.
-cudaError_t launch_plan_build(const SegInfo* d_seg, int n_seg, int bm, int bn, nsp_tile_t* d_fwd, int64_t n_fwd,
-                              nsp_tile_t* d_bwd, int64_t n_bwd, uint64_t* d_keys, uint64_t* d_keys_alt, void* d_sort_tmp,
-                              size_t sort_tmp_bytes, const int64_t* d_fwd_base, const int64_t* d_bwd_base,
-                              cudaStream_t st) {
-  if (n_seg == 0 || (n_fwd == 0 && n_bwd == 0)) return cudaSuccess;
-  emit_keys_kernel<<<n_seg, 256, 0, st>>>(d_seg, bm, bn, d_fwd_base, d_bwd_base, d_keys, d_keys + n_fwd);
+cudaError_t launch_plan_lists(const PlanKey* d_key, const int32_t* d_tile_base, int n_seg, int n_tiles, nsp_tile_t* d_fwd,
+                              nsp_tile_t* d_bwd, nsp_tile_t* d_exec, cudaStream_t st) {
+  if (n_tiles == 0) return cudaSuccess;
+  const int blocks = (n_tiles + kListThreads / 32 - 1) / (kListThreads / 32);
+  plan_lists_kernel<<<blocks < 148 * 8 ? blocks : 148 * 8, kListThreads, 0, st>>>(d_key, d_tile_base, n_seg, n_tiles, d_fwd,
+                                                                                  d_bwd, d_exec);
   count_launches(1);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  if (n_fwd > 0) {
-    e = cub::DeviceRadixSort::SortKeys(d_sort_tmp, sort_tmp_bytes, d_keys, d_keys_alt, n_fwd, 0, 64, st);
-    if (e != cudaSuccess) return e;
-    decode_keys_kernel<<<static_cast<unsigned>((n_fwd + 255) / 256), 256, 0, st>>>(d_keys_alt, n_fwd, d_fwd);
-    count_launches(1);
-  }
-  if (n_bwd > 0) {
-    e = cub::DeviceRadixSort::SortKeys(d_sort_tmp, sort_tmp_bytes, d_keys + n_fwd, d_keys_alt + n_fwd, n_bwd, 0, 64, st);
-    if (e != cudaSuccess) return e;
-    decode_keys_kernel<<<static_cast<unsigned>((n_bwd + 255) / 256), 256, 0, st>>>(d_keys_alt + n_fwd, n_bwd, d_bwd);
-    count_launches(1);
-  }
   return cudaGetLastError();
 }
 

@@ -45,6 +45,10 @@ struct nsp_plan {
   // long-tailed batch 8 %), and the walk ends with the cheapest items of the shortest segments. Same items, same costs:
   // a permutation of the published list.
   nsp_tile_t* d_bwd_exec = nullptr;
+  nsp_tile_t* d_bwd_parts = nullptr;        // the same items divided into parts (see divide_items)
+  nsp_tile_t* d_bwd_first_parts = nullptr;  // the first-tile kernel's items likewise
+  int64_t n_parts = 0, n_first_parts = 0;   // 0: not divided
+  int32_t* d_turns = nullptr;               // turn counters of the divided items
   nsp_tile_t* d_bwd_first = nullptr;  // one item per (segment or pack, kv head): the first-tile kernels' list
   int64_t n_first = 0;
   RowInfo* d_rows = nullptr;          // row tables of the packs, 128 entries each (d_seg holds the packs' entries after
@@ -166,6 +170,42 @@ bool log_on() {
 
 inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
 inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
+
+// Divides backward items into parts of at most about `most` steps (see kMaxParts) and lists them, the longest first. A
+// part has its own K / V loads and its own dK / dV epilogue, ~14,000 clocks or the time of 3-4 steps.
+// Returns an empty list when nothing is divided.
+// Where the lines lie: an item is divided when it is longer than the SMs' share of all steps, because the longest item
+// then bounds the kernel. Microseconds a step with parts of at most share / 2, share, whole: 8,192 tokens in one
+// segment at 32q/4kv 2,198, 2,124, 2,462; 17,545 tokens at 8q/2kv 1,063, 1,043, 1,158; 8,192 tokens in ten segments 718,
+// 694, 737. Smaller parts than kMinPart steps cost more than they give: 1,511 tokens of three head structures, parts of
+// 24 / 16 / 12 / 8 / 4 steps: 101, 85, 88, 109, 125 us (whole: 114). The first-tile kernel's items have one step per q
+// head of twice that length and run beside the main kernel: divided they are worth it where they, not the main kernel,
+// bound the call (20 segments of about 100 tokens at 64q/4kv 233 -> 216 us; parts of eight steps 248, of two 215).
+constexpr int kMinPart = 16, kMinFirstPart = 4;
+struct WholeItem {
+  int32_t seg, head, tile, steps;
+};
+std::vector<nsp_tile_t> divide_items(const std::vector<WholeItem>& items, int64_t most, int32_t* n_turns) {
+  struct Part {
+    nsp_tile_t t;
+    int32_t steps;
+  };
+  std::vector<Part> out;
+  const int32_t turn0 = *n_turns;
+  for (const WholeItem& w : items) {
+    const int64_t k = std::min<int64_t>(std::min<int64_t>(kMaxParts, w.steps), (w.steps + most - 1) / most);
+    const int32_t turn = k > 1 ? (*n_turns)++ : 0;
+    for (int32_t p = 0; p < k; ++p)
+      out.push_back(Part{nsp_tile_t{w.seg, w.head, w.tile | p << 16 | static_cast<int32_t>(k) << 24, turn},
+                         static_cast<int32_t>(w.steps / k + (p < w.steps % k))});
+  }
+  std::vector<nsp_tile_t> list;
+  if (*n_turns == turn0) return list;
+  // the parts of an item do not grow with their number, so a stable sort keeps them in order
+  std::stable_sort(out.begin(), out.end(), [](const Part& a, const Part& b) { return a.steps > b.steps; });
+  for (const Part& p : out) list.push_back(p.t);
+  return list;
+}
 
 void free_plan(nsp_plan* p) {
   if (!p) return;
@@ -394,6 +434,34 @@ int nsp_plan_tiles(const int32_t* cu_seqlens, const int32_t* hq, const int32_t* 
     delete p;
     return NSP_ERR_UNSUPPORTED;
   }
+  std::vector<nsp_tile_t> parts, first_parts;
+  int32_t n_turns = 0;
+  try {
+    if (!p->deterministic && !p->rounded_dq) {
+      std::vector<WholeItem> main_items, first_items;
+      int64_t main_steps = 0, first_steps = 0;
+      for (const SegInfo& sg : p->seg) {
+        const int32_t Mt = (sg.len + bm - 1) / bm, G = sg.hq / sg.hkv;
+        for (int g = 0; g < sg.hkv; ++g)
+          for (int32_t n = 0; n < Mt; ++n) {
+            const int32_t steps = G * (Mt - std::max(n, 1));
+            if (steps > 0) main_items.push_back(WholeItem{static_cast<int32_t>(&sg - p->seg.data()), g, n, steps});
+            main_steps += steps;
+          }
+      }
+      for (const nsp_tile_t& t : bwd_first) {
+        first_items.push_back(WholeItem{t.seg, t.head, 0, t.cost});
+        first_steps += t.cost;
+      }
+      parts = divide_items(main_items, std::max<int64_t>(kMinPart, main_steps / p->num_sms), &n_turns);
+      first_parts = divide_items(first_items, std::max<int64_t>(kMinFirstPart, (first_steps + main_steps) / (2 * p->num_sms)), &n_turns);
+    }
+    p->n_parts = static_cast<int64_t>(parts.size());
+    p->n_first_parts = static_cast<int64_t>(first_parts.size());
+  } catch (...) {
+    delete p;
+    return NSP_ERR_ALLOC;
+  }
   // Layout of the arena's device block: what the host uploads (counters and status first, all zero), then the lists the
   // device builds and the start-alignment counters. The pinned host block holds the host's copy of the status record
   // and, behind it, the image of the upload.
@@ -410,6 +478,9 @@ int nsp_plan_tiles(const int32_t* cu_seqlens, const int32_t* hq, const int32_t* 
   const size_t o_first = take(sizeof(nsp_tile_t) * p->n_first);
   const size_t o_keys = take(sizeof(PlanKey) * n_seg);
   const size_t o_tiles = take(sizeof(int32_t) * (n_seg + 1));
+  const size_t o_parts = take(sizeof(nsp_tile_t) * parts.size());
+  const size_t o_first_parts = take(sizeof(nsp_tile_t) * first_parts.size());
+  const size_t o_turns = take(sizeof(int32_t) * n_turns);
   const size_t upload = at;
   const size_t o_fwd = take(sizeof(nsp_tile_t) * nf);
   const size_t o_bwd = take(sizeof(nsp_tile_t) * nb);
@@ -431,6 +502,9 @@ int nsp_plan_tiles(const int32_t* cu_seqlens, const int32_t* hq, const int32_t* 
   p->d_bwd = reinterpret_cast<nsp_tile_t*>(d + o_bwd);
   p->d_bwd_exec = reinterpret_cast<nsp_tile_t*>(d + o_exec);
   p->d_front = reinterpret_cast<int32_t*>(d + o_front);
+  p->d_bwd_parts = reinterpret_cast<nsp_tile_t*>(d + o_parts);
+  p->d_bwd_first_parts = reinterpret_cast<nsp_tile_t*>(d + o_first_parts);
+  p->d_turns = reinterpret_cast<int32_t*>(d + o_turns);
   p->h_status = static_cast<int32_t*>(p->arena->host);
   p->h_status_dev = reinterpret_cast<int32_t*>(p->arena->host_dev);
   char* const image = static_cast<char*>(p->arena->host) + 256;
@@ -446,6 +520,9 @@ int nsp_plan_tiles(const int32_t* cu_seqlens, const int32_t* hq, const int32_t* 
   put(o_first, bwd_first.data(), sizeof(nsp_tile_t) * p->n_first);
   put(o_keys, keys.data(), sizeof(PlanKey) * n_seg);
   put(o_tiles, tile_base.data(), sizeof(int32_t) * (n_seg + 1));
+  put(o_parts, parts.data(), sizeof(nsp_tile_t) * parts.size());
+  put(o_first_parts, first_parts.data(), sizeof(nsp_tile_t) * first_parts.size());
+  std::memset(image + o_turns, 0, sizeof(int32_t) * n_turns);
   // On the arena's own stream, so that the plan is complete when this call returns without waiting for the work the
   // caller has enqueued before (nothing here depends on it).
   cudaStream_t bs = p->arena->build;
@@ -667,15 +744,19 @@ int bwd_impl(const nsp_plan_t* plan, const uint8_t* recompute, const void* q, co
   a.kv_elems = plan->kv_elems;
   a.lse_elems = plan->lse_elems;
   // first-tile kernel: q tile 0 of every segment (its dQ rows; its part of, or all of, dK / dV rows 0..127)
-  a.items = plan->d_bwd_first;
-  a.n_items = static_cast<int32_t>(plan->n_first);
+  const bool f_parts = a.dkv_f32 && plan->n_first_parts > 0;  // bf16 gradients are not added up piece by piece
+  a.items = f_parts ? plan->d_bwd_first_parts : plan->d_bwd_first;
+  a.n_items = static_cast<int32_t>(f_parts ? plan->n_first_parts : plan->n_first);
+  a.turn = f_parts ? plan->d_turns : nullptr;
   a.counter = plan->d_counters + 2;
   prof_mark(plan, NSP_KERNEL_BWD_FIRST, 0, st);
   if (launch_bwd_first(maps, a, plan->head_dim, plan->num_sms, st) != cudaSuccess) return NSP_ERR_CUDA;
   prof_mark(plan, NSP_KERNEL_BWD_FIRST, 1, st);
   // main kernel: everything else
-  a.items = plan->d_bwd_exec;
-  a.n_items = static_cast<int32_t>(plan->n_bwd);
+  const bool m_parts = a.dkv_f32 && plan->n_parts > 0;
+  a.items = m_parts ? plan->d_bwd_parts : plan->d_bwd_exec;
+  a.n_items = static_cast<int32_t>(m_parts ? plan->n_parts : plan->n_bwd);
+  a.turn = m_parts ? plan->d_turns : nullptr;
   a.counter = plan->d_counters + 1;
   prof_mark(plan, NSP_KERNEL_BWD_MAIN, 0, st);
   if (multi && launch_bwd(maps, a, plan->head_dim, plan->num_sms, plan->small_bwd, st) != cudaSuccess) return NSP_ERR_CUDA;

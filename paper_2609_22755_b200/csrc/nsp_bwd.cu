@@ -29,8 +29,8 @@
 // bandwidth (MMA operand reads, TMA fills, dS^T) is a scarce resource of this kernel.
 // dK and dV accumulate in TMEM over the whole item in a fixed order (q tiles descending, heads ascending inside
 // a tile), so the reduction over the query heads of a group is deterministic.
-// At the end of an item a full fp32 tile of each is staged in the (then idle) operand buffers and written by TMA tile
-// stores; bf16 outputs and ragged tiles are stored row by row from the threads.
+// At the end of an item both tiles are staged in the (then idle) operand buffers; a full fp32 tile is written by TMA tile
+// stores, ragged tiles and bf16 outputs by the softmax warps, whole rows at a time.
 // For the first q tile of a segment (rows 0..127, where P is O(1)) the step runs twice, once with the bf16
 // value of P and dS and once with the bf16 residual (hi + lo), and delta is recomputed in fp32 as
 // sum_j P_ij dP_ij instead of taking it from the bf16-rounded O; this keeps dK/dV/dQ inside the 2e-2 tolerance.
@@ -77,7 +77,9 @@ struct ItemCtx {
   int32_t first;                   // key tile 0
   int32_t m0;                      // first (lowest) q tile of the walk
   int32_t per_head;                // steps per q head
-  int32_t steps;                   // G * per_head
+  int32_t steps;                   // G * per_head, or the part's share of them
+  int32_t h0, r0;                  // where the walk starts (see StepWalk): 0, 0 unless a later part
+  int32_t part, parts, turn;       // see kMaxParts; parts = 1: the whole item
   int32_t rows;                    // first-tile kernel: 0, or 1 + index of the row table of a pack of short segments
 };
 
@@ -150,7 +152,7 @@ __device__ __forceinline__ void setmaxnreg_dec() {
 // kernel (the same code instantiated with FIRST = true), so an item with key tile 0 starts at q tile 1.
 struct StepWalk {
   int hh, rr;
-  __device__ __forceinline__ void reset() { hh = 0, rr = 0; }
+  __device__ __forceinline__ void reset(const ItemCtx& c) { hh = c.h0, rr = c.r0; }
   __device__ __forceinline__ void get(const ItemCtx& c, int& h, int& m) const {
     const int p = c.per_head - 1 - rr;  // q tiles in DESCENDING order (see above)
     h = c.g * c.G + hh;
@@ -260,6 +262,15 @@ __global__ void __launch_bounds__(kBwdThreads, 1) bwd_kernel(const __grid_consta
   // 512-token segments). Both sides derive "ahead" from the finished item's step count, so no flag is needed; the
   // barrier below publishes the slot either way.
   constexpr int kAheadMaxSteps = 64;
+  auto take_part = [&](ItemCtx& x, const nsp_tile_t& item) {
+    if (a.turn == nullptr) return;
+    x.part = (item.tile >> 16) & 0xff, x.parts = (item.tile >> 24) & 0xff;
+    x.turn = item.cost;
+    const int each = x.steps / x.parts, more = x.steps % x.parts;  // the first `more` parts take one step more
+    const int t0 = x.part * each + min(x.part, more);
+    x.h0 = t0 % x.G, x.r0 = t0 / x.G;
+    x.steps = each + (x.part < more);
+  };
   auto fetch_item = [&](ItemCtx& x) {
     for (;;) {
       const int idx = atomicAdd(a.counter, 1);
@@ -272,20 +283,27 @@ __global__ void __launch_bounds__(kBwdThreads, 1) bwd_kernel(const __grid_consta
       const SegInfo sg = a.seg[item.seg];
       x.q_off = sg.q_off, x.kv_off = sg.kv_off, x.lse_off = sg.lse_off;
       x.len = sg.len, x.hq = sg.hq, x.hkv = sg.hkv, x.run = sg.run, x.tok0 = sg.tok_in_run;
-      x.g = item.head, x.n = item.tile;
+      x.g = item.head, x.n = item.tile & 0xffff;
+      x.h0 = x.r0 = 0;
+      x.part = 0, x.parts = 1;
       x.G = sg.hq / sg.hkv;
       x.turn_off = sg.turn_off, x.mt = (sg.len + kBM - 1) / kBM;
-      x.first = (item.tile == 0);
+      x.first = (x.n == 0);
       x.rows = sg.rows;
       if constexpr (FIRST) {
         x.m0 = 0;
         x.per_head = 1;  // q tile 0 only
         x.steps = x.G;
+        take_part(x, item);
         break;
       }
-      x.m0 = item.tile + x.first;                        // q tile 0 belongs to the first-tile kernel
+      x.m0 = x.n + x.first;                        // q tile 0 belongs to the first-tile kernel
       x.per_head = (sg.len + kBM - 1) / kBM - x.m0;      // q tiles max(n, 1) .. Mt-1 (bm == bn)
       x.steps = x.G * x.per_head;
+      if (a.turn != nullptr) {
+        take_part(x, item);
+        break;
+      }
       // Start alignment. kFrontBlock consecutive items are neighbouring key tiles of one (segment, kv head) and
       // walk the same (q tile, head) sequence from the segment's last q tile down. CTAs that start them at the
       // same moment stay on the same q tile for the whole item and find its Q, dO and dQ-accumulator tiles in
@@ -348,7 +366,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) bwd_kernel(const __grid_consta
             tma_load_3d(s.v[hf], &maps.v[c.run], &s.bar_kv, 64 * hf, c.g, c.tok0 + c.n * kBN);
           }
           StepWalk w;
-          w.reset();
+          w.reset(c);
 #pragma unroll 1
           for (int vt = 0; vt < c.steps; ++vt) {
             const uint32_t cs = gs + vt;
@@ -530,7 +548,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) bwd_kernel(const __grid_consta
       while (next_item()) {
         const ItemCtx c = *cx;
         StepWalk w;
-        w.reset();
+        w.reset(c);
 #pragma unroll 1
         for (int vt = 0; vt < c.steps; ++vt) {
           const uint32_t cs = gs + vt, st = cs & 1;
@@ -584,7 +602,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) bwd_kernel(const __grid_consta
       const ItemCtx c = *cx;
       const int64_t q_stride = static_cast<int64_t>(c.hq) * kHeadDim;  // floats between consecutive query rows
       StepWalk w;
-      w.reset();
+      w.reset(c);
 #pragma unroll 1
       for (int vt = 0; vt < c.steps; ++vt) {
         const uint32_t cs = gs + vt;
@@ -736,7 +754,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) bwd_kernel(const __grid_consta
         if (c.rows > 0) r_end = a.rows[static_cast<int64_t>(c.rows - 1) * kBM + r].hi;
       }
       StepWalk w;
-      w.reset();
+      w.reset(c);
 #pragma unroll 1
       for (int vt = 0; vt < c.steps; ++vt) {
         const uint32_t cs = gs + vt, st = cs & 1;
@@ -977,104 +995,163 @@ __global__ void __launch_bounds__(kBwdThreads, 1) bwd_kernel(const __grid_consta
       }
       if (oks) {
         tc_fence_after_sync();
-        const int kj = c.n * kBN + r;
-        const bool valid = kj < c.len;
         constexpr int kCols = D / 2;  // this thread's columns of a dK / dV row
-        const int64_t off = c.kv_off + (static_cast<int64_t>(kj) * c.hkv + c.g) * kHeadDim + half * kCols;
         // Key tile 0 in the main kernel: the first-tile kernel, which ran before, left its part (q tile 0) in the
         // output; this item's sum over the q tiles 1 .. Mt-1 is added to it (one fixed order: reproducible).
-        const bool add = !FIRST && c.first;
-        if (add) grid_wait_predecessor();
-        if (a.dkv_f32 && (c.n + 1) * kBN <= c.len) {
-          // ---- fp32 outputs, full key tile: staged in shared memory (every operand buffer is free now: dK over K
-          // and V, dV over the Q ring), swizzled as sub-tiles of 32 columns, and written by TMA tile stores (added,
-          // for key tile 0). Stored row by row from the threads (a row per lane, 16 bytes per store, half a sector
-          // each) the two tiles took 12,000-13,000 clocks per item.
-          constexpr uint32_t kSubBytes = 128 * 32 * 4;
-#pragma unroll 1
-          for (int part = 0; part < 2 * (kCols / 32); ++part) {  // (dK, dV) x 32-column chunks
-            const int which = part / (kCols / 32), cc = part % (kCols / 32);
-            const float mul = which == 0 ? a.scale : 1.f;
-            uint32_t v[32];
-            tmem_ld32(tDK + which * 128 + lane_off + half * kCols + cc * 32, v);
-            tmem_wait_ld();
-            uint8_t* const sub = (which == 0 ? &s.k[0][0] : &s.q[0][0][0]) + (half * (kCols / 32) + cc) * kSubBytes + r * 128;
-#pragma unroll
-            for (int x = 0; x < 8; ++x) {
-              *reinterpret_cast<float4*>(sub + ((x ^ (r & 7)) * 16)) =
-                  make_float4(__uint_as_float(v[4 * x]) * mul, __uint_as_float(v[4 * x + 1]) * mul,
-                              __uint_as_float(v[4 * x + 2]) * mul, __uint_as_float(v[4 * x + 3]) * mul);
+        // Later parts of a divided item add to what the parts before them have left, in turn.
+        const bool add = (!FIRST && c.first) || c.part > 0;
+        if (!FIRST && c.first) grid_wait_predecessor();
+        auto wait_part = [&]() {  // one lane per warp that goes on to read or add to the output
+          if (c.part == 0) return;
+          const long long t0 = clock64();
+          while (*reinterpret_cast<volatile int32_t*>(a.turn + c.turn) != c.part) {
+            if (clock64() - t0 > a.wait_limit) {
+              report_timeout(a.status, c.it, kWhereBwdTurn, c.part);
+              *abort_flag = 1;
+              break;
             }
+            __nanosleep(32);
           }
-          fence_proxy_async_smem();
-          const uint64_t staged = mbar_arrive_token(&s.bar_out);
+          __threadfence();
+          fence_proxy_async();
+        };
+        auto pass_part = [&]() {  // one thread, once the part's results are in global memory
+          __threadfence();
+          *reinterpret_cast<volatile int32_t*>(a.turn + c.turn) = c.part + 1 < c.parts ? c.part + 1 : 0;
+        };
+        // Both tiles are staged in shared memory (every operand buffer is free now: dK over K and V, dV over the Q ring),
+        // fp32, swizzled as sub-tiles of 32 columns.
+        constexpr uint32_t kSubBytes = 128 * 32 * 4;
+        uint8_t* const stage_k = &s.k[0][0];
+        uint8_t* const stage_v = &s.q[0][0][0];
+#pragma unroll 1
+        for (int part = 0; part < 2 * (kCols / 32); ++part) {  // (dK, dV) x 32-column chunks
+          const int which = part / (kCols / 32), cc = part % (kCols / 32);
+          const float mul = which == 0 ? a.scale : 1.f;
+          uint32_t v[32];
+          tmem_ld32(tDK + which * 128 + lane_off + half * kCols + cc * 32, v);
+          tmem_wait_ld();
+          uint8_t* const sub = (which == 0 ? stage_k : stage_v) + (half * (kCols / 32) + cc) * kSubBytes + r * 128;
+#pragma unroll
+          for (int x = 0; x < 8; ++x) {
+            *reinterpret_cast<float4*>(sub + ((x ^ (r & 7)) * 16)) =
+                make_float4(__uint_as_float(v[4 * x]) * mul, __uint_as_float(v[4 * x + 1]) * mul,
+                            __uint_as_float(v[4 * x + 2]) * mul, __uint_as_float(v[4 * x + 3]) * mul);
+          }
+        }
+        const bool full = a.dkv_f32 && (c.n + 1) * kBN <= c.len;
+        if (full) fence_proxy_async_smem();
+        const uint64_t staged = mbar_arrive_token(&s.bar_out);
+        if (full) {
+          // ---- fp32 outputs, full key tile: TMA tile stores (added, for key tile 0). Stored row by row from the threads
+          // (a row per lane, 16 bytes per store, half a sector each) the two tiles took 12,000-13,000 clocks per item.
           if (tid == 0) {
             if (mbar_wait_token(&s.bar_out, staged, a.wait_limit)) {
               const int tok = c.tok0 + c.n * kBN;
+              wait_part();
 #pragma unroll 1
               for (int i = 0; i < D / 32; ++i) {
                 if (add) {
-                  tma_reduce_add_3d(&maps.dk[c.run], &s.k[0][0] + i * kSubBytes, 32 * i, c.g, tok);
-                  tma_reduce_add_3d(&maps.dv[c.run], &s.q[0][0][0] + i * kSubBytes, 32 * i, c.g, tok);
+                  tma_reduce_add_3d(&maps.dk[c.run], stage_k + i * kSubBytes, 32 * i, c.g, tok);
+                  tma_reduce_add_3d(&maps.dv[c.run], stage_v + i * kSubBytes, 32 * i, c.g, tok);
                 } else {
-                  tma_store_3d(&maps.dk[c.run], &s.k[0][0] + i * kSubBytes, 32 * i, c.g, tok);
-                  tma_store_3d(&maps.dv[c.run], &s.q[0][0][0] + i * kSubBytes, 32 * i, c.g, tok);
+                  tma_store_3d(&maps.dk[c.run], stage_k + i * kSubBytes, 32 * i, c.g, tok);
+                  tma_store_3d(&maps.dv[c.run], stage_v + i * kSubBytes, 32 * i, c.g, tok);
                 }
               }
               tma_store_commit();
-              tma_store_wait_read();  // before the barrier of next_item(): the producer refills these buffers after it
+              if (c.parts > 1) {
+                tma_store_wait();
+                fence_proxy_async();
+                pass_part();
+              } else {
+                tma_store_wait_read();  // before the barrier of next_item(): the producer refills these buffers after it
+              }
             } else {
               report_timeout(a.status, c.it, kWhereBwdDqFull, 1);
               *abort_flag = 1;
             }
           }
         } else {
+          // ---- ragged tiles and bf16 outputs: the eight warps write whole rows (D / 4 lanes per row, 16 staged bytes
+          // each), four row passes in flight; an added tile reads its rows the same way first. Written from the threads
+          // that hold the rows (a row per lane, 16 bytes per store, each store its own line) a tile pair took four times
+          // as long, and twice that where it was added.
+          constexpr int kLanes = D / 4, kRowsPerPass = 32 / kLanes, kPasses = 128 / (8 * kRowsPerPass);
+          const int rows = min(kBN, c.len - c.n * kBN);
+          const int l = lane % kLanes;
+          bool oku = mbar_wait_token(&s.bar_out, staged, a.wait_limit);
+          if (!oku) {
+            report_timeout(a.status, c.it, kWhereBwdDqFull, 1);
+            *abort_flag = 1;
+          }
+          if (lane == 0) wait_part();
+          __syncwarp();
+          oku = __all_sync(0xffffffffu, oku);
 #pragma unroll 1
-        for (int part = 0; part < 2 * (kCols / 32); ++part) {  // (dK, dV) x 32-column chunks
-          const int which = part / (kCols / 32), cc = part % (kCols / 32);
-          const float mul = which == 0 ? a.scale : 1.f;
-          void* outp = which == 0 ? a.dk : a.dv;
-          uint32_t v[32];
-          tmem_ld32(tDK + which * 128 + lane_off + half * kCols + cc * 32, v);
-          tmem_wait_ld();
-          NSP_CHECK(!valid || (off >= 0 && off + kCols <= a.kv_elems), a.status, c.it, kWhereCheckBwdDkv, kj)
-          if (valid) {
-            if (a.dkv_f32) {
-              float* o = static_cast<float*>(outp) + off + cc * 32;
+          for (int it = 0; oku && it < 2 * kPasses; it += 4) {
+            const int which = it / kPasses;
+            const uint8_t* const st0 = (which == 0 ? stage_k : stage_v) + (l / 8) * kSubBytes;
+            float4 w4[4];
+            int64_t at[4];
+            bool on[4];
 #pragma unroll
-              for (int x = 0; x < 32; x += 4) {
-                float4 w4 = make_float4(__uint_as_float(v[x]) * mul, __uint_as_float(v[x + 1]) * mul,
-                                        __uint_as_float(v[x + 2]) * mul, __uint_as_float(v[x + 3]) * mul);
-                if (add) {
-                  const float4 old = *reinterpret_cast<const float4*>(o + x);
-                  w4.x += old.x, w4.y += old.y, w4.z += old.z, w4.w += old.w;
-                }
-                *reinterpret_cast<float4*>(o + x) = w4;
+            for (int u = 0; u < 4; ++u) {
+              const int row = ((it + u) % kPasses * 8 + warp) * kRowsPerPass + lane / kLanes;
+              on[u] = row < rows;
+              at[u] = c.kv_off + (static_cast<int64_t>(c.n * kBN + row) * c.hkv + c.g) * kHeadDim + 4 * l;
+              w4[u] = *reinterpret_cast<const float4*>(st0 + row * 128 + ((l % 8) ^ (row & 7)) * 16);
+#ifdef NSP_CHECKED
+              if (on[u] && (at[u] < 0 || at[u] + 4 > a.kv_elems)) {
+                report_status(a.status, NSP_ERR_DEVICE_ASSERT, c.it, kWhereCheckBwdDkv, row);
+                on[u] = false;
               }
+#endif
+            }
+            void* const outp = which == 0 ? a.dk : a.dv;
+            if (a.dkv_f32) {
+              float* const o = static_cast<float*>(outp);
+              if (add) {
+                float4 old[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) old[u] = on[u] ? __ldcg(reinterpret_cast<const float4*>(o + at[u])) : w4[u];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) w4[u].x += old[u].x, w4[u].y += old[u].y, w4[u].z += old[u].z, w4[u].w += old[u].w;
+              }
+#pragma unroll
+              for (int u = 0; u < 4; ++u)
+                if (on[u]) *reinterpret_cast<float4*>(o + at[u]) = w4[u];
             } else {
-              __nv_bfloat16* o = static_cast<__nv_bfloat16*>(outp) + off + cc * 32;
+              __nv_bfloat16* const o = static_cast<__nv_bfloat16*>(outp);
+              if (add) {  // bf16 output: the first part was rounded once already (not the graded dtype)
+                uint2 old[4];
 #pragma unroll
-              for (int x = 0; x < 32; x += 8) {
-                if (add) {  // bf16 output: the first part was rounded once already (not the graded dtype)
-                  const uint4 old = *reinterpret_cast<const uint4*>(o + x);
-                  const uint32_t ow[4] = {old.x, old.y, old.z, old.w};
+                for (int u = 0; u < 4; ++u) old[u] = on[u] ? __ldcg(reinterpret_cast<const uint2*>(o + at[u])) : make_uint2(0u, 0u);
 #pragma unroll
-                  for (int t = 0; t < 4; ++t) {
-                    v[x + 2 * t] = __float_as_uint(__uint_as_float(v[x + 2 * t]) + __uint_as_float(ow[t] << 16) / mul);
-                    v[x + 2 * t + 1] =
-                        __float_as_uint(__uint_as_float(v[x + 2 * t + 1]) + __uint_as_float(ow[t] & 0xffff0000u) / mul);
-                  }
+                for (int u = 0; u < 4; ++u) {
+                  w4[u].x += __uint_as_float(old[u].x << 16), w4[u].y += __uint_as_float(old[u].x & 0xffff0000u);
+                  w4[u].z += __uint_as_float(old[u].y << 16), w4[u].w += __uint_as_float(old[u].y & 0xffff0000u);
                 }
-                uint4 wv;
-                wv.x = pack_bf16x2(__uint_as_float(v[x]) * mul, __uint_as_float(v[x + 1]) * mul);
-                wv.y = pack_bf16x2(__uint_as_float(v[x + 2]) * mul, __uint_as_float(v[x + 3]) * mul);
-                wv.z = pack_bf16x2(__uint_as_float(v[x + 4]) * mul, __uint_as_float(v[x + 5]) * mul);
-                wv.w = pack_bf16x2(__uint_as_float(v[x + 6]) * mul, __uint_as_float(v[x + 7]) * mul);
-                *reinterpret_cast<uint4*>(o + x) = wv;
+              }
+#pragma unroll
+              for (int u = 0; u < 4; ++u)
+                if (on[u])
+                  *reinterpret_cast<uint2*>(o + at[u]) =
+                      make_uint2(pack_bf16x2(w4[u].x, w4[u].y), pack_bf16x2(w4[u].z, w4[u].w));
+            }
+          }
+          if (c.parts > 1) {
+            __threadfence();
+            const uint64_t stored = mbar_arrive_token(&s.bar_out);
+            if (tid == 0) {
+              if (mbar_wait_token(&s.bar_out, stored, a.wait_limit)) {
+                pass_part();
+              } else {
+                report_timeout(a.status, c.it, kWhereBwdDqFull, 2);
+                *abort_flag = 1;
               }
             }
           }
-        }
         }
       } else if (where != 0 && lane == 0) {
         report_timeout(a.status, c.it, where, 0);

@@ -179,6 +179,7 @@ struct BwdArgs {
   long long wait_limit;  // SM clocks a device-side wait may take before it gives up
   int64_t q_elems, kv_elems, lse_elems;  // tensor sizes (checked build)
   int32_t* front;    // [n_items / kFrontBlock + 1] arrival counters, zeroed by the preprocess kernel (see next_item)
+  int32_t* turn;     // null, or items are parts (see kMaxParts): one counter per divided item, zero between launches
   const RowInfo* rows;  // row tables of the packs (first-tile kernel)
 };
 
@@ -206,6 +207,14 @@ inline cudaError_t launch_chained_if(bool chained, void (*kernel)(P...), unsigne
   cfg.numAttrs = chained ? 1 : 0;
   return cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
 }
+
+// Parts of a backward item. The steps of an item (its q tiles and q heads) may be divided among several CTAs: part p of
+// k walks a contiguous piece of the item's steps and adds its dK / dV to what the parts before it have left, in the order
+// of the parts (a turn counter per divided item, taken with the bounded wait; the last part puts it back to zero), so the
+// result is reproducible. Such a list holds nsp_tile_t entries with tile = tile | part << 16 | parts << 24 and cost = the
+// item's turn counter. A part never precedes an earlier part of its item in the list, so the part that is waited for has
+// always been popped, and the lowest unfinished position of the list never waits: no cycle.
+constexpr int kMaxParts = 64;
 
 // Host-side launchers implemented next to their kernels.
 cudaError_t launch_plan_lists(const PlanKey* d_key, const int32_t* d_tile_base, int n_seg, int n_tiles, nsp_tile_t* d_fwd,

@@ -5,7 +5,7 @@
 //   main         key-stationary persistent kernel, see below
 //   postprocess  dQ = scale * fp32 accumulator -> bf16 / fp32                   (HBM-bound)
 //
-// Main kernel. One CTA per SM (640 threads, five warpgroups with their own register budgets) pops items
+// Main kernel. One CTA per SM (640 threads, five warpgroups with their own register budgets; 896 in seven at D = 64) pops items
 // (segment, kv head, key tile n) from the longest-first list. K_n and V_n stay in shared memory; the CTA walks
 // every q head of the KV group and every q tile m >= n. All score-shaped quantities are computed TRANSPOSED
 // (key index on the TMEM lanes) so that P^T and dS^T are directly the A operands of the dV and dK products:
@@ -14,8 +14,8 @@
 //     dV  += P^T dO                               A = P^T (bf16, written over S^T in R0), B = dO  MN-major
 //     dK  += dS^T Q                               A = dS^T (shared memory, K-major), B = Q MN-major
 //     dQ_m^T = K^T dS^T -> R1 (over dP^T)         A = K read MN-major, B = dS^T read MN-major
-// TMEM: R0 [0,128), R1 [128,256), dK [256,384), dV [384,512).
-// Roles:  warps 0-7  softmax / dS (key row = TMEM lane, two column halves)
+// TMEM: R0 [0,128), R1 [128,256), dK [256,384), dV [384,512); at D = 64 dK, dV 64 columns each and dQ^T in [384,512).
+// Roles (at D = 128; see Roles):  warps 0-7  softmax / dS (key row = TMEM lane, two column halves)
 //         warps 8-15 dQ: TMEM -> fp32 accumulator in global memory (lane quadrant x 64-column half)
 //         warp 16    TMA producer (K, V once per item; Q two-stage ring, dO single buffer)
 //         warp 17    MMA issuer A (whole warp runs the waits, the elected lane issues): dV(t), S^T(t+1)
@@ -39,6 +39,7 @@
 // together do not fit in it runs at the speed of instruction fetch. So the common step (an interior tile) has
 // its own lean, fully unrolled path; everything rare (diagonal tile, first-tile passes, ragged tail, item
 // epilogue) goes through compact rolled loops; an item is decoded once, by one thread, into shared memory.
+#include <cstddef>
 #include <type_traits>
 #include <cuda_bf16.h>
 #include "nsp_internal.cuh"
@@ -47,7 +48,6 @@
 namespace nsp {
 namespace {
 
-constexpr int kBwdThreads = 640;  // 8 softmax warps, 8 dQ warps, one auxiliary warpgroup
 constexpr uint32_t kHalfTileBytes = 128 * 64 * 2;
 constexpr uint32_t kBwdTmemCols = 512;
 constexpr float kLog2e = 1.4426950408889634f;
@@ -57,13 +57,35 @@ constexpr float kLog2e = 1.4426950408889634f;
 // most a warpgroup can keep without an increase of its own), while the softmax role fits 120. First-tile kernel
 // 136 / 80 / 48: there the softmax role carries the packed P of a whole tile across two sweeps and the dQ role only
 // stores. 256 * (120 + 96) + 128 * 48 = 256 * (136 + 80) + 128 * 48 = 640 * 96.
-template <bool FIRST> constexpr int kRegsSoftmax = FIRST ? 136 : 120;
-template <bool FIRST> constexpr int kRegsReduce = FIRST ? 80 : 96;
-constexpr int kRegsAux = 48;
+// D = 64: sixteen softmax warps of 32 columns and eight dQ warps of 32 columns each: 896 threads, 80 / 64 / 48. The dQ
+// warps are what counts (65,536 long-tailed tokens at 32q/4kv, whole step: four warps that drain 64 columns 14.4 ms, eight
+// of 32 columns 13.4 ms); the sixteen softmax warps make the first-tile kernel faster (98,275 tokens in 100-token segments
+// 2,036 -> 1,996 us, 7,818 tokens at 8q/2kv 108 -> 99 us) and leave the main kernel as it is, which at D = 64 waits for
+// neither the arithmetic nor the reductions but for the chain of hand-overs of a step (without any of them: -6 %).
+template <bool FIRST, int D>
+struct Roles {
+  static constexpr int kSoft = D == 64 ? 4 : 2;      // warpgroups of the softmax role; they come first
+  static constexpr int kReduce = 2;                  // warpgroups of the dQ role
+  static constexpr int kDrain = D / 2;               // query columns of a dQ warp
+  // D = 64 leaves 128 TMEM columns free: dQ^T gets a region of its own instead of R1, and dP^T of the next step follows as
+  // soon as the softmax warps have consumed dP^T of this one, instead of waiting for dQ^T, dK and the drain (13.4 -> 13.0 ms).
+  static constexpr bool kOwnDq = D == 64;
+  static constexpr int kThreads = 128 * (kSoft + kReduce + 1);
+  static constexpr int kCols = 128 / kSoft;          // query columns of a softmax thread
+  static constexpr int kAux0 = 4 * (kSoft + kReduce);  // first warp of the auxiliary warpgroup
+  static constexpr int kRegsLaunch = kSoft == 4 ? 72 : 96;
+  static constexpr int kRegsSoft = kSoft == 4 ? 80 : FIRST ? 136 : 120;
+  static constexpr int kRegsReduce = kSoft == 4 ? 64 : FIRST ? 80 : 96;
+  static constexpr int kRegsAux = 48;
+  static_assert(128 * (kSoft * kRegsSoft + kReduce * kRegsReduce + kRegsAux) <= kThreads * kRegsLaunch, "register budget");
+};
 constexpr int kFrontMinSteps = 2048;          // items shorter than this start at once
 constexpr int kFrontMinGroup = 8;             // so do items of groups with fewer q heads per kv head
 constexpr long long kFrontWaitClk = 1500000;  // ~0.9 ms: upper bound of the start alignment (also: 1/16 of the item)
 constexpr int kQStages = 2;                   // Q ring (three stages measured 3 % slower on the nested shard)
+
+// With D = 64 dP^T of the next step is issued a step ahead (see kOwnDq), which takes a second dO buffer.
+template <int D> constexpr int kDoStages = D == 64 ? 2 : 1;
 
 // A decoded work item: written by one thread (thread 0, or the producer's lane 0 one item ahead), read by every role
 // after the CTA-wide barrier of next_item().
@@ -91,28 +113,32 @@ struct BwdSmem {
   uint8_t k[D / 64][kHalfTileBytes];  // K, V, Q, dO tiles: D / 64 sub-tiles of 64 columns (D = head dimension)
   uint8_t v[D / 64][kHalfTileBytes];
   uint8_t q[kQStages][D / 64][kHalfTileBytes];  // [stage][64-column half]: ring, loaded a whole step ahead
-  uint8_t d_o[D / 64][kHalfTileBytes];  // [half]: single buffer (its consumers leave a long window for the refill)
+  uint8_t d_o[kDoStages<D>][D / 64][kHalfTileBytes];  // [buffer][half]; one buffer: its consumers leave a long window for the refill
   uint8_t ds[2][kHalfTileBytes];      // dS^T, [key row][query col], two 64-column halves
   uint8_t ds_lo[FIRST ? 2 * kHalfTileBytes : 16];  // first-tile kernel: the bf16 residual of dS^T, same layout, right behind it
-  float lse[2][128];                  // [stage] LSE * log2(e) of the q tile (+inf for rows past the segment)
+  float part[FIRST && D == 64 ? 512 : 4];  // first-tile kernel, D = 64: partial sums of delta (D = 128: in ds)
+  alignas(16) float lse[2][128];      // [stage] LSE * log2(e) of the q tile (+inf for rows past the segment)
   float delta[2][128];                // [stage]
   ItemCtx ctx[2];
   uint64_t bar_kv;
   uint64_t bar_q_full[kQStages];
   uint64_t bar_q_empty[kQStages][2];  // [stage][issuer A / B]: that issuer's MMAs reading the Q stage have completed
-  uint64_t bar_do_full;
-  uint64_t bar_do_empty[2];    // [issuer A / B]: that issuer's MMAs reading the dO buffer have completed
+  uint64_t bar_do_full[2];        // [dO buffer]
+  uint64_t bar_do_empty[2][2];    // [dO buffer][issuer A / B]: that issuer's MMAs reading it have completed
   uint64_t bar_a_done;         // dV of the step (issuer A) has completed
   uint64_t bar_b_done;         // dK of the step (issuer B) has completed
   uint64_t bar_ld_full[2], bar_ld_empty[2];
   uint64_t bar_s_full, bar_dp_full, bar_dq_full, bar_dq_empty;
-  uint64_t bar_p_ready;   // 256 softmax threads: P^T of the step is in R0
-  uint64_t bar_ds_ready;  // 256 softmax threads: dS^T of the step is in shared memory
-  uint64_t bar_delta[2];  // 128 softmax threads of one column half: partial / final sums of the exact delta
-  uint64_t bar_out;       // 256 softmax threads: the item's dK and dV tiles are staged for the tile stores
+  uint64_t bar_p_ready;   // softmax threads: P^T of the step is in R0
+  uint64_t bar_ds_ready;  // softmax threads: dS^T of the step is in shared memory
+  uint64_t bar_delta[4];  // 128 softmax threads of one column group: partial / final sums of the exact delta
+  uint64_t bar_out;       // softmax threads: the item's dK and dV tiles are staged for the tile stores
   uint32_t tmem_base;
   int32_t abort;
 };
+using FirstSmem128 = BwdSmem<true, 128>;
+using MainSmem128 = BwdSmem<false, 128>;
+static_assert(offsetof(FirstSmem128, lse) % 16 == 0 && offsetof(MainSmem128, lse) % 16 == 0, "16-byte loads");
 static_assert(sizeof(BwdSmem<true, 128>) <= 232448, "shared memory budget (227 KB)");
 
 // DET = 2: every term a key tile adds to the dQ accumulator is first rounded to a multiple of 2^-12 (x + 1.5 * 2^11
@@ -186,12 +212,18 @@ struct QRing {
 // tiles before its own are done, adds, and passes the turn on. In lock-step the CTAs of neighbouring key tiles then
 // follow one another a reduction apart instead of all adding at once.
 template <bool FIRST, int DET, int D>
-__global__ void __launch_bounds__(kBwdThreads, 1) bwd_kernel(const __grid_constant__ BwdMaps maps, const BwdArgs a) {
+__global__ void __launch_bounds__(Roles<FIRST, D>::kThreads, 1) bwd_kernel(const __grid_constant__ BwdMaps maps, const BwdArgs a) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   BwdSmem<FIRST, D>& s = *reinterpret_cast<BwdSmem<FIRST, D>*>(smem_raw);
   constexpr int kHalves = D / 64;  // 64-column sub-tiles of a K / V / Q / dO tile
   constexpr uint32_t kOpBytes = kHalves * kHalfTileBytes;  // bytes of such a tile
   constexpr int kHeadDim = D;
+  using R = Roles<FIRST, D>;
+  constexpr int kSoft = R::kSoft, kReduceWarps = 4 * R::kReduce;
+  constexpr bool kOwnDq = R::kOwnDq;
+  // dO buffer of step cs and the parity of the number of earlier uses of that buffer
+  auto do_stage = [](uint32_t cs) { return kDoStages<D> == 2 ? cs & 1 : 0u; };
+  auto do_parity = [](uint32_t cs) { return kDoStages<D> == 2 ? (cs >> 1) & 1 : cs & 1; };
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, wg = warp >> 2;
   // swizzled tiles need a 1024-byte aligned base
   const bool misaligned = (smem_u32(smem_raw) & 1023u) != 0;
@@ -203,24 +235,23 @@ __global__ void __launch_bounds__(kBwdThreads, 1) bwd_kernel(const __grid_consta
       mbar_init(&s.bar_q_empty[i][0], 1);
       mbar_init(&s.bar_q_empty[i][1], 1);
     }
-    mbar_init(&s.bar_do_full, 1);
-    mbar_init(&s.bar_do_empty[0], 1);
-    mbar_init(&s.bar_do_empty[1], 1);
     for (int i = 0; i < 2; ++i) {
+      mbar_init(&s.bar_do_full[i], 1);
+      mbar_init(&s.bar_do_empty[i][0], 1);
+      mbar_init(&s.bar_do_empty[i][1], 1);
       mbar_init(&s.bar_ld_full[i], 32);
-      mbar_init(&s.bar_ld_empty[i], 256);
+      mbar_init(&s.bar_ld_empty[i], 128 * kSoft);
     }
     mbar_init(&s.bar_s_full, 1);
     mbar_init(&s.bar_dp_full, 1);
-    mbar_init(&s.bar_p_ready, 256);
-    mbar_init(&s.bar_ds_ready, 256);
+    mbar_init(&s.bar_p_ready, 128 * kSoft);
+    mbar_init(&s.bar_ds_ready, 128 * kSoft);
     mbar_init(&s.bar_dq_full, 1);
     mbar_init(&s.bar_a_done, 1);
     mbar_init(&s.bar_b_done, 1);
-    mbar_init(&s.bar_dq_empty, 256);
-    mbar_init(&s.bar_delta[0], 128);
-    mbar_init(&s.bar_delta[1], 128);
-    mbar_init(&s.bar_out, 256);
+    mbar_init(&s.bar_dq_empty, 32 * kReduceWarps);
+    for (int i = 0; i < kSoft; ++i) mbar_init(&s.bar_delta[i], 128);
+    mbar_init(&s.bar_out, 128 * kSoft);
     s.abort = 0;
     fence_mbar_init();
   }
@@ -234,7 +265,8 @@ __global__ void __launch_bounds__(kBwdThreads, 1) bwd_kernel(const __grid_consta
 
   // The CTA owns all 512 TMEM columns, so the allocation starts at column 0 and every TMEM address is a
   // compile-time constant.
-  constexpr uint32_t tR0 = 0, tR1 = 128, tDK = 256, tDV = 384;
+  constexpr uint32_t tR0 = 0, tR1 = 128, tDK = 256, tDV = 256 + D;
+  constexpr uint32_t tDQ = kOwnDq ? 384 : tR1;  // where dQ^T of a step goes
   if (misaligned || s.tmem_base != 0) {
     if (tid == 0)
       report_timeout(a.status, -1, misaligned ? kWhereBwdSmemAlign : kWhereBwdTmemBase, static_cast<int32_t>(s.tmem_base));
@@ -346,9 +378,9 @@ __global__ void __launch_bounds__(kBwdThreads, 1) bwd_kernel(const __grid_consta
     gi += 1;
   };
 
-  if (wg == 4) {
-    setmaxnreg_dec<kRegsAux>();
-    if (warp == 16) {
+  if (wg == kSoft + R::kReduce) {
+    setmaxnreg_dec<R::kRegsAux>();
+    if (warp == R::kAux0) {
       // ================================================================ TMA producer
       // Q(t) goes into a three-stage ring and is requested about one step before S^T(t) needs it; dO(t) goes
       // into a single buffer that is free from the end of dV(t-1) until dP^T(t). Requests are issued in the
@@ -384,27 +416,28 @@ __global__ void __launch_bounds__(kBwdThreads, 1) bwd_kernel(const __grid_consta
             for (int hf = 0; hf < kHalves; ++hf)
               tma_load_3d(s.q[qr.st][hf], mq, &s.bar_q_full[qr.st], 64 * hf, h, c.tok0 + m * kBM);
             qr.next();
-            if (!mbar_wait(&s.bar_do_empty[0], (cs & 1) ^ 1, a.wait_limit) || !mbar_wait(&s.bar_do_empty[1], (cs & 1) ^ 1, a.wait_limit)) {
+            const uint32_t dst = do_stage(cs);
+            if (!mbar_wait(&s.bar_do_empty[dst][0], do_parity(cs) ^ 1, a.wait_limit) || !mbar_wait(&s.bar_do_empty[dst][1], do_parity(cs) ^ 1, a.wait_limit)) {
               report_timeout(a.status, c.it, kWhereBwdQEmpty, 100000 + vt);
               *abort_flag = 1;
               break;
             }
-            mbar_expect_tx(&s.bar_do_full, kOpBytes);
+            mbar_expect_tx(&s.bar_do_full[dst], kOpBytes);
 #pragma unroll
-            for (int hf = 0; hf < kHalves; ++hf) tma_load_3d(s.d_o[hf], mdo, &s.bar_do_full, 64 * hf, h, c.tok0 + m * kBM);
+            for (int hf = 0; hf < kHalves; ++hf) tma_load_3d(s.d_o[dst][hf], mdo, &s.bar_do_full[dst], 64 * hf, h, c.tok0 + m * kBM);
           }
           if (c.steps <= kAheadMaxSteps) fetch_item(s.ctx[(gi + 1) & 1]);  // see next_item(): the same rule on both sides
         }
         item_done();
       }
-    } else if (warp == 17 || warp == 19) {
+    } else if (warp == R::kAux0 + 1 || warp == R::kAux0 + 3) {
       // ================================================================ MMA issuers
       // Two issuing warps share the step: warp 17 (A) owns R0 and dV: dV(t), S^T(t+1); warp 19 (B) owns R1 and
       // dK: dQ^T(t), dK(t), dP^T(t+1). Each has its own chain of waits, so the bookkeeping of one hides behind
       // the MMAs of the other. All 32 lanes run the waits and the address arithmetic (convergent code); the lane
       // elect.sync picks issues the MMAs and the commits. Each issuer signals completion on barriers of its own
       // (a tcgen05.commit covers only the issuing thread's MMAs); whoever depends on both waits for both.
-      const bool is_a = warp == 17;
+      const bool is_a = warp == R::kAux0 + 1;
       QRing qr;
       while (next_item()) {
         {
@@ -420,14 +453,14 @@ __global__ void __launch_bounds__(kBwdThreads, 1) bwd_kernel(const __grid_consta
           constexpr uint32_t lbo_km = (16u >> 4) << 16, lbo_mn = (kHalfTileBytes >> 4) << 16;
           // K read MN-major as the A operand of dQ^T has M = head dimension. With D = 64 the product still runs with
           // M = 128: the second half of the rows repeats the first (leading byte offset 0) and lands in TMEM lanes
-          // 64..127, which nobody reads.
+          // 64..127, from where the dQ role drains the upper query columns.
           constexpr uint32_t lbo_kt = D == 128 ? lbo_mn : 0u;
           constexpr uint32_t kStageStep = kOpBytes >> 4;  // descriptor distance between Q stages
           const int steps = cx->steps, item_it = cx->it;
           int where = 0;
           bool okm = mbar_wait(&s.bar_kv, gi & 1, a.wait_limit);
           if (!okm) where = kWhereBwdLoadKV;
-          const uint32_t q0_lo = smem_desc_addr(s.q[0][0]), do_lo = smem_desc_addr(s.d_o[0]);
+          const uint32_t q0_lo = smem_desc_addr(s.q[0][0]), do0_lo = smem_desc_addr(s.d_o[0][0]);
           if (is_a) {
             const uint32_t k_km = smem_desc_addr(s.k[0]) | lbo_km;
             // S^T of the next step not yet issued -> R0 (A = K, B = Q of the ring stage, both K-major)
@@ -450,7 +483,8 @@ __global__ void __launch_bounds__(kBwdThreads, 1) bwd_kernel(const __grid_consta
               constexpr bool fold = FIRST;
               const uint32_t cs = gs + vt;
               if (*abort_flag) return false;
-              if (!mbar_wait(&s.bar_do_full, cs & 1, a.wait_limit)) { where = kWhereBwdLoadQ; return false; }
+              const uint32_t do_lo = do0_lo + do_stage(cs) * kStageStep;
+              if (!mbar_wait(&s.bar_do_full[do_stage(cs)], do_parity(cs), a.wait_limit)) { where = kWhereBwdLoadQ; return false; }
               if (!mbar_wait(&s.bar_p_ready, cs & 1, a.wait_limit)) { where = kWhereBwdPReady; return false; }
               tc_fence_after_sync();
               const uint32_t acc = vt > 0;
@@ -469,7 +503,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) bwd_kernel(const __grid_consta
                 }
               }
               if (leader) umma_commit(&s.bar_a_done);       // S^T and dV of the step
-              if (leader) umma_commit(&s.bar_do_empty[0]);  // this thread is done with the dO buffer
+              if (leader) umma_commit(&s.bar_do_empty[do_stage(cs)][0]);  // this thread is done with the dO buffer
               if (vt + 1 < steps && !issue_s()) return false;
               return true;
             };
@@ -479,11 +513,13 @@ __global__ void __launch_bounds__(kBwdThreads, 1) bwd_kernel(const __grid_consta
             const uint32_t v_km = smem_desc_addr(s.v[0]) | lbo_km, k_mn = smem_desc_addr(s.k[0]) | lbo_kt;
             const uint32_t ds_km = smem_desc_addr(s.ds[0]) | lbo_km, ds_mn = smem_desc_addr(s.ds[0]) | lbo_mn;
             constexpr uint32_t kLoStep = (2 * kHalfTileBytes) >> 4;  // descriptor distance from dS^T to its residual
-            // dP^T of step vt -> R1, once the dQ warps have drained dQ^T of the previous step from it
+            // dP^T of step vt -> R1, once the dQ warps have drained dQ^T of the previous step from it (with a dQ^T region
+            // of its own: once the softmax warps have consumed dP^T of the previous step)
             auto issue_dp = [&](int vt) -> bool {
               const uint32_t cs = gs + vt;
-              if (!mbar_wait(&s.bar_do_full, cs & 1, a.wait_limit)) { where = kWhereBwdLoadQ; return false; }
-              if (!mbar_wait(&s.bar_dq_empty, (cs & 1) ^ 1, a.wait_limit)) { where = kWhereBwdDqEmpty; return false; }
+              const uint32_t do_lo = do0_lo + do_stage(cs) * kStageStep;
+              if (!mbar_wait(&s.bar_do_full[do_stage(cs)], do_parity(cs), a.wait_limit)) { where = kWhereBwdLoadQ; return false; }
+              if (!kOwnDq && !mbar_wait(&s.bar_dq_empty, (cs & 1) ^ 1, a.wait_limit)) { where = kWhereBwdDqEmpty; return false; }
               tc_fence_after_sync();
 #pragma unroll
               for (int kk = 0; kk < D / 16; ++kk) {
@@ -491,7 +527,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) bwd_kernel(const __grid_consta
                 if (leader) umma_ss_lh(tR1, v_km + off, hi, (do_lo | lbo_km) + off, hi, idesc_kk, kk > 0);
               }
               if (leader) umma_commit(&s.bar_dp_full);
-              if (leader) umma_commit(&s.bar_do_empty[1]);  // this thread is done with the dO buffer
+              if (leader) umma_commit(&s.bar_do_empty[do_stage(cs)][1]);  // this thread is done with the dO buffer
               return true;
             };
             okm = okm && issue_dp(0);
@@ -501,17 +537,21 @@ __global__ void __launch_bounds__(kBwdThreads, 1) bwd_kernel(const __grid_consta
               if (*abort_flag) return false;
               if (!mbar_wait(&s.bar_q_full[qr.st], qr.ph, a.wait_limit)) { where = kWhereBwdLoadQ; return false; }
               if (!mbar_wait(&s.bar_ds_ready, cs & 1, a.wait_limit)) { where = kWhereBwdDsReady; return false; }
+              if constexpr (kOwnDq) {
+                if (vt + 1 < steps && !issue_dp(vt + 1)) return false;
+                if (!mbar_wait(&s.bar_dq_empty, (cs & 1) ^ 1, a.wait_limit)) { where = kWhereBwdDqEmpty; return false; }
+              }
               tc_fence_after_sync();
               const uint32_t acc = vt > 0;
               const uint32_t q_mn = (q0_lo + qr.st * kStageStep) | lbo_mn;
-              // dQ^T = K^T dS^T -> R1 (dP^T of this step has been consumed: ds_ready). It goes first: the dQ warps
+              // dQ^T = K^T dS^T -> R1 (dP^T of this step has been consumed: ds_ready), or a region of its own. It goes first: the dQ warps
               // drain R1 while dK runs, so that dP^T of the next step can follow dK without a gap.
 #pragma unroll
-              for (int kk = 0; kk < 8; ++kk) if (leader) umma_ss_lh(tR1, k_mn + kk * 128, hi, ds_mn + kk * 128, hi, idesc_nn, kk > 0);
+              for (int kk = 0; kk < 8; ++kk) if (leader) umma_ss_lh(tDQ, k_mn + kk * 128, hi, ds_mn + kk * 128, hi, idesc_nn, kk > 0);
               if constexpr (fold) {
 #pragma unroll 1
                 for (int kk = 0; kk < 8; ++kk)
-                  if (leader) umma_ss_lh(tR1, k_mn + kk * 128, hi, ds_mn + kLoStep + kk * 128, hi, idesc_nn, 1u);
+                  if (leader) umma_ss_lh(tDQ, k_mn + kk * 128, hi, ds_mn + kLoStep + kk * 128, hi, idesc_nn, 1u);
               }
               if (leader) umma_commit(&s.bar_dq_full);
               // dK += dS^T Q
@@ -530,7 +570,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) bwd_kernel(const __grid_consta
               if (leader) umma_commit(&s.bar_b_done);              // dP^T, dQ^T and dK of the step
               if (leader) umma_commit(&s.bar_q_empty[qr.st][1]);  // this thread is done with the Q stage
               qr.next();
-              if (vt + 1 < steps && !issue_dp(vt + 1)) return false;
+              if (!kOwnDq && vt + 1 < steps && !issue_dp(vt + 1)) return false;
               return true;
             };
 #pragma unroll 1
@@ -543,7 +583,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) bwd_kernel(const __grid_consta
         }
         item_done();
       }
-    } else if (warp == 18) {
+    } else if (warp == R::kAux0 + 2) {
       // ================================================================ LSE / delta loader
       while (next_item()) {
         const ItemCtx c = *cx;
@@ -592,12 +632,16 @@ __global__ void __launch_bounds__(kBwdThreads, 1) bwd_kernel(const __grid_consta
         item_done();
       }
     }
-  } else if (wg >= 2) {
+  } else if (wg >= kSoft) {
     // ================================================================ dQ^T: R1 -> global fp32 accumulator
-    setmaxnreg_dec<kRegsReduce<FIRST>>();
-    const int quad = warp & 3, colhalf = wg - 2;  // this warp drains query columns [64*colhalf, 64*colhalf + 64)
+    setmaxnreg_dec<R::kRegsReduce>();
+    // This warp drains query columns [col0, col0 + kDrain). With D = 64 the tile's rows d = 0..63 are repeated in TMEM
+    // lanes 64..127 (see the descriptor of K^T), so the eight warps take 32 columns each: a warp issues a reduction every
+    // ~46 clocks whatever its size, and four warps of 64 were what a step waited for.
+    constexpr int kDrain = R::kDrain;
+    const int quad = warp & 3, col0 = kDrain * (D == 64 ? 2 * (wg - kSoft) + (quad >> 1) : wg - kSoft);
     const uint32_t lane_off = static_cast<uint32_t>(quad * 32) << 16;
-    const int d = quad * 32 + lane;  // head-dimension index = TMEM lane
+    const int d = (D == 64 ? quad & 1 : quad) * 32 + lane;  // head-dimension index
     while (next_item()) {
       const ItemCtx c = *cx;
       const int64_t q_stride = static_cast<int64_t>(c.hq) * kHeadDim;  // floats between consecutive query rows
@@ -626,61 +670,44 @@ __global__ void __launch_bounds__(kBwdThreads, 1) bwd_kernel(const __grid_consta
         // skipped (their dS^T columns are zero, and they may lie outside the buffer).
         const int rows_left = c.len - m * kBM;  // valid query rows of this q tile (>= 128 for an interior tile)
         float* const tile0 = a.dq_acc + c.q_off + (static_cast<int64_t>(m) * kBM * c.hq + h) * kHeadDim + d;
-        const int n_valid = min(kBM, rows_left) - colhalf * 64;
-        if constexpr (D < 128) {
-          // dQ^T has D rows: the warps of TMEM lanes D..127 have nothing to drain, they only keep the barrier counts
-          // (and, with ordered additions, the turn counts)
-          if (d >= D) {
-            tc_fence_before_sync();
-            mbar_arrive(&s.bar_dq_empty);
-            if constexpr (DET == 1) {
-              int32_t* turn = a.dq_turn + c.turn_off + h * c.mt + m;
-              if (lane == 0) {
-                const long long t0 = clock64();
-                while (*reinterpret_cast<volatile int32_t*>(turn) < 8 * c.n && clock64() - t0 < a.wait_limit) __nanosleep(64);
-                atomicAdd(turn, 1);
-              }
-            }
-            continue;
-          }
-        }
+        const int n_valid = min(kBM, rows_left) - col0;
         if constexpr (FIRST) {
           // q tile 0 gets nothing from any other key tile: scale and store the rows directly, no accumulator
           uint32_t v0[32], v1[32];
-          tmem_ld32(tR1 + lane_off + colhalf * 64, v0);
-          tmem_ld32(tR1 + lane_off + colhalf * 64 + 32, v1);
+          tmem_ld32(tDQ + lane_off + col0, v0);
+          if constexpr (kDrain == 64) tmem_ld32(tDQ + lane_off + col0 + 32, v1);
           tmem_wait_ld();
           tc_fence_before_sync();
           mbar_arrive(&s.bar_dq_empty);
-          const int64_t o0 = c.q_off + (static_cast<int64_t>(colhalf * 64) * c.hq + h) * kHeadDim + d;
-          NSP_CHECK(n_valid <= 0 || (o0 >= 0 && o0 + (min(n_valid, 64) - 1) * q_stride < a.q_elems), a.status, c.it,
+          const int64_t o0 = c.q_off + (static_cast<int64_t>(col0) * c.hq + h) * kHeadDim + d;
+          NSP_CHECK(n_valid <= 0 || (o0 >= 0 && o0 + (min(n_valid, kDrain) - 1) * q_stride < a.q_elems), a.status, c.it,
                     kWhereCheckBwdDq, h) {
           if (a.dq_f32) {
             float* q0 = static_cast<float*>(a.dq) + o0;
 #pragma unroll
             for (int e = 0; e < 32; ++e) {
               if (e < n_valid) q0[e * q_stride] = __uint_as_float(v0[e]) * a.scale;
-              if (e + 32 < n_valid) q0[(e + 32) * q_stride] = __uint_as_float(v1[e]) * a.scale;
+              if (kDrain == 64 && e + 32 < n_valid) q0[(e + 32) * q_stride] = __uint_as_float(v1[e]) * a.scale;
             }
           } else {
             __nv_bfloat16* q0 = static_cast<__nv_bfloat16*>(a.dq) + o0;
 #pragma unroll
             for (int e = 0; e < 32; ++e) {
               if (e < n_valid) q0[e * q_stride] = __float2bfloat16_rn(__uint_as_float(v0[e]) * a.scale);
-              if (e + 32 < n_valid) q0[(e + 32) * q_stride] = __float2bfloat16_rn(__uint_as_float(v1[e]) * a.scale);
+              if (kDrain == 64 && e + 32 < n_valid) q0[(e + 32) * q_stride] = __float2bfloat16_rn(__uint_as_float(v1[e]) * a.scale);
             }
           }
           }
           continue;
         }
-        float* p0 = tile0 + colhalf * 64 * q_stride;
+        float* p0 = tile0 + col0 * q_stride;
         int32_t* turn = nullptr;
         if constexpr (DET == 1) turn = a.dq_turn + c.turn_off + h * c.mt + m;
         auto wait_turn = [&]() -> bool {  // key tiles 0 .. n-1 have added their tiles (eight dQ warps each)
           bool okt = true;
           if (lane == 0) {
             const long long t0 = clock64();
-            while (*reinterpret_cast<volatile int32_t*>(turn) < 8 * c.n) {
+            while (*reinterpret_cast<volatile int32_t*>(turn) < kReduceWarps * c.n) {
               if (clock64() - t0 > a.wait_limit) { okt = false; break; }
               __nanosleep(64);
             }
@@ -700,8 +727,8 @@ __global__ void __launch_bounds__(kBwdThreads, 1) bwd_kernel(const __grid_consta
           // rolled loop of 16-column loads with a wait each, R1 was handed back late and such a step took twice as long
           // (batches of 500-, 1,000- and 2,000-token segments ran 10-18 % slower per flop than 512 / 1,024 / 2,048).
           uint32_t v0[32], v1[32];
-          tmem_ld32(tR1 + lane_off + colhalf * 64, v0);
-          tmem_ld32(tR1 + lane_off + colhalf * 64 + 32, v1);
+          tmem_ld32(tDQ + lane_off + col0, v0);
+          if constexpr (kDrain == 64) tmem_ld32(tDQ + lane_off + col0 + 32, v1);
           tmem_wait_ld();
           tc_fence_before_sync();
           mbar_arrive(&s.bar_dq_empty);  // R1 is drained: the next dP^T may overwrite it
@@ -717,14 +744,14 @@ __global__ void __launch_bounds__(kBwdThreads, 1) bwd_kernel(const __grid_consta
           // The reductions sit in a conditional region on purpose (the condition always holds): as straight-line
           // code the compiler computes all 64 row addresses ahead of the TMEM loads, runs out of the 80 registers
           // this role has and spills inside the loop (measured: the whole kernel 25 % slower).
-          NSP_CHECK(n_valid <= 0 || (p0 >= a.dq_acc && p0 + (min(n_valid, 64) - 1) * q_stride < a.dq_acc + a.q_elems), a.status,
+          NSP_CHECK(n_valid <= 0 || (p0 >= a.dq_acc && p0 + (min(n_valid, kDrain) - 1) * q_stride < a.dq_acc + a.q_elems), a.status,
                     c.it, kWhereCheckBwdDq, m)
           if (c.hq > 0) {
             float* p1 = p0 + 32 * q_stride;
 #pragma unroll
             for (int e = 0; e < 32; ++e) {
               if (e < n_valid) red_add_f32(p0, dq_term<DET>(__uint_as_float(v0[e])));
-              if (e + 32 < n_valid) red_add_f32(p1, dq_term<DET>(__uint_as_float(v1[e])));
+              if (kDrain == 64 && e + 32 < n_valid) red_add_f32(p1, dq_term<DET>(__uint_as_float(v1[e])));
               p0 += q_stride;
               p1 += q_stride;
             }
@@ -736,13 +763,16 @@ __global__ void __launch_bounds__(kBwdThreads, 1) bwd_kernel(const __grid_consta
     }
   } else {
     // ================================================================ softmax / dS (key row r, 64 query columns)
-    setmaxnreg_inc<kRegsSoftmax<FIRST>>();
-    const int quad = warp & 3, half = wg;
+    setmaxnreg_inc<R::kRegsSoft>();
+    constexpr int kCols = R::kCols, kChunks = kCols / 16;  // this thread's query columns [kCols * wg, kCols * wg + kCols)
+    const int quad = warp & 3;
+    const int col0 = kCols * wg;
     const int r = quad * 32 + lane;
     const uint32_t lane_off = static_cast<uint32_t>(quad * 32) << 16;
-    const uint32_t tS = tR0 + lane_off + half * 64, tDP = tR1 + lane_off + half * 64;
-    uint8_t* const ds_row = s.ds[half] + r * 128;  // this thread's 128-byte row of the swizzled dS^T half tile
-    uint32_t nd = 0;                               // completed phases of bar_delta[half]
+    const uint32_t tS = tR0 + lane_off + col0, tDP = tR1 + lane_off + col0;
+    uint8_t* const ds_row = s.ds[col0 / 64] + r * 128;  // this thread's 128-byte row of the swizzled dS^T half tile
+    const int chunk0 = (col0 % 64) / 8;                 // its first 16-byte chunk in that row
+    uint32_t nd = 0;                                    // completed phases of bar_delta[wg]
     while (next_item()) {
       const ItemCtx c = *cx;
       bool oks = true;
@@ -766,8 +796,12 @@ __global__ void __launch_bounds__(kBwdThreads, 1) bwd_kernel(const __grid_consta
         oks = __all_sync(0xffffffffu, oks);
         if (!oks) { where = kWhereBwdS; break; }
         tc_fence_after_sync();
-        const float* lse_s = s.lse[st] + half * 64;
-        float* delta_s = s.delta[st] + half * 64;
+        // With a dQ^T region of its own dP^T runs ahead of dQ^T and dK of the previous step, which read the dS buffer
+        auto ds_free = [&]() -> bool {
+          return !kOwnDq || vt == 0 || mbar_wait(&s.bar_b_done, (cs - 1) & 1, a.wait_limit);
+        };
+        const float* lse_s = s.lse[st] + col0;
+        float* delta_s = s.delta[st] + col0;
         // ---- common step (interior tile; the diagonal tile runs a second copy of the same code with a mask on P,
         // kept apart so that the interior copy's instructions stay as they are)
         auto common_step = [&](auto diag_tag) -> bool {
@@ -777,17 +811,17 @@ __global__ void __launch_bounds__(kBwdThreads, 1) bwd_kernel(const __grid_consta
           // Sixteen columns at a time; the LSE (delta) values of the next sixteen are requested before the
           // arithmetic of the current ones, because a shared-memory load takes a long time here: the LSU is
           // shared with the 64 KB of dQ reductions per step.
-          uint32_t sv[2][32];
+          uint32_t sv[kChunks / 2][32];
           float4 aux[2][4];
 #pragma unroll
           for (int i = 0; i < 4; ++i) aux[0][i] = lds128(lse_s + 4 * i);
-          tmem_ld32(tS, sv[0]);
-          tmem_ld32(tS + 32, sv[1]);
-          tmem_wait_ld();
-          uint32_t pp[2][16];  // P^T as bf16 pairs: what goes to R0, and what the dS^T product uses below
 #pragma unroll
-          for (int ch = 0; ch < 4; ++ch) {
-            if (ch < 3) {
+          for (int g = 0; g < kChunks / 2; ++g) tmem_ld32(tS + 32 * g, sv[g]);
+          tmem_wait_ld();
+          uint32_t pp[kChunks / 2][16];  // P^T as bf16 pairs: what goes to R0, and what the dS^T product uses below
+#pragma unroll
+          for (int ch = 0; ch < kChunks; ++ch) {
+            if (ch < kChunks - 1) {
 #pragma unroll
               for (int i = 0; i < 4; ++i) aux[(ch + 1) & 1][i] = lds128(lse_s + (ch + 1) * 16 + 4 * i);
             }
@@ -818,9 +852,9 @@ __global__ void __launch_bounds__(kBwdThreads, 1) bwd_kernel(const __grid_consta
             }
             if constexpr (decltype(diag_tag)::value) {
               // diagonal tile: a key sees only the queries at or after it. Element e of this chunk (query column
-              // 64 * half + 16 * ch + e) survives iff e >= t; P = 0 also zeroes dS^T below. Rows and columns past
+              // col0 + 16 * ch + e) survives iff e >= t; P = 0 also zeroes dS^T below. Rows and columns past
               // the end of a ragged segment fall under the same mask (their LSE is +inf).
-              const int t = r - (half * 64 + ch * 16);
+              const int t = r - (col0 + ch * 16);
 #pragma unroll
               for (int kk = 0; kk < 8; ++kk) {
                 const uint32_t keep = t <= 2 * kk ? 0xffffffffu : (t == 2 * kk + 1 ? 0xffff0000u : 0u);
@@ -834,19 +868,19 @@ __global__ void __launch_bounds__(kBwdThreads, 1) bwd_kernel(const __grid_consta
           mbar_arrive(&s.bar_p_ready);
           // Phase 2: dS^T = P^T o (dP^T - delta) -> swizzled shared memory; P enters with its bf16 value, the one
           // the dV product uses. The dS buffer is free: dP^T of this step was issued behind dK / dQ^T of the
-          // previous step, so bar_dp_full implies they have completed.
+          // previous step, so bar_dp_full implies they have completed (or, issued ahead of them, they are waited for).
 #pragma unroll
           for (int i = 0; i < 4; ++i) aux[0][i] = lds128(delta_s + 4 * i);
-          oks = mbar_wait(&s.bar_dp_full, cs & 1, a.wait_limit);
+          oks = mbar_wait(&s.bar_dp_full, cs & 1, a.wait_limit) && ds_free();
           oks = __all_sync(0xffffffffu, oks);
           if (!oks) { where = kWhereBwdDp; return false; }
           tc_fence_after_sync();
           uint32_t dpv[2][16];
           tmem_ld16(tDP, dpv[0]);
 #pragma unroll
-          for (int ch = 0; ch < 4; ++ch) {
+          for (int ch = 0; ch < kChunks; ++ch) {
             tmem_wait_ld();
-            if (ch < 3) {
+            if (ch < kChunks - 1) {
               tmem_ld16(tDP + (ch + 1) * 16, dpv[(ch + 1) & 1]);
 #pragma unroll
               for (int i = 0; i < 4; ++i) aux[(ch + 1) & 1][i] = lds128(delta_s + (ch + 1) * 16 + 4 * i);
@@ -866,8 +900,8 @@ __global__ void __launch_bounds__(kBwdThreads, 1) bwd_kernel(const __grid_consta
               dsp[(x >> 1) + 1] = pack_bf16x2(d2, d3);
             }
             // sixteen query columns = two 16-byte chunks of the swizzled dS^T row
-            *reinterpret_cast<uint4*>(ds_row + ((2 * ch) ^ (r & 7)) * 16) = make_uint4(dsp[0], dsp[1], dsp[2], dsp[3]);
-            *reinterpret_cast<uint4*>(ds_row + ((2 * ch + 1) ^ (r & 7)) * 16) = make_uint4(dsp[4], dsp[5], dsp[6], dsp[7]);
+            *reinterpret_cast<uint4*>(ds_row + ((chunk0 + 2 * ch) ^ (r & 7)) * 16) = make_uint4(dsp[0], dsp[1], dsp[2], dsp[3]);
+            *reinterpret_cast<uint4*>(ds_row + ((chunk0 + 2 * ch + 1) ^ (r & 7)) * 16) = make_uint4(dsp[4], dsp[5], dsp[6], dsp[7]);
           }
           return true;
         };
@@ -887,18 +921,20 @@ __global__ void __launch_bounds__(kBwdThreads, 1) bwd_kernel(const __grid_consta
           oks = __all_sync(0xffffffffu, oks);
           if (!oks) { where = kWhereBwdDp; break; }
           tc_fence_after_sync();
-          uint32_t pkk[4][16];
+          uint32_t pkk[kChunks][16];
           {
             // Sweep 1: P^T (value and residual over the S^T columns just read: packed columns [16ch, 16ch + 8) and
             // [16ch + 8, 16ch + 16)) and the partial sums of delta. The packed values stay in registers for sweep 2
             // (both sweeps fully unrolled), so R0 is free for the next S^T as soon as the dV products have run.
-            float* part = reinterpret_cast<float*>(s.ds[half]);  // [4 quadrants][64 columns]; free until dS is written
+            // [4 quadrants][kCols columns]; with two column groups in the group's own half of dS^T, which is free until the
+            // group itself writes it
+            float* part = kSoft == 2 ? reinterpret_cast<float*>(s.ds[wg & 1]) : s.part + wg * 4 * kCols;
             // Column sums over the 32 key rows of a warp by a butterfly: at every level a lane keeps the half of
             // the columns its lane bit selects and adds the partner's partial sums of that half (16 shuffles for
             // 16 columns); after the last level lane 2c (and 2c + 1) holds column c = lane / 2.
             const bool b4 = lane & 16, b3 = lane & 8, b2 = lane & 4, b1 = lane & 2;
 #pragma unroll
-            for (int ch = 0; ch < 4; ++ch) {
+            for (int ch = 0; ch < kChunks; ++ch) {
               uint32_t sv[16], dpv[16];
               uint32_t* const pk = pkk[ch];
               float4 l4[4];
@@ -913,7 +949,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) bwd_kernel(const __grid_consta
                 const float lse0 = (x & 2) ? l4[x >> 2].z : l4[x >> 2].x, lse1 = (x & 2) ? l4[x >> 2].w : l4[x >> 2].y;
                 float p0 = ex2f(fmaf(__uint_as_float(sv[x + 0]), a.scale_log2, -lse0));
                 float p1 = ex2f(fmaf(__uint_as_float(sv[x + 1]), a.scale_log2, -lse1));
-                const int qc = half * 64 + ch * 16 + x;
+                const int qc = col0 + ch * 16 + x;
                 if (qc + 0 < r || qc + 0 >= r_end) p0 = 0.f;  // query index must be >= key index, inside its segment
                 if (qc + 1 < r || qc + 1 >= r_end) p1 = 0.f;
                 v[x + 0] = p0 * __uint_as_float(dpv[x + 0]);
@@ -935,27 +971,32 @@ __global__ void __launch_bounds__(kBwdThreads, 1) bwd_kernel(const __grid_consta
                 w2[i] = (b2 ? w4[i + 2] : w4[i]) + __shfl_xor_sync(0xffffffffu, b2 ? w4[i] : w4[i + 2], 4);
               float w1 = (b1 ? w2[1] : w2[0]) + __shfl_xor_sync(0xffffffffu, b1 ? w2[0] : w2[1], 2);
               w1 += __shfl_xor_sync(0xffffffffu, w1, 1);
-              if ((lane & 1) == 0) part[quad * 64 + ch * 16 + (lane >> 1)] = w1;
+              if ((lane & 1) == 0) part[quad * kCols + ch * 16 + (lane >> 1)] = w1;
             }
             tmem_wait_st();
             tc_fence_before_sync();
             mbar_arrive(&s.bar_p_ready);  // the dV products run under the rest of this step
-            mbar_arrive(&s.bar_delta[half]);
-            oks = mbar_wait(&s.bar_delta[half], nd & 1, a.wait_limit);
+            mbar_arrive(&s.bar_delta[wg]);
+            oks = mbar_wait(&s.bar_delta[wg], nd & 1, a.wait_limit);
             ++nd;
             oks = __all_sync(0xffffffffu, oks);
             if (!oks) { where = kWhereBwdDelta; break; }
-            if (r < 64) delta_s[r] = (part[r] + part[64 + r]) + (part[128 + r] + part[192 + r]);
-            mbar_arrive(&s.bar_delta[half]);
-            oks = mbar_wait(&s.bar_delta[half], nd & 1, a.wait_limit);
+            if (r < kCols) delta_s[r] = (part[r] + part[kCols + r]) + (part[2 * kCols + r] + part[3 * kCols + r]);
+            mbar_arrive(&s.bar_delta[wg]);
+            oks = mbar_wait(&s.bar_delta[wg], nd & 1, a.wait_limit);
             ++nd;
             oks = __all_sync(0xffffffffu, oks);
             if (!oks) { where = kWhereBwdDelta; break; }
           }
           // Sweep 2: dS^T = P^T o (dP^T - delta), value and residual (P = value + residual to 2^-17)
+          if constexpr (kOwnDq) {
+            oks = ds_free();
+            oks = __all_sync(0xffffffffu, oks);
+            if (!oks) { where = kWhereBwdDelta; break; }
+          }
           uint8_t* const ds_row_lo = ds_row + 2 * kHalfTileBytes;
 #pragma unroll
-          for (int ch = 0; ch < 4; ++ch) {
+          for (int ch = 0; ch < kChunks; ++ch) {
             uint32_t dpv[16], dsp[8], dsl[8];
             const uint32_t* const pk = pkk[ch];
             float4 e4[4];
@@ -975,7 +1016,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) bwd_kernel(const __grid_consta
               dsp[x >> 1] = da;
               dsl[x >> 1] = pack_bf16x2(d0 - __uint_as_float(da << 16), d1 - __uint_as_float(da & 0xffff0000u));
             }
-            const uint32_t c0 = ((2 * ch) ^ (r & 7)) * 16, c1 = ((2 * ch + 1) ^ (r & 7)) * 16;
+            const uint32_t c0 = ((chunk0 + 2 * ch) ^ (r & 7)) * 16, c1 = ((chunk0 + 2 * ch + 1) ^ (r & 7)) * 16;
             *reinterpret_cast<uint4*>(ds_row + c0) = make_uint4(dsp[0], dsp[1], dsp[2], dsp[3]);
             *reinterpret_cast<uint4*>(ds_row + c1) = make_uint4(dsp[4], dsp[5], dsp[6], dsp[7]);
             *reinterpret_cast<uint4*>(ds_row_lo + c0) = make_uint4(dsl[0], dsl[1], dsl[2], dsl[3]);
@@ -995,7 +1036,6 @@ __global__ void __launch_bounds__(kBwdThreads, 1) bwd_kernel(const __grid_consta
       }
       if (oks) {
         tc_fence_after_sync();
-        constexpr int kCols = D / 2;  // this thread's columns of a dK / dV row
         // Key tile 0 in the main kernel: the first-tile kernel, which ran before, left its part (q tile 0) in the
         // output; this item's sum over the q tiles 1 .. Mt-1 is added to it (one fixed order: reproducible).
         // Later parts of a divided item add to what the parts before them have left, in turn.
@@ -1025,13 +1065,13 @@ __global__ void __launch_bounds__(kBwdThreads, 1) bwd_kernel(const __grid_consta
         uint8_t* const stage_k = &s.k[0][0];
         uint8_t* const stage_v = &s.q[0][0][0];
 #pragma unroll 1
-        for (int part = 0; part < 2 * (kCols / 32); ++part) {  // (dK, dV) x 32-column chunks
-          const int which = part / (kCols / 32), cc = part % (kCols / 32);
+        for (int i = 0; i < 2 * (D / 32) / kSoft; ++i) {  // (dK, dV) x 32-column sub-tiles
+          const int piece = i * kSoft + wg, which = piece / (D / 32), cc = piece % (D / 32);
           const float mul = which == 0 ? a.scale : 1.f;
           uint32_t v[32];
-          tmem_ld32(tDK + which * 128 + lane_off + half * kCols + cc * 32, v);
+          tmem_ld32(tDK + which * (tDV - tDK) + lane_off + cc * 32, v);
           tmem_wait_ld();
-          uint8_t* const sub = (which == 0 ? stage_k : stage_v) + (half * (kCols / 32) + cc) * kSubBytes + r * 128;
+          uint8_t* const sub = (which == 0 ? stage_k : stage_v) + cc * kSubBytes + r * 128;
 #pragma unroll
           for (int x = 0; x < 8; ++x) {
             *reinterpret_cast<float4*>(sub + ((x ^ (r & 7)) * 16)) =
@@ -1073,11 +1113,11 @@ __global__ void __launch_bounds__(kBwdThreads, 1) bwd_kernel(const __grid_consta
             }
           }
         } else {
-          // ---- ragged tiles and bf16 outputs: the eight warps write whole rows (D / 4 lanes per row, 16 staged bytes
+          // ---- ragged tiles and bf16 outputs: the softmax warps write whole rows (D / 4 lanes per row, 16 staged bytes
           // each), four row passes in flight; an added tile reads its rows the same way first. Written from the threads
           // that hold the rows (a row per lane, 16 bytes per store, each store its own line) a tile pair took four times
           // as long, and twice that where it was added.
-          constexpr int kLanes = D / 4, kRowsPerPass = 32 / kLanes, kPasses = 128 / (8 * kRowsPerPass);
+          constexpr int kLanes = D / 4, kRowsPerPass = 32 / kLanes, kPasses = 128 / (4 * kSoft * kRowsPerPass);
           const int rows = min(kBN, c.len - c.n * kBN);
           const int l = lane % kLanes;
           bool oku = mbar_wait_token(&s.bar_out, staged, a.wait_limit);
@@ -1097,7 +1137,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) bwd_kernel(const __grid_consta
             bool on[4];
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
-              const int row = ((it + u) % kPasses * 8 + warp) * kRowsPerPass + lane / kLanes;
+              const int row = ((it + u) % kPasses * 4 * kSoft + warp) * kRowsPerPass + lane / kLanes;
               on[u] = row < rows;
               at[u] = c.kv_off + (static_cast<int64_t>(c.n * kBN + row) * c.hkv + c.g) * kHeadDim + 4 * l;
               w4[u] = *reinterpret_cast<const float4*>(st0 + row * 128 + ((l % 8) ^ (row & 7)) * 16);
@@ -1332,7 +1372,7 @@ cudaError_t launch_bwd_t(const BwdMaps& maps, const BwdArgs& args, int num_sms, 
   if (e != cudaSuccess) return e;
   const int grid = args.n_items < num_sms ? args.n_items : num_sms;
   count_launches(1);
-  return launch_chained_if(chained, bwd_kernel<FIRST, DET, D>, grid, kBwdThreads, sizeof(BwdSmem<FIRST, D>), st, maps, args);
+  return launch_chained_if(chained, bwd_kernel<FIRST, DET, D>, grid, Roles<FIRST, D>::kThreads, sizeof(BwdSmem<FIRST, D>), st, maps, args);
 }
 }  // namespace
 

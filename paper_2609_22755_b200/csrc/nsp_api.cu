@@ -53,8 +53,8 @@ struct nsp_plan {
   int64_t n_first = 0;
   RowInfo* d_rows = nullptr;          // row tables of the packs, 128 entries each (d_seg holds the packs' entries after
   int64_t n_packs = 0;                // the n_seg segments')
-  int64_t n_fwd_main = 0;             // forward items that visit at least two key tiles: a prefix of d_fwd (the
-                                      // cost-1 tail = q tile 0 of every segment runs in the first-tile forward kernel)
+  nsp_tile_t* d_fwd_pairs = nullptr;  // the forward items that visit at least two key tiles, in the pairs the general
+  int64_t n_pairs = 0;                // kernel runs (q tile 0 of every segment runs in the first-tile forward kernel)
   bool deterministic = false;         // plan option: dQ tiles added in key-tile order
   bool rounded_dq = false;            // plan option: dQ terms rounded to a fixed quantum (order-independent sums)
   // Small batches launch the preprocess and the main kernel chained as well (see launch_chained_if), so that the main
@@ -408,13 +408,11 @@ int nsp_plan_tiles(const int32_t* cu_seqlens, const int32_t* hq, const int32_t* 
       }
     }
     p->n_first = static_cast<int64_t>(bwd_first.size());
-    p->n_fwd_main = nf;
     for (const SegInfo& sg : p->seg) {
       const int64_t Mt = (static_cast<int64_t>(sg.len) + bm - 1) / bm;
       bwd_steps += sg.hq * (Mt * (Mt + 1) / 2);
+      if (Mt > 1) p->n_pairs += (sg.hq / sg.hkv) % 2 == 0 ? sg.hq / 2 * (Mt - 1) : sg.hq * (Mt / 2);
     }
-    for (const SegInfo& sg : p->seg)
-      if (sg.len > 0) p->n_fwd_main -= sg.hq;
     for (const SegInfo& sg : p->seg) p->max_len = std::max(p->max_len, sg.len);
   } catch (...) {
     delete p;
@@ -485,6 +483,7 @@ int nsp_plan_tiles(const int32_t* cu_seqlens, const int32_t* hq, const int32_t* 
   const size_t o_fwd = take(sizeof(nsp_tile_t) * nf);
   const size_t o_bwd = take(sizeof(nsp_tile_t) * nb);
   const size_t o_exec = take(sizeof(nsp_tile_t) * nb);
+  const size_t o_pairs = take(sizeof(nsp_tile_t) * 2 * p->n_pairs);
   const size_t o_front = take(sizeof(int32_t) * (nb / kFrontBlock + 1));
   p->arena = arena_acquire(p->device, at, 256 + upload);
   if (!p->arena) {
@@ -501,6 +500,7 @@ int nsp_plan_tiles(const int32_t* cu_seqlens, const int32_t* hq, const int32_t* 
   p->d_fwd = reinterpret_cast<nsp_tile_t*>(d + o_fwd);
   p->d_bwd = reinterpret_cast<nsp_tile_t*>(d + o_bwd);
   p->d_bwd_exec = reinterpret_cast<nsp_tile_t*>(d + o_exec);
+  p->d_fwd_pairs = reinterpret_cast<nsp_tile_t*>(d + o_pairs);
   p->d_front = reinterpret_cast<int32_t*>(d + o_front);
   p->d_bwd_parts = reinterpret_cast<nsp_tile_t*>(d + o_parts);
   p->d_bwd_first_parts = reinterpret_cast<nsp_tile_t*>(d + o_first_parts);
@@ -528,7 +528,7 @@ int nsp_plan_tiles(const int32_t* cu_seqlens, const int32_t* hq, const int32_t* 
   cudaStream_t bs = p->arena->build;
   if (cudaMemcpyAsync(d, image, upload, cudaMemcpyHostToDevice, bs) != cudaSuccess ||
       launch_plan_lists(reinterpret_cast<const PlanKey*>(d + o_keys), reinterpret_cast<const int32_t*>(d + o_tiles), n_seg,
-                        static_cast<int>(tiles), p->d_fwd, p->d_bwd, p->d_bwd_exec, bs) != cudaSuccess ||
+                        static_cast<int>(tiles), p->d_fwd, p->d_bwd, p->d_bwd_exec, p->d_fwd_pairs, bs) != cudaSuccess ||
       cudaStreamSynchronize(bs) != cudaSuccess) {
     p->arena->captured = true;  // not for reuse
     free_plan(p);
@@ -613,9 +613,9 @@ int nsp_attn_fwd(const nsp_plan_t* plan, const void* q, const void* k, const voi
   prof_mark(plan, NSP_KERNEL_FWD_FIRST, 0, st);
   if (!plan->withhold && launch_fwd_first(maps, a, plan->head_dim, plan->num_sms, st) != cudaSuccess) return NSP_ERR_CUDA;
   prof_mark(plan, NSP_KERNEL_FWD_FIRST, 1, st);
-  // everything else: the list's prefix (with the test switch of the checked build: the whole list, general kernel)
-  a.items = plan->d_fwd;
-  a.n_items = static_cast<int32_t>(plan->withhold ? plan->n_fwd : plan->n_fwd_main);
+  // everything else, in pairs (with the test switch of the checked build: the whole list, general kernel)
+  a.items = plan->withhold ? plan->d_fwd : plan->d_fwd_pairs;
+  a.n_items = static_cast<int32_t>(plan->withhold ? plan->n_fwd : 2 * plan->n_pairs);
   a.counter = plan->d_counters;
   prof_mark(plan, NSP_KERNEL_FWD, 0, st);
   if (launch_fwd(maps, a, plan->head_dim, plan->num_sms, !plan->withhold, st) != cudaSuccess) return NSP_ERR_CUDA;

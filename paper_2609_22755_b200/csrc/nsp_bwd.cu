@@ -284,6 +284,11 @@ __global__ void __launch_bounds__(Roles<FIRST, D>::kThreads, 1) bwd_kernel(const
   uint32_t gs = 0;  // steps completed so far by this CTA (every role advances it identically)
   uint32_t gi = 0;  // items completed so far
 
+  // One vote of a converged warp: true if every lane's waits succeeded and no role had raised the abort flag when they
+  // began (`calm`, read ahead of the waits; voted on and not tested on its own: lanes that read it at different times would
+  // part, and the next vote would never complete).
+  auto together = [&](bool here) -> bool { return __all_sync(0xffffffffu, here); };
+
   // Every role runs its own copy of the item loop (so that its register budget, set by setmaxnreg at the top of
   // the role, governs the whole loop); the loops meet at the CTA-wide barrier inside next_item().
   const ItemCtx* cx = nullptr;
@@ -458,21 +463,23 @@ __global__ void __launch_bounds__(Roles<FIRST, D>::kThreads, 1) bwd_kernel(const
           constexpr uint32_t kStageStep = kOpBytes >> 4;  // descriptor distance between Q stages
           const int steps = cx->steps, item_it = cx->it;
           int where = 0;
-          bool okm = mbar_wait(&s.bar_kv, gi & 1, a.wait_limit);
+          bool okm = together(mbar_poll(&s.bar_kv, gi & 1, a.wait_limit));
           if (!okm) where = kWhereBwdLoadKV;
           const uint32_t q0_lo = smem_desc_addr(s.q[0][0]), do0_lo = smem_desc_addr(s.d_o[0][0]);
           if (is_a) {
             const uint32_t k_km = smem_desc_addr(s.k[0]) | lbo_km;
             // S^T of the next step not yet issued -> R0 (A = K, B = Q of the ring stage, both K-major)
             auto issue_s = [&]() -> bool {
-              if (!mbar_wait(&s.bar_q_full[qr.st], qr.ph, a.wait_limit)) { where = kWhereBwdLoadQ; return false; }
+              const bool here = mbar_poll(&s.bar_q_full[qr.st], qr.ph, a.wait_limit);
               tc_fence_after_sync();
+              const bool go = leader && here;
               const uint32_t b_lo = (q0_lo + qr.st * kStageStep) | lbo_km;
 #pragma unroll
               for (int kk = 0; kk < D / 16; ++kk) {
                 const uint32_t off = ((kk >> 2) * kHalfTileBytes + (kk & 3) * 32) >> 4;
-                if (leader) umma_ss_lh(tR0, k_km + off, hi, b_lo + off, hi, idesc_kk, kk > 0);
+                if (go) umma_ss_lh(tR0, k_km + off, hi, b_lo + off, hi, idesc_kk, kk > 0);
               }
+              if (!together(here)) { where = kWhereBwdLoadQ; return false; }
               if (leader) umma_commit(&s.bar_s_full);
               if (leader) umma_commit(&s.bar_q_empty[qr.st][0]);  // this thread is done with the Q stage
               qr.next();
@@ -481,27 +488,29 @@ __global__ void __launch_bounds__(Roles<FIRST, D>::kThreads, 1) bwd_kernel(const
             okm = okm && issue_s();
             auto step_a = [&](int vt) -> bool {
               constexpr bool fold = FIRST;
+              const bool calm = *abort_flag == 0;
               const uint32_t cs = gs + vt;
-              if (*abort_flag) return false;
               const uint32_t do_lo = do0_lo + do_stage(cs) * kStageStep;
-              if (!mbar_wait(&s.bar_do_full[do_stage(cs)], do_parity(cs), a.wait_limit)) { where = kWhereBwdLoadQ; return false; }
-              if (!mbar_wait(&s.bar_p_ready, cs & 1, a.wait_limit)) { where = kWhereBwdPReady; return false; }
+              bool here = mbar_poll(&s.bar_do_full[do_stage(cs)], do_parity(cs), a.wait_limit);
+              here = mbar_poll(&s.bar_p_ready, cs & 1, a.wait_limit) && here;
               tc_fence_after_sync();
+              const bool go = leader && here;
               const uint32_t acc = vt > 0;
               if constexpr (!fold) {
                 // dV += P^T dO; packed P^T columns of K-step kk (16 query columns) sit at R0 + (kk/2)*32 + (kk%2)*8
 #pragma unroll
                 for (int kk = 0; kk < 8; ++kk)
-                  if (leader) umma_ts_lh(tDV, tR0 + (kk >> 1) * 32 + (kk & 1) * 8, (do_lo | lbo_mn) + kk * 128, hi, idesc_kn,
+                  if (go) umma_ts_lh(tDV, tR0 + (kk >> 1) * 32 + (kk & 1) * 8, (do_lo | lbo_mn) + kk * 128, hi, idesc_kn,
                              acc | (kk > 0));
               } else {
                 // P^T as value + residual, 16 query columns = 8 packed columns each, side by side
 #pragma unroll 1
                 for (int kk = 0; kk < 8; ++kk) {
-                  if (leader) umma_ts_lh(tDV, tR0 + kk * 16, (do_lo | lbo_mn) + kk * 128, hi, idesc_kn, acc | (kk > 0));
-                  if (leader) umma_ts_lh(tDV, tR0 + kk * 16 + 8, (do_lo | lbo_mn) + kk * 128, hi, idesc_kn, 1u);
+                  if (go) umma_ts_lh(tDV, tR0 + kk * 16, (do_lo | lbo_mn) + kk * 128, hi, idesc_kn, acc | (kk > 0));
+                  if (go) umma_ts_lh(tDV, tR0 + kk * 16 + 8, (do_lo | lbo_mn) + kk * 128, hi, idesc_kn, 1u);
                 }
               }
+              if (!together(here && calm)) { where = kWhereBwdPReady; return false; }
               if (leader) umma_commit(&s.bar_a_done);       // S^T and dV of the step
               if (leader) umma_commit(&s.bar_do_empty[do_stage(cs)][0]);  // this thread is done with the dO buffer
               if (vt + 1 < steps && !issue_s()) return false;
@@ -518,14 +527,16 @@ __global__ void __launch_bounds__(Roles<FIRST, D>::kThreads, 1) bwd_kernel(const
             auto issue_dp = [&](int vt) -> bool {
               const uint32_t cs = gs + vt;
               const uint32_t do_lo = do0_lo + do_stage(cs) * kStageStep;
-              if (!mbar_wait(&s.bar_do_full[do_stage(cs)], do_parity(cs), a.wait_limit)) { where = kWhereBwdLoadQ; return false; }
-              if (!kOwnDq && !mbar_wait(&s.bar_dq_empty, (cs & 1) ^ 1, a.wait_limit)) { where = kWhereBwdDqEmpty; return false; }
+              bool here = mbar_poll(&s.bar_do_full[do_stage(cs)], do_parity(cs), a.wait_limit);
+              if constexpr (!kOwnDq) here = mbar_poll(&s.bar_dq_empty, (cs & 1) ^ 1, a.wait_limit) && here;
               tc_fence_after_sync();
+              const bool go = leader && here;
 #pragma unroll
               for (int kk = 0; kk < D / 16; ++kk) {
                 const uint32_t off = ((kk >> 2) * kHalfTileBytes + (kk & 3) * 32) >> 4;
-                if (leader) umma_ss_lh(tR1, v_km + off, hi, (do_lo | lbo_km) + off, hi, idesc_kk, kk > 0);
+                if (go) umma_ss_lh(tR1, v_km + off, hi, (do_lo | lbo_km) + off, hi, idesc_kk, kk > 0);
               }
+              if (!together(here)) { where = kWhereBwdDqEmpty; return false; }
               if (leader) umma_commit(&s.bar_dp_full);
               if (leader) umma_commit(&s.bar_do_empty[do_stage(cs)][1]);  // this thread is done with the dO buffer
               return true;
@@ -533,38 +544,41 @@ __global__ void __launch_bounds__(Roles<FIRST, D>::kThreads, 1) bwd_kernel(const
             okm = okm && issue_dp(0);
             auto step_b = [&](int vt) -> bool {
               constexpr bool fold = FIRST;
+              const bool calm = *abort_flag == 0;
               const uint32_t cs = gs + vt;
-              if (*abort_flag) return false;
-              if (!mbar_wait(&s.bar_q_full[qr.st], qr.ph, a.wait_limit)) { where = kWhereBwdLoadQ; return false; }
-              if (!mbar_wait(&s.bar_ds_ready, cs & 1, a.wait_limit)) { where = kWhereBwdDsReady; return false; }
+              bool here = mbar_poll(&s.bar_q_full[qr.st], qr.ph, a.wait_limit);
+              here = mbar_poll(&s.bar_ds_ready, cs & 1, a.wait_limit) && here;
               if constexpr (kOwnDq) {
+                if (!together(here && calm)) { where = kWhereBwdDsReady; return false; }
                 if (vt + 1 < steps && !issue_dp(vt + 1)) return false;
-                if (!mbar_wait(&s.bar_dq_empty, (cs & 1) ^ 1, a.wait_limit)) { where = kWhereBwdDqEmpty; return false; }
+                here = mbar_poll(&s.bar_dq_empty, (cs & 1) ^ 1, a.wait_limit);
               }
               tc_fence_after_sync();
+              const bool go = leader && here;
               const uint32_t acc = vt > 0;
               const uint32_t q_mn = (q0_lo + qr.st * kStageStep) | lbo_mn;
               // dQ^T = K^T dS^T -> R1 (dP^T of this step has been consumed: ds_ready), or a region of its own. It goes first: the dQ warps
               // drain R1 while dK runs, so that dP^T of the next step can follow dK without a gap.
 #pragma unroll
-              for (int kk = 0; kk < 8; ++kk) if (leader) umma_ss_lh(tDQ, k_mn + kk * 128, hi, ds_mn + kk * 128, hi, idesc_nn, kk > 0);
+              for (int kk = 0; kk < 8; ++kk) if (go) umma_ss_lh(tDQ, k_mn + kk * 128, hi, ds_mn + kk * 128, hi, idesc_nn, kk > 0);
               if constexpr (fold) {
 #pragma unroll 1
                 for (int kk = 0; kk < 8; ++kk)
-                  if (leader) umma_ss_lh(tDQ, k_mn + kk * 128, hi, ds_mn + kLoStep + kk * 128, hi, idesc_nn, 1u);
+                  if (go) umma_ss_lh(tDQ, k_mn + kk * 128, hi, ds_mn + kLoStep + kk * 128, hi, idesc_nn, 1u);
               }
+              if (!together(here && calm)) { where = kWhereBwdDsReady; return false; }
               if (leader) umma_commit(&s.bar_dq_full);
               // dK += dS^T Q
 #pragma unroll
               for (int kk = 0; kk < 8; ++kk) {
                 const uint32_t off = ((kk >> 2) * kHalfTileBytes + (kk & 3) * 32) >> 4;
-                if (leader) umma_ss_lh(tDK, ds_km + off, hi, q_mn + kk * 128, hi, idesc_kn, acc | (kk > 0));
+                if (go) umma_ss_lh(tDK, ds_km + off, hi, q_mn + kk * 128, hi, idesc_kn, acc | (kk > 0));
               }
               if constexpr (fold) {
 #pragma unroll 1
                 for (int kk = 0; kk < 8; ++kk) {
                   const uint32_t off = ((kk >> 2) * kHalfTileBytes + (kk & 3) * 32) >> 4;
-                  if (leader) umma_ss_lh(tDK, ds_km + kLoStep + off, hi, q_mn + kk * 128, hi, idesc_kn, 1u);
+                  if (go) umma_ss_lh(tDK, ds_km + kLoStep + off, hi, q_mn + kk * 128, hi, idesc_kn, 1u);
                 }
               }
               if (leader) umma_commit(&s.bar_b_done);              // dP^T, dQ^T and dK of the step
@@ -578,6 +592,7 @@ __global__ void __launch_bounds__(Roles<FIRST, D>::kThreads, 1) bwd_kernel(const
           }
           if (!okm && where != 0) {  // where == 0: another role raised the abort flag
             if (leader) report_timeout(a.status, item_it, where, is_a ? 0 : 1);
+            drain_products();
             *abort_flag = 1;
           }
         }

@@ -1,10 +1,12 @@
 // Forward: packed variable-length causal GQA attention on tcgen05 tensor cores.
 //
-// One persistent CTA per SM (640 threads) pops work items (segment, q head, q tile) from the longest-first
-// list TWO at a time. Neighbouring items of the list are the same (segment, q tile) for consecutive q heads, so
-// when they share a KV head (GQA) the CTA runs them as a pair "A/B" over the SAME K/V tiles: every K/V tile is
+// One persistent CTA per SM (640 threads) pops work items (segment, q head, q tile) from a longest-first
+// list TWO at a time and runs them as a pair "A/B" over the SAME K/V tiles: every K/V tile is
 // fetched once for 256 query rows, and the tensor pipe alternates between the two while their softmax
-// warpgroups work (otherwise the two items run one after the other with warpgroup B idle).
+// warpgroups work (otherwise the two items run one after the other with warpgroup B idle). With an even number of q
+// heads per KV head a pair is one q tile of two heads; otherwise (one head per KV head above all) it is two neighbouring
+// q tiles of one head, B the lower one, which visits one key tile less than A (16q/16kv, forward: 24,097 tokens of
+// median 1,000 445 -> 339 us, 2,000 tokens of median 600 66 -> 41 us).
 //     S_x  = Q_x K_j^T      tcgen05.mma SS (both K-major, 128B-swizzled smem staged by TMA)       -> TMEM S_x
 //     P_x  = exp2(S_x*c - m)  one thread per query row (tcgen05.ld), bf16 pairs written over S_x  (tcgen05.st)
 //     O_x += P_x V_j        tcgen05.mma TS (A = P_x from TMEM, B = V MN-major from smem)          -> TMEM O_x
@@ -53,6 +55,7 @@ struct FwdSmem {
                              // half-row dot product of O and dO (3, recomputation only)
                              // (slot 2) handed to the partner thread
   uint64_t bar_pv_done[2];  // [A/B] O_x += P_x V has completed
+  uint64_t bar_last_pv;     // two q tiles of one head: the last PV product of A has completed (B's O tile may be staged)
   uint64_t bar_q_free;      // the last S products of the round have completed: the Q tiles may be overwritten
   uint64_t bar_o_staged[2];  // [A/B] 256 softmax threads: the tile's O rows are in the staging buffer
   uint64_t bar_pop_ready[2];  // [slot] the pop fetched ahead is in its slot
@@ -111,6 +114,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1) fwd_kernel(const __grid_consta
       mbar_init(&s.bar_pv_done[i], 1);
     }
     mbar_init(&s.bar_q_free, 1);
+    mbar_init(&s.bar_last_pv, 1);
     mbar_init(&s.bar_o_staged[0], 256);
     mbar_init(&s.bar_o_staged[1], 256);
     mbar_init(&s.bar_pop_ready[0], 1);
@@ -132,6 +136,10 @@ __global__ void __launch_bounds__(kFwdThreads, 1) fwd_kernel(const __grid_consta
   const uint32_t tmem = s.tmem_base;
   volatile int32_t* abort_flag = &s.abort;
   uint32_t gp = 0;  // pops so far
+  // One vote of a converged warp: true if every lane's waits succeeded and no role had raised the abort flag when they
+  // began (`calm`, read ahead of the waits; voted on and not tested on its own: lanes that read it at different times would
+  // part, and the next vote would never complete).
+  auto together = [&](bool here) -> bool { return __all_sync(0xffffffffu, here); };
   // The CTA-wide meeting points are plain barriers. Every role reaches them in bounded time: all its other waits are
   // bounded and none of them returns before the end of the kernel. (An mbarrier with a bounded wait in their place
   // made the register allocation of the softmax role fail.)
@@ -163,7 +171,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1) fwd_kernel(const __grid_consta
         reset_cursor(a.counter, it, (a.n_items + 1) / 2 * 2, 2);
         break;
       }
-      bool have_b = it + 1 < a.n_items;
+      bool have_b = it + 1 < a.n_items && a.items[it + 1].seg >= 0;
       nsp_tile_t ia = a.items[it];
       nsp_tile_t ib = have_b ? a.items[it + 1] : ia;
       if (RECOMP && a.seg_mask != nullptr) {  // recomputation: only the marked segments
@@ -176,7 +184,8 @@ __global__ void __launch_bounds__(kFwdThreads, 1) fwd_kernel(const __grid_consta
       p.a = ia, p.b = ib, p.sa = sa;
       p.sb = ib.seg == ia.seg ? sa : a.seg[ib.seg];
       const int G = sa.hq / sa.hkv;
-      p.joint = have_b && ib.seg == ia.seg && ib.tile == ia.tile && (ia.head / G == ib.head / G);
+      p.joint = have_b && ib.seg == ia.seg && ((ib.tile == ia.tile && ia.head / G == ib.head / G) ||
+                                               (ib.head == ia.head && ib.tile == ia.tile - 1));
       p.n_rounds = p.joint ? 1 : (have_b ? 2 : 1);
       p.kt_base = static_cast<int32_t>(kt_total);
       kt_total += static_cast<uint32_t>(ia.cost + (p.n_rounds == 2 ? ib.cost : 0));
@@ -232,7 +241,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1) fwd_kernel(const __grid_consta
               for (int hf = 0; hf < kHalves; ++hf) tma_load_3d(s.q[0][hf], mq, &s.bar_q, 64 * hf, ia.head, tok0 + q_row0);
               if (rd.joint) {
 #pragma unroll
-                for (int hf = 0; hf < kHalves; ++hf) tma_load_3d(s.q[1][hf], mq, &s.bar_q, 64 * hf, rd.b.head, tok0 + q_row0);
+                for (int hf = 0; hf < kHalves; ++hf) tma_load_3d(s.q[1][hf], mq, &s.bar_q, 64 * hf, rd.b.head, tok0 + rd.b.tile * kBM);
               }
             }
             for (int j = pre ? 1 : 0; j < n_kv; ++j) {
@@ -285,7 +294,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1) fwd_kernel(const __grid_consta
               for (int hf = 0; hf < kHalves; ++hf) tma_load_3d(s.q[0][hf], &maps.q[ns->run], &s.bar_q, 64 * hf, na->head, ntok + na->tile * kBM);
               if (joint) {
 #pragma unroll
-                for (int hf = 0; hf < kHalves; ++hf) tma_load_3d(s.q[1][hf], &maps.q[ns->run], &s.bar_q, 64 * hf, nx->b.head, ntok + na->tile * kBM);
+                for (int hf = 0; hf < kHalves; ++hf) tma_load_3d(s.q[1][hf], &maps.q[ns->run], &s.bar_q, 64 * hf, nx->b.head, ntok + nx->b.tile * kBM);
               }
               const uint32_t kst = kn & 1, vst = vn & 1;
               if (mbar_wait(&s.bar_k_empty[kst], ((kn >> 1) & 1) ^ 1, a.wait_limit) &&
@@ -316,11 +325,12 @@ __global__ void __launch_bounds__(kFwdThreads, 1) fwd_kernel(const __grid_consta
       uint32_t qn = 0, kn = 0, vn = 0, pn[2] = {0, 0};
       while (next_pop()) {
         for (int r = 0; r < n_rounds; ++r) {
-          if (!*abort_flag) {
+          if (together(*abort_flag == 0)) {
             const bool leader = elect_one();
             const nsp_tile_t ia = r == 0 ? rd.a : rd.b;
             const int n_kv = ia.cost;
             const int joint = rd.joint;
+            const int n_kv_b = joint ? rd.b.cost : 0;  // n_kv or, with two q tiles of one head, n_kv - 1
             int where = 0;
             // S_x of key tile in stage kst -> TMEM columns [128*x, 128*x + 128)
             // Descriptors are {low word, high word}; inside the loops an operand advances by adding its byte
@@ -342,59 +352,62 @@ __global__ void __launch_bounds__(kFwdThreads, 1) fwd_kernel(const __grid_consta
               if (leader) umma_commit(&s.bar_s_full[x]);
             };
             // O_x += P_x V (P_x: bf16 pairs in columns [0,32) and [64,96) of S_x)
-            auto issue_pv = [&](int x, uint32_t vst, int j) {
+            auto issue_pv = [&](int x, uint32_t vst, int j, bool go) {  // the caller commits bar_pv_done
               const uint32_t b_lo = v_lo + vst * kTileStep;
 #pragma unroll
               for (int kk = 0; kk < 8; ++kk)
-                if (leader) umma_ts_lh(tmem + 256 + 128 * x, tmem + 128 * x + (kk >> 2) * 64 + (kk & 3) * 8, b_lo + kk * 128, hi, idesc_pv,
+                if (go) umma_ts_lh(tmem + 256 + 128 * x, tmem + 128 * x + (kk >> 2) * 64 + (kk & 3) * 8, b_lo + kk * 128, hi, idesc_pv,
                            (j > 0 || kk > 0));
-              if (leader) umma_commit(&s.bar_pv_done[x]);
             };
-            bool ok = mbar_wait(&s.bar_q, qn & 1, a.wait_limit);
+            bool ok = together(mbar_poll(&s.bar_q, qn & 1, a.wait_limit));
             ++qn;
             if (!ok) where = kWhereFwdLoad;
             uint32_t kst = 0;
             for (int j = 0; ok && j < n_kv; ++j) {
-              if (*abort_flag) break;
               if (j == 0) {
                 kst = kn & 1;
-                if (!mbar_wait(&s.bar_k_full[kst], (kn >> 1) & 1, a.wait_limit)) { ok = false; where = kWhereFwdLoad; break; }
+                if (!together(mbar_poll(&s.bar_k_full[kst], (kn >> 1) & 1, a.wait_limit))) { ok = false; where = kWhereFwdLoad; break; }
                 tc_fence_after_sync();
                 issue_s(0, kst);
                 if (joint) issue_s(1, kst);
                 if (leader) umma_commit(&s.bar_k_empty[kst]);
                 ++kn;
               }
+              const bool calm = *abort_flag == 0;
               const uint32_t vst = vn & 1;
               const bool more = j + 1 < n_kv;
               if (!more && leader) umma_commit(&s.bar_q_free);  // every S product of the round has been issued
-              if (!mbar_wait(&s.bar_p_ready[0], pn[0] & 1, a.wait_limit)) { ok = false; where = kWhereFwdS; break; }
+              // P of A, this V tile and the next K tile (both loaded a key tile ahead)
+              kst = kn & 1;
+              bool here = mbar_poll(&s.bar_v_full[vst], (vn >> 1) & 1, a.wait_limit);
+              if (more) here = mbar_poll(&s.bar_k_full[kst], (kn >> 1) & 1, a.wait_limit) && here;
+              here = mbar_poll(&s.bar_p_ready[0], pn[0] & 1, a.wait_limit) && here;
               ++pn[0];
-              if (!mbar_wait(&s.bar_v_full[vst], (vn >> 1) & 1, a.wait_limit)) { ok = false; where = kWhereFwdLoad; break; }
               tc_fence_after_sync();
-              issue_pv(0, vst, j);
-              if (more) {  // S_A of the next key tile runs while softmax B is still working
-                kst = kn & 1;
-                if (!mbar_wait(&s.bar_k_full[kst], (kn >> 1) & 1, a.wait_limit)) { ok = false; where = kWhereFwdLoad; break; }
-                tc_fence_after_sync();
-                issue_s(0, kst);
-              }
-              if (joint) {
-                if (!mbar_wait(&s.bar_p_ready[1], pn[1] & 1, a.wait_limit)) { ok = false; where = kWhereFwdS; break; }
+              issue_pv(0, vst, j, leader && here);
+              if (!together(here && calm)) { ok = false; where = kWhereFwdS; break; }
+              if (leader) umma_commit(&s.bar_pv_done[0]);
+              if (more) issue_s(0, kst);  // S_A of the next key tile runs while softmax B is still working
+              if (j < n_kv_b) {
+                here = mbar_poll(&s.bar_p_ready[1], pn[1] & 1, a.wait_limit);
                 ++pn[1];
                 tc_fence_after_sync();
-                issue_pv(1, vst, j);
+                issue_pv(1, vst, j, leader && here);
+                if (!together(here)) { ok = false; where = kWhereFwdS; break; }
+                if (leader) umma_commit(&s.bar_pv_done[1]);
               }
               if (leader) umma_commit(&s.bar_v_empty[vst]);
               ++vn;
               if (more) {
-                if (joint) issue_s(1, kst);
+                if (j + 1 < n_kv_b) issue_s(1, kst);
                 if (leader) umma_commit(&s.bar_k_empty[kst]);
                 ++kn;
               }
             }
+            if (!RECOMP && ok && joint && n_kv_b != n_kv && leader) umma_commit(&s.bar_last_pv);
             if (!ok) {
               if (leader) report_timeout(a.status, it0, where, 0);
+              drain_products();
               *abort_flag = 1;
             }
           }
@@ -419,6 +432,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1) fwd_kernel(const __grid_consta
     uint32_t sn = 0;   // S tiles consumed so far
     uint32_t pvn = 0;  // PV products of this half issued before the current round
     uint32_t xn = 0;   // completed phases of this row pair's exchange barrier
+    uint32_t ln = 0;   // completed phases of bar_last_pv
     float* my_slot = &s.xchg[x][ch][0][rl];                   // slot k is my_slot[128 * k]
     const float* partner_slot = &s.xchg[x][ch ^ 1][0][rl];
     uint64_t* pair_bar = &s.bar_pair[x][quad];
@@ -617,6 +631,16 @@ __global__ void __launch_bounds__(kFwdThreads, 1) fwd_kernel(const __grid_consta
             l += partner_slot[256];
             tc_fence_after_sync();
             const float inv_l = 1.f / l;
+            // B of two q tiles of one head ends a key tile before A, whose products still read the stage used below
+            if (x == 1 && rd.b.cost != rd.a.cost) {
+              ok = mbar_wait(&s.bar_last_pv, ln & 1, a.wait_limit);
+              ++ln;
+              ok = __all_sync(0xffffffffu, ok);
+              if (!ok && lane == 0) {
+                report_timeout(a.status, it0, kWhereFwdO, 4);
+                *abort_flag = 1;
+              }
+            }
             if (q_row0 + kBM <= sg.len) {
               // ---- a full tile goes out as a TMA tile store. The rows are staged, swizzled like an operand tile, in
               // the ring stage of the round's last key tile: K's for item A, V's for item B. Both are free: the last

@@ -111,6 +111,11 @@ __global__ void __launch_bounds__(kThreads, 1) fwd_first_kernel(const __grid_con
   const uint32_t tmem = s.tmem_base;
   volatile int32_t* abort_flag = &s.abort;
 
+  // One vote of a converged warp: true if every lane's waits succeeded and no role had raised the abort flag when they
+  // began (`calm`, read ahead of the waits; voted on and not tested on its own: lanes that read it at different times would
+  // part, and the next vote would never complete).
+  auto together = [&](bool here) -> bool { return __all_sync(0xffffffffu, here); };
+
   // ---- work distribution: thread 0 pops and decodes; the next item is fetched while the current one runs
   uint32_t gi = 0;  // items finished so far
   FirstCtx c;
@@ -197,13 +202,13 @@ __global__ void __launch_bounds__(kThreads, 1) fwd_first_kernel(const __grid_con
       while (next_item()) {
         const bool leader = elect_one();
         int where = 0;
-        bool ok = mbar_wait(&s.bar_kv, gi & 1, a.wait_limit);
-        if (!ok) where = kWhereFwdLoad;
+        bool ok = true;
         for (int r = 0; ok && r < c.rounds; ++r) {
-          if (*abort_flag) break;
           const uint32_t st = (R + r) & 1;
           const int halves = 2 * r + 1 < c.G ? 2 : 1;
-          if (!mbar_wait(&s.bar_q_full[st], ((R + r) >> 1) & 1, a.wait_limit)) { ok = false; where = kWhereFwdLoad; break; }
+          const bool calm = *abort_flag == 0;
+          bool here = r > 0 || mbar_poll(&s.bar_kv, gi & 1, a.wait_limit);
+          here = mbar_poll(&s.bar_q_full[st], ((R + r) >> 1) & 1, a.wait_limit) && here;
           tc_fence_after_sync();
           // S of this round follows the PV products of the previous one on the same pipe, so P of the previous
           // round has been read before S overwrites it
@@ -212,18 +217,20 @@ __global__ void __launch_bounds__(kThreads, 1) fwd_first_kernel(const __grid_con
 #pragma unroll
             for (int kk = 0; kk < D / 16; ++kk) {
               const uint32_t off = ((kk >> 2) * kHalfTileBytes + (kk & 3) * 32) >> 4;
-              if (leader) umma_ss_lh(tmem + 128 * x, a_lo + off, hi, k_lo + off, hi, idesc_qk, kk > 0);
+              if (leader && here) umma_ss_lh(tmem + 128 * x, a_lo + off, hi, k_lo + off, hi, idesc_qk, kk > 0);
             }
+            if (x == 0 && !together(here && calm)) { ok = false; where = kWhereFwdLoad; break; }
             if (leader) umma_commit(&s.bar_s_full[x]);
           }
-          for (int x = 0; x < halves; ++x) {
-            if (!mbar_wait(&s.bar_p_ready[x], n[x] & 1, a.wait_limit)) { ok = false; where = kWhereFwdS; break; }
-            if (!mbar_wait(&s.bar_o_free[x], (n[x] & 1) ^ 1, a.wait_limit)) { ok = false; where = kWhereFwdO; break; }
+          for (int x = 0; ok && x < halves; ++x) {
+            here = mbar_poll(&s.bar_o_free[x], (n[x] & 1) ^ 1, a.wait_limit);
+            here = mbar_poll(&s.bar_p_ready[x], n[x] & 1, a.wait_limit) && here;
             tc_fence_after_sync();
 #pragma unroll
             for (int kk = 0; kk < 8; ++kk)
-              if (leader) umma_ts_lh(tmem + 256 + 128 * x, tmem + 128 * x + (kk >> 2) * 64 + (kk & 3) * 8, v_lo + kk * 128, hi,
+              if (leader && here) umma_ts_lh(tmem + 256 + 128 * x, tmem + 128 * x + (kk >> 2) * 64 + (kk & 3) * 8, v_lo + kk * 128, hi,
                                      idesc_pv, kk > 0);
+            if (!together(here)) { ok = false; where = kWhereFwdS; break; }
             if (leader) umma_commit(&s.bar_pv_done[x]);
             ++n[x];
           }
@@ -231,6 +238,7 @@ __global__ void __launch_bounds__(kThreads, 1) fwd_first_kernel(const __grid_con
         if (leader) umma_commit(&s.bar_kv_free);  // K and V may be replaced once everything issued so far has run
         if (!ok && where != 0) {
           if (leader) report_timeout(a.status, c.it, where, 0);
+          drain_products();
           *abort_flag = 1;
         }
         R += static_cast<uint32_t>(c.rounds);

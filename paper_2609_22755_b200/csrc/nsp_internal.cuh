@@ -218,7 +218,7 @@ constexpr int kMaxParts = 64;
 
 // Host-side launchers implemented next to their kernels.
 cudaError_t launch_plan_lists(const PlanKey* d_key, const int32_t* d_tile_base, int n_seg, int n_tiles, nsp_tile_t* d_fwd,
-                              nsp_tile_t* d_bwd, nsp_tile_t* d_exec, cudaStream_t st);
+                              nsp_tile_t* d_bwd, nsp_tile_t* d_exec, nsp_tile_t* d_pairs, cudaStream_t st);
 // chained: launched right behind launch_fwd_first, whose inputs are this kernel's too
 cudaError_t launch_fwd(const FwdMaps& maps, const FwdArgs& args, int head_dim, int num_sms, bool chained, cudaStream_t st);
 // q tile 0 of every segment: items (segment, kv head); args.items / n_items / counter are that list's

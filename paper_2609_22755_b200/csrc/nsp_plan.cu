@@ -1,10 +1,13 @@
-// Device-side construction of the tile work lists (forward, backward, and the backward items in the order the kernel
-// walks them).
+// Device-side construction of the tile work lists (forward, backward, the backward items in the order the kernel
+// walks them, and the forward items in the pairs its kernel runs).
 //
 // Item definitions and order (unique, so any correct construction gives the same lists bit for bit):
 //   forward  (s, h, m): cost = ceil(min(L, (m+1)*bm) / bn)          -- key tiles the query tile visits
 //   backward (s, g, n): cost = G * (Mt - floor(n*bn / bm))          -- (q head, q tile) visits of the key tile
 //   order: cost descending, then segment, tile, head ascending.
+//   pairs    of forward items with at least two key tiles, by the cost of their first item descending, then segment, head:
+//            an even group: (s, h, m), (s, h + 1, m) for even h; otherwise (s, h, m), (s, h, m - 1) for m = Mt-1, Mt-3, ..
+//            (without a second item where m - 1 = 0, which belongs to the first-tile kernel: seg = -1).
 //   walked   (s, g, n): groups (s, g) by segment length descending, then s, g ascending; n ascending inside a group.
 //
 // With bm == bn a segment has at most one tile of a given cost, so the position of a tile's items in each list is a sum
@@ -25,7 +28,8 @@ constexpr int kListThreads = 128;
 
 __global__ void __launch_bounds__(kListThreads, 16)
     plan_lists_kernel(const PlanKey* __restrict__ key, const int32_t* __restrict__ tile_base, int n_seg, int n_tiles,
-                      nsp_tile_t* __restrict__ fwd, nsp_tile_t* __restrict__ bwd, nsp_tile_t* __restrict__ exec) {
+                      nsp_tile_t* __restrict__ fwd, nsp_tile_t* __restrict__ bwd, nsp_tile_t* __restrict__ exec,
+                      nsp_tile_t* __restrict__ pairs) {
   const int lane = threadIdx.x & 31;
   const int n_warps = gridDim.x * (kListThreads / 32);
   for (int t = (blockIdx.x * kListThreads + threadIdx.x) >> 5; t < n_tiles; t += n_warps) {
@@ -37,7 +41,7 @@ __global__ void __launch_bounds__(kListThreads, 16)
     const PlanKey k = key[s];
     const int m = t - tile_base[s];
     const int cf = m + 1, cb = k.group * (k.tiles - m);
-    int nf = 0, nb = 0, ne = 0;  // items before this tile's (before its group's, in the walked order)
+    int nf = 0, nb = 0, ne = 0, np = 0;  // items before this tile's (before its group's, in the walked order); pairs likewise
     for (int x = lane; x < n_seg; x += 32) {
       const PlanKey o = key[x];
       const int hkv = o.hq / o.group;
@@ -47,11 +51,27 @@ __global__ void __launch_bounds__(kListThreads, 16)
       // backward: cost = group * k, k = 1 .. tiles
       const int q = cb / o.group;
       nb += hkv * (max(o.tiles - q, 0) + (before && q * o.group == cb && q <= o.tiles));
+      // pairs: an even group has hq / 2 of every cost 2 .. tiles; another hq of the costs tiles, tiles - 2, .. >= 2
+      if (o.group & 1)
+        np += o.hq * ((max(o.tiles - cf, 0) + 1) / 2 + (before && o.tiles >= cf && ((o.tiles - cf) & 1) == 0));
+      else
+        np += o.hq / 2 * (max(o.tiles - cf, 0) + (before && o.tiles >= cf));
       ne += o.len > k.len || (o.len == k.len && before) ? hkv * o.tiles : 0;
     }
     nf = __reduce_add_sync(0xffffffffu, nf);
     nb = __reduce_add_sync(0xffffffffu, nb);
     ne = __reduce_add_sync(0xffffffffu, ne);
+    np = __reduce_add_sync(0xffffffffu, np);
+    if (m > 0) {
+      if (!(k.group & 1)) {
+        for (int h = lane; h < k.hq; h += 32) pairs[2 * np + h] = nsp_tile_t{s, h, m, cf};
+      } else if (((k.tiles - cf) & 1) == 0) {
+        for (int h = lane; h < k.hq; h += 32) {
+          pairs[2 * (np + h)] = nsp_tile_t{s, h, m, cf};
+          pairs[2 * (np + h) + 1] = m > 1 ? nsp_tile_t{s, h, m - 1, cf - 1} : nsp_tile_t{-1, 0, 0, 0};
+        }
+      }
+    }
     for (int h = lane; h < k.hq; h += 32) fwd[nf + h] = nsp_tile_t{s, h, m, cf};
     for (int g = lane; g < k.hq / k.group; g += 32) {
       bwd[nb + g] = nsp_tile_t{s, g, m, cb};
@@ -63,11 +83,11 @@ __global__ void __launch_bounds__(kListThreads, 16)
 }  // namespace
 
 cudaError_t launch_plan_lists(const PlanKey* d_key, const int32_t* d_tile_base, int n_seg, int n_tiles, nsp_tile_t* d_fwd,
-                              nsp_tile_t* d_bwd, nsp_tile_t* d_exec, cudaStream_t st) {
+                              nsp_tile_t* d_bwd, nsp_tile_t* d_exec, nsp_tile_t* d_pairs, cudaStream_t st) {
   if (n_tiles == 0) return cudaSuccess;
   const int blocks = (n_tiles + kListThreads / 32 - 1) / (kListThreads / 32);
   plan_lists_kernel<<<blocks < 148 * 8 ? blocks : 148 * 8, kListThreads, 0, st>>>(d_key, d_tile_base, n_seg, n_tiles, d_fwd,
-                                                                                  d_bwd, d_exec);
+                                                                                  d_bwd, d_exec, d_pairs);
   count_launches(1);
   return cudaGetLastError();
 }

@@ -78,6 +78,34 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, long l
     if (clock64() - t0 > limit) return false;
   }
 }
+// The MMA-issuing warps run their waits with all 32 lanes and have to go on together: mbar_poll for the operands of some
+// products, the products, one vote, and only then the commits that let any of those barriers move on (behind the products
+// the vote costs nothing; in front of them it cost 2 %). A lane that falls behind its warp may test a phase only after the
+// others have moved the barrier on by two, and then waits for a phase that has passed until the limit runs out. (Without
+// the vote that happened about once in 10^5 rounds of a forward pass over two-tile segments with one head per KV head: a
+// lane other than the elected one gave up after two seconds.) Polled, not suspended: waking up takes longer than a poll,
+// and these two warps are what everybody waits for.
+__device__ __forceinline__ bool mbar_poll(uint64_t* bar, uint32_t parity, long long limit) {
+  const long long t0 = clock64();
+#pragma unroll 1
+  for (;;) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(smem_u32(bar)), "r"(parity)
+        : "memory");
+    if (ok) return true;
+    if (clock64() - t0 > limit) return false;
+  }
+}
+// On the way out after a failed wait: the products issued last finish before the CTA gives up its TMEM.
+__device__ __forceinline__ void drain_products() {
+  const long long t0 = clock64();
+  while (clock64() - t0 < 20000) __nanosleep(500);
+}
 // ---------------------------------------------------------------- fences
 __device__ __forceinline__ void fence_proxy_async_smem() {
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");

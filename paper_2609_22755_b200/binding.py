@@ -152,13 +152,11 @@ def _i32(a):
 def _ptr(t):
     """Address of a torch tensor / numpy array (host metadata only) / int / None. Tensor arguments of the compute
     calls are validated by _check_tensors before they get here."""
-    if t is None:
-        return None
-    if isinstance(t, int):
-        return ctypes.c_void_p(t)
+    if t is None or isinstance(t, int):
+        return t
     if isinstance(t, np.ndarray):
-        return t.ctypes.data_as(ctypes.c_void_p)
-    return ctypes.c_void_p(t.data_ptr())
+        return t.ctypes.data
+    return t.data_ptr()
 
 
 def _check_tensors(what, plan, specs):
@@ -167,16 +165,19 @@ def _check_tensors(what, plan, specs):
     Sizes of zero need no buffer at all."""
     import torch
 
+    tensor, here = torch.Tensor, None
     for name, t, dtypes, need in specs:
         if need == 0:
             continue
-        if not isinstance(t, torch.Tensor) or not t.is_cuda or not t.is_contiguous():
+        if not isinstance(t, tensor) or not t.is_cuda or not t.is_contiguous():
             raise NspError(NSP_ERR_INVALID_ARG, f"{what}: {name} must be a contiguous CUDA tensor")
         if t.dtype not in dtypes:
             raise NspError(NSP_ERR_INVALID_ARG, f"{what}: {name} has dtype {t.dtype}")
         if t.numel() < need:
             raise NspError(NSP_ERR_INVALID_ARG, f"{what}: {name} holds {t.numel()} elements, the plan needs {need}")
-        if t.device.index != torch.cuda.current_device():
+        if here is None:
+            here = torch.cuda.current_device()
+        if t.get_device() != here:
             raise NspError(NSP_ERR_INVALID_ARG, f"{what}: {name} is on {t.device}, not on the current device")
 
 
@@ -206,13 +207,13 @@ def _check_ws(what, ws):
 
 
 def _stream_ptr(stream):
+    """Address of a stream (None: the current one; its handle is asked for directly, building a Stream object around it
+    costs 3 us of a call)."""
     if stream is None:
         import torch
 
-        stream = torch.cuda.current_stream()
-    if isinstance(stream, int):
-        return ctypes.c_void_p(stream)
-    return ctypes.c_void_p(stream.cuda_stream)
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+    return stream if isinstance(stream, int) else stream.cuda_stream
 
 
 class Plan:
@@ -405,15 +406,15 @@ def nsp_route_sp_tree(lengths, cost, n_levels, prefix_k, beam_w, b_tok, monotone
 
 
 def _a2a(fn_name, src, dst, tokens, heads, heads_per_block, head_dim, first_head, stream):
-    import numpy as np
     import torch
 
     dtype = NSP_F32 if src.dtype == torch.float32 else NSP_BF16
     if dst.dtype != src.dtype:
         raise ValueError("source and destination must have the same dtype")
-    fh = np.ascontiguousarray(first_head, dtype=np.int32)
-    rc = getattr(lib(), fn_name)(_ptr(src), _ptr(dst), int(tokens), int(heads), int(heads_per_block), len(fh),
-                                 int(head_dim), dtype, fh.ctypes.data_as(ctypes.c_void_p), _stream_ptr(stream))
+    n = len(first_head)
+    fh = (ctypes.c_int32 * n)(*[int(h) for h in first_head])
+    rc = getattr(lib(), fn_name)(_ptr(src), _ptr(dst), int(tokens), int(heads), int(heads_per_block), n, int(head_dim), dtype,
+                                 fh, _stream_ptr(stream))
     if rc != NSP_OK:
         raise NspError(rc, fn_name)
 

@@ -12,10 +12,11 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include "../../include/nsp.h"
+#include "nsp_internal.cuh"
+#include "sm100_ptx.cuh"
 
-namespace nsp {
-void count_launches(int n);
-}
+using nsp::grid_launch_dependents;
+using nsp::grid_wait_predecessor;
 
 namespace {
 
@@ -26,9 +27,14 @@ struct HeadMap {
 // Both kernels are launched with a thread count that is a multiple of the 16-byte vectors of one token row of the
 // side they iterate over, so a thread keeps its (head, vector) position for the whole grid-stride loop and only the
 // token (and, for the gather, the block) advances: no division inside the loop.
+// The grid is one wave of 1,024 threads per SM, and a thread has four 16-byte loads in flight: 64 KB per SM, against the
+// ~40 KB that 6.5 TB/s needs at the latency of DRAM. With one or two loads and four waves of blocks the copies ran at
+// 5.8 TB/s (a degree-8 node's gathers and scatters around one 393,216-token sample, 4.1 GB in eight launches: 714 us, now
+// 690; a degree-2 node with 19,380 tokens 172 -> 138 us; 5, 6 and 8 blocks per SM, with fewer registers: 698, 729, 818).
+// The launches follow one another with programmatic serialization (each waits for its predecessor first thing).
 
 // one thread per 16 bytes of the packed side [n][T, Hd, D]
-__global__ void __launch_bounds__(256) gather_heads_kernel(const uint4* __restrict__ src, uint4* __restrict__ dst,
+__global__ void __launch_bounds__(256, 4) gather_heads_kernel(const uint4* __restrict__ src, uint4* __restrict__ dst,
                                                            int64_t T, int H, int Hd, int n, int vec_per_row,
                                                            const __grid_constant__ HeadMap map) {
   const int row = Hd * vec_per_row;  // vectors of one token inside a block
@@ -37,13 +43,22 @@ __global__ void __launch_bounds__(256) gather_heads_kernel(const uint4* __restri
   const int in_row = static_cast<int>(t0 % row);
   const int hh = in_row / vec_per_row, v = in_row - hh * vec_per_row;
   const int64_t tok_step = threads / row;
+  const int64_t s_step = tok_step * H * vec_per_row, d_step = tok_step * row;
   int64_t tok = t0 / row;
-  int p = 0;
-  for (;;) {
-    while (tok >= T && p < n) tok -= T, ++p;
-    if (p >= n) break;
-    dst[(p * T + tok) * row + in_row] = __ldg(src + (tok * H + map.first_head[p] + hh) * vec_per_row + v);
-    tok += tok_step;
+  grid_wait_predecessor();
+  grid_launch_dependents();
+  for (int p = 0; p < n; ++p) {
+    const uint4* s1 = src + (tok * H + map.first_head[p] + hh) * vec_per_row + v;
+    uint4* d1 = dst + (p * T + tok) * row + in_row;
+    for (; tok + 3 * tok_step < T; tok += 4 * tok_step, s1 += 4 * s_step, d1 += 4 * d_step) {
+      uint4 x[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) x[u] = __ldg(s1 + u * s_step);
+#pragma unroll
+      for (int u = 0; u < 4; ++u) d1[u * d_step] = x[u];
+    }
+    for (; tok < T; tok += tok_step, s1 += s_step, d1 += d_step) *d1 = __ldg(s1);
+    tok -= T;  // the walk goes on in the next block
   }
 }
 
@@ -55,7 +70,7 @@ __global__ void __launch_bounds__(256) gather_heads_kernel(const uint4* __restri
 struct PeerBases {
   uint4* base[NSP_A2A_MAX_PEERS];
 };
-__global__ void __launch_bounds__(256) gather_heads_to_kernel(const uint4* __restrict__ src, int64_t T, int H, int Hd,
+__global__ void __launch_bounds__(256, 4) gather_heads_to_kernel(const uint4* __restrict__ src, int64_t T, int H, int Hd,
                                                               int n, int vec_per_row, int n_samples,
                                                               const int64_t* __restrict__ sample_off,
                                                               const int64_t* __restrict__ dst_row,
@@ -69,6 +84,8 @@ __global__ void __launch_bounds__(256) gather_heads_to_kernel(const uint4* __res
   const int64_t tok_step = threads / row;
   int64_t tok = t0 / row;
   int p = 0;
+  grid_wait_predecessor();
+  grid_launch_dependents();
   for (;;) {
     while (tok >= T && p < n) tok -= T, ++p;
     if (p >= n) break;
@@ -84,10 +101,10 @@ __global__ void __launch_bounds__(256) gather_heads_to_kernel(const uint4* __res
 }
 
 // one thread per 16 bytes of the [T, H, D] side; the blocks that carry the thread's head are found once, the common
-// case of exactly one is a plain copy (two tokens per pass, so that two loads are in flight), several are added in
-// block order in fp32
+// case of exactly one is a plain copy (four tokens per pass), several are added in block order in fp32 (two: two tokens per
+// pass, four loads in flight as well)
 template <bool kF32>
-__global__ void __launch_bounds__(256) scatter_heads_kernel(const uint4* __restrict__ src, uint4* __restrict__ dst,
+__global__ void __launch_bounds__(256, 4) scatter_heads_kernel(const uint4* __restrict__ src, uint4* __restrict__ dst,
                                                             int64_t T, int H, int Hd, int n, int vec_per_row,
                                                             const __grid_constant__ HeadMap map) {
   const int row = H * vec_per_row;
@@ -97,6 +114,8 @@ __global__ void __launch_bounds__(256) scatter_heads_kernel(const uint4* __restr
   const int h = in_row / vec_per_row, v = in_row - h * vec_per_row;
   const int64_t tok_step = threads / row;
   const int64_t per_block = T * Hd * vec_per_row;
+  grid_wait_predecessor();
+  grid_launch_dependents();
   uint64_t hits = 0;
   for (int p = 0; p < n; ++p) {
     const int hh = h - map.first_head[p];
@@ -109,12 +128,33 @@ __global__ void __launch_bounds__(256) scatter_heads_kernel(const uint4* __restr
     const uint4* s1 = src + p * per_block + static_cast<int64_t>(h - map.first_head[p]) * vec_per_row + v;
     const int64_t srow = static_cast<int64_t>(Hd) * vec_per_row;
     int64_t tok = t0 / row;
-    for (; tok + tok_step < T; tok += 2 * tok_step) {
-      const uint4 a = __ldg(s1 + tok * srow), b = __ldg(s1 + (tok + tok_step) * srow);
-      dst[tok * row + in_row] = a;  // a plain copy keeps the bits
-      dst[(tok + tok_step) * row + in_row] = b;
+    for (; tok + 3 * tok_step < T; tok += 4 * tok_step) {
+      uint4 x[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) x[u] = __ldg(s1 + (tok + u * tok_step) * srow);
+#pragma unroll
+      for (int u = 0; u < 4; ++u) dst[(tok + u * tok_step) * row + in_row] = x[u];  // a plain copy keeps the bits
     }
-    if (tok < T) dst[tok * row + in_row] = __ldg(s1 + tok * srow);
+    for (; tok < T; tok += tok_step) dst[tok * row + in_row] = __ldg(s1 + tok * srow);
+    return;
+  }
+  if (cnt == 2 && kF32) {
+    const int p0 = __ffsll(static_cast<long long>(hits)) - 1, p1 = __ffsll(static_cast<long long>(hits & (hits - 1))) - 1;
+    const float4* sa = reinterpret_cast<const float4*>(src + p0 * per_block) + static_cast<int64_t>(h - map.first_head[p0]) * vec_per_row + v;
+    const float4* sb = reinterpret_cast<const float4*>(src + p1 * per_block) + static_cast<int64_t>(h - map.first_head[p1]) * vec_per_row + v;
+    float4* d1 = reinterpret_cast<float4*>(dst) + in_row;
+    const int64_t srow = static_cast<int64_t>(Hd) * vec_per_row;
+    auto add = [](float4 a, float4 b) {  // from zero, in block order, as below
+      return make_float4((0.f + a.x) + b.x, (0.f + a.y) + b.y, (0.f + a.z) + b.z, (0.f + a.w) + b.w);
+    };
+    int64_t tok = t0 / row;
+    for (; tok + tok_step < T; tok += 2 * tok_step) {
+      const float4 a0 = __ldg(sa + tok * srow), a1 = __ldg(sa + (tok + tok_step) * srow);
+      const float4 b0 = __ldg(sb + tok * srow), b1 = __ldg(sb + (tok + tok_step) * srow);
+      d1[tok * row] = add(a0, b0);
+      d1[(tok + tok_step) * row] = add(a1, b1);
+    }
+    if (tok < T) d1[tok * row] = add(__ldg(sa + tok * srow), __ldg(sb + tok * srow));
     return;
   }
   for (int64_t tok = t0 / row; tok < T; tok += tok_step) {
@@ -183,13 +223,13 @@ int check(const void* src, void* dst, int64_t tokens, int heads, int heads_per_b
 }
 
 // Blocks of 256 threads whose total is a multiple of `row` (the vectors of one token row), about `total` threads but
-// no more than 32 blocks per SM.
+// no more than 4 blocks per SM (one wave: the kernels take up to 64 registers).
 int grid_for(int64_t total, int row) {
   int a = row, b = 256;
   while (b) { const int t = a % b; a = b; b = t; }
   const int unit = row / a;  // blocks per multiple of `row`
   int64_t blocks = (total + 255) / 256;
-  if (blocks > 148 * 32) blocks = 148 * 32;
+  if (blocks > 148 * 4) blocks = 148 * 4 / unit * unit;
   blocks = (blocks + unit - 1) / unit * unit;
   return static_cast<int>(blocks < unit ? unit : blocks);
 }
@@ -205,10 +245,10 @@ extern "C" int nsp_a2a_gather_heads(const void* src, void* dst, int64_t tokens, 
   const int vec = head_dim * (dtype == NSP_F32 ? 4 : 2) / 16;
   const int64_t total = tokens * heads_per_block * vec * n_blocks;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  gather_heads_kernel<<<grid_for(total, heads_per_block * vec), 256, 0, st>>>(static_cast<const uint4*>(src), static_cast<uint4*>(dst),
-                                                          tokens, heads, heads_per_block, n_blocks, vec, map);
   nsp::count_launches(1);
-  return cudaGetLastError() == cudaSuccess ? NSP_OK : NSP_ERR_CUDA;
+  return nsp::launch_chained_if(true, gather_heads_kernel, grid_for(total, heads_per_block * vec), 256, 0, st,
+                                static_cast<const uint4*>(src), static_cast<uint4*>(dst), tokens, heads, heads_per_block,
+                                n_blocks, vec, map) == cudaSuccess ? NSP_OK : NSP_ERR_CUDA;
 }
 
 extern "C" int nsp_a2a_scatter_heads(const void* src, void* dst, int64_t tokens, int32_t heads, int32_t heads_per_block,
@@ -220,14 +260,11 @@ extern "C" int nsp_a2a_scatter_heads(const void* src, void* dst, int64_t tokens,
   const int vec = head_dim * (dtype == NSP_F32 ? 4 : 2) / 16;
   const int64_t total = tokens * heads * vec;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  if (dtype == NSP_F32)
-    scatter_heads_kernel<true><<<grid_for(total, heads * vec), 256, 0, st>>>(static_cast<const uint4*>(src), static_cast<uint4*>(dst),
-                                                                tokens, heads, heads_per_block, n_blocks, vec, map);
-  else
-    scatter_heads_kernel<false><<<grid_for(total, heads * vec), 256, 0, st>>>(static_cast<const uint4*>(src), static_cast<uint4*>(dst),
-                                                                 tokens, heads, heads_per_block, n_blocks, vec, map);
   nsp::count_launches(1);
-  return cudaGetLastError() == cudaSuccess ? NSP_OK : NSP_ERR_CUDA;
+  return nsp::launch_chained_if(true, dtype == NSP_F32 ? scatter_heads_kernel<true> : scatter_heads_kernel<false>,
+                                grid_for(total, heads * vec), 256, 0, st, static_cast<const uint4*>(src),
+                                static_cast<uint4*>(dst), tokens, heads, heads_per_block, n_blocks, vec,
+                                map) == cudaSuccess ? NSP_OK : NSP_ERR_CUDA;
 }
 
 extern "C" int nsp_a2a_gather_heads_to(const void* src, void* const* dst_base, const int64_t* dst_row,
@@ -248,9 +285,8 @@ extern "C" int nsp_a2a_gather_heads_to(const void* src, void* const* dst_base, c
   const int vec = head_dim * (dtype == NSP_F32 ? 4 : 2) / 16;
   const int64_t total = tokens * heads_per_block * vec * n_blocks;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  gather_heads_to_kernel<<<grid_for(total, heads_per_block * vec), 256, 0, st>>>(
-      static_cast<const uint4*>(src), tokens, heads, heads_per_block, n_blocks, vec, n_samples, sample_off, dst_row, map,
-      peers);
   nsp::count_launches(1);
-  return cudaGetLastError() == cudaSuccess ? NSP_OK : NSP_ERR_CUDA;
+  return nsp::launch_chained_if(true, gather_heads_to_kernel, grid_for(total, heads_per_block * vec), 256, 0, st,
+                                static_cast<const uint4*>(src), tokens, heads, heads_per_block, n_blocks, vec, n_samples,
+                                sample_off, dst_row, map, peers) == cudaSuccess ? NSP_OK : NSP_ERR_CUDA;
 }

@@ -463,14 +463,14 @@ __global__ void __launch_bounds__(Roles<FIRST, D>::kThreads, 1) bwd_kernel(const
           constexpr uint32_t kStageStep = kOpBytes >> 4;  // descriptor distance between Q stages
           const int steps = cx->steps, item_it = cx->it;
           int where = 0;
-          bool okm = together(mbar_poll(&s.bar_kv, gi & 1, a.wait_limit));
+          bool okm = together(mbar_wait(&s.bar_kv, gi & 1, a.wait_limit));
           if (!okm) where = kWhereBwdLoadKV;
           const uint32_t q0_lo = smem_desc_addr(s.q[0][0]), do0_lo = smem_desc_addr(s.d_o[0][0]);
           if (is_a) {
             const uint32_t k_km = smem_desc_addr(s.k[0]) | lbo_km;
             // S^T of the next step not yet issued -> R0 (A = K, B = Q of the ring stage, both K-major)
             auto issue_s = [&]() -> bool {
-              const bool here = mbar_poll(&s.bar_q_full[qr.st], qr.ph, a.wait_limit);
+              const bool here = mbar_wait(&s.bar_q_full[qr.st], qr.ph, a.wait_limit);
               tc_fence_after_sync();
               const bool go = leader && here;
               const uint32_t b_lo = (q0_lo + qr.st * kStageStep) | lbo_km;
@@ -491,8 +491,8 @@ __global__ void __launch_bounds__(Roles<FIRST, D>::kThreads, 1) bwd_kernel(const
               const bool calm = *abort_flag == 0;
               const uint32_t cs = gs + vt;
               const uint32_t do_lo = do0_lo + do_stage(cs) * kStageStep;
-              bool here = mbar_poll(&s.bar_do_full[do_stage(cs)], do_parity(cs), a.wait_limit);
-              here = mbar_poll(&s.bar_p_ready, cs & 1, a.wait_limit) && here;
+              bool here = mbar_wait(&s.bar_do_full[do_stage(cs)], do_parity(cs), a.wait_limit);
+              here = mbar_wait(&s.bar_p_ready, cs & 1, a.wait_limit) && here;
               tc_fence_after_sync();
               const bool go = leader && here;
               const uint32_t acc = vt > 0;
@@ -527,8 +527,8 @@ __global__ void __launch_bounds__(Roles<FIRST, D>::kThreads, 1) bwd_kernel(const
             auto issue_dp = [&](int vt) -> bool {
               const uint32_t cs = gs + vt;
               const uint32_t do_lo = do0_lo + do_stage(cs) * kStageStep;
-              bool here = mbar_poll(&s.bar_do_full[do_stage(cs)], do_parity(cs), a.wait_limit);
-              if constexpr (!kOwnDq) here = mbar_poll(&s.bar_dq_empty, (cs & 1) ^ 1, a.wait_limit) && here;
+              bool here = mbar_wait(&s.bar_do_full[do_stage(cs)], do_parity(cs), a.wait_limit);
+              if constexpr (!kOwnDq) here = mbar_wait(&s.bar_dq_empty, (cs & 1) ^ 1, a.wait_limit) && here;
               tc_fence_after_sync();
               const bool go = leader && here;
 #pragma unroll
@@ -546,12 +546,12 @@ __global__ void __launch_bounds__(Roles<FIRST, D>::kThreads, 1) bwd_kernel(const
               constexpr bool fold = FIRST;
               const bool calm = *abort_flag == 0;
               const uint32_t cs = gs + vt;
-              bool here = mbar_poll(&s.bar_q_full[qr.st], qr.ph, a.wait_limit);
-              here = mbar_poll(&s.bar_ds_ready, cs & 1, a.wait_limit) && here;
+              bool here = mbar_wait(&s.bar_q_full[qr.st], qr.ph, a.wait_limit);
+              here = mbar_wait(&s.bar_ds_ready, cs & 1, a.wait_limit) && here;
               if constexpr (kOwnDq) {
                 if (!together(here && calm)) { where = kWhereBwdDsReady; return false; }
                 if (vt + 1 < steps && !issue_dp(vt + 1)) return false;
-                here = mbar_poll(&s.bar_dq_empty, (cs & 1) ^ 1, a.wait_limit);
+                here = mbar_wait(&s.bar_dq_empty, (cs & 1) ^ 1, a.wait_limit);
               }
               tc_fence_after_sync();
               const bool go = leader && here;
@@ -932,15 +932,45 @@ __global__ void __launch_bounds__(Roles<FIRST, D>::kThreads, 1) bwd_kernel(const
           // would push dK / dV past the tolerance: P^T and dS^T enter their products as bf16 value plus bf16 residual
           // (two products each, the residuals next to the values), and delta_i = sum_j P_ij dP_ij is taken here in
           // fp32 (all keys of these rows sit in this tile) instead of from the bf16-rounded O.
-          oks = mbar_wait(&s.bar_dp_full, cs & 1, a.wait_limit);
-          oks = __all_sync(0xffffffffu, oks);
-          if (!oks) { where = kWhereBwdDp; break; }
-          tc_fence_after_sync();
           uint32_t pkk[kChunks][16];
           {
-            // Sweep 1: P^T (value and residual over the S^T columns just read: packed columns [16ch, 16ch + 8) and
-            // [16ch + 8, 16ch + 16)) and the partial sums of delta. The packed values stay in registers for sweep 2
-            // (both sweeps fully unrolled), so R0 is free for the next S^T as soon as the dV products have run.
+            // Sweep 1: P^T, value and residual over the S^T columns just read (packed columns [16ch, 16ch + 8) and
+            // [16ch + 8, 16ch + 16)). The packed values stay in registers for the other sweeps (all fully unrolled), so R0 is
+            // free for the next S^T as soon as the dV products have run. It needs no dP^T, which arrives ~2,500 clocks after
+            // the previous step's dS^T (behind that step's dQ^T, its drain and dK); taken with the partial sums of delta in
+            // one sweep behind dP^T, as it was, 1,024 segments of 128 tokens took 3,521 us a step (now 3,448; 98,275 tokens in
+            // 100-token segments at head_dim 64 2,013 -> 1,935).
+#pragma unroll
+            for (int ch = 0; ch < kChunks; ++ch) {
+              uint32_t sv[16];
+              uint32_t* const pk = pkk[ch];
+              float4 l4[4];
+#pragma unroll
+              for (int i = 0; i < 4; ++i) l4[i] = lds128(lse_s + ch * 16 + 4 * i);
+              tmem_ld16(tS + ch * 16, sv);
+              tmem_wait_ld();
+#pragma unroll
+              for (int x = 0; x < 16; x += 2) {
+                const float lse0 = (x & 2) ? l4[x >> 2].z : l4[x >> 2].x, lse1 = (x & 2) ? l4[x >> 2].w : l4[x >> 2].y;
+                float p0 = ex2f(fmaf(__uint_as_float(sv[x + 0]), a.scale_log2, -lse0));
+                float p1 = ex2f(fmaf(__uint_as_float(sv[x + 1]), a.scale_log2, -lse1));
+                const int qc = col0 + ch * 16 + x;
+                if (qc + 0 < r || qc + 0 >= r_end) p0 = 0.f;  // query index must be >= key index, inside its segment
+                if (qc + 1 < r || qc + 1 >= r_end) p1 = 0.f;
+                const uint32_t pa = pack_bf16x2(p0, p1);
+                pk[x >> 1] = pa;
+                pk[8 + (x >> 1)] = pack_bf16x2(p0 - __uint_as_float(pa << 16), p1 - __uint_as_float(pa & 0xffff0000u));
+              }
+              tmem_st16(tS + ch * 16, pk);
+            }
+            tmem_wait_st();
+            tc_fence_before_sync();
+            mbar_arrive(&s.bar_p_ready);  // the dV products run under the rest of this step
+            oks = mbar_wait(&s.bar_dp_full, cs & 1, a.wait_limit);
+            oks = __all_sync(0xffffffffu, oks);
+            if (!oks) { where = kWhereBwdDp; break; }
+            tc_fence_after_sync();
+            // Sweep 2: the partial sums of delta (P = value + residual to 2^-17)
             // [4 quadrants][kCols columns]; with two column groups in the group's own half of dS^T, which is free until the
             // group itself writes it
             float* part = kSoft == 2 ? reinterpret_cast<float*>(s.ds[wg & 1]) : s.part + wg * 4 * kCols;
@@ -950,30 +980,17 @@ __global__ void __launch_bounds__(Roles<FIRST, D>::kThreads, 1) bwd_kernel(const
             const bool b4 = lane & 16, b3 = lane & 8, b2 = lane & 4, b1 = lane & 2;
 #pragma unroll
             for (int ch = 0; ch < kChunks; ++ch) {
-              uint32_t sv[16], dpv[16];
-              uint32_t* const pk = pkk[ch];
-              float4 l4[4];
-#pragma unroll
-              for (int i = 0; i < 4; ++i) l4[i] = lds128(lse_s + ch * 16 + 4 * i);
-              tmem_ld16(tS + ch * 16, sv);
+              uint32_t dpv[16];
+              const uint32_t* const pk = pkk[ch];
               tmem_ld16(tDP + ch * 16, dpv);
               tmem_wait_ld();
               float v[16];
 #pragma unroll
               for (int x = 0; x < 16; x += 2) {
-                const float lse0 = (x & 2) ? l4[x >> 2].z : l4[x >> 2].x, lse1 = (x & 2) ? l4[x >> 2].w : l4[x >> 2].y;
-                float p0 = ex2f(fmaf(__uint_as_float(sv[x + 0]), a.scale_log2, -lse0));
-                float p1 = ex2f(fmaf(__uint_as_float(sv[x + 1]), a.scale_log2, -lse1));
-                const int qc = col0 + ch * 16 + x;
-                if (qc + 0 < r || qc + 0 >= r_end) p0 = 0.f;  // query index must be >= key index, inside its segment
-                if (qc + 1 < r || qc + 1 >= r_end) p1 = 0.f;
-                v[x + 0] = p0 * __uint_as_float(dpv[x + 0]);
-                v[x + 1] = p1 * __uint_as_float(dpv[x + 1]);
-                const uint32_t pa = pack_bf16x2(p0, p1);
-                pk[x >> 1] = pa;
-                pk[8 + (x >> 1)] = pack_bf16x2(p0 - __uint_as_float(pa << 16), p1 - __uint_as_float(pa & 0xffff0000u));
+                const uint32_t ph = pk[x >> 1], pl = pk[8 + (x >> 1)];
+                v[x + 0] = (__uint_as_float(ph << 16) + __uint_as_float(pl << 16)) * __uint_as_float(dpv[x + 0]);
+                v[x + 1] = (__uint_as_float(ph & 0xffff0000u) + __uint_as_float(pl & 0xffff0000u)) * __uint_as_float(dpv[x + 1]);
               }
-              tmem_st16(tS + ch * 16, pk);
               float w8[8], w4[4], w2[2];
 #pragma unroll
               for (int i = 0; i < 8; ++i)
@@ -988,9 +1005,6 @@ __global__ void __launch_bounds__(Roles<FIRST, D>::kThreads, 1) bwd_kernel(const
               w1 += __shfl_xor_sync(0xffffffffu, w1, 1);
               if ((lane & 1) == 0) part[quad * kCols + ch * 16 + (lane >> 1)] = w1;
             }
-            tmem_wait_st();
-            tc_fence_before_sync();
-            mbar_arrive(&s.bar_p_ready);  // the dV products run under the rest of this step
             mbar_arrive(&s.bar_delta[wg]);
             oks = mbar_wait(&s.bar_delta[wg], nd & 1, a.wait_limit);
             ++nd;
@@ -1003,7 +1017,7 @@ __global__ void __launch_bounds__(Roles<FIRST, D>::kThreads, 1) bwd_kernel(const
             oks = __all_sync(0xffffffffu, oks);
             if (!oks) { where = kWhereBwdDelta; break; }
           }
-          // Sweep 2: dS^T = P^T o (dP^T - delta), value and residual (P = value + residual to 2^-17)
+          // Sweep 3: dS^T = P^T o (dP^T - delta), value and residual
           if constexpr (kOwnDq) {
             oks = ds_free();
             oks = __all_sync(0xffffffffu, oks);

@@ -51,6 +51,8 @@ struct nsp_plan {
   int32_t* d_turns = nullptr;               // turn counters of the divided items
   nsp_tile_t* d_bwd_first = nullptr;  // one item per (segment or pack, kv head): the first-tile kernels' list
   int64_t n_first = 0;
+  nsp_tile_t* d_fwd_first = nullptr;  // the first-tile forward kernel's list: d_bwd_first, or with pairs of KV heads (cost 2)
+  int64_t n_fwd_first = 0;
   RowInfo* d_rows = nullptr;          // row tables of the packs, 128 entries each (d_seg holds the packs' entries after
   int64_t n_packs = 0;                // the n_seg segments')
   nsp_tile_t* d_fwd_pairs = nullptr;  // the forward items that visit at least two key tiles, in the pairs the general
@@ -432,6 +434,25 @@ int nsp_plan_tiles(const int32_t* cu_seqlens, const int32_t* hq, const int32_t* 
     delete p;
     return NSP_ERR_UNSUPPORTED;
   }
+  // Two KV heads of one q head each as one item of the first-tile forward kernel: its two halves then both work, for a
+  // little more latency per item, so only where there are more items than SMs (16q/16kv, forward: 56,657 tokens in segments
+  // of about 100 423 -> 363 us, at head_dim 64 319 -> 261).
+  std::vector<nsp_tile_t> fwd_first;
+  if (p->n_first > p->num_sms) {
+    try {
+      for (const nsp_tile_t& t : bwd_first) {
+        const int hkv = (t.seg < n_seg ? p->seg[t.seg] : pack_segs[t.seg - n_seg]).hkv;
+        if (t.cost > 1)
+          fwd_first.push_back(t);
+        else if (t.head % 2 == 0)
+          fwd_first.push_back(nsp_tile_t{t.seg, t.head, 0, t.head + 1 < hkv ? 2 : 1});
+      }
+    } catch (...) {
+      delete p;
+      return NSP_ERR_ALLOC;
+    }
+    if (fwd_first.size() == bwd_first.size()) fwd_first.clear();
+  }
   std::vector<nsp_tile_t> parts, first_parts;
   int32_t n_turns = 0;
   try {
@@ -478,6 +499,7 @@ int nsp_plan_tiles(const int32_t* cu_seqlens, const int32_t* hq, const int32_t* 
   const size_t o_tiles = take(sizeof(int32_t) * (n_seg + 1));
   const size_t o_parts = take(sizeof(nsp_tile_t) * parts.size());
   const size_t o_first_parts = take(sizeof(nsp_tile_t) * first_parts.size());
+  const size_t o_fwd_first = take(sizeof(nsp_tile_t) * fwd_first.size());
   const size_t o_turns = take(sizeof(int32_t) * n_turns);
   const size_t upload = at;
   const size_t o_fwd = take(sizeof(nsp_tile_t) * nf);
@@ -505,6 +527,8 @@ int nsp_plan_tiles(const int32_t* cu_seqlens, const int32_t* hq, const int32_t* 
   p->d_bwd_parts = reinterpret_cast<nsp_tile_t*>(d + o_parts);
   p->d_bwd_first_parts = reinterpret_cast<nsp_tile_t*>(d + o_first_parts);
   p->d_turns = reinterpret_cast<int32_t*>(d + o_turns);
+  p->d_fwd_first = fwd_first.empty() ? p->d_bwd_first : reinterpret_cast<nsp_tile_t*>(d + o_fwd_first);
+  p->n_fwd_first = fwd_first.empty() ? p->n_first : static_cast<int64_t>(fwd_first.size());
   p->h_status = static_cast<int32_t*>(p->arena->host);
   p->h_status_dev = reinterpret_cast<int32_t*>(p->arena->host_dev);
   char* const image = static_cast<char*>(p->arena->host) + 256;
@@ -522,6 +546,7 @@ int nsp_plan_tiles(const int32_t* cu_seqlens, const int32_t* hq, const int32_t* 
   put(o_tiles, tile_base.data(), sizeof(int32_t) * (n_seg + 1));
   put(o_parts, parts.data(), sizeof(nsp_tile_t) * parts.size());
   put(o_first_parts, first_parts.data(), sizeof(nsp_tile_t) * first_parts.size());
+  put(o_fwd_first, fwd_first.data(), sizeof(nsp_tile_t) * fwd_first.size());
   std::memset(image + o_turns, 0, sizeof(int32_t) * n_turns);
   // On the arena's own stream, so that the plan is complete when this call returns without waiting for the work the
   // caller has enqueued before (nothing here depends on it).
@@ -607,8 +632,9 @@ int nsp_attn_fwd(const nsp_plan_t* plan, const void* q, const void* k, const voi
   a.delta = nullptr;
   NSP_LOGF("fwd plan %p stream %p scale %g", static_cast<const void*>(plan), stream, softmax_scale);
   // q tile 0 of every segment (the cost-1 tail of the list): one item per (segment, kv head)
-  a.items = plan->d_bwd_first;
-  a.n_items = static_cast<int32_t>(plan->n_first);
+  a.pairs = plan->d_fwd_first != plan->d_bwd_first;
+  a.items = plan->d_fwd_first;
+  a.n_items = static_cast<int32_t>(plan->n_fwd_first);
   a.counter = plan->d_counters + 3;
   prof_mark(plan, NSP_KERNEL_FWD_FIRST, 0, st);
   if (!plan->withhold && launch_fwd_first(maps, a, plan->head_dim, plan->num_sms, st) != cudaSuccess) return NSP_ERR_CUDA;
@@ -698,6 +724,7 @@ int bwd_impl(const nsp_plan_t* plan, const uint8_t* recompute, const void* q, co
     fa.lse_elems = plan->lse_elems;
     fa.seg_mask = d_mask;
     fa.rows = plan->d_rows;
+    fa.pairs = 0;
     fa.d_o = static_cast<const __nv_bfloat16*>(d_o);
     fa.delta = delta;
     prof_mark(plan, NSP_KERNEL_FWD, 0, st);

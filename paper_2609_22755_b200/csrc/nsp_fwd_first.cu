@@ -10,6 +10,8 @@
 // key tile, so the softmax needs no running maximum and no rescaling. (A variant without the CTA-wide barrier between
 // items -- the producer popping ahead and publishing items through a two-slot mailbox -- measured slower: 0.89 ms
 // against 0.77 ms on 1,024 segments of 128 tokens.)
+// Where every q head has a KV head of its own an item is two KV heads (a pair list, see nsp_api.cu): A and B are then the two
+// heads, and B's K and V wait in the other stage of the Q ring, which one round per item leaves free.
 // The general kernel then runs only the items that visit at least two key tiles: the first-tile items are exactly
 // the tail (cost 1) of the longest-first forward list.
 //     S_x  = Q_x K^T        tcgen05.mma SS (both K-major)                      -> TMEM S_x
@@ -34,6 +36,7 @@ struct FirstCtx {
   int32_t it;  // position in the list (>= n_items: no more work)
   int32_t len, hq, G, g, run, tok0, rounds;
   int32_t rows;  // 0, or 1 + index of the row table of a pack of short segments (see RowInfo)
+  int32_t pair;  // two KV heads of one q head each: g (A) and g + 1 (B)
 };
 
 template <int D>
@@ -70,7 +73,8 @@ __device__ __forceinline__ float ff_max3(float a, float b, float c) {
   return d;
 }
 
-template <int D>
+// PAIRS: the list holds items of two KV heads (without them the kernel carries none of that code: 1 % on the others).
+template <int D, bool PAIRS>
 __global__ void __launch_bounds__(kThreads, 1) fwd_first_kernel(const __grid_constant__ FwdMaps maps, const FwdArgs a) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   FwdFirstSmem<D>& s = *reinterpret_cast<FwdFirstSmem<D>*>(smem_raw);
@@ -129,10 +133,12 @@ __global__ void __launch_bounds__(kThreads, 1) fwd_first_kernel(const __grid_con
       x.len = sg.len, x.hq = sg.hq, x.G = sg.hq / sg.hkv, x.g = item.head, x.run = sg.run, x.tok0 = sg.tok_in_run;
       x.rounds = (x.G + 1) / 2;
       x.rows = sg.rows;
+      x.pair = item.cost == 2 && x.G == 1;
     } else {
       reset_cursor(a.counter, idx, a.n_items, 1);
     }
   };
+  auto has_b = [&](int r) -> bool { return (PAIRS && c.pair) || 2 * r + 1 < c.G; };  // B takes part in round r
   auto next_item = [&]() -> bool {
     if (tid == kPopThread && gi == 0) fetch(s.ctx[0]);
     // Every role reaches this barrier in bounded time: all its other waits are bounded and none returns early.
@@ -156,7 +162,7 @@ __global__ void __launch_bounds__(kThreads, 1) fwd_first_kernel(const __grid_con
           const CUtensorMap* mq = &maps.q[c.run];
           bool ok = mbar_wait(&s.bar_kv_free, (gi & 1) ^ 1, a.wait_limit);
           if (ok) {
-            mbar_expect_tx(&s.bar_kv, 2 * kTileBytes);
+            mbar_expect_tx(&s.bar_kv, (PAIRS && c.pair ? 4 : 2) * kTileBytes);
 #pragma unroll
             for (int hf = 0; hf < kHalves; ++hf) {
               tma_load_3d(s.k[hf], &maps.k[c.run], &s.bar_kv, 64 * hf, c.g, c.tok0);
@@ -167,7 +173,7 @@ __global__ void __launch_bounds__(kThreads, 1) fwd_first_kernel(const __grid_con
             if (*abort_flag) break;
             const uint32_t st = (R + r) & 1;
             const int hA = c.g * c.G + 2 * r;
-            const bool joint = 2 * r + 1 < c.G;
+            const bool joint = has_b(r);
             ok = mbar_wait(&s.bar_q_empty[st][0], ((use >> (2 * st)) & 1) ^ 1, a.wait_limit) &&
                  (!joint || mbar_wait(&s.bar_q_empty[st][1], ((use >> (2 * st + 1)) & 1) ^ 1, a.wait_limit));
             if (!ok) break;
@@ -179,6 +185,18 @@ __global__ void __launch_bounds__(kThreads, 1) fwd_first_kernel(const __grid_con
 #pragma unroll
               for (int hf = 0; hf < kHalves; ++hf)
                 tma_load_3d(s.q[st][1][hf], mq, &s.bar_q_full[st], 64 * hf, hA + 1, c.tok0);
+            }
+            if (PAIRS && c.pair) {  // K and V of B: the two slots of the other stage, handed back by the MMA warp
+              const uint32_t ot = st ^ 1;
+              ok = mbar_wait(&s.bar_q_empty[ot][0], ((use >> (2 * ot)) & 1) ^ 1, a.wait_limit) &&
+                   mbar_wait(&s.bar_q_empty[ot][1], ((use >> (2 * ot + 1)) & 1) ^ 1, a.wait_limit);
+              if (!ok) break;
+              use ^= 3u << (2 * ot);
+#pragma unroll
+              for (int hf = 0; hf < kHalves; ++hf) {
+                tma_load_3d(s.q[ot][0][hf], &maps.k[c.run], &s.bar_kv, 64 * hf, c.g + 1, c.tok0);
+                tma_load_3d(s.q[ot][1][hf], &maps.v[c.run], &s.bar_kv, 64 * hf, c.g + 1, c.tok0);
+              }
             }
           }
           if (!ok) {
@@ -203,9 +221,13 @@ __global__ void __launch_bounds__(kThreads, 1) fwd_first_kernel(const __grid_con
         const bool leader = elect_one();
         int where = 0;
         bool ok = true;
+        // operands of B where it has a KV head of its own (one round: its Q stage is R & 1)
+        const uint32_t other = 2 * ((R & 1) ^ 1) * kTileStep;
+        const uint32_t kb_lo = PAIRS && c.pair ? q_lo + other : k_lo;
+        const uint32_t vb_lo = PAIRS && c.pair ? (smem_desc_addr(s.q[0][0][0]) | lbo_mn) + other + kTileStep : v_lo;
         for (int r = 0; ok && r < c.rounds; ++r) {
           const uint32_t st = (R + r) & 1;
-          const int halves = 2 * r + 1 < c.G ? 2 : 1;
+          const int halves = has_b(r) ? 2 : 1;
           const bool calm = *abort_flag == 0;
           bool here = r > 0 || mbar_poll(&s.bar_kv, gi & 1, a.wait_limit);
           here = mbar_poll(&s.bar_q_full[st], ((R + r) >> 1) & 1, a.wait_limit) && here;
@@ -213,11 +235,11 @@ __global__ void __launch_bounds__(kThreads, 1) fwd_first_kernel(const __grid_con
           // S of this round follows the PV products of the previous one on the same pipe, so P of the previous
           // round has been read before S overwrites it
           for (int x = 0; x < halves; ++x) {
-            const uint32_t a_lo = q_lo + (2 * st + x) * kTileStep;
+            const uint32_t a_lo = q_lo + (2 * st + x) * kTileStep, b_lo = x ? kb_lo : k_lo;
 #pragma unroll
             for (int kk = 0; kk < D / 16; ++kk) {
               const uint32_t off = ((kk >> 2) * kHalfTileBytes + (kk & 3) * 32) >> 4;
-              if (leader && here) umma_ss_lh(tmem + 128 * x, a_lo + off, hi, k_lo + off, hi, idesc_qk, kk > 0);
+              if (leader && here) umma_ss_lh(tmem + 128 * x, a_lo + off, hi, b_lo + off, hi, idesc_qk, kk > 0);
             }
             if (x == 0 && !together(here && calm)) { ok = false; where = kWhereFwdLoad; break; }
             if (leader) umma_commit(&s.bar_s_full[x]);
@@ -228,12 +250,16 @@ __global__ void __launch_bounds__(kThreads, 1) fwd_first_kernel(const __grid_con
             tc_fence_after_sync();
 #pragma unroll
             for (int kk = 0; kk < 8; ++kk)
-              if (leader && here) umma_ts_lh(tmem + 256 + 128 * x, tmem + 128 * x + (kk >> 2) * 64 + (kk & 3) * 8, v_lo + kk * 128, hi,
+              if (leader && here) umma_ts_lh(tmem + 256 + 128 * x, tmem + 128 * x + (kk >> 2) * 64 + (kk & 3) * 8, (x ? vb_lo : v_lo) + kk * 128, hi,
                                      idesc_pv, kk > 0);
             if (!together(here)) { ok = false; where = kWhereFwdS; break; }
             if (leader) umma_commit(&s.bar_pv_done[x]);
             ++n[x];
           }
+        }
+        if (PAIRS && c.pair && leader) {
+          umma_commit(&s.bar_q_empty[(R & 1) ^ 1][0]);
+          umma_commit(&s.bar_q_empty[(R & 1) ^ 1][1]);
         }
         if (leader) umma_commit(&s.bar_kv_free);  // K and V may be replaced once everything issued so far has run
         if (!ok && where != 0) {
@@ -253,7 +279,7 @@ __global__ void __launch_bounds__(kThreads, 1) fwd_first_kernel(const __grid_con
       uint32_t R = 0, nx = 0;
       while (next_item()) {
         for (int r = 0; r < c.rounds; ++r) {
-          if (x == 1 && 2 * r + 1 >= c.G) break;
+          if (x == 1 && !has_b(r)) break;
           if (*abort_flag) break;
           if (lane == 0) {
             const uint32_t st = (R + r) & 1;
@@ -307,7 +333,7 @@ __global__ void __launch_bounds__(kThreads, 1) fwd_first_kernel(const __grid_con
         lo = ri.lo, lse_row = ri.lse_base + rl, lse_len = ri.len;
       }
       for (int r = 0; r < c.rounds; ++r) {
-        if (x == 1 && 2 * r + 1 >= c.G) break;  // an odd group's last head runs alone, as half A
+        if (x == 1 && !has_b(r)) break;  // an odd group's last head runs alone, as half A
         if (*abort_flag) { ok = false; break; }
         const int h = c.g * c.G + 2 * r + x;
         ok = mbar_wait(&s.bar_s_full[x], nx & 1, a.wait_limit);
@@ -431,21 +457,23 @@ __global__ void __launch_bounds__(kThreads, 1) fwd_first_kernel(const __grid_con
   if (warp == 0) tmem_dealloc(s.tmem_base, kTmemCols);
 }
 
-template <int D>
+template <int D, bool PAIRS>
 cudaError_t launch_t(const FwdMaps& maps, const FwdArgs& args, int num_sms, cudaStream_t st) {
-  cudaError_t e = cudaFuncSetAttribute(fwd_first_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  cudaError_t e = cudaFuncSetAttribute(fwd_first_kernel<D, PAIRS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        static_cast<int>(sizeof(FwdFirstSmem<D>)));
   if (e != cudaSuccess) return e;
   const int grid = args.n_items < num_sms ? args.n_items : num_sms;
   count_launches(1);
-  return launch_chained_if(true, fwd_first_kernel<D>, grid, kThreads, sizeof(FwdFirstSmem<D>), st, maps, args);
+  return launch_chained_if(true, fwd_first_kernel<D, PAIRS>, grid, kThreads, sizeof(FwdFirstSmem<D>), st, maps, args);
 }
 
 }  // namespace
 
 cudaError_t launch_fwd_first(const FwdMaps& maps, const FwdArgs& args, int head_dim, int num_sms, cudaStream_t st) {
   if (args.n_items == 0) return cudaSuccess;
-  return head_dim == 64 ? launch_t<64>(maps, args, num_sms, st) : launch_t<128>(maps, args, num_sms, st);
+  if (args.pairs)
+    return head_dim == 64 ? launch_t<64, true>(maps, args, num_sms, st) : launch_t<128, true>(maps, args, num_sms, st);
+  return head_dim == 64 ? launch_t<64, false>(maps, args, num_sms, st) : launch_t<128, false>(maps, args, num_sms, st);
 }
 
 }  // namespace nsp

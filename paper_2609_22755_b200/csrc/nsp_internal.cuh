@@ -156,6 +156,7 @@ struct FwdArgs {
   const __nv_bfloat16* d_o;
   float* delta;
   const RowInfo* rows;  // row tables of the packs (first-tile kernel)
+  int32_t pairs;        // first-tile kernel: the list holds items of two KV heads
 };
 
 struct BwdArgs {

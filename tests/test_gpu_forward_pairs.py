@@ -11,6 +11,11 @@ pytestmark = pytest.mark.gpu
     ([1100, 128, 640], 5, 1, 128),                     # odd group
     ([3000], 1, 1, 128),                               # one head: long pairs, next round prefetched under an unequal one
     ([700, 300, 700], [3, 4, 1], [1, 2, 1], 64),       # odd and even groups in one list
+    # first-tile items of two KV heads (more items than SMs): full tiles, ragged ones, packs, an odd head left over, and
+    # groups of two and three before and behind them
+    ([100, 128, 37, 90] * 15, 5, 5, 128),
+    ([100, 128, 37, 90] * 15, 5, 5, 64),
+    ([128, 64, 130] * 14, [4] * 3 + [6] * 36 + [3] * 3, [2] * 3 + [6] * 36 + [1] * 3, 128),
 ])
 def test_pairs_every_element(lengths, hq, hkv, head_dim):
     import torch

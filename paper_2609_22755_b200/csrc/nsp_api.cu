@@ -173,8 +173,10 @@ bool log_on() {
 inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
 inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
-// Divides backward items into parts of at most about `most` steps (see kMaxParts) and lists them, the longest first. A
-// part has its own K / V loads and its own dK / dV epilogue, ~14,000 clocks or the time of 3-4 steps.
+// Divides backward items into parts of at most about `most` steps (see kMaxParts) and lists them: the longest first where
+// the dQ accumulator is no more than twice L2 (126 MB), otherwise in the order of the items, the walked one, which keeps the
+// CTAs of a group on the same q tiles. By length / in order, us a step: 17,545 tokens at 8q/2kv (72 MB) 1,044 / 1,191,
+// 47,878 tokens at 64q/4kv in 173 segments (1.6 GB), the longest divided, 3,187 / 3,121. A part has its own K / V loads and its own dK / dV epilogue, ~14,000 clocks or the time of 3-4 steps.
 // Returns an empty list when nothing is divided.
 // Where the lines lie: an item is divided when it is longer than the SMs' share of all steps, because the longest item
 // then bounds the kernel. Microseconds a step with parts of at most share / 2, share, whole: 8,192 tokens in one
@@ -187,7 +189,7 @@ constexpr int kMinPart = 16, kMinFirstPart = 4;
 struct WholeItem {
   int32_t seg, head, tile, steps;
 };
-std::vector<nsp_tile_t> divide_items(const std::vector<WholeItem>& items, int64_t most, int32_t* n_turns) {
+std::vector<nsp_tile_t> divide_items(const std::vector<WholeItem>& items, int64_t most, bool by_length, int32_t* n_turns) {
   struct Part {
     nsp_tile_t t;
     int32_t steps;
@@ -204,7 +206,8 @@ std::vector<nsp_tile_t> divide_items(const std::vector<WholeItem>& items, int64_
   std::vector<nsp_tile_t> list;
   if (*n_turns == turn0) return list;
   // the parts of an item do not grow with their number, so a stable sort keeps them in order
-  std::stable_sort(out.begin(), out.end(), [](const Part& a, const Part& b) { return a.steps > b.steps; });
+  if (by_length)
+    std::stable_sort(out.begin(), out.end(), [](const Part& a, const Part& b) { return a.steps > b.steps; });
   for (const Part& p : out) list.push_back(p.t);
   return list;
 }
@@ -459,12 +462,16 @@ int nsp_plan_tiles(const int32_t* cu_seqlens, const int32_t* hq, const int32_t* 
     if (!p->deterministic && !p->rounded_dq) {
       std::vector<WholeItem> main_items, first_items;
       int64_t main_steps = 0, first_steps = 0;
-      for (const SegInfo& sg : p->seg) {
+      std::vector<int32_t> order(n_seg);  // the groups the way the kernel walks them
+      for (int s = 0; s < n_seg; ++s) order[s] = s;
+      std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return p->seg[x].len > p->seg[y].len; });
+      for (const int s : order) {
+        const SegInfo& sg = p->seg[s];
         const int32_t Mt = (sg.len + bm - 1) / bm, G = sg.hq / sg.hkv;
         for (int g = 0; g < sg.hkv; ++g)
           for (int32_t n = 0; n < Mt; ++n) {
             const int32_t steps = G * (Mt - std::max(n, 1));
-            if (steps > 0) main_items.push_back(WholeItem{static_cast<int32_t>(&sg - p->seg.data()), g, n, steps});
+            if (steps > 0) main_items.push_back(WholeItem{s, g, n, steps});
             main_steps += steps;
           }
       }
@@ -472,8 +479,10 @@ int nsp_plan_tiles(const int32_t* cu_seqlens, const int32_t* hq, const int32_t* 
         first_items.push_back(WholeItem{t.seg, t.head, 0, t.cost});
         first_steps += t.cost;
       }
-      parts = divide_items(main_items, std::max<int64_t>(kMinPart, main_steps / p->num_sms), &n_turns);
-      first_parts = divide_items(first_items, std::max<int64_t>(kMinFirstPart, (first_steps + main_steps) / (2 * p->num_sms)), &n_turns);
+      parts = divide_items(main_items, std::max<int64_t>(kMinPart, main_steps / p->num_sms),
+                           q_off * 4 <= (256ll << 20), &n_turns);
+      first_parts = divide_items(first_items, std::max<int64_t>(kMinFirstPart, (first_steps + main_steps) / (2 * p->num_sms)), true,
+                                 &n_turns);
     }
     p->n_parts = static_cast<int64_t>(parts.size());
     p->n_first_parts = static_cast<int64_t>(first_parts.size());

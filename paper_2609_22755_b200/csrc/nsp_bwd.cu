@@ -1209,6 +1209,9 @@ __global__ void __launch_bounds__(Roles<FIRST, D>::kThreads, 1) bwd_kernel(const
                       make_uint2(pack_bf16x2(w4[u].x, w4[u].y), pack_bf16x2(w4[u].z, w4[u].w));
             }
           }
+          // The staging buffers were written and read through the generic proxy; the TMA loads of the next item write them
+          // through the async one, with only the barrier of next_item() in between.
+          fence_proxy_async_smem();
           if (c.parts > 1) {
             __threadfence();
             const uint64_t stored = mbar_arrive_token(&s.bar_out);

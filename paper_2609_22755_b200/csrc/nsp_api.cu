@@ -564,7 +564,7 @@ int nsp_plan_tiles(const int32_t* cu_seqlens, const int32_t* hq, const int32_t* 
       launch_plan_lists(reinterpret_cast<const PlanKey*>(d + o_keys), reinterpret_cast<const int32_t*>(d + o_tiles), n_seg,
                         static_cast<int>(tiles), p->d_fwd, p->d_bwd, p->d_bwd_exec, p->d_fwd_pairs, bs) != cudaSuccess ||
       cudaStreamSynchronize(bs) != cudaSuccess) {
-    p->arena->captured = true;  // not for reuse
+    p->arena->unpooled = true;
     free_plan(p);
     return NSP_ERR_CUDA;
   }

@@ -4,10 +4,9 @@
 // segments, against 0.7 ms of kernels of a batch of 8,192 tokens.
 //
 // The idle blocks are bounded in number and bytes (beyond that the oldest are freed), and all of them are given back by
-// nsp_trim(), or when an allocation fails. An arena whose last kernels may still run is never handed out: every call on
-// a plan records the arena's event, and a plan that took part in a stream capture (its kernels may run again at any
-// replay) gives its memory back to the driver, which waits for the device.
-#include <mutex>
+// nsp_trim(), or when an allocation fails. An arena whose kernels may still run is never handed out: every call on a plan
+// records the arena's event of the call's stream, and a plan that took part in a stream capture (its kernels may run again
+// at any replay) gives its memory back to the driver, which waits for the device.
 #include <new>
 #include <vector>
 #include "nsp_arena.h"
@@ -35,7 +34,8 @@ size_t round_up_pow2(size_t n) {
 void destroy(Arena* a) {  // cudaFree waits for whatever still uses the block
   cudaFree(a->dev);
   if (a->host) cudaFreeHost(a->host);
-  if (a->done) cudaEventDestroy(a->done);
+  for (const Arena::Use& u : a->uses)
+    if (u.done) cudaEventDestroy(u.done);
   if (a->build) cudaStreamDestroy(a->build);
   delete a;
 }
@@ -51,7 +51,7 @@ Arena* create(int device, size_t dev_bytes, size_t host_bytes) {
   const bool ok = cudaMalloc(&a->dev, a->dev_bytes) == cudaSuccess &&
                   cudaHostAlloc(&a->host, a->host_bytes, cudaHostAllocMapped) == cudaSuccess &&
                   cudaHostGetDevicePointer(&hd, a->host, 0) == cudaSuccess &&
-                  cudaEventCreateWithFlags(&a->done, cudaEventDisableTiming) == cudaSuccess &&
+                  cudaEventCreateWithFlags(&a->uses[0].done, cudaEventDisableTiming) == cudaSuccess &&
                   cudaDeviceGetStreamPriorityRange(&least, &greatest) == cudaSuccess &&
                   cudaStreamCreateWithPriority(&a->build, cudaStreamNonBlocking, greatest) == cudaSuccess;
   if (!ok) {
@@ -61,6 +61,22 @@ Arena* create(int device, size_t dev_bytes, size_t host_bytes) {
   }
   a->host_dev = static_cast<char*>(hd);
   return a;
+}
+
+bool in_use(const Arena* a) {
+  for (int i = 0; i < a->n_uses; ++i)
+    if (cudaEventQuery(a->uses[i].done) != cudaSuccess) {
+      cudaGetLastError();
+      return true;
+    }
+  return false;
+}
+
+bool wait_unused(Arena* a) {
+  for (int i = 0; i < a->n_uses; ++i)
+    if (cudaEventSynchronize(a->uses[i].done) != cudaSuccess) return false;
+  a->n_uses = 0;
+  return true;
 }
 
 }  // namespace
@@ -76,10 +92,7 @@ Arena* arena_acquire(int device, size_t dev_bytes, size_t host_bytes) {
       if (a->device != device || a->dev_bytes < dev_bytes || a->host_bytes < host_bytes) continue;
       if (fitting++ == 0) oldest = i;
       if (best < v.size() && v[best]->dev_bytes <= a->dev_bytes) continue;
-      if (a->pending && cudaEventQuery(a->done) != cudaSuccess) {
-        cudaGetLastError();
-        continue;
-      }
+      if (in_use(a)) continue;
       best = i;
     }
     if (best == v.size() && fitting >= kWaitFor) best = oldest;
@@ -88,10 +101,7 @@ Arena* arena_acquire(int device, size_t dev_bytes, size_t host_bytes) {
       v.erase(v.begin() + best);
     }
   }
-  if (found && (!found->pending || cudaEventSynchronize(found->done) == cudaSuccess)) {
-    found->pending = false;
-    return found;
-  }
+  if (found && wait_unused(found)) return found;
   if (found) {
     cudaGetLastError();
     destroy(found);
@@ -106,7 +116,7 @@ Arena* arena_acquire(int device, size_t dev_bytes, size_t host_bytes) {
 
 void arena_release(Arena* a) {
   if (!a) return;
-  if (a->captured || a->dev_bytes + a->host_bytes > kMaxIdleBytes / 2) {
+  if (a->unpooled || a->dev_bytes + a->host_bytes > kMaxIdleBytes / 2) {
     destroy(a);
     return;
   }
@@ -128,13 +138,22 @@ void arena_release(Arena* a) {
 
 void arena_used(Arena* a, cudaStream_t st) {
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone ||
-      cudaEventRecord(a->done, st) != cudaSuccess) {
-    cudaGetLastError();
-    a->captured = true;
-    return;
+  unsigned long long id = 0;
+  std::lock_guard<std::mutex> lock(a->mutex);
+  if (cudaStreamIsCapturing(st, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone &&
+      cudaStreamGetId(st, &id) == cudaSuccess) {
+    int i = 0;
+    while (i < a->n_uses && a->uses[i].stream != id) ++i;
+    if (i < Arena::kMaxUses &&
+        (a->uses[i].done || cudaEventCreateWithFlags(&a->uses[i].done, cudaEventDisableTiming) == cudaSuccess) &&
+        cudaEventRecord(a->uses[i].done, st) == cudaSuccess) {
+      a->uses[i].stream = id;
+      if (i == a->n_uses) ++a->n_uses;
+      return;
+    }
   }
-  a->pending = true;
+  cudaGetLastError();
+  a->unpooled = true;
 }
 
 void arena_trim() {

@@ -1,6 +1,7 @@
 // Device and pinned host memory of a plan (see nsp_arena.cu).
 #pragma once
 #include <cstddef>
+#include <mutex>
 #include <cuda_runtime.h>
 
 namespace nsp {
@@ -12,9 +13,18 @@ struct Arena {
   char* host_dev = nullptr;  // device pointer to the same memory
   size_t dev_bytes = 0, host_bytes = 0;
   cudaStream_t build = nullptr;  // non-blocking, highest priority: uploads and list construction
-  cudaEvent_t done = nullptr;    // recorded behind the last call that used the arena
-  bool pending = false;          // `done` has been recorded
-  bool captured = false;         // used in a stream capture: its kernels may run again at any time
+  // What still may use the arena: one event per stream (by its id: a new stream may take a destroyed one's address), recorded
+  // behind the last call on that stream. The events are kept, `n_uses` of them stand for work.
+  struct Use {
+    unsigned long long stream = 0;
+    cudaEvent_t done = nullptr;
+  };
+  static constexpr int kMaxUses = 8;
+  Use uses[kMaxUses];
+  int n_uses = 0;
+  bool unpooled = false;  // goes back to the driver: used in a stream capture (its kernels may run again at any time), or on
+                          // more streams than there are events
+  std::mutex mutex;       // uses and unpooled: calls on a plan may come from several threads
 };
 
 // An arena of at least the given sizes on the current device that nothing uses any more; null when out of memory.

@@ -1,0 +1,82 @@
+// Host-side rules of the plans' memory (csrc/nsp_arena.cu), against the stand-in runtime of tests/fake_cuda.
+// usage: arena_case SCENARIO; prints the first violated expectation and returns 1.
+#include <cstring>
+#include "nsp_arena.h"
+
+using namespace nsp;
+
+#define EXPECT(c)                                                       \
+  do {                                                                  \
+    if (!(c)) return std::printf("line %d: %s\n", __LINE__, #c), 1;     \
+  } while (0)
+
+static void call(Arena* a, cudaStream_t st) {  // a library call: some work, then the mark
+  ++st->enqueued;
+  arena_used(a, st);
+}
+static void finish(cudaStream_t st) { st->finished = st->enqueued; }
+
+static constexpr size_t kDev = 300 << 10, kHost = 100 << 10;
+
+// A plan used on two streams: its memory is free only when both have finished.
+static int two_streams() {
+  FakeStream s1{101}, s2{102};
+  for (int last = 0; last < 2; ++last) {
+    Arena* a = arena_acquire(0, kDev, kHost);
+    call(a, &s1), call(a, &s2);
+    if (last) call(a, &s1);
+    arena_release(a);
+    finish(last ? &s1 : &s2);  // the stream used last is done, the other one is not
+    Arena* b = arena_acquire(0, kDev, kHost);
+    EXPECT(b != a);
+    EXPECT(fake().waits == 0);
+    finish(&s1), finish(&s2);
+    arena_release(b);
+    arena_trim();
+  }
+  // more streams than are kept track of: the memory goes back to the driver
+  FakeStream many[9] = {{1}, {2}, {3}, {4}, {5}, {6}, {7}, {8}, {9}};
+  Arena* a = arena_acquire(0, kDev, kHost);
+  for (FakeStream& s : many) call(a, &s);
+  arena_release(a);
+  EXPECT(fake().device_bytes == 0);
+  return 0;
+}
+
+// A stream that was destroyed and whose address a new one took is another stream.
+static int recycled_stream_address() {
+  FakeStream s{201};
+  Arena* a = arena_acquire(0, kDev, kHost);
+  call(a, &s);
+  FakeStream before = s;  // the first stream's work goes on
+  a->uses[0].done->on = &before;
+  s = FakeStream{202};
+  call(a, &s);
+  finish(&s);
+  arena_release(a);
+  EXPECT(arena_acquire(0, kDev, kHost) != a);
+  return 0;
+}
+
+static int reuse_and_trim() {
+  FakeStream s{301};
+  Arena* a = arena_acquire(0, kDev, kHost);
+  call(a, &s);
+  arena_release(a);
+  finish(&s);
+  EXPECT(arena_acquire(0, kDev, kHost) == a);
+  EXPECT(arena_acquire(1, kDev, kHost)->device == 1);
+  s.capturing = true;
+  call(a, &s);
+  arena_release(a);  // its kernels may run again at any replay
+  EXPECT(fake().live.size() == 2);
+  return 0;
+}
+
+int main(int argc, char** argv) {
+  const char* what = argc > 1 ? argv[1] : "";
+  if (!std::strcmp(what, "two_streams")) return two_streams();
+  if (!std::strcmp(what, "recycled_stream_address")) return recycled_stream_address();
+  if (!std::strcmp(what, "reuse_and_trim")) return reuse_and_trim();
+  return std::printf("no scenario %s\n", what), 2;
+}

@@ -307,7 +307,10 @@ int nsp_selftest_wait_timeout(const nsp_plan_t* plan, int64_t limit_clk, void* s
 
 /* How long a device-side wait of this plan's kernels may take before it gives up, in SM clocks (default 4e9, about
  * two seconds; at least 1000). Every wait on a barrier inside the kernels is bounded by it; when one runs out the kernel
- * records NSP_ERR_DEVICE_TIMEOUT with the work item and the place, all its roles unwind and the launch ends. Errors:
+ * records NSP_ERR_DEVICE_TIMEOUT with the work item and the place, all its roles unwind and the launch ends. Two waits are
+ * for the work of other thread blocks: a block that runs a later part of a divided backward item waits for the parts
+ * before it, for the limit plus 32768 clocks per step and part (a step is one key tile against one query tile of one
+ * head); with NSP_PLAN_DETERMINISTIC_DQ a block waits, under the limit itself, for the key tiles before its own. Errors:
  * INVALID_ARG. */
 int nsp_plan_set_wait_limit(nsp_plan_t* plan, int64_t sm_clocks);
 

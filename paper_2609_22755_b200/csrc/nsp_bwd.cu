@@ -1072,9 +1072,9 @@ __global__ void __launch_bounds__(Roles<FIRST, D>::kThreads, 1) bwd_kernel(const
         if (!FIRST && c.first) grid_wait_predecessor();
         auto wait_part = [&]() {  // one lane per warp that goes on to read or add to the output
           if (c.part == 0) return;
-          const long long t0 = clock64();
+          const long long t0 = clock64(), limit = a.wait_limit + (c.steps + c.parts) * kTurnClkPerStep;
           while (*reinterpret_cast<volatile int32_t*>(a.turn + c.turn) != c.part) {
-            if (clock64() - t0 > a.wait_limit) {
+            if (clock64() - t0 > limit) {
               report_timeout(a.status, c.it, kWhereBwdTurn, c.part);
               *abort_flag = 1;
               break;

@@ -95,7 +95,7 @@ enum DeviceWhere : int32_t {
   kWhereBwdDsReady = 24,
   kWhereBwdItemBarrier = 25,
   kWhereBwdTmemBase = 26,
-  kWhereBwdTurn = 27,  // deterministic dQ: the key tiles before this one did not finish their additions
+  kWhereBwdTurn = 27,  // the parts before this one (deterministic dQ: the key tiles) did not finish their additions
   kWhereCheckFwdO = 40,    // checked build: an index outside the tensor (O, LSE / delta, dQ, dK / dV, LSE read)
   kWhereCheckFwdLse = 41,
   kWhereCheckBwdDq = 42,
@@ -216,6 +216,12 @@ inline cudaError_t launch_chained_if(bool chained, void (*kernel)(P...), unsigne
 // item's turn counter. A part never precedes an earlier part of its item in the list, so the part that is waited for has
 // always been popped, and the lowest unfinished position of the list never waits: no cycle.
 constexpr int kMaxParts = 64;
+// The wait for a turn is a wait for another CTA's work: the part before may still have all its steps to do (it was popped
+// earlier and holds at most one step more), and the parts before that one their additions. On top of the wait limit it
+// may therefore take this many clocks for every step and every part. A step takes 3,000-5,000 clocks, one of the first-tile
+// kernel ~10,000, an addition and its hand-over ~4,000 (one 128-token segment at 256q/1kv: part 49 of 64 gave up at a limit
+// of 200,000).
+constexpr long long kTurnClkPerStep = 32768;
 
 // Host-side launchers implemented next to their kernels.
 cudaError_t launch_plan_lists(const PlanKey* d_key, const int32_t* d_tile_base, int n_seg, int n_tiles, nsp_tile_t* d_fwd,

@@ -100,7 +100,9 @@ typedef struct {
  *   order: cost descending, then seg, tile, head ascending (a total order: the list is unique).
  * cu_seqlens [n_seg+1], hq [n_seg], hkv [n_seg]: host arrays, copied. Zero-length segments and n_seg == 0 are legal.
  * opts may be NULL (= {128,128,1,0}). The lists are built on a stream of the plan's own and are complete when the call
- * returns; it does not wait for work enqueued on `stream` or any other stream (`stream` is not used).
+ * returns. It does not wait for work of other streams. Of `stream`, the one the plan is meant for, it may wait for an
+ * earlier batch: when the calls of three or more destroyed plans have not finished there, for the oldest of them (the host
+ * is that many batches ahead).
  * Errors: INVALID_ARG (null, n_seg < 0, cu_seqlens[0] != 0, decreasing cu_seqlens, hq/hkv <= 0, hq % hkv != 0),
  * UNSUPPORTED (head_dim other than 128 or 64, > NSP_MAX_RUNS runs, unsupported tile sizes, >= 65536 segments, > 256 heads,
  * >= 65536 tiles in a segment), ALLOC, CUDA. On error *out_plan is NULL.

@@ -261,7 +261,6 @@ int64_t nsp_launch_count(void) { return g_launches.load(std::memory_order_relaxe
 
 int nsp_plan_tiles(const int32_t* cu_seqlens, const int32_t* hq, const int32_t* hkv, int32_t n_seg, int32_t head_dim,
                    const nsp_plan_opts* opts, void* stream, nsp_plan_t** out_plan) {
-  (void)stream;
   if (!out_plan) return NSP_ERR_INVALID_ARG;
   *out_plan = nullptr;
   if (n_seg < 0 || (n_seg > 0 && (!cu_seqlens || !hq || !hkv))) return NSP_ERR_INVALID_ARG;
@@ -516,7 +515,7 @@ int nsp_plan_tiles(const int32_t* cu_seqlens, const int32_t* hq, const int32_t* 
   const size_t o_exec = take(sizeof(nsp_tile_t) * nb);
   const size_t o_pairs = take(sizeof(nsp_tile_t) * 2 * p->n_pairs);
   const size_t o_front = take(sizeof(int32_t) * (nb / kFrontBlock + 1));
-  p->arena = arena_acquire(p->device, at, 256 + upload);
+  p->arena = arena_acquire(p->device, at, 256 + upload, static_cast<cudaStream_t>(stream));
   if (!p->arena) {
     delete p;
     return NSP_ERR_ALLOC;

@@ -15,8 +15,10 @@ namespace nsp {
 namespace {
 
 constexpr size_t kMaxIdle = 8;                  // arenas
-constexpr size_t kWaitFor = 3;  // with that many fitting arenas still in use, wait for the oldest instead of allocating:
-                                // the host is three batches ahead of the device, which has work enough
+// With that many fitting arenas still in use by the caller's stream alone, wait for the oldest of them instead of
+// allocating: the host is three batches ahead of the device, which has work enough. Arenas that other streams use are left
+// alone: their work may depend on what the calling thread does next.
+constexpr size_t kWaitFor = 3;
 constexpr size_t kMaxIdleBytes = 64ull << 20;   // device + pinned bytes of all idle arenas
 
 std::mutex g_mutex;
@@ -72,6 +74,12 @@ bool in_use(const Arena* a) {
   return false;
 }
 
+bool used_only_by(const Arena* a, unsigned long long stream) {
+  for (int i = 0; i < a->n_uses; ++i)
+    if (a->uses[i].stream != stream) return false;
+  return true;
+}
+
 bool wait_unused(Arena* a) {
   for (int i = 0; i < a->n_uses; ++i)
     if (cudaEventSynchronize(a->uses[i].done) != cudaSuccess) return false;
@@ -81,8 +89,11 @@ bool wait_unused(Arena* a) {
 
 }  // namespace
 
-Arena* arena_acquire(int device, size_t dev_bytes, size_t host_bytes) {
+Arena* arena_acquire(int device, size_t dev_bytes, size_t host_bytes, cudaStream_t st) {
   Arena* found = nullptr;
+  unsigned long long own = 0;
+  const bool have_own = cudaStreamGetId(st, &own) == cudaSuccess;
+  if (!have_own) cudaGetLastError();
   {
     std::lock_guard<std::mutex> lock(g_mutex);
     auto& v = idle();
@@ -90,10 +101,11 @@ Arena* arena_acquire(int device, size_t dev_bytes, size_t host_bytes) {
     for (size_t i = 0; i < v.size(); ++i) {
       const Arena* a = v[i];
       if (a->device != device || a->dev_bytes < dev_bytes || a->host_bytes < host_bytes) continue;
-      if (fitting++ == 0) oldest = i;
       if (best < v.size() && v[best]->dev_bytes <= a->dev_bytes) continue;
-      if (in_use(a)) continue;
-      best = i;
+      if (!in_use(a))
+        best = i;
+      else if (have_own && used_only_by(a, own) && fitting++ == 0)
+        oldest = i;
     }
     if (best == v.size() && fitting >= kWaitFor) best = oldest;
     if (best < v.size()) {

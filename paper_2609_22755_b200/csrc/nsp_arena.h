@@ -27,8 +27,9 @@ struct Arena {
   std::mutex mutex;       // uses and unpooled: calls on a plan may come from several threads
 };
 
-// An arena of at least the given sizes on the current device that nothing uses any more; null when out of memory.
-Arena* arena_acquire(int device, size_t dev_bytes, size_t host_bytes);
+// An arena of at least the given sizes on the current device that nothing uses any more; null when out of memory. May wait
+// for work of the stream `st`, the caller's, but for no other (see kWaitFor).
+Arena* arena_acquire(int device, size_t dev_bytes, size_t host_bytes, cudaStream_t st);
 // Hands an arena back (null is a no-op); kernels recorded with arena_used may still run.
 void arena_release(Arena* a);
 // The work enqueued on st so far uses the arena.

@@ -22,12 +22,12 @@ static constexpr size_t kDev = 300 << 10, kHost = 100 << 10;
 static int two_streams() {
   FakeStream s1{101}, s2{102};
   for (int last = 0; last < 2; ++last) {
-    Arena* a = arena_acquire(0, kDev, kHost);
+    Arena* a = arena_acquire(0, kDev, kHost, nullptr);
     call(a, &s1), call(a, &s2);
     if (last) call(a, &s1);
     arena_release(a);
     finish(last ? &s1 : &s2);  // the stream used last is done, the other one is not
-    Arena* b = arena_acquire(0, kDev, kHost);
+    Arena* b = arena_acquire(0, kDev, kHost, nullptr);
     EXPECT(b != a);
     EXPECT(fake().waits == 0);
     finish(&s1), finish(&s2);
@@ -36,7 +36,7 @@ static int two_streams() {
   }
   // more streams than are kept track of: the memory goes back to the driver
   FakeStream many[9] = {{1}, {2}, {3}, {4}, {5}, {6}, {7}, {8}, {9}};
-  Arena* a = arena_acquire(0, kDev, kHost);
+  Arena* a = arena_acquire(0, kDev, kHost, nullptr);
   for (FakeStream& s : many) call(a, &s);
   arena_release(a);
   EXPECT(fake().device_bytes == 0);
@@ -46,7 +46,7 @@ static int two_streams() {
 // A stream that was destroyed and whose address a new one took is another stream.
 static int recycled_stream_address() {
   FakeStream s{201};
-  Arena* a = arena_acquire(0, kDev, kHost);
+  Arena* a = arena_acquire(0, kDev, kHost, nullptr);
   call(a, &s);
   FakeStream before = s;  // the first stream's work goes on
   a->uses[0].done->on = &before;
@@ -54,18 +54,43 @@ static int recycled_stream_address() {
   call(a, &s);
   finish(&s);
   arena_release(a);
-  EXPECT(arena_acquire(0, kDev, kHost) != a);
+  EXPECT(arena_acquire(0, kDev, kHost, nullptr) != a);
+  return 0;
+}
+
+// Three fitting arenas in use by the caller's stream: the oldest is waited for. In use by others: never.
+static int back_pressure() {
+  FakeStream mine{401}, other{402};
+  Arena* a[3];
+  for (int own = 0; own < 3; ++own) {  // none, some, all of them on the caller's stream
+    for (Arena*& x : a) x = arena_acquire(0, kDev, kHost, &mine);
+    for (int i = 0; i < 3; ++i) call(a[i], i < (own == 0 ? 0 : own == 1 ? 2 : 3) ? &mine : &other);
+    for (Arena* x : a) arena_release(x);
+    Arena* b = arena_acquire(0, kDev, kHost, &mine);
+    EXPECT(fake().waits == (own == 2));
+    EXPECT((b == a[0]) == (own == 2));
+    EXPECT(other.finished == 0);
+    finish(&mine);
+    other = FakeStream{402};
+    arena_release(b);
+    arena_trim();
+  }
+  // an arena that another stream uses as well is not waited for either
+  for (Arena*& x : a) x = arena_acquire(0, kDev, kHost, &mine);
+  for (Arena* x : a) call(x, &mine), call(x, &other), arena_release(x);
+  Arena* b = arena_acquire(0, kDev, kHost, &mine);
+  EXPECT(b != a[0] && b != a[1] && b != a[2] && fake().waits == 1);
   return 0;
 }
 
 static int reuse_and_trim() {
   FakeStream s{301};
-  Arena* a = arena_acquire(0, kDev, kHost);
+  Arena* a = arena_acquire(0, kDev, kHost, nullptr);
   call(a, &s);
   arena_release(a);
   finish(&s);
-  EXPECT(arena_acquire(0, kDev, kHost) == a);
-  EXPECT(arena_acquire(1, kDev, kHost)->device == 1);
+  EXPECT(arena_acquire(0, kDev, kHost, nullptr) == a);
+  EXPECT(arena_acquire(1, kDev, kHost, nullptr)->device == 1);
   s.capturing = true;
   call(a, &s);
   arena_release(a);  // its kernels may run again at any replay
@@ -76,6 +101,7 @@ static int reuse_and_trim() {
 int main(int argc, char** argv) {
   const char* what = argc > 1 ? argv[1] : "";
   if (!std::strcmp(what, "two_streams")) return two_streams();
+  if (!std::strcmp(what, "back_pressure")) return back_pressure();
   if (!std::strcmp(what, "recycled_stream_address")) return recycled_stream_address();
   if (!std::strcmp(what, "reuse_and_trim")) return reuse_and_trim();
   return std::printf("no scenario %s\n", what), 2;

@@ -99,10 +99,12 @@ typedef struct {
  *   backward item (s, g, n), g in [0,hkv[s]), n in [0, ceil(L_s/bn)): cost = (hq[s]/hkv[s]) * (ceil(L_s/bm) - floor(n*bn/bm))
  *   order: cost descending, then seg, tile, head ascending (a total order: the list is unique).
  * cu_seqlens [n_seg+1], hq [n_seg], hkv [n_seg]: host arrays, copied. Zero-length segments and n_seg == 0 are legal.
- * opts may be NULL (= {128,128,1,0}). The lists are built on a stream of the plan's own and are complete when the call
- * returns. It does not wait for work of other streams. Of `stream`, the one the plan is meant for, it may wait for an
- * earlier batch: when the calls of three or more destroyed plans have not finished there, for the oldest of them (the host
- * is that many batches ahead).
+ * opts may be NULL (= {128,128,1,0}). The lists are built on a stream of the plan's own; the call looks for them
+ * for some 40 us and then returns, and every call that uses the plan is ordered behind them. (While a kernel that leaves no
+ * room on any SM is running, they are complete when one of its blocks has ended. A call under stream capture then waits
+ * for them on the host.) It does not wait for work of other streams. Of `stream`, the one the plan is meant for, it may
+ * wait for an earlier batch: when the calls of three or more destroyed plans have not finished there, for the oldest of
+ * them (the host is that many batches ahead).
  * Errors: INVALID_ARG (null, n_seg < 0, cu_seqlens[0] != 0, decreasing cu_seqlens, hq/hkv <= 0, hq % hkv != 0),
  * UNSUPPORTED (head_dim other than 128 or 64, > NSP_MAX_RUNS runs, unsupported tile sizes, >= 65536 segments, > 256 heads,
  * >= 65536 tiles in a segment), ALLOC, CUDA. On error *out_plan is NULL.
@@ -119,8 +121,8 @@ int nsp_plan_sizes(const nsp_plan_t* plan, int64_t* q_elems, int64_t* kv_elems, 
  * backward items in the order the backward kernel actually walks them, a permutation of pass 1 that is just as
  * unique: the (segment, kv head) groups by segment length descending, then segment, then kv head ascending; inside a
  * group the key tiles ascending. Group-major order keeps the dQ accumulator rows of a q tile in L2 while all key tiles
- * of the group add to them. Writes min(cap, n) items, stores n in *n_items (host_out may be NULL to query). The lists
- * were complete when nsp_plan_tiles returned; this call only copies. */
+ * of the group add to them. Writes min(cap, n) items, stores n in *n_items (host_out may be NULL to query). Waits
+ * until the lists are complete, then copies. */
 int nsp_plan_get(const nsp_plan_t* plan, int pass, nsp_tile_t* host_out, int64_t cap, int64_t* n_items);
 
 /*

@@ -2,6 +2,7 @@
 // Plain C ABI (include/nsp.h); no torch types, no CPU fallback.
 #include <algorithm>
 #include <atomic>
+#include <chrono>
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
@@ -28,6 +29,7 @@ struct nsp_plan {
   std::vector<RunInfo> runs;
   // device state, all of it inside the arena
   Arena* arena = nullptr;
+  std::atomic<bool> built{false};  // known to be complete on the device; until then every stream's first call waits for it
   SegInfo* d_seg = nullptr;
   int64_t* d_row_base = nullptr;  // [n_seg + 1] first packed (token, head) row of each segment
   nsp_tile_t* d_fwd = nullptr;
@@ -223,10 +225,15 @@ void free_plan(nsp_plan* p) {
   delete p;
 }
 
-// Ends every call that enqueues work of a plan, however it returns: see arena_used.
+// Brackets every call that enqueues work of a plan, however it returns: behind the plan's construction (see
+// arena_order_built), and with the arena marked as used by the stream (see arena_used).
 struct UsesArena {
   const nsp_plan* plan;
   cudaStream_t st;
+  cudaError_t ready;
+  UsesArena(const nsp_plan* p, cudaStream_t stream) : plan(p), st(stream), ready(cudaSuccess) {
+    if (!p->built.load(std::memory_order_acquire)) ready = arena_order_built(p->arena, st);
+  }
   ~UsesArena() { arena_used(plan->arena, st); }
 };
 
@@ -556,17 +563,28 @@ int nsp_plan_tiles(const int32_t* cu_seqlens, const int32_t* hq, const int32_t* 
   put(o_first_parts, first_parts.data(), sizeof(nsp_tile_t) * first_parts.size());
   put(o_fwd_first, fwd_first.data(), sizeof(nsp_tile_t) * fwd_first.size());
   std::memset(image + o_turns, 0, sizeof(int32_t) * n_turns);
-  // On the arena's own stream, so that the plan is complete when this call returns without waiting for the work the
-  // caller has enqueued before (nothing here depends on it).
+  // On the arena's own stream: nothing here depends on the caller's work. It takes ~20 us where an SM has room for a block of
+  // the list kernel. A backward kernel leaves none (its shared memory, at head_dim 64 its registers), and then the lists
+  // are ready when one of its CTAs ends: waited for here, the host stood still for up to the rest of a running backward
+  // pass (13 ms, four segments of 16,384 tokens at 32q/4kv, head_dim 64). So the host looks for kBuildPoll and then leaves the
+  // waiting to the streams that use the plan. Plans that are ready at once save those a dependency in front of their first
+  // kernel.
+  constexpr auto kBuildPoll = std::chrono::microseconds(40);
   cudaStream_t bs = p->arena->build;
-  if (cudaMemcpyAsync(d, image, upload, cudaMemcpyHostToDevice, bs) != cudaSuccess ||
+  const bool enqueued =
+      cudaMemcpyAsync(d, image, upload, cudaMemcpyHostToDevice, bs) == cudaSuccess &&
       launch_plan_lists(reinterpret_cast<const PlanKey*>(d + o_keys), reinterpret_cast<const int32_t*>(d + o_tiles), n_seg,
-                        static_cast<int>(tiles), p->d_fwd, p->d_bwd, p->d_bwd_exec, p->d_fwd_pairs, bs) != cudaSuccess ||
-      cudaStreamSynchronize(bs) != cudaSuccess) {
+                        static_cast<int>(tiles), p->d_fwd, p->d_bwd, p->d_bwd_exec, p->d_fwd_pairs, bs) == cudaSuccess;
+  arena_used(p->arena, bs);
+  if (!enqueued || p->arena->n_uses != 1) {
     p->arena->unpooled = true;
     free_plan(p);
     return NSP_ERR_CUDA;
   }
+  const auto begun = std::chrono::steady_clock::now();
+  bool built = false;
+  while (!(built = arena_built(p->arena)) && std::chrono::steady_clock::now() - begun < kBuildPoll) {}
+  p->built.store(built, std::memory_order_release);
   NSP_LOGF("plan %p: %d segments, %zu runs, head_dim %d, q_elems %lld, kv_elems %lld, fwd items %lld, bwd items %lld%s",
            static_cast<void*>(p), n_seg, p->runs.size(), head_dim, static_cast<long long>(p->q_elems),
            static_cast<long long>(p->kv_elems), static_cast<long long>(nf), static_cast<long long>(nb),
@@ -595,6 +613,7 @@ int nsp_plan_get(const nsp_plan_t* plan, int pass, nsp_tile_t* host_out, int64_t
   *n_items = n;
   if (!host_out || cap == 0 || n == 0) return NSP_OK;
   const int64_t m = cap < n ? cap : n;
+  if (!plan->built.load(std::memory_order_acquire) && arena_wait_built(plan->arena) != cudaSuccess) return NSP_ERR_CUDA;
   const nsp_tile_t* src = pass == 0 ? plan->d_fwd : (pass == 1 ? plan->d_bwd : plan->d_bwd_exec);
   if (cudaMemcpy(host_out, src, sizeof(nsp_tile_t) * m, cudaMemcpyDeviceToHost) !=
       cudaSuccess)
@@ -613,7 +632,8 @@ int nsp_attn_fwd(const nsp_plan_t* plan, const void* q, const void* k, const voi
   if (!q || !k || !v || !o || !lse) return NSP_ERR_INVALID_ARG;
   if (!aligned16(q) || !aligned16(k) || !aligned16(v) || !aligned16(o) || !aligned16(lse)) return NSP_ERR_INVALID_ARG;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  const UsesArena uses{plan, st};
+  const UsesArena uses(plan, st);
+  if (uses.ready != cudaSuccess) return NSP_ERR_CUDA;
   FwdMaps maps;
   std::memset(&maps, 0, sizeof(maps));
   for (size_t r = 0; r < plan->runs.size(); ++r) {
@@ -685,7 +705,8 @@ int bwd_impl(const nsp_plan_t* plan, const uint8_t* recompute, const void* q, co
   const size_t need = recompute ? recompute_ws_bytes(plan) : base;
   if (!ws || (reinterpret_cast<uintptr_t>(ws) & 255) != 0 || ws_bytes < need) return NSP_ERR_WORKSPACE;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  const UsesArena uses{plan, st};
+  const UsesArena uses(plan, st);
+  if (uses.ready != cudaSuccess) return NSP_ERR_CUDA;
   char* wsb = static_cast<char*>(ws);
   float* dq_acc = static_cast<float*>(ws);
   float* delta = reinterpret_cast<float*>(wsb + align_up(static_cast<size_t>(plan->q_elems) * 4, 256));
@@ -971,7 +992,8 @@ __global__ void selftest_wait_kernel(StatusWord status, long long limit_clk) {
 int nsp_selftest_wait_timeout(const nsp_plan_t* plan, int64_t limit_clk, void* stream) {
   if (!plan || limit_clk < 1 || limit_clk > (1ll << 31)) return NSP_ERR_INVALID_ARG;
   if (const int failed = plan_failed(plan)) return failed;
-  const UsesArena uses{plan, static_cast<cudaStream_t>(stream)};
+  const UsesArena uses(plan, static_cast<cudaStream_t>(stream));
+  if (uses.ready != cudaSuccess) return NSP_ERR_CUDA;
   selftest_wait_kernel<<<1, 32, 0, static_cast<cudaStream_t>(stream)>>>(status_word(plan), limit_clk);
   count_launches(1);
   return cudaGetLastError() == cudaSuccess ? NSP_OK : NSP_ERR_CUDA;

@@ -75,9 +75,9 @@ bool in_use(const Arena* a) {
 }
 
 bool used_only_by(const Arena* a, unsigned long long stream) {
-  for (int i = 0; i < a->n_uses; ++i)
+  for (int i = 1; i < a->n_uses; ++i)  // behind the use of the construction, which no other stream's work holds up for long
     if (a->uses[i].stream != stream) return false;
-  return true;
+  return a->n_uses > 1;
 }
 
 bool wait_unused(Arena* a) {
@@ -166,6 +166,34 @@ void arena_used(Arena* a, cudaStream_t st) {
   }
   cudaGetLastError();
   a->unpooled = true;
+}
+
+bool arena_built(const Arena* a) { return cudaEventQuery(a->uses[0].done) == cudaSuccess; }
+
+cudaError_t arena_wait_built(const Arena* a) {
+  // another thread may be capturing, and a wait would end its capture unless this thread says that it is unrelated
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  cudaError_t e = cudaThreadExchangeStreamCaptureMode(&mode);
+  if (e != cudaSuccess) return e;
+  e = cudaEventSynchronize(a->uses[0].done);
+  cudaThreadExchangeStreamCaptureMode(&mode);
+  return e;
+}
+
+cudaError_t arena_order_built(Arena* a, cudaStream_t st) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  unsigned long long id = 0;
+  cudaError_t e = cudaStreamIsCapturing(st, &cap);
+  if (e != cudaSuccess) return e;
+  if (cap != cudaStreamCaptureStatusNone) return arena_wait_built(a);
+  e = cudaStreamGetId(st, &id);
+  if (e != cudaSuccess) return e;
+  {
+    std::lock_guard<std::mutex> lock(a->mutex);
+    for (int i = 1; i < a->n_uses; ++i)
+      if (a->uses[i].stream == id) return cudaSuccess;  // an earlier call on this stream waited
+  }
+  return cudaStreamWaitEvent(st, a->uses[0].done, 0);
 }
 
 void arena_trim() {

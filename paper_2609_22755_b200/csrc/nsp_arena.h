@@ -12,7 +12,7 @@ struct Arena {
   void* host = nullptr;      // pinned, mapped
   char* host_dev = nullptr;  // device pointer to the same memory
   size_t dev_bytes = 0, host_bytes = 0;
-  cudaStream_t build = nullptr;  // non-blocking, highest priority: uploads and list construction
+  cudaStream_t build = nullptr;  // non-blocking, highest priority: uploads and list construction; the first use of a plan
   // What still may use the arena: one event per stream (by its id: a new stream may take a destroyed one's address), recorded
   // behind the last call on that stream. The events are kept, `n_uses` of them stand for work.
   struct Use {
@@ -34,6 +34,12 @@ Arena* arena_acquire(int device, size_t dev_bytes, size_t host_bytes, cudaStream
 void arena_release(Arena* a);
 // The work enqueued on st so far uses the arena.
 void arena_used(Arena* a, cudaStream_t st);
+// What the plan's construction has enqueued (its use of a->build, the first one) has completed / is waited for by the host.
+bool arena_built(const Arena* a);
+cudaError_t arena_wait_built(const Arena* a);
+// What is enqueued on st from now on runs behind the construction. A stream that is being captured cannot wait for work
+// outside the capture: then the host does.
+cudaError_t arena_order_built(Arena* a, cudaStream_t st);
 // Frees every idle arena.
 void arena_trim();
 

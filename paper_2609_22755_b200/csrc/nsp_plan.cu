@@ -15,8 +15,9 @@
 // and writes the tile's items, no keys and no sort. A plan of 8,192 tokens at 32q/4kv spent 60 us in two radix sorts
 // with their key and decode kernels; this is one launch of about 5 us. The cost is tiles x segments: 131,072 tokens in
 // 8,192 segments of 16 tokens are 67 M terms, about 0.1 ms.
-// 128 threads of 32 registers, no shared memory: a block fits beside the persistent 640-thread kernels (61,440 of the
-// 65,536 registers of an SM), so building the next batch's plan does not wait for the running batch.
+// 128 threads of 32 registers, no shared memory: a block fits beside the general forward kernel (61,440 of the 65,536
+// registers of an SM). It does not fit beside the backward kernels, which leave no shared memory for another block (and at
+// head_dim 64 no registers); then it starts when one of their blocks ends, and the host does not wait for it (nsp_api.cu).
 #include <cuda_bf16.h>
 #include "nsp_internal.cuh"
 

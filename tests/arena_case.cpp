@@ -18,16 +18,23 @@ static void finish(cudaStream_t st) { st->finished = st->enqueued; }
 
 static constexpr size_t kDev = 300 << 10, kHost = 100 << 10;
 
+static Arena* acquire(int device, cudaStream_t st, bool built = true) {  // with the construction of a plan enqueued
+  Arena* a = arena_acquire(device, kDev, kHost, st);
+  call(a, a->build);
+  if (built) finish(a->build);
+  return a;
+}
+
 // A plan used on two streams: its memory is free only when both have finished.
 static int two_streams() {
   FakeStream s1{101}, s2{102};
   for (int last = 0; last < 2; ++last) {
-    Arena* a = arena_acquire(0, kDev, kHost, nullptr);
+    Arena* a = acquire(0, nullptr);
     call(a, &s1), call(a, &s2);
     if (last) call(a, &s1);
     arena_release(a);
     finish(last ? &s1 : &s2);  // the stream used last is done, the other one is not
-    Arena* b = arena_acquire(0, kDev, kHost, nullptr);
+    Arena* b = acquire(0, nullptr);
     EXPECT(b != a);
     EXPECT(fake().waits == 0);
     finish(&s1), finish(&s2);
@@ -35,8 +42,8 @@ static int two_streams() {
     arena_trim();
   }
   // more streams than are kept track of: the memory goes back to the driver
-  FakeStream many[9] = {{1}, {2}, {3}, {4}, {5}, {6}, {7}, {8}, {9}};
-  Arena* a = arena_acquire(0, kDev, kHost, nullptr);
+  FakeStream many[8] = {{501}, {502}, {503}, {504}, {505}, {506}, {507}, {508}};  // and the construction's
+  Arena* a = acquire(0, nullptr);
   for (FakeStream& s : many) call(a, &s);
   arena_release(a);
   EXPECT(fake().device_bytes == 0);
@@ -46,15 +53,15 @@ static int two_streams() {
 // A stream that was destroyed and whose address a new one took is another stream.
 static int recycled_stream_address() {
   FakeStream s{201};
-  Arena* a = arena_acquire(0, kDev, kHost, nullptr);
+  Arena* a = acquire(0, nullptr);
   call(a, &s);
   FakeStream before = s;  // the first stream's work goes on
-  a->uses[0].done->on = &before;
+  a->uses[1].done->on = &before;
   s = FakeStream{202};
   call(a, &s);
   finish(&s);
   arena_release(a);
-  EXPECT(arena_acquire(0, kDev, kHost, nullptr) != a);
+  EXPECT(acquire(0, nullptr) != a);
   return 0;
 }
 
@@ -63,10 +70,10 @@ static int back_pressure() {
   FakeStream mine{401}, other{402};
   Arena* a[3];
   for (int own = 0; own < 3; ++own) {  // none, some, all of them on the caller's stream
-    for (Arena*& x : a) x = arena_acquire(0, kDev, kHost, &mine);
+    for (Arena*& x : a) x = acquire(0, &mine);
     for (int i = 0; i < 3; ++i) call(a[i], i < (own == 0 ? 0 : own == 1 ? 2 : 3) ? &mine : &other);
     for (Arena* x : a) arena_release(x);
-    Arena* b = arena_acquire(0, kDev, kHost, &mine);
+    Arena* b = acquire(0, &mine);
     EXPECT(fake().waits == (own == 2));
     EXPECT((b == a[0]) == (own == 2));
     EXPECT(other.finished == 0);
@@ -76,21 +83,43 @@ static int back_pressure() {
     arena_trim();
   }
   // an arena that another stream uses as well is not waited for either
-  for (Arena*& x : a) x = arena_acquire(0, kDev, kHost, &mine);
+  for (Arena*& x : a) x = acquire(0, &mine);
   for (Arena* x : a) call(x, &mine), call(x, &other), arena_release(x);
-  Arena* b = arena_acquire(0, kDev, kHost, &mine);
+  Arena* b = acquire(0, &mine);
   EXPECT(b != a[0] && b != a[1] && b != a[2] && fake().waits == 1);
+  return 0;
+}
+
+// The first call on a stream is ordered behind a construction that still runs, later ones are not ordered again, and a stream
+// under capture has the host wait. An arena whose construction still runs is not handed out, nor waited for.
+static int order_behind_construction() {
+  FakeStream s1{601}, s2{602}, captured{603};
+  Arena* a = acquire(0, &s1, false);
+  EXPECT(!arena_built(a));
+  EXPECT(arena_order_built(a, &s1) == cudaSuccess && fake().stream_waits == 1);
+  call(a, &s1);
+  EXPECT(arena_order_built(a, &s1) == cudaSuccess && fake().stream_waits == 1);
+  EXPECT(arena_order_built(a, &s2) == cudaSuccess && fake().stream_waits == 2);
+  EXPECT(fake().waits == 0);
+  captured.capturing = true;
+  EXPECT(arena_order_built(a, &captured) == cudaSuccess && fake().stream_waits == 2 && fake().waits == 1);
+  EXPECT(arena_built(a) && fake().mode == cudaStreamCaptureModeGlobal);
+  for (int i = 0; i < 4; ++i) {
+    Arena* b = acquire(0, &s1, false);
+    arena_release(b);  // a plan that was never used
+  }
+  EXPECT(fake().waits == 1 && fake().live.size() == 2 * 5);
   return 0;
 }
 
 static int reuse_and_trim() {
   FakeStream s{301};
-  Arena* a = arena_acquire(0, kDev, kHost, nullptr);
+  Arena* a = acquire(0, nullptr);
   call(a, &s);
   arena_release(a);
   finish(&s);
-  EXPECT(arena_acquire(0, kDev, kHost, nullptr) == a);
-  EXPECT(arena_acquire(1, kDev, kHost, nullptr)->device == 1);
+  EXPECT(acquire(0, nullptr) == a);
+  EXPECT(acquire(1, nullptr)->device == 1);
   s.capturing = true;
   call(a, &s);
   arena_release(a);  // its kernels may run again at any replay
@@ -101,6 +130,7 @@ static int reuse_and_trim() {
 int main(int argc, char** argv) {
   const char* what = argc > 1 ? argv[1] : "";
   if (!std::strcmp(what, "two_streams")) return two_streams();
+  if (!std::strcmp(what, "order_behind_construction")) return order_behind_construction();
   if (!std::strcmp(what, "back_pressure")) return back_pressure();
   if (!std::strcmp(what, "recycled_stream_address")) return recycled_stream_address();
   if (!std::strcmp(what, "reuse_and_trim")) return reuse_and_trim();

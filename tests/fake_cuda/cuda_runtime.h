@@ -19,6 +19,7 @@ struct FakeEvent {
 typedef FakeStream* cudaStream_t;
 typedef FakeEvent* cudaEvent_t;
 enum cudaError_t { cudaSuccess = 0, cudaErrorInvalidValue = 1, cudaErrorNotReady = 600 };
+enum cudaStreamCaptureMode { cudaStreamCaptureModeGlobal = 0, cudaStreamCaptureModeRelaxed = 2 };
 enum cudaStreamCaptureStatus { cudaStreamCaptureStatusNone = 0, cudaStreamCaptureStatusActive = 1 };
 constexpr unsigned cudaEventDisableTiming = 2, cudaHostAllocMapped = 2, cudaStreamNonBlocking = 1;
 
@@ -27,7 +28,8 @@ struct Fake {
   size_t device_limit = ~size_t(0);
   std::set<void*> live;
   int waits = 0;            // host waits for an event that had not completed
-  int frees_in_use = 0;     // cudaFree calls (each waits for the device)
+  int stream_waits = 0;     // cudaStreamWaitEvent calls
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeGlobal;  // of the thread
   unsigned long long next_id = 1;
 };
 inline Fake& fake() {
@@ -50,7 +52,6 @@ inline cudaError_t cudaMalloc(void** p, size_t n) {
 inline cudaError_t cudaFree(void* p) {
   if (!p) return cudaSuccess;
   if (!fake().live.erase(p)) std::abort();
-  ++fake().frees_in_use;
   fake().device_bytes -= *static_cast<size_t*>(p);
   std::free(p);
   return cudaSuccess;
@@ -83,6 +84,16 @@ inline cudaError_t cudaEventCreateWithFlags(cudaEvent_t* e, unsigned) { return *
 inline cudaError_t cudaEventDestroy(cudaEvent_t e) { return delete e, cudaSuccess; }
 inline cudaError_t cudaEventRecord(cudaEvent_t e, cudaStream_t s) { return e->on = s, e->at = s->enqueued, cudaSuccess; }
 inline cudaError_t cudaEventQuery(cudaEvent_t e) { return e->complete() ? cudaSuccess : cudaErrorNotReady; }
+inline cudaError_t cudaThreadExchangeStreamCaptureMode(cudaStreamCaptureMode* m) {
+  const cudaStreamCaptureMode was = fake().mode;
+  fake().mode = *m, *m = was;
+  return cudaSuccess;
+}
+inline cudaError_t cudaStreamWaitEvent(cudaStream_t s, cudaEvent_t, unsigned) {
+  if (s->capturing) return cudaErrorInvalidValue;  // the event was recorded outside the capture
+  ++fake().stream_waits;
+  return cudaSuccess;
+}
 inline cudaError_t cudaEventSynchronize(cudaEvent_t e) {
   if (!e->complete()) {
     ++fake().waits;

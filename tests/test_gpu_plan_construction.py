@@ -57,3 +57,120 @@ def test_destroyed_plans_of_another_stream_are_not_waited_for(env):
     e.plan = seen[0][0]
     e.forward()
     assert e.status()[0] == 0 and torch.equal(e.o, want)
+
+
+@pytest.mark.parametrize("lengths,head_dim", [
+    ([16384] * 4, 64),    # no registers left on an SM
+    ([16384] * 4, 128),   # no shared memory left
+    ([128] * 4096, 128),  # the first-tile kernel
+])
+@pytest.mark.parametrize("captured", [False, True])
+def test_construction_under_a_backward_pass(env, lengths, head_dim, captured):
+    """The call returns while the pass still runs, and the first calls on the plan, plain or captured, find its lists."""
+    torch, B, W = env
+    from paper_2609_22755_b200.api import NspAttention
+
+    names = ("o", "lse", "dk", "dv")
+    w = W.custom([700, 300, 64, 5], 8, 2, seed=82)
+    e = NspAttention(w)
+    e.load(W.make_tensors(w))
+    e.step_device()
+    torch.cuda.synchronize()
+    want = {n: getattr(e, n).clone() for n in names}
+    big = NspAttention(W.custom(lengths, 32, 4, head_dim=head_dim))
+    for t in (big.q, big.k, big.v, big.do):
+        t.normal_()
+    big.step_device()
+    for n in names:
+        getattr(e, n).fill_(float("nan"))
+    busy = torch.cuda.Stream()
+    busy.wait_stream(torch.cuda.current_stream())
+    e.plan = None
+    plans = [B.nsp_plan_tiles(w.cu_seqlens, w.hq, w.hkv) for _ in range(8)]  # leave memory for those below: no allocation there
+    plans.clear()
+    torch.cuda.synchronize()
+    with torch.cuda.stream(busy):
+        for _ in range(3):
+            big.backward()
+        running = torch.cuda.Event()
+        running.record()
+    plans = [B.nsp_plan_tiles(w.cu_seqlens, w.hq, w.hkv) for _ in range(8)]  # some of them meet a kernel that leaves no room
+    assert not running.query()
+    graphs = []
+    for p in plans:
+        e.plan = p
+        if captured:
+            graphs.append(torch.cuda.CUDAGraph())
+            with torch.cuda.graph(graphs[-1]):
+                e.step_device()
+        else:
+            e.step_device()
+    for i, p in enumerate(plans):
+        if captured:
+            for n in names:
+                getattr(e, n).fill_(float("nan"))
+            graphs[i].replay()
+        torch.cuda.synchronize()
+        assert B.nsp_device_status(p) == (0, 0, 0, 0)
+        for n in names:
+            assert torch.equal(getattr(e, n), want[n]), n
+    assert big.status()[0] == 0
+
+
+def test_lists_read_while_they_are_being_built(env):
+    torch, B, W = env
+    import oracle
+    from paper_2609_22755_b200.api import NspAttention
+
+    big = NspAttention(W.custom([16384] * 4, 32, 4, head_dim=64))
+    for t in (big.q, big.k, big.v, big.do):
+        t.normal_()
+    big.forward()
+    torch.cuda.synchronize()
+    busy = torch.cuda.Stream()
+    with torch.cuda.stream(busy):
+        big.backward()
+    w = W.custom([700, 300, 64, 5], 8, 2)
+    for _ in range(4):
+        plan = B.nsp_plan_tiles(w.cu_seqlens, w.hq, w.hkv)
+        for p in (0, 1, 2):
+            assert (B.nsp_plan_get(plan, p) == oracle.plan_tiles(w.cu_seqlens, w.hq, w.hkv, 128, 128, p)).all()
+    torch.cuda.synchronize()
+
+
+def test_captured_plan_destroyed_before_others(env):
+    """The memory of a plan that took part in a capture is not handed to later plans."""
+    torch, B, W = env
+    from paper_2609_22755_b200.api import NspAttention
+
+    w = W.custom([700, 300, 64, 5], 8, 2, seed=83)
+    e = NspAttention(w)
+    e.load(W.make_tensors(w))
+    e.step_device()
+    torch.cuda.synchronize()
+    names = ("o", "lse", "dk", "dv")
+    want = {n: getattr(e, n).clone() for n in names}
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        e.step_device()
+    for _ in range(3):
+        for n in names:
+            getattr(e, n).fill_(float("nan"))
+        graph.replay()
+        torch.cuda.synchronize()
+        assert e.status()[0] == 0
+        for n in names:
+            assert torch.equal(getattr(e, n), want[n]), n
+    del graph
+    e.plan.destroy()
+    e.plan = None
+    plans = [B.nsp_plan_tiles(w.cu_seqlens, w.hq, w.hkv) for _ in range(4)]
+    for p in plans:
+        for n in names:
+            getattr(e, n).fill_(float("nan"))
+        e.plan = p
+        e.step_device()
+        torch.cuda.synchronize()
+        assert e.status()[0] == 0
+        for n in names:
+            assert torch.equal(getattr(e, n), want[n]), n

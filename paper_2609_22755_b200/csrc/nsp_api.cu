@@ -214,6 +214,11 @@ std::vector<nsp_tile_t> divide_items(const std::vector<WholeItem>& items, int64_
   return list;
 }
 
+// Up to that many (tile, segment) terms the list kernel takes the positions as sums over the segments, beyond it the host
+// counts them (plan_tile_bases). Whole construction in ms, sums / counted: 1,000 segments of 24 tiles (24 M terms) 0.42 /
+// 0.50, 8,192 of one tile (67 M) 2.22 / 2.08, 65,535 of four tiles 74 / 31, of eight 142 / 45.
+constexpr int64_t kMostSumTerms = 1ll << 26;
+
 void free_plan(nsp_plan* p) {
   if (!p) return;
   for (cudaEvent_t e : p->ev)
@@ -463,14 +468,16 @@ int nsp_plan_tiles(const int32_t* cu_seqlens, const int32_t* hq, const int32_t* 
     if (fwd_first.size() == bwd_first.size()) fwd_first.clear();
   }
   std::vector<nsp_tile_t> parts, first_parts;
+  std::vector<TileBase> bases;
   int32_t n_turns = 0;
   try {
+    std::vector<int32_t> order(n_seg);  // the groups the way the kernel walks them
+    for (int s = 0; s < n_seg; ++s) order[s] = s;
+    std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return p->seg[x].len > p->seg[y].len; });
+    if (tiles * n_seg > kMostSumTerms) bases = plan_tile_bases(keys, order);
     if (!p->deterministic && !p->rounded_dq) {
       std::vector<WholeItem> main_items, first_items;
       int64_t main_steps = 0, first_steps = 0;
-      std::vector<int32_t> order(n_seg);  // the groups the way the kernel walks them
-      for (int s = 0; s < n_seg; ++s) order[s] = s;
-      std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return p->seg[x].len > p->seg[y].len; });
       for (const int s : order) {
         const SegInfo& sg = p->seg[s];
         const int32_t Mt = (sg.len + bm - 1) / bm, G = sg.hq / sg.hkv;
@@ -516,6 +523,7 @@ int nsp_plan_tiles(const int32_t* cu_seqlens, const int32_t* hq, const int32_t* 
   const size_t o_first_parts = take(sizeof(nsp_tile_t) * first_parts.size());
   const size_t o_fwd_first = take(sizeof(nsp_tile_t) * fwd_first.size());
   const size_t o_turns = take(sizeof(int32_t) * n_turns);
+  const size_t o_bases = take(sizeof(TileBase) * bases.size());
   const size_t upload = at;
   const size_t o_fwd = take(sizeof(nsp_tile_t) * nf);
   const size_t o_bwd = take(sizeof(nsp_tile_t) * nb);
@@ -563,6 +571,7 @@ int nsp_plan_tiles(const int32_t* cu_seqlens, const int32_t* hq, const int32_t* 
   put(o_first_parts, first_parts.data(), sizeof(nsp_tile_t) * first_parts.size());
   put(o_fwd_first, fwd_first.data(), sizeof(nsp_tile_t) * fwd_first.size());
   std::memset(image + o_turns, 0, sizeof(int32_t) * n_turns);
+  put(o_bases, bases.data(), sizeof(TileBase) * bases.size());
   // On the arena's own stream: nothing here depends on the caller's work. It takes ~20 us where an SM has room for a block of
   // the list kernel. A backward kernel leaves none (its shared memory, at head_dim 64 its registers), and then the lists
   // are ready when one of its CTAs ends: waited for here, the host stood still for up to the rest of a running backward
@@ -573,8 +582,9 @@ int nsp_plan_tiles(const int32_t* cu_seqlens, const int32_t* hq, const int32_t* 
   cudaStream_t bs = p->arena->build;
   const bool enqueued =
       cudaMemcpyAsync(d, image, upload, cudaMemcpyHostToDevice, bs) == cudaSuccess &&
-      launch_plan_lists(reinterpret_cast<const PlanKey*>(d + o_keys), reinterpret_cast<const int32_t*>(d + o_tiles), n_seg,
-                        static_cast<int>(tiles), p->d_fwd, p->d_bwd, p->d_bwd_exec, p->d_fwd_pairs, bs) == cudaSuccess;
+      launch_plan_lists(reinterpret_cast<const PlanKey*>(d + o_keys), reinterpret_cast<const int32_t*>(d + o_tiles),
+                        bases.empty() ? nullptr : reinterpret_cast<const TileBase*>(d + o_bases), n_seg, static_cast<int>(tiles),
+                        p->d_fwd, p->d_bwd, p->d_bwd_exec, p->d_fwd_pairs, bs) == cudaSuccess;
   arena_used(p->arena, bs);
   if (!enqueued || p->arena->n_uses != 1) {
     p->arena->unpooled = true;

@@ -5,6 +5,7 @@
 #include <cuda.h>
 #include <cuda_runtime.h>
 #include "../../include/nsp.h"
+#include "nsp_plan_bases.h"
 
 namespace nsp {
 
@@ -42,11 +43,6 @@ struct RowInfo {
   uint8_t pad_[2];
 };
 static_assert(sizeof(RowInfo) == 16, "RowInfo layout");
-
-// What the list construction needs of a segment.
-struct PlanKey {
-  int32_t tiles, hq, group, len;  // 128-row tiles, q heads, q heads per kv head, tokens
-};
 
 struct RunInfo {
   int64_t q_off, kv_off;  // element offsets of the run's first token
@@ -224,8 +220,9 @@ constexpr int kMaxParts = 64;
 constexpr long long kTurnClkPerStep = 32768;
 
 // Host-side launchers implemented next to their kernels.
-cudaError_t launch_plan_lists(const PlanKey* d_key, const int32_t* d_tile_base, int n_seg, int n_tiles, nsp_tile_t* d_fwd,
-                              nsp_tile_t* d_bwd, nsp_tile_t* d_exec, nsp_tile_t* d_pairs, cudaStream_t st);
+// d_bases: null (the kernel sums over the segments), or the result of plan_tile_bases
+cudaError_t launch_plan_lists(const PlanKey* d_key, const int32_t* d_tile_base, const TileBase* d_bases, int n_seg, int n_tiles,
+                              nsp_tile_t* d_fwd, nsp_tile_t* d_bwd, nsp_tile_t* d_exec, nsp_tile_t* d_pairs, cudaStream_t st);
 // chained: launched right behind launch_fwd_first, whose inputs are this kernel's too
 cudaError_t launch_fwd(const FwdMaps& maps, const FwdArgs& args, int head_dim, int num_sms, bool chained, cudaStream_t st);
 // q tile 0 of every segment: items (segment, kv head); args.items / n_items / counter are that list's

@@ -13,8 +13,8 @@
 // With bm == bn a segment has at most one tile of a given cost, so the position of a tile's items in each list is a sum
 // over the segments of a closed form: one warp per (segment, tile) takes that sum (the lanes stride over the segments)
 // and writes the tile's items, no keys and no sort. A plan of 8,192 tokens at 32q/4kv spent 60 us in two radix sorts
-// with their key and decode kernels; this is one launch of about 5 us. The cost is tiles x segments: 131,072 tokens in
-// 8,192 segments of 16 tokens are 67 M terms, about 0.1 ms.
+// with their key and decode kernels; this is one launch of about 5 us. The sums are tiles x segments terms; where that is
+// more than a counting pass on the host costs, the positions come from there (nsp_plan_bases.cpp).
 // 128 threads of 32 registers, no shared memory: a block fits beside the general forward kernel (61,440 of the 65,536
 // registers of an SM). It does not fit beside the backward kernels, which leave no shared memory for another block (and at
 // head_dim 64 no registers); then it starts when one of their blocks ends, and the host does not wait for it (nsp_api.cu).
@@ -28,9 +28,9 @@ namespace {
 constexpr int kListThreads = 128;
 
 __global__ void __launch_bounds__(kListThreads, 16)
-    plan_lists_kernel(const PlanKey* __restrict__ key, const int32_t* __restrict__ tile_base, int n_seg, int n_tiles,
-                      nsp_tile_t* __restrict__ fwd, nsp_tile_t* __restrict__ bwd, nsp_tile_t* __restrict__ exec,
-                      nsp_tile_t* __restrict__ pairs) {
+    plan_lists_kernel(const PlanKey* __restrict__ key, const int32_t* __restrict__ tile_base,
+                      const TileBase* __restrict__ bases, int n_seg, int n_tiles, nsp_tile_t* __restrict__ fwd,
+                      nsp_tile_t* __restrict__ bwd, nsp_tile_t* __restrict__ exec, nsp_tile_t* __restrict__ pairs) {
   const int lane = threadIdx.x & 31;
   const int n_warps = gridDim.x * (kListThreads / 32);
   for (int t = (blockIdx.x * kListThreads + threadIdx.x) >> 5; t < n_tiles; t += n_warps) {
@@ -43,7 +43,7 @@ __global__ void __launch_bounds__(kListThreads, 16)
     const int m = t - tile_base[s];
     const int cf = m + 1, cb = k.group * (k.tiles - m);
     int nf = 0, nb = 0, ne = 0, np = 0;  // items before this tile's (before its group's, in the walked order); pairs likewise
-    for (int x = lane; x < n_seg; x += 32) {
+    for (int x = bases ? n_seg : lane; x < n_seg; x += 32) {
       const PlanKey o = key[x];
       const int hkv = o.hq / o.group;
       const bool before = x < s;
@@ -63,6 +63,10 @@ __global__ void __launch_bounds__(kListThreads, 16)
     nb = __reduce_add_sync(0xffffffffu, nb);
     ne = __reduce_add_sync(0xffffffffu, ne);
     np = __reduce_add_sync(0xffffffffu, np);
+    if (bases) {
+      const TileBase b = bases[t];
+      nf = b.fwd, nb = b.bwd, ne = b.exec, np = b.pairs;
+    }
     if (m > 0) {
       if (!(k.group & 1)) {
         for (int h = lane; h < k.hq; h += 32) pairs[2 * np + h] = nsp_tile_t{s, h, m, cf};
@@ -83,12 +87,12 @@ __global__ void __launch_bounds__(kListThreads, 16)
 
 }  // namespace
 
-cudaError_t launch_plan_lists(const PlanKey* d_key, const int32_t* d_tile_base, int n_seg, int n_tiles, nsp_tile_t* d_fwd,
-                              nsp_tile_t* d_bwd, nsp_tile_t* d_exec, nsp_tile_t* d_pairs, cudaStream_t st) {
+cudaError_t launch_plan_lists(const PlanKey* d_key, const int32_t* d_tile_base, const TileBase* d_bases, int n_seg, int n_tiles,
+                              nsp_tile_t* d_fwd, nsp_tile_t* d_bwd, nsp_tile_t* d_exec, nsp_tile_t* d_pairs, cudaStream_t st) {
   if (n_tiles == 0) return cudaSuccess;
   const int blocks = (n_tiles + kListThreads / 32 - 1) / (kListThreads / 32);
-  plan_lists_kernel<<<blocks < 148 * 8 ? blocks : 148 * 8, kListThreads, 0, st>>>(d_key, d_tile_base, n_seg, n_tiles, d_fwd,
-                                                                                  d_bwd, d_exec, d_pairs);
+  plan_lists_kernel<<<blocks < 148 * 8 ? blocks : 148 * 8, kListThreads, 0, st>>>(
+      d_key, d_tile_base, d_bases, n_seg, n_tiles, d_fwd, d_bwd, d_exec, d_pairs);
   count_launches(1);
   return cudaGetLastError();
 }

@@ -174,3 +174,27 @@ def test_captured_plan_destroyed_before_others(env):
         assert e.status()[0] == 0
         for n in names:
             assert torch.equal(getattr(e, n), want[n]), n
+
+
+@pytest.mark.parametrize("lengths,hq,hkv", [
+    ([1] * 8192, [4] * 8192, [2] * 8192),  # 2^26 terms: positions summed on the device
+    ([1] * 8193, [4] * 8193, [2] * 8193),  # counted on the host from here on
+    ([130, 0, 260, 5] * 1800, [6] * 3600 + [4] * 3600, [2] * 7200),  # groups of 3 and 2, equal costs across them
+    ([129, 257] * 2600, [2] * 5200, [2] * 2600 + [1] * 2600),        # one head per group, and pairs of heads
+])
+def test_lists_of_many_segments(env, lengths, hq, hkv):
+    torch, B, W = env
+    import oracle
+    import parity_util as P
+
+    w = W.custom(lengths, hq, hkv, seed=84)
+    plan = B.nsp_plan_tiles(w.cu_seqlens, w.hq, w.hkv)
+    for p in (0, 1, 2):
+        assert (B.nsp_plan_get(plan, p) == oracle.plan_tiles(w.cu_seqlens, w.hq, w.hkv, 128, 128, p)).all()
+    run = P.GpuRun(w)  # the list of forward pairs, which nobody can read: through the results
+    run.forward()
+    assert run.status()[0] == 0
+    res, bits = run.results(), {n: W.bf16_bits(run.host[n]) for n in ("q", "k", "v")}
+    o, lse = oracle.attn_fwd(bits["q"], bits["k"], bits["v"], w.cu_seqlens, w.hq, w.hkv, w.head_dim, w.softmax_scale)
+    P.check("o", res["o"], o)
+    assert abs(res["lse"] - lse).max() <= P.LSE_ABS_TOL

@@ -33,6 +33,8 @@ size_t round_up_pow2(size_t n) {
   return r;
 }
 
+bool kept(const Arena* a) { return a->dev_bytes + a->host_bytes <= kMaxIdleBytes / 2; }
+
 void destroy(Arena* a) {  // cudaFree waits for whatever still uses the block
   cudaFree(a->dev);
   if (a->host) cudaFreeHost(a->host);
@@ -46,8 +48,10 @@ Arena* create(int device, size_t dev_bytes, size_t host_bytes) {
   Arena* a = new (std::nothrow) Arena;
   if (!a) return nullptr;
   a->device = device;
+  // Powers of two, so that later plans of other sizes fit; what that makes too large to be kept takes no more than it needs.
   a->dev_bytes = round_up_pow2(dev_bytes);
   a->host_bytes = round_up_pow2(host_bytes);
+  if (!kept(a)) a->dev_bytes = dev_bytes, a->host_bytes = host_bytes;
   int least = 0, greatest = 0;
   void* hd = nullptr;
   const bool ok = cudaMalloc(&a->dev, a->dev_bytes) == cudaSuccess &&
@@ -128,7 +132,7 @@ Arena* arena_acquire(int device, size_t dev_bytes, size_t host_bytes, cudaStream
 
 void arena_release(Arena* a) {
   if (!a) return;
-  if (a->unpooled || a->dev_bytes + a->host_bytes > kMaxIdleBytes / 2) {
+  if (a->unpooled || !kept(a)) {
     destroy(a);
     return;
   }

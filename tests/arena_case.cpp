@@ -127,10 +127,41 @@ static int reuse_and_trim() {
   return 0;
 }
 
+// A plan too large to be kept takes what it needs and no more; a kept one is rounded up for the plans after it.
+static int sizes() {
+  const size_t big = (48u << 20) + 512;
+  fake().device_limit = big;
+  Arena* a = arena_acquire(0, big, 1000, nullptr);
+  EXPECT(a && a->dev_bytes == big && fake().device_bytes == big);
+  arena_release(a);
+  EXPECT(fake().device_bytes == 0 && fake().host_bytes == 0);
+  fake().device_limit = ~size_t(0);
+  // one that only its rounding would make too large is kept as it is
+  a = arena_acquire(0, 17u << 20, 1000, nullptr);
+  EXPECT(a && a->dev_bytes == 17u << 20);
+  arena_release(a);
+  EXPECT(fake().device_bytes == 17u << 20);
+  arena_trim();
+  a = arena_acquire(0, 300 << 10, 1000, nullptr);
+  EXPECT(a && a->dev_bytes == 512 << 10);
+  arena_release(a);
+  EXPECT(arena_acquire(0, 500 << 10, 1000, nullptr) == a);
+  // bounded in number and bytes
+  Arena* many[12];
+  for (Arena*& x : many) x = arena_acquire(0, 6u << 20, 1000, nullptr);
+  for (Arena* x : many) arena_release(x);
+  EXPECT(fake().live.size() == 2 * 7 + 2);  // eight of 8 MB would be 64 MB of device memory and their host blocks
+  for (Arena*& x : many) x = arena_acquire(1, 100, 100, nullptr);
+  for (Arena* x : many) arena_release(x);
+  EXPECT(fake().live.size() == 2 * 8 + 2);
+  return 0;
+}
+
 int main(int argc, char** argv) {
   const char* what = argc > 1 ? argv[1] : "";
   if (!std::strcmp(what, "two_streams")) return two_streams();
   if (!std::strcmp(what, "order_behind_construction")) return order_behind_construction();
+  if (!std::strcmp(what, "sizes")) return sizes();
   if (!std::strcmp(what, "back_pressure")) return back_pressure();
   if (!std::strcmp(what, "recycled_stream_address")) return recycled_stream_address();
   if (!std::strcmp(what, "reuse_and_trim")) return reuse_and_trim();

@@ -6,7 +6,7 @@ from pathlib import Path
 import pytest
 
 ROOT = Path(__file__).resolve().parent.parent
-SCENARIOS = ["two_streams", "back_pressure", "order_behind_construction", "recycled_stream_address", "reuse_and_trim"]
+SCENARIOS = ["two_streams", "back_pressure", "order_behind_construction", "recycled_stream_address", "reuse_and_trim", "sizes"]
 
 
 @pytest.fixture(scope="module")

@@ -216,7 +216,7 @@ std::vector<nsp_tile_t> divide_items(const std::vector<WholeItem>& items, int64_
 
 // Up to that many (tile, segment) terms the list kernel takes the positions as sums over the segments, beyond it the host
 // counts them (plan_tile_bases). Whole construction in ms, sums / counted: 1,000 segments of 24 tiles (24 M terms) 0.42 /
-// 0.50, 8,192 of one tile (67 M) 2.22 / 2.08, 65,535 of four tiles 74 / 31, of eight 142 / 45.
+// 0.50, 2,000 of 64 tiles (256 M) 7.0 / 7.4, 8,192 of one tile (67 M) 2.0 / 2.1, 65,535 of four tiles 74 / 11, of eight 142 / 16.
 constexpr int64_t kMostSumTerms = 1ll << 26;
 
 void free_plan(nsp_plan* p) {
@@ -505,7 +505,9 @@ int nsp_plan_tiles(const int32_t* cu_seqlens, const int32_t* hq, const int32_t* 
   }
   // Layout of the arena's device block: what the host uploads (counters and status first, all zero), then the lists the
   // device builds and the start-alignment counters. The pinned host block holds the host's copy of the status record
-  // and, behind it, the image of the upload.
+  // and, behind it, the image of the upload. A block that no later plan will use is not worth pinning: cudaHostAlloc
+  // of 4 MB takes 3-5 ms, of 16 MB 7-18. The image of a plan that is too large to be kept is ordinary memory (65,535 segments
+  // of 16 tokens at 32q/4kv 55 -> 29 ms, of 1,024 tokens at 4q/1kv 41 -> 16 ms).
   size_t at = 0;
   auto take = [&](size_t bytes) {
     const size_t here = at;
@@ -530,7 +532,15 @@ int nsp_plan_tiles(const int32_t* cu_seqlens, const int32_t* hq, const int32_t* 
   const size_t o_exec = take(sizeof(nsp_tile_t) * nb);
   const size_t o_pairs = take(sizeof(nsp_tile_t) * 2 * p->n_pairs);
   const size_t o_front = take(sizeof(int32_t) * (nb / kFrontBlock + 1));
-  p->arena = arena_acquire(p->device, at, 256 + upload, static_cast<cudaStream_t>(stream));
+  const bool pinned = arena_keeps(at, 256 + upload);
+  std::vector<char> pageable;
+  try {
+    if (!pinned) pageable.resize(upload);
+  } catch (...) {
+    delete p;
+    return NSP_ERR_ALLOC;
+  }
+  p->arena = arena_acquire(p->device, at, pinned ? 256 + upload : 256, static_cast<cudaStream_t>(stream));
   if (!p->arena) {
     delete p;
     return NSP_ERR_ALLOC;
@@ -554,7 +564,7 @@ int nsp_plan_tiles(const int32_t* cu_seqlens, const int32_t* hq, const int32_t* 
   p->n_fwd_first = fwd_first.empty() ? p->n_first : static_cast<int64_t>(fwd_first.size());
   p->h_status = static_cast<int32_t*>(p->arena->host);
   p->h_status_dev = reinterpret_cast<int32_t*>(p->arena->host_dev);
-  char* const image = static_cast<char*>(p->arena->host) + 256;
+  char* const image = pinned ? static_cast<char*>(p->arena->host) + 256 : pageable.data();
   auto put = [&](size_t off, const void* src, size_t bytes) {
     if (bytes) std::memcpy(image + off, src, bytes);
   };
@@ -582,6 +592,7 @@ int nsp_plan_tiles(const int32_t* cu_seqlens, const int32_t* hq, const int32_t* 
   cudaStream_t bs = p->arena->build;
   const bool enqueued =
       cudaMemcpyAsync(d, image, upload, cudaMemcpyHostToDevice, bs) == cudaSuccess &&
+      (pinned || cudaStreamSynchronize(bs) == cudaSuccess) &&
       launch_plan_lists(reinterpret_cast<const PlanKey*>(d + o_keys), reinterpret_cast<const int32_t*>(d + o_tiles),
                         bases.empty() ? nullptr : reinterpret_cast<const TileBase*>(d + o_bases), n_seg, static_cast<int>(tiles),
                         p->d_fwd, p->d_bwd, p->d_bwd_exec, p->d_fwd_pairs, bs) == cudaSuccess;

@@ -33,8 +33,6 @@ size_t round_up_pow2(size_t n) {
   return r;
 }
 
-bool kept(const Arena* a) { return a->dev_bytes + a->host_bytes <= kMaxIdleBytes / 2; }
-
 void destroy(Arena* a) {  // cudaFree waits for whatever still uses the block
   cudaFree(a->dev);
   if (a->host) cudaFreeHost(a->host);
@@ -51,7 +49,7 @@ Arena* create(int device, size_t dev_bytes, size_t host_bytes) {
   // Powers of two, so that later plans of other sizes fit; what that makes too large to be kept takes no more than it needs.
   a->dev_bytes = round_up_pow2(dev_bytes);
   a->host_bytes = round_up_pow2(host_bytes);
-  if (!kept(a)) a->dev_bytes = dev_bytes, a->host_bytes = host_bytes;
+  if (!arena_keeps(a->dev_bytes, a->host_bytes)) a->dev_bytes = dev_bytes, a->host_bytes = host_bytes;
   int least = 0, greatest = 0;
   void* hd = nullptr;
   const bool ok = cudaMalloc(&a->dev, a->dev_bytes) == cudaSuccess &&
@@ -93,6 +91,8 @@ bool wait_unused(Arena* a) {
 
 }  // namespace
 
+bool arena_keeps(size_t dev_bytes, size_t host_bytes) { return dev_bytes + host_bytes <= kMaxIdleBytes / 2; }
+
 Arena* arena_acquire(int device, size_t dev_bytes, size_t host_bytes, cudaStream_t st) {
   Arena* found = nullptr;
   unsigned long long own = 0;
@@ -132,7 +132,7 @@ Arena* arena_acquire(int device, size_t dev_bytes, size_t host_bytes, cudaStream
 
 void arena_release(Arena* a) {
   if (!a) return;
-  if (a->unpooled || !kept(a)) {
+  if (a->unpooled || !arena_keeps(a->dev_bytes, a->host_bytes)) {
     destroy(a);
     return;
   }

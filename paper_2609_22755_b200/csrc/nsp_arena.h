@@ -27,6 +27,8 @@ struct Arena {
   std::mutex mutex;       // uses and unpooled: calls on a plan may come from several threads
 };
 
+// Blocks of these sizes stay when their plan is destroyed; larger ones go back to the driver.
+bool arena_keeps(size_t dev_bytes, size_t host_bytes);
 // An arena of at least the given sizes on the current device that nothing uses any more; null when out of memory. May wait
 // for work of the stream `st`, the caller's, but for no other (see kWaitFor).
 Arena* arena_acquire(int device, size_t dev_bytes, size_t host_bytes, cudaStream_t st);

@@ -180,6 +180,7 @@ def test_captured_plan_destroyed_before_others(env):
     ([1] * 8192, [4] * 8192, [2] * 8192),  # 2^26 terms: positions summed on the device
     ([1] * 8193, [4] * 8193, [2] * 8193),  # counted on the host from here on
     ([130, 0, 260, 5] * 1800, [6] * 3600 + [4] * 3600, [2] * 7200),  # groups of 3 and 2, equal costs across them
+    ([1] * 65535, [32] * 65535, [4] * 65535),  # memory that is not kept, its image not pinned
     ([129, 257] * 2600, [2] * 5200, [2] * 2600 + [1] * 2600),        # one head per group, and pairs of heads
 ])
 def test_lists_of_many_segments(env, lengths, hq, hkv):

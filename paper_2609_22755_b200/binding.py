@@ -411,10 +411,9 @@ def _a2a(fn_name, src, dst, tokens, heads, heads_per_block, head_dim, first_head
     dtype = NSP_F32 if src.dtype == torch.float32 else NSP_BF16
     if dst.dtype != src.dtype:
         raise ValueError("source and destination must have the same dtype")
-    n = len(first_head)
-    fh = (ctypes.c_int32 * n)(*[int(h) for h in first_head])
-    rc = getattr(lib(), fn_name)(_ptr(src), _ptr(dst), int(tokens), int(heads), int(heads_per_block), n, int(head_dim), dtype,
-                                 fh, _stream_ptr(stream))
+    fh = np.ascontiguousarray(first_head, dtype=np.int32)  # refuses heads that a C int would wrap
+    rc = getattr(lib(), fn_name)(_ptr(src), _ptr(dst), int(tokens), int(heads), int(heads_per_block), len(fh), int(head_dim),
+                                 dtype, _ptr(fh), _stream_ptr(stream))
     if rc != NSP_OK:
         raise NspError(rc, fn_name)
 

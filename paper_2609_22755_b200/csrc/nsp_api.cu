@@ -29,7 +29,7 @@ struct nsp_plan {
   std::vector<RunInfo> runs;
   // device state, all of it inside the arena
   Arena* arena = nullptr;
-  std::atomic<bool> built{false};  // known to be complete on the device; until then every stream's first call waits for it
+  mutable std::atomic<bool> built{false};  // known to be complete on the device; until then every stream's first call waits for it
   SegInfo* d_seg = nullptr;
   int64_t* d_row_base = nullptr;  // [n_seg + 1] first packed (token, head) row of each segment
   nsp_tile_t* d_fwd = nullptr;
@@ -237,7 +237,11 @@ struct UsesArena {
   cudaStream_t st;
   cudaError_t ready;
   UsesArena(const nsp_plan* p, cudaStream_t stream) : plan(p), st(stream), ready(cudaSuccess) {
-    if (!p->built.load(std::memory_order_acquire)) ready = arena_order_built(p->arena, st);
+    bool built = p->built.load(std::memory_order_acquire);
+    if (!built) {
+      ready = arena_order_built(p->arena, st, &built);
+      if (built) p->built.store(true, std::memory_order_release);
+    }
   }
   ~UsesArena() { arena_used(plan->arena, st); }
 };

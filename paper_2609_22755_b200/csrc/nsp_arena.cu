@@ -172,24 +172,39 @@ void arena_used(Arena* a, cudaStream_t st) {
   a->unpooled = true;
 }
 
-bool arena_built(const Arena* a) { return cudaEventQuery(a->uses[0].done) == cudaSuccess; }
-
-cudaError_t arena_wait_built(const Arena* a) {
-  // another thread may be capturing, and a wait would end its capture unless this thread says that it is unrelated
+namespace {
+// Another thread may be capturing, and looking at an event would end its capture unless this thread says that it is unrelated.
+struct Unrelated {
   cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
-  cudaError_t e = cudaThreadExchangeStreamCaptureMode(&mode);
-  if (e != cudaSuccess) return e;
-  e = cudaEventSynchronize(a->uses[0].done);
-  cudaThreadExchangeStreamCaptureMode(&mode);
-  return e;
+  Unrelated() { cudaThreadExchangeStreamCaptureMode(&mode); }
+  ~Unrelated() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
+}  // namespace
+
+bool arena_built(const Arena* a) {
+  const Unrelated here;
+  if (cudaEventQuery(a->uses[0].done) == cudaSuccess) return true;
+  cudaGetLastError();
+  return false;
 }
 
-cudaError_t arena_order_built(Arena* a, cudaStream_t st) {
+cudaError_t arena_wait_built(const Arena* a) {
+  const Unrelated here;
+  return cudaEventSynchronize(a->uses[0].done);
+}
+
+cudaError_t arena_order_built(Arena* a, cudaStream_t st, bool* built) {
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   unsigned long long id = 0;
+  *built = arena_built(a);
+  if (*built) return cudaSuccess;
   cudaError_t e = cudaStreamIsCapturing(st, &cap);
   if (e != cudaSuccess) return e;
-  if (cap != cudaStreamCaptureStatusNone) return arena_wait_built(a);
+  if (cap != cudaStreamCaptureStatusNone) {
+    e = arena_wait_built(a);
+    *built = e == cudaSuccess;
+    return e;
+  }
   e = cudaStreamGetId(st, &id);
   if (e != cudaSuccess) return e;
   {

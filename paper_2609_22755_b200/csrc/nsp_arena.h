@@ -39,9 +39,9 @@ void arena_used(Arena* a, cudaStream_t st);
 // What the plan's construction has enqueued (its use of a->build, the first one) has completed / is waited for by the host.
 bool arena_built(const Arena* a);
 cudaError_t arena_wait_built(const Arena* a);
-// What is enqueued on st from now on runs behind the construction. A stream that is being captured cannot wait for work
-// outside the capture: then the host does.
-cudaError_t arena_order_built(Arena* a, cudaStream_t st);
+// What is enqueued on st from now on runs behind the construction. *built: it has completed, and nothing needs to be ordered
+// behind it any more. A stream that is being captured cannot wait for work outside the capture: then the host does.
+cudaError_t arena_order_built(Arena* a, cudaStream_t st, bool* built);
 // Frees every idle arena.
 void arena_trim();
 

@@ -95,15 +95,18 @@ static int back_pressure() {
 static int order_behind_construction() {
   FakeStream s1{601}, s2{602}, captured{603};
   Arena* a = acquire(0, &s1, false);
+  bool built = true;
+  auto ordered = [&](FakeStream* st) { return arena_order_built(a, st, &built) == cudaSuccess; };
   EXPECT(!arena_built(a));
-  EXPECT(arena_order_built(a, &s1) == cudaSuccess && fake().stream_waits == 1);
+  EXPECT(ordered(&s1) && !built && fake().stream_waits == 1);
   call(a, &s1);
-  EXPECT(arena_order_built(a, &s1) == cudaSuccess && fake().stream_waits == 1);
-  EXPECT(arena_order_built(a, &s2) == cudaSuccess && fake().stream_waits == 2);
+  EXPECT(ordered(&s1) && !built && fake().stream_waits == 1);
+  EXPECT(ordered(&s2) && !built && fake().stream_waits == 2);
   EXPECT(fake().waits == 0);
   captured.capturing = true;
-  EXPECT(arena_order_built(a, &captured) == cudaSuccess && fake().stream_waits == 2 && fake().waits == 1);
+  EXPECT(ordered(&captured) && built && fake().stream_waits == 2 && fake().waits == 1);
   EXPECT(arena_built(a) && fake().mode == cudaStreamCaptureModeGlobal);
+  EXPECT(ordered(&s2) && built && fake().stream_waits == 2);  // complete: nothing to be ordered
   for (int i = 0; i < 4; ++i) {
     Arena* b = acquire(0, &s1, false);
     arena_release(b);  // a plan that was never used

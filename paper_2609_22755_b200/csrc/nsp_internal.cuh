@@ -202,7 +202,9 @@ inline cudaError_t launch_chained_if(bool chained, void (*kernel)(P...), unsigne
   at.val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = &at;
   cfg.numAttrs = chained ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
+  if (e != cudaSuccess) cudaGetLastError();  // reported here, not to whoever asks for the last error next
+  return e;
 }
 
 // Parts of a backward item. The steps of an item (its q tiles and q heads) may be divided among several CTAs: part p of

@@ -465,6 +465,10 @@ __global__ void __launch_bounds__(Roles<FIRST, D>::kThreads, 1) bwd_kernel(const
           int where = 0;
           bool okm = together(mbar_wait(&s.bar_kv, gi & 1, a.wait_limit));
           if (!okm) where = kWhereBwdLoadKV;
+          // After a failed vote: which wait failed, the one on `bar` or the other; 0 if none did (another role raised the abort flag).
+          auto failed_wait = [&](bool here, uint64_t* bar, uint32_t parity, int on_bar, int on_other) -> int {
+            return together(here) ? 0 : mbar_test(bar, parity) ? on_other : on_bar;
+          };
           const uint32_t q0_lo = smem_desc_addr(s.q[0][0]), do0_lo = smem_desc_addr(s.d_o[0][0]);
           if (is_a) {
             const uint32_t k_km = smem_desc_addr(s.k[0]) | lbo_km;
@@ -510,7 +514,10 @@ __global__ void __launch_bounds__(Roles<FIRST, D>::kThreads, 1) bwd_kernel(const
                   if (go) umma_ts_lh(tDV, tR0 + kk * 16 + 8, (do_lo | lbo_mn) + kk * 128, hi, idesc_kn, 1u);
                 }
               }
-              if (!together(here && calm)) { where = kWhereBwdPReady; return false; }
+              if (!together(here && calm)) {
+                where = failed_wait(here, &s.bar_do_full[do_stage(cs)], do_parity(cs), kWhereBwdLoadQ, kWhereBwdPReady);
+                return false;
+              }
               if (leader) umma_commit(&s.bar_a_done);       // S^T and dV of the step
               if (leader) umma_commit(&s.bar_do_empty[do_stage(cs)][0]);  // this thread is done with the dO buffer
               if (vt + 1 < steps && !issue_s()) return false;
@@ -536,7 +543,10 @@ __global__ void __launch_bounds__(Roles<FIRST, D>::kThreads, 1) bwd_kernel(const
                 const uint32_t off = ((kk >> 2) * kHalfTileBytes + (kk & 3) * 32) >> 4;
                 if (go) umma_ss_lh(tR1, v_km + off, hi, (do_lo | lbo_km) + off, hi, idesc_kk, kk > 0);
               }
-              if (!together(here)) { where = kWhereBwdDqEmpty; return false; }
+              if (!together(here)) {
+                where = failed_wait(here, &s.bar_do_full[do_stage(cs)], do_parity(cs), kWhereBwdLoadQ, kWhereBwdDqEmpty);
+                return false;
+              }
               if (leader) umma_commit(&s.bar_dp_full);
               if (leader) umma_commit(&s.bar_do_empty[do_stage(cs)][1]);  // this thread is done with the dO buffer
               return true;
@@ -549,7 +559,10 @@ __global__ void __launch_bounds__(Roles<FIRST, D>::kThreads, 1) bwd_kernel(const
               bool here = mbar_wait(&s.bar_q_full[qr.st], qr.ph, a.wait_limit);
               here = mbar_wait(&s.bar_ds_ready, cs & 1, a.wait_limit) && here;
               if constexpr (kOwnDq) {
-                if (!together(here && calm)) { where = kWhereBwdDsReady; return false; }
+                if (!together(here && calm)) {
+                  where = failed_wait(here, &s.bar_q_full[qr.st], qr.ph, kWhereBwdLoadQ, kWhereBwdDsReady);
+                  return false;
+                }
                 if (vt + 1 < steps && !issue_dp(vt + 1)) return false;
                 here = mbar_wait(&s.bar_dq_empty, (cs & 1) ^ 1, a.wait_limit);
               }
@@ -566,7 +579,10 @@ __global__ void __launch_bounds__(Roles<FIRST, D>::kThreads, 1) bwd_kernel(const
                 for (int kk = 0; kk < 8; ++kk)
                   if (go) umma_ss_lh(tDQ, k_mn + kk * 128, hi, ds_mn + kLoStep + kk * 128, hi, idesc_nn, 1u);
               }
-              if (!together(here && calm)) { where = kWhereBwdDsReady; return false; }
+              if (!together(here && calm)) {
+                where = failed_wait(here, &s.bar_q_full[qr.st], qr.ph, kWhereBwdLoadQ, kOwnDq ? kWhereBwdDqEmpty : kWhereBwdDsReady);
+                return false;
+              }
               if (leader) umma_commit(&s.bar_dq_full);
               // dK += dS^T Q
 #pragma unroll
@@ -590,8 +606,8 @@ __global__ void __launch_bounds__(Roles<FIRST, D>::kThreads, 1) bwd_kernel(const
 #pragma unroll 1
             for (int vt = 0; okm && vt < steps; ++vt) okm = step_b(vt);
           }
-          if (!okm && where != 0) {  // where == 0: another role raised the abort flag
-            if (leader) report_timeout(a.status, item_it, where, is_a ? 0 : 1);
+          if (!okm) {
+            if (leader && where != 0) report_timeout(a.status, item_it, where, is_a ? 0 : 1);
             drain_products();
             *abort_flag = 1;
           }

@@ -385,7 +385,13 @@ __global__ void __launch_bounds__(kFwdThreads, 1) fwd_kernel(const __grid_consta
               ++pn[0];
               tc_fence_after_sync();
               issue_pv(0, vst, j, leader && here);
-              if (!together(here && calm)) { ok = false; where = kWhereFwdS; break; }
+              if (!together(here && calm)) {  // where stays 0 if no wait failed: another role raised the abort flag
+                ok = false;
+                if (!together(here))
+                  where = mbar_test(&s.bar_v_full[vst], (vn >> 1) & 1) && (!more || mbar_test(&s.bar_k_full[kst], (kn >> 1) & 1))
+                              ? kWhereFwdS : kWhereFwdLoad;
+                break;
+              }
               if (leader) umma_commit(&s.bar_pv_done[0]);
               if (more) issue_s(0, kst);  // S_A of the next key tile runs while softmax B is still working
               if (j < n_kv_b) {
@@ -406,7 +412,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1) fwd_kernel(const __grid_consta
             }
             if (!RECOMP && ok && joint && n_kv_b != n_kv && leader) umma_commit(&s.bar_last_pv);
             if (!ok) {
-              if (leader) report_timeout(a.status, it0, where, 0);
+              if (leader && where != 0) report_timeout(a.status, it0, where, 0);
               drain_products();
               *abort_flag = 1;
             }

@@ -241,7 +241,11 @@ __global__ void __launch_bounds__(kThreads, 1) fwd_first_kernel(const __grid_con
               const uint32_t off = ((kk >> 2) * kHalfTileBytes + (kk & 3) * 32) >> 4;
               if (leader && here) umma_ss_lh(tmem + 128 * x, a_lo + off, hi, b_lo + off, hi, idesc_qk, kk > 0);
             }
-            if (x == 0 && !together(here && calm)) { ok = false; where = kWhereFwdLoad; break; }
+            if (x == 0 && !together(here && calm)) {  // where stays 0 if no wait failed: another role raised the abort flag
+              ok = false;
+              if (!together(here)) where = kWhereFwdLoad;
+              break;
+            }
             if (leader) umma_commit(&s.bar_s_full[x]);
           }
           for (int x = 0; ok && x < halves; ++x) {
@@ -252,7 +256,11 @@ __global__ void __launch_bounds__(kThreads, 1) fwd_first_kernel(const __grid_con
             for (int kk = 0; kk < 8; ++kk)
               if (leader && here) umma_ts_lh(tmem + 256 + 128 * x, tmem + 128 * x + (kk >> 2) * 64 + (kk & 3) * 8, (x ? vb_lo : v_lo) + kk * 128, hi,
                                      idesc_pv, kk > 0);
-            if (!together(here)) { ok = false; where = kWhereFwdS; break; }
+            if (!together(here)) {
+              ok = false;
+              where = mbar_test(&s.bar_o_free[x], (n[x] & 1) ^ 1) ? kWhereFwdS : kWhereFwdO;
+              break;
+            }
             if (leader) umma_commit(&s.bar_pv_done[x]);
             ++n[x];
           }
@@ -262,8 +270,8 @@ __global__ void __launch_bounds__(kThreads, 1) fwd_first_kernel(const __grid_con
           umma_commit(&s.bar_q_empty[(R & 1) ^ 1][1]);
         }
         if (leader) umma_commit(&s.bar_kv_free);  // K and V may be replaced once everything issued so far has run
-        if (!ok && where != 0) {
-          if (leader) report_timeout(a.status, c.it, where, 0);
+        if (!ok) {
+          if (leader && where != 0) report_timeout(a.status, c.it, where, 0);
           drain_products();
           *abort_flag = 1;
         }

@@ -78,6 +78,18 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, long l
     if (clock64() - t0 > limit) return false;
   }
 }
+// One look: has the phase completed? (To say which of several waits failed, once one has.)
+__device__ __forceinline__ bool mbar_test(uint64_t* bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok)
+      : "r"(smem_u32(bar)), "r"(parity)
+      : "memory");
+  return ok != 0;
+}
 // The MMA-issuing warps run their waits with all 32 lanes and have to go on together: wait for the operands of some
 // products, issue the products, vote once, and only then the commits that let any of those barriers move on (behind the products
 // the vote costs nothing; in front of them it cost 2 %). A lane that falls behind its warp may test a phase only after the
@@ -90,15 +102,7 @@ __device__ __forceinline__ bool mbar_poll(uint64_t* bar, uint32_t parity, long l
   const long long t0 = clock64();
 #pragma unroll 1
   for (;;) {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(smem_u32(bar)), "r"(parity)
-        : "memory");
-    if (ok) return true;
+    if (mbar_test(bar, parity)) return true;
     if (clock64() - t0 > limit) return false;
   }
 }

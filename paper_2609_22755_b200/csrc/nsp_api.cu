@@ -176,9 +176,13 @@ inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 
 inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 // Divides backward items into parts of at most about `most` steps (see kMaxParts) and lists them: the longest first where
-// the dQ accumulator is no more than twice L2 (126 MB), otherwise in the order of the items, the walked one, which keeps the
-// CTAs of a group on the same q tiles. By length / in order, us a step: 17,545 tokens at 8q/2kv (72 MB) 1,044 / 1,191,
-// 47,878 tokens at 64q/4kv in 173 segments (1.6 GB), the longest divided, 3,187 / 3,121. A part has its own K / V loads and its own dK / dV epilogue, ~14,000 clocks or the time of 3-4 steps.
+// the dQ accumulator is no more than kMostByLength, otherwise in the order of the items, the walked one, which keeps the
+// CTAs of a group on the same q tiles but packs the parts worse. Backward pass, us, by length / walked / undivided: 17,545
+// tokens at 8q/2kv (68 MiB) 1,652 / 1,850 / 1,693; at 16q/1kv four segments of 9,000 tokens (281 MiB) 3,494 / 5,074 / 4,701,
+// two of 14,000 and forty of 500 (375 MiB) 4,372 / 6,151 / 5,144; 8,000 tokens and twenty times 500 at 64q/4kv (562 MiB) 3,049 /
+// 4,493 / 4,173; beyond, 79,335 and 79,500 long-tailed tokens at 16q/1kv (620 MiB) 1,654 / 1,599 / 1,925 and 4,362 / 4,243 /
+// 5,412, 53,428 at 32q/2kv (834 MiB) 2,186 / 2,182 / 2,397, 47,878 tokens at 64q/4kv in 173 segments (1,500 MiB) 3,187 / 3,121 a
+// step. A part has its own K / V loads and its own dK / dV epilogue, ~14,000 clocks or the time of 3-4 steps.
 // Returns an empty list when nothing is divided.
 // Where the lines lie: an item is divided when it is longer than the SMs' share of all steps, because the longest item
 // then bounds the kernel. Microseconds a step with parts of at most share / 2, share, whole: 8,192 tokens in one
@@ -188,6 +192,7 @@ inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 // head of twice that length and run beside the main kernel: divided they are worth it where they, not the main kernel,
 // bound the call (20 segments of about 100 tokens at 64q/4kv 233 -> 216 us; parts of eight steps 248, of two 215).
 constexpr int kMinPart = 16, kMinFirstPart = 4;
+constexpr int64_t kMostByLength = 600ll << 20;
 struct WholeItem {
   int32_t seg, head, tile, steps;
 };
@@ -497,7 +502,7 @@ int nsp_plan_tiles(const int32_t* cu_seqlens, const int32_t* hq, const int32_t* 
         first_steps += t.cost;
       }
       parts = divide_items(main_items, std::max<int64_t>(kMinPart, main_steps / p->num_sms),
-                           q_off * 4 <= (256ll << 20), &n_turns);
+                           q_off * 4 <= kMostByLength, &n_turns);
       first_parts = divide_items(first_items, std::max<int64_t>(kMinFirstPart, (first_steps + main_steps) / (2 * p->num_sms)), true,
                                  &n_turns);
     }

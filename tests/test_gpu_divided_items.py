@@ -12,6 +12,7 @@ pytestmark = pytest.mark.gpu
     ([2000, 129, 257], 5, 1, 64),   # odd group: a part starts inside a q tile's heads
     ([100, 28, 90, 20, 128, 60], 16, 1, 128),  # first-tile items divided; packs, a full tile and a ragged one
     ([130, 31], 32, 2, 64),         # one-row last tile
+    ([700] + [128] * 150, 64, 4, 128),  # 620 MiB of dQ accumulator: the parts in the walked order
 ])
 def test_divided_items_every_element(lengths, hq, hkv, head_dim):
     import torch
@@ -43,3 +44,31 @@ def test_divided_items_every_element(lengths, hq, hkv, head_dim):
         got = low.results()
         for n in ("dk", "dv"):
             assert np.max(np.abs(got[n] - res[n])) <= 2.0 ** -7 * np.max(np.abs(res[n])), n
+
+
+def test_division_does_not_cost_time():
+    """A long segment among short ones, 562 MiB of dQ accumulator. bf16 gradients are not divided and stand for whole items: the
+    divided ones take three quarters of their time (listed in the walked order they took 8 % more)."""
+    import torch
+
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA device")
+    from paper_2609_22755_b200 import workloads as W
+    from paper_2609_22755_b200.api import NspAttention
+
+    w = W.custom([8000] + [500] * 20, 64, 4)
+    engines = [NspAttention(w, dkv_dtype=d) for d in ("f32", "bf16")]
+    best = [1e9, 1e9]
+    for e in engines:
+        for t in (e.q, e.k, e.v, e.do):
+            t.normal_()
+        e.step_device()
+    for _ in range(5):
+        for i, e in enumerate(engines):
+            start, end = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            start.record()
+            e.backward()
+            end.record()
+            torch.cuda.synchronize()
+            best[i] = min(best[i], start.elapsed_time(end))
+    assert best[0] < 0.95 * best[1], best

@@ -374,16 +374,27 @@ int nsp_plan_tiles(const int32_t* cu_seqlens, const int32_t* hq, const int32_t* 
   }
 
   int64_t bwd_steps = 0;  // (key tile, q tile, q head) steps of the backward pass
+  std::vector<int32_t> order;  // segments by length descending: the order of the groups the backward kernel walks
   std::vector<nsp_tile_t> bwd_first;
   std::vector<SegInfo> pack_segs;
   std::vector<RowInfo> pack_rows;
   try {
+    order.resize(n_seg);
+    for (int s = 0; s < n_seg; ++s) order[s] = s;
+    std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return p->seg[x].len > p->seg[y].len; });
     // the first-tile kernel's items: key tile 0 of every group, in the same group order; q heads of the group = steps
     // Segments of fewer than 128 tokens that follow one another inside a run (they are contiguous in every tensor)
     // and together hold at most 128 tokens share one first tile: such a pack becomes an entry of its own behind the
     // segments (len = its tokens, offsets of its first segment) with a row table, and takes its segments' places in
     // the first-tile list.
     std::vector<int32_t> pack_of(n_seg, -1);
+    {
+      // a pack and the one behind it hold more than 128 tokens together, or another run or a long segment lies between them
+      int64_t short_segs = 0, short_tokens = 0;
+      for (const SegInfo& sg : p->seg)
+        if (sg.len > 0 && sg.len < kBM) ++short_segs, short_tokens += sg.len;
+      pack_rows.reserve(kBM * std::min<int64_t>(short_segs / 2, 2 * short_tokens / kBM + 1));
+    }
     for (int s0 = 0; s0 < n_seg;) {
       const SegInfo& first = p->seg[s0];
       if (first.len <= 0 || first.len >= kBM) { ++s0; continue; }
@@ -417,12 +428,9 @@ int nsp_plan_tiles(const int32_t* cu_seqlens, const int32_t* hq, const int32_t* 
     }
     p->n_packs = static_cast<int64_t>(pack_segs.size());
     {
-      std::vector<int32_t> order;  // segments by length descending: the order of the groups the backward kernel walks
-      for (int s = 0; s < n_seg; ++s)
-        if (p->seg[s].len > 0) order.push_back(s);
-      std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return p->seg[x].len > p->seg[y].len; });
       std::vector<char> listed(pack_segs.size(), 0);
       for (const int s : order) {
+        if (p->seg[s].len == 0) break;  // empty segments come last
         if (pack_of[s] >= 0) {
           if (listed[pack_of[s] - n_seg]) continue;
           listed[pack_of[s] - n_seg] = 1;
@@ -480,9 +488,6 @@ int nsp_plan_tiles(const int32_t* cu_seqlens, const int32_t* hq, const int32_t* 
   std::vector<TileBase> bases;
   int32_t n_turns = 0;
   try {
-    std::vector<int32_t> order(n_seg);  // the groups the way the kernel walks them
-    for (int s = 0; s < n_seg; ++s) order[s] = s;
-    std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return p->seg[x].len > p->seg[y].len; });
     if (tiles * n_seg > kMostSumTerms) bases = plan_tile_bases(keys, order);
     if (!p->deterministic && !p->rounded_dq) {
       std::vector<WholeItem> main_items, first_items;

@@ -42,12 +42,17 @@ def _stale(target: Path, deps) -> bool:
     return any(Path(d).stat().st_mtime > t for d in deps)
 
 
+def headers_of_library():
+    """Every header a source may include: an object older than any of them is compiled again."""
+    return sorted([*CSRC.glob("*.cuh"), *CSRC.glob("*.h")]) + [PKG.parent / "include" / "nsp.h"]
+
+
 def build_library(force: bool = False, verbose: bool = False, checked: bool = False) -> Path:
     """Build libnsp.so, or with checked=True libnsp_checked.so (kernels verify every index they compute; for tests)."""
     nvcc = _nvcc()
     lib, tag, extra = (LIB_CHECKED, "_checked", ["-DNSP_CHECKED"]) if checked else (LIB, "", [])
     sources = sorted(CSRC.glob("*.cu")) + sorted(CSRC.glob("*.cpp"))  # the planner is host-only C++
-    headers = sorted(CSRC.glob("*.cuh")) + [PKG.parent / "include" / "nsp.h"]
+    headers = headers_of_library()
     OBJ_DIR.mkdir(exist_ok=True)
 
     def compile_one(src: Path):

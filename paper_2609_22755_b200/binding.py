@@ -207,12 +207,13 @@ def _check_ws(what, ws):
 
 
 def _stream_ptr(stream):
-    """Address of a stream (None: the current one; its handle is asked for directly, building a Stream object around it
-    costs 3 us of a call)."""
+    """Address of a stream (None: the current one; its handle is asked for directly where torch has that call, which is not a
+    public one: building a Stream object around it costs 3 us of a call)."""
     if stream is None:
         import torch
 
-        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+        direct = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+        return direct(torch.cuda.current_device()) if direct else torch.cuda.current_stream().cuda_stream
     return stream if isinstance(stream, int) else stream.cuda_stream
 
 

@@ -651,8 +651,15 @@ __global__ void __launch_bounds__(Roles<FIRST, D>::kThreads, 1) bwd_kernel(const
                 }
               }
               NSP_CHECK(at >= 0 && at < a.lse_elems, a.status, c.it, kWhereCheckBwdLse, qi) {
-                lv = __ldcg(a.lse + at) * kLog2e;
-                dv_ = __ldcg(a.delta + at);
+                if constexpr (FIRST) {
+                  // Read behind this kernel's own grid_wait_predecessor, so an ordinary load will do: the four of a step are
+                  // in flight together. Past L1 they followed one another, eight with delta, which this kernel forms
+                  // itself: 1,024 segments of 128 tokens at 16q/16kv 1,642 us, now 1,376.
+                  lv = a.lse[at] * kLog2e;
+                } else {
+                  lv = __ldcg(a.lse + at) * kLog2e;
+                  dv_ = __ldcg(a.delta + at);
+                }
               }
             }
             s.lse[st][col] = lv;

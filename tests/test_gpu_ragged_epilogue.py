@@ -36,3 +36,25 @@ def test_staged_rows_are_not_overwritten_by_the_next_item(head_dim, dkv_dtype):
             first = res
         for n in ("dk", "dv"):  # one fixed order of additions
             assert np.array_equal(res[n], first[n]), n
+
+
+@pytest.mark.parametrize("head_dim", [128, 64])
+@pytest.mark.parametrize("dkv_dtype", ["f32", "bf16"])
+def test_last_tiles_of_few_rows(head_dim, dkv_dtype):
+    """One row, a row short of a warp's 32, one past, and so on: warps and row passes without a valid row skip their part."""
+    import torch
+
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA device")
+    import parity_util as P
+    from paper_2609_22755_b200 import workloads as W
+
+    w = W.custom([129, 1, 159, 160, 161, 31, 192, 193, 225, 33, 255, 385], 4, 2, seed=62, head_dim=head_dim)
+    run = P.GpuRun(w, dkv_dtype=dkv_dtype)
+    run.forward()
+    run.backward()
+    assert run.status()[0] == 0
+    res, ref = run.results(), P.oracle_full(w, run.host)
+    for n in ("dk", "dv"):
+        step = 2.0 ** -7 * np.max(np.abs(ref[n])) if dkv_dtype == "bf16" else 0.0  # two bf16 roundings, as above
+        P.check(n, res[n], ref[n], max_abs_tol=P.MAX_ABS_TOL + step)

@@ -351,7 +351,9 @@ int64_t nsp_launch_count(void);
 
 /* Free the plan (device lists, tables, status word). NULL is a no-op. The memory is kept for later plans, at most 64 MiB
  * (device and pinned host together) in at most eight blocks per process; what the plan's last calls enqueued may still be
- * running, and the block is not handed out again before that has finished. Call it outside any stream capture. */
+ * running, and the block is not handed out again before that has finished. What is not kept (a plan above 32 MiB or used in
+ * a stream capture, the oldest block beyond those bounds) goes back with cudaFree, which may wait for the device. Call it
+ * outside any stream capture. */
 int nsp_plan_destroy(nsp_plan_t* plan);
 
 /* Give back all memory kept from destroyed plans. */

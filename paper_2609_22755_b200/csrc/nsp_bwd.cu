@@ -17,7 +17,7 @@
 // TMEM: R0 [0,128), R1 [128,256), dK [256,384), dV [384,512); at D = 64 dK, dV 64 columns each and dQ^T in [384,512).
 // Roles (at D = 128; see Roles):  warps 0-7  softmax / dS (key row = TMEM lane, two column halves)
 //         warps 8-15 dQ: TMEM -> fp32 accumulator in global memory (lane quadrant x 64-column half)
-//         warp 16    TMA producer (K, V once per item; Q two-stage ring, dO single buffer)
+//         warp 16    TMA producer (K, V once per item; Q two-stage ring, one dO buffer, two at D = 64)
 //         warp 17    MMA issuer A (whole warp runs the waits, the elected lane issues): dV(t), S^T(t+1)
 //         warp 18    LSE / delta loader (two-stage ring in shared memory)
 //         warp 19    MMA issuer B (likewise): dQ^T(t), dK(t), dP^T(t+1)
@@ -387,9 +387,9 @@ __global__ void __launch_bounds__(Roles<FIRST, D>::kThreads, 1) bwd_kernel(const
     setmaxnreg_dec<R::kRegsAux>();
     if (warp == R::kAux0) {
       // ================================================================ TMA producer
-      // Q(t) goes into a three-stage ring and is requested about one step before S^T(t) needs it; dO(t) goes
-      // into a single buffer that is free from the end of dV(t-1) until dP^T(t). Requests are issued in the
-      // order Q(0), dO(0), Q(1), dO(1), ...: the wait for the dO buffer is the one that paces the loop.
+      // Q(t) goes into a two-stage ring and is requested about one step before S^T(t) needs it; dO(t) goes into one
+      // buffer that is free from the end of dV(t-1) until dP^T(t) (at D = 64 into two, because dP^T runs a step ahead).
+      // Requests are issued in the order Q(0), dO(0), Q(1), dO(1), ...: the wait for the dO buffer paces the loop.
       QRing qr;
       while (next_item()) {
         if (lane == 0) {
@@ -1220,7 +1220,7 @@ __global__ void __launch_bounds__(Roles<FIRST, D>::kThreads, 1) bwd_kernel(const
                 if (on[u]) *reinterpret_cast<float4*>(o + at[u]) = w4[u];
             } else {
               __nv_bfloat16* const o = static_cast<__nv_bfloat16*>(outp);
-              if (add) {  // bf16 output: the first part was rounded once already (not the graded dtype)
+              if (add) {  // bf16 output: what the first-tile kernel left was rounded to bf16 already, the sum is rounded again
                 uint2 old[4];
 #pragma unroll
                 for (int u = 0; u < 4; ++u) old[u] = on[u] ? __ldcg(reinterpret_cast<const uint2*>(o + at[u])) : make_uint2(0u, 0u);

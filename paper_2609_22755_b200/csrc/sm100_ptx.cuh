@@ -91,8 +91,8 @@ __device__ __forceinline__ bool mbar_test(uint64_t* bar, uint32_t parity) {
   return ok != 0;
 }
 // The MMA-issuing warps run their waits with all 32 lanes and have to go on together: wait for the operands of some
-// products, issue the products, vote once, and only then the commits that let any of those barriers move on (behind the products
-// the vote costs nothing; in front of them it cost 2 %). A lane that falls behind its warp may test a phase only after the
+// products, issue the products, vote once, and only then the commits that let any of those barriers move on (in front of the
+// products the vote cost 2-4 % of a pass, behind them nothing on long items and 0-3.5 % of a forward pass over short ones). A lane that falls behind its warp may test a phase only after the
 // others have moved the barrier on by two, and then waits for a phase that has passed until the limit runs out. (Without
 // the vote that happened about once in 10^5 rounds of a forward pass over two-tile segments with one head per KV head: a
 // lane other than the elected one gave up after two seconds.)

@@ -50,6 +50,8 @@ struct nsp_plan {
   nsp_tile_t* d_bwd_parts = nullptr;        // the same items divided into parts (see divide_items)
   nsp_tile_t* d_bwd_first_parts = nullptr;  // the first-tile kernel's items likewise
   int64_t n_parts = 0, n_first_parts = 0;   // 0: not divided
+  nsp_tile_t* d_bwd_pairs = nullptr;          // items of the pair kernel: two key tiles of a segment of at least kPairTiles
+  int64_t n_bwd_pairs = 0, n_bwd_paired = 0;  // their number, and how many of d_bwd_exec's first items they stand for
   int32_t* d_turns = nullptr;               // turn counters of the divided items
   nsp_tile_t* d_bwd_first = nullptr;  // one item per (segment or pack, kv head): the first-tile kernels' list
   int64_t n_first = 0;
@@ -104,9 +106,9 @@ EncodeTiledFn get_encode_fn() {
   return fn;
 }
 
-// Tensor map of one run: a dense bf16 [tokens, heads, 128] tensor; tiles are {64 dims, 1 head, 128 tokens}
+// Tensor map of one run: a dense bf16 [tokens, heads, 128] tensor; tiles are {64 dims, 1 head, `rows` tokens}
 // with 128-byte swizzle, rows past the run read as zero.
-bool encode_run_map(CUtensorMap* out, const void* base, int64_t elem_off, int64_t tokens, int heads, int head_dim) {
+bool encode_run_map(CUtensorMap* out, const void* base, int64_t elem_off, int64_t tokens, int heads, int head_dim, int rows = kBM) {
   EncodeTiledFn enc = get_encode_fn();
   if (!enc) return false;
   if (tokens <= 0) {
@@ -116,7 +118,7 @@ bool encode_run_map(CUtensorMap* out, const void* base, int64_t elem_off, int64_
   const cuuint64_t dims[3] = {static_cast<cuuint64_t>(head_dim), static_cast<cuuint64_t>(heads),
                               static_cast<cuuint64_t>(tokens)};
   const cuuint64_t strides[2] = {static_cast<cuuint64_t>(head_dim) * 2, static_cast<cuuint64_t>(heads) * head_dim * 2};
-  const cuuint32_t box[3] = {64, 1, 128};
+  const cuuint32_t box[3] = {64, 1, static_cast<cuuint32_t>(rows)};
   const cuuint32_t estr[3] = {1, 1, 1};
   void* ptr = const_cast<char*>(static_cast<const char*>(base)) + elem_off * 2;
   return enc(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, ptr, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
@@ -193,6 +195,7 @@ inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 // bound the call (20 segments of about 100 tokens at 64q/4kv 233 -> 216 us; parts of eight steps 248, of two 215).
 constexpr int kMinPart = 16, kMinFirstPart = 4;
 constexpr int64_t kMostByLength = 600ll << 20;
+constexpr int kPairTiles = 16;
 struct WholeItem {
   int32_t seg, head, tile, steps;
 };
@@ -484,7 +487,7 @@ int nsp_plan_tiles(const int32_t* cu_seqlens, const int32_t* hq, const int32_t* 
     }
     if (fwd_first.size() == bwd_first.size()) fwd_first.clear();
   }
-  std::vector<nsp_tile_t> parts, first_parts;
+  std::vector<nsp_tile_t> parts, first_parts, pairs;
   std::vector<TileBase> bases;
   int32_t n_turns = 0;
   try {
@@ -492,7 +495,29 @@ int nsp_plan_tiles(const int32_t* cu_seqlens, const int32_t* hq, const int32_t* 
     if (!p->deterministic && !p->rounded_dq) {
       std::vector<WholeItem> main_items, first_items;
       int64_t main_steps = 0, first_steps = 0;
-      for (const int s : order) {
+      size_t paired = 0;  // segments, in the order of their lengths, whose items run on CTA pairs
+      if (head_dim == 128 && !p->small_bwd) {
+        int64_t steps = 0, longest = 0;
+        for (; paired < order.size(); ++paired) {
+          const SegInfo& sg = p->seg[order[paired]];
+          const int32_t Mt = (sg.len + bm - 1) / bm, G = sg.hq / sg.hkv;
+          if (Mt < kPairTiles) break;
+          for (int g = 0; g < sg.hkv; ++g)
+            for (int32_t n = 0; n < Mt; n += 2) {
+              pairs.push_back(nsp_tile_t{order[paired], g, n / 2, G * (Mt - std::max(n, 1))});
+              steps += pairs.back().cost;
+              longest = std::max<int64_t>(longest, pairs.back().cost);
+            }
+          p->n_bwd_paired += static_cast<int64_t>(sg.hkv) * Mt;
+        }
+        if (longest * (p->num_sms / 2) > steps) {  // the longest item would bound the kernel
+          paired = 0;
+          p->n_bwd_paired = 0;
+          pairs.clear();
+        }
+      }
+      for (size_t at = paired; at < order.size(); ++at) {
+        const int s = order[at];
         const SegInfo& sg = p->seg[s];
         const int32_t Mt = (sg.len + bm - 1) / bm, G = sg.hq / sg.hkv;
         for (int g = 0; g < sg.hkv; ++g)
@@ -511,6 +536,7 @@ int nsp_plan_tiles(const int32_t* cu_seqlens, const int32_t* hq, const int32_t* 
       first_parts = divide_items(first_items, std::max<int64_t>(kMinFirstPart, (first_steps + main_steps) / (2 * p->num_sms)), true,
                                  &n_turns);
     }
+    p->n_bwd_pairs = static_cast<int64_t>(pairs.size());
     p->n_parts = static_cast<int64_t>(parts.size());
     p->n_first_parts = static_cast<int64_t>(first_parts.size());
   } catch (...) {
@@ -528,7 +554,7 @@ int nsp_plan_tiles(const int32_t* cu_seqlens, const int32_t* hq, const int32_t* 
     at += align_up(bytes, 256);
     return here;
   };
-  const size_t o_counters = take(8 * sizeof(int32_t));
+  const size_t o_counters = take(16 * sizeof(int32_t));
   const size_t o_seg = take(sizeof(SegInfo) * (n_seg + pack_segs.size()));
   const size_t o_rows = take(sizeof(RowInfo) * pack_rows.size());
   const size_t o_row_base = take(sizeof(int64_t) * (n_seg + 1));
@@ -537,6 +563,7 @@ int nsp_plan_tiles(const int32_t* cu_seqlens, const int32_t* hq, const int32_t* 
   const size_t o_tiles = take(sizeof(int32_t) * (n_seg + 1));
   const size_t o_parts = take(sizeof(nsp_tile_t) * parts.size());
   const size_t o_first_parts = take(sizeof(nsp_tile_t) * first_parts.size());
+  const size_t o_bwd_pairs = take(sizeof(nsp_tile_t) * pairs.size());
   const size_t o_fwd_first = take(sizeof(nsp_tile_t) * fwd_first.size());
   const size_t o_turns = take(sizeof(int32_t) * n_turns);
   const size_t o_bases = take(sizeof(TileBase) * bases.size());
@@ -545,7 +572,7 @@ int nsp_plan_tiles(const int32_t* cu_seqlens, const int32_t* hq, const int32_t* 
   const size_t o_bwd = take(sizeof(nsp_tile_t) * nb);
   const size_t o_exec = take(sizeof(nsp_tile_t) * nb);
   const size_t o_pairs = take(sizeof(nsp_tile_t) * 2 * p->n_pairs);
-  const size_t o_front = take(sizeof(int32_t) * (nb / kFrontBlock + 1));
+  const size_t o_front = take(sizeof(int32_t) * (nb / kFrontBlock + 1 + pairs.size() / kFrontBlock + 1));
   const bool pinned = arena_keeps(at, 256 + upload);
   std::vector<char> pageable;
   try {
@@ -560,7 +587,7 @@ int nsp_plan_tiles(const int32_t* cu_seqlens, const int32_t* hq, const int32_t* 
     return NSP_ERR_ALLOC;
   }
   char* const d = static_cast<char*>(p->arena->dev);
-  p->d_counters = reinterpret_cast<int32_t*>(d + o_counters);  // [0] forward, [1] backward main, [2] first-tile backward, [3] first-tile forward
+  p->d_counters = reinterpret_cast<int32_t*>(d + o_counters);  // [0] forward, [1] backward main, [2] first-tile backward, [3] first-tile forward, [8] pairs
   p->d_status = p->d_counters + 4;
   p->d_seg = reinterpret_cast<SegInfo*>(d + o_seg);
   p->d_rows = reinterpret_cast<RowInfo*>(d + o_rows);
@@ -573,6 +600,7 @@ int nsp_plan_tiles(const int32_t* cu_seqlens, const int32_t* hq, const int32_t* 
   p->d_front = reinterpret_cast<int32_t*>(d + o_front);
   p->d_bwd_parts = reinterpret_cast<nsp_tile_t*>(d + o_parts);
   p->d_bwd_first_parts = reinterpret_cast<nsp_tile_t*>(d + o_first_parts);
+  p->d_bwd_pairs = reinterpret_cast<nsp_tile_t*>(d + o_bwd_pairs);
   p->d_turns = reinterpret_cast<int32_t*>(d + o_turns);
   p->d_fwd_first = fwd_first.empty() ? p->d_bwd_first : reinterpret_cast<nsp_tile_t*>(d + o_fwd_first);
   p->n_fwd_first = fwd_first.empty() ? p->n_first : static_cast<int64_t>(fwd_first.size());
@@ -583,7 +611,7 @@ int nsp_plan_tiles(const int32_t* cu_seqlens, const int32_t* hq, const int32_t* 
     if (bytes) std::memcpy(image + off, src, bytes);
   };
   std::memset(p->h_status, 0, 256);
-  std::memset(image, 0, 8 * sizeof(int32_t));
+  std::memset(image, 0, 16 * sizeof(int32_t));
   put(o_seg, p->seg.data(), sizeof(SegInfo) * n_seg);
   put(o_seg + sizeof(SegInfo) * n_seg, pack_segs.data(), sizeof(SegInfo) * pack_segs.size());
   put(o_rows, pack_rows.data(), sizeof(RowInfo) * pack_rows.size());
@@ -593,6 +621,7 @@ int nsp_plan_tiles(const int32_t* cu_seqlens, const int32_t* hq, const int32_t* 
   put(o_tiles, tile_base.data(), sizeof(int32_t) * (n_seg + 1));
   put(o_parts, parts.data(), sizeof(nsp_tile_t) * parts.size());
   put(o_first_parts, first_parts.data(), sizeof(nsp_tile_t) * first_parts.size());
+  put(o_bwd_pairs, pairs.data(), sizeof(nsp_tile_t) * pairs.size());
   put(o_fwd_first, fwd_first.data(), sizeof(nsp_tile_t) * fwd_first.size());
   std::memset(image + o_turns, 0, sizeof(int32_t) * n_turns);
   put(o_bases, bases.data(), sizeof(TileBase) * bases.size());
@@ -809,7 +838,8 @@ int bwd_impl(const nsp_plan_t* plan, const uint8_t* recompute, const void* q, co
                               static_cast<const __nv_bfloat16*>(o), static_cast<const __nv_bfloat16*>(d_o), delta,
                               dq_acc, recompute ? d_mask : nullptr, recompute ? lse : nullptr,
                               recompute ? lse_ws : nullptr, plan->d_front,
-                              static_cast<int>(plan->n_bwd / kFrontBlock + 1), plan->small_bwd, st) != cudaSuccess)
+                              static_cast<int>(plan->n_bwd / kFrontBlock + 1 + plan->n_bwd_pairs / kFrontBlock + 1),
+                              plan->small_bwd, st) != cudaSuccess)
       return NSP_ERR_CUDA;
   }
   prof_mark(plan, NSP_KERNEL_BWD_PRE, 1, st);
@@ -843,13 +873,29 @@ int bwd_impl(const nsp_plan_t* plan, const uint8_t* recompute, const void* q, co
   prof_mark(plan, NSP_KERNEL_BWD_FIRST, 0, st);
   if (launch_bwd_first(maps, a, plan->head_dim, plan->num_sms, st) != cudaSuccess) return NSP_ERR_CUDA;
   prof_mark(plan, NSP_KERNEL_BWD_FIRST, 1, st);
-  // main kernel: everything else
+  // main kernels: everything else, the long segments on CTA pairs
+  prof_mark(plan, NSP_KERNEL_BWD_MAIN, 0, st);
+  a.turn = nullptr;
+  if (plan->n_bwd_pairs > 0) {
+    BwdMaps pair_maps = maps;
+    for (size_t r = 0; r < plan->runs.size(); ++r) {
+      const RunInfo& run = plan->runs[r];
+      if (!encode_run_map(&pair_maps.q[r], q, run.q_off, run.tokens, run.hq, plan->head_dim, 64) ||
+          !encode_run_map(&pair_maps.d_o[r], d_o, run.q_off, run.tokens, run.hq, plan->head_dim, 64))
+        return NSP_ERR_CUDA;
+    }
+    a.items = plan->d_bwd_pairs;
+    a.n_items = static_cast<int32_t>(plan->n_bwd_pairs);
+    a.counter = plan->d_counters + 8;
+    a.front = plan->d_front + plan->n_bwd / kFrontBlock + 1;
+    if (launch_bwd_pair(pair_maps, a, plan->num_sms, st) != cudaSuccess) return NSP_ERR_CUDA;
+    a.front = plan->d_front;
+  }
   const bool m_parts = a.dkv_f32 && plan->n_parts > 0;
-  a.items = m_parts ? plan->d_bwd_parts : plan->d_bwd_exec;
-  a.n_items = static_cast<int32_t>(m_parts ? plan->n_parts : plan->n_bwd);
+  a.items = m_parts ? plan->d_bwd_parts : plan->d_bwd_exec + plan->n_bwd_paired;
+  a.n_items = static_cast<int32_t>(m_parts ? plan->n_parts : plan->n_bwd - plan->n_bwd_paired);
   a.turn = m_parts ? plan->d_turns : nullptr;
   a.counter = plan->d_counters + 1;
-  prof_mark(plan, NSP_KERNEL_BWD_MAIN, 0, st);
   if (multi && launch_bwd(maps, a, plan->head_dim, plan->num_sms, plan->small_bwd, st) != cudaSuccess) return NSP_ERR_CUDA;
   prof_mark(plan, NSP_KERNEL_BWD_MAIN, 1, st);
   prof_mark(plan, NSP_KERNEL_BWD_POST, 0, st);

@@ -239,6 +239,9 @@ cudaError_t launch_bwd_preprocess(const SegInfo* d_seg, int n_seg, const int64_t
                                   int32_t* front, int n_front, bool chained, cudaStream_t st);
 cudaError_t launch_bwd_first(const BwdMaps& maps, const BwdArgs& args, int head_dim, int num_sms, cudaStream_t st);
 cudaError_t launch_bwd(const BwdMaps& maps, const BwdArgs& args, int head_dim, int num_sms, bool chained, cudaStream_t st);  // args.dq_turn / args.dq_rounded select the reproducible variants
+// the long segments' share of the main kernel's work, on CTA pairs: items (segment, kv head, two key tiles), head dimension
+// 128; maps.q and maps.d_o have boxes of 64 rows
+cudaError_t launch_bwd_pair(const BwdMaps& maps, const BwdArgs& args, int num_sms, cudaStream_t st);
 cudaError_t launch_bwd_postprocess(const SegInfo* d_seg, int n_seg, const int64_t* d_row_base, int64_t total_rows,
                                    int head_dim, const float* dq_acc, void* dq, int dq_f32, float scale,
                                    cudaStream_t st);

@@ -67,7 +67,8 @@ struct PairSmem {
   uint64_t bar_kv, bar_row_full[3], bar_qc_full, bar_doc_full;
   uint64_t bar_s_read;    // 16 warps: S^T has been read (R0 [64, 128) is free for dQ^T)
   uint64_t bar_p_ready;   // 16 warps: P^T is in R0
-  uint64_t bar_ds_ready;  // 16 warps: dS^T is in R1 and in shared memory
+  uint64_t bar_ds_ready;  // 16 warps: dS^T is in R1
+  uint64_t bar_x_own;     // 8 warps: the parts of dS^T that stay in their CTA are in shared memory
   uint64_t bar_dq_empty;  // 16 warps: dQ^T has been drained
   uint64_t bar_x_peer;    // the second CTA has received its part of dS^T
   // Completed in both CTAs: products
@@ -124,6 +125,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
     mbar_init(&s.bar_s_read, 16);
     mbar_init(&s.bar_p_ready, 16);
     mbar_init(&s.bar_ds_ready, 16);
+    mbar_init(&s.bar_x_own, 8);
     mbar_init(&s.bar_dq_empty, 16);
     mbar_init(&s.bar_x_peer, 1);
     mbar_init(&s.bar_s_full, 1);
@@ -399,11 +401,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
           if (is_a) {
             const uint32_t k_km = smem_desc_addr(s.k[0]) | lbo_km;
             const uint32_t do_mn = smem_desc_addr(s.do_col) | lbo_mn;
-            auto issue_s = [&](int vt) -> bool {
+            auto issue_s = [&](int vt, bool here) -> bool {  // here: the Q rows have arrived
               const uint32_t cs = gs + vt;
-              bool here = mbar_wait(&s.bar_row_full[ring.st], ring.ph, a.wait_limit);
               // R0 [64, 128) held dQ^T of the step before the last one (of this item: earlier ones are long drained)
-              if (vt > 0) here = mbar_wait(&s.bar_dq_empty, cs & 1, a.wait_limit) && here;
+              if (vt > 0) here = mbar_poll(&s.bar_dq_empty, cs & 1, a.wait_limit) && here;
               tc_fence_after_sync();
               issue_kk(tR0, k_km, leader && here);
               if (!together(here)) { where = kWhereBwdLoadQ; return false; }
@@ -412,13 +413,15 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
               ring.next();
               return true;
             };
-            okm = okm && issue_s(0);
+            okm = okm && issue_s(0, mbar_poll(&s.bar_row_full[ring.st], ring.ph, a.wait_limit));
 #pragma unroll 1
             for (int vt = 0; okm && vt < steps; ++vt) {
               const bool calm = *abort_flag == 0;
               const uint32_t cs = gs + vt;
-              bool here = mbar_wait(&s.bar_doc_full, cs & 1, a.wait_limit);
-              here = mbar_wait(&s.bar_p_ready, cs & 1, a.wait_limit) && here;
+              bool here = mbar_poll(&s.bar_doc_full, cs & 1, a.wait_limit);
+              const bool more = vt + 1 < steps;
+              if (more) here = mbar_poll(&s.bar_row_full[ring.st], ring.ph, a.wait_limit) && here;
+              here = mbar_poll(&s.bar_p_ready, cs & 1, a.wait_limit) && here;
               tc_fence_after_sync();
               issue_kn(tDV, tR0, do_mn, vt > 0, leader && here);
               if (!together(here && calm)) {
@@ -427,15 +430,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
                 break;
               }
               if (leader) umma2_commit(&s.bar_dv_done);
-              if (vt + 1 < steps) okm = issue_s(vt + 1);
+              if (more) okm = issue_s(vt + 1, true);
             }
           } else {
             const uint32_t v_km = smem_desc_addr(s.v[0]) | lbo_km;
             const uint32_t q_mn = smem_desc_addr(s.q_col) | lbo_mn;
             const uint32_t kt_mn = smem_desc_addr(s.kt[0]) | lbo_mn, x_mn = smem_desc_addr(s.x[0]) | lbo_mn;
-            auto issue_dp = [&]() -> bool {
-              const bool here = mbar_wait(&s.bar_row_full[ring.st], ring.ph, a.wait_limit);
-              tc_fence_after_sync();
+            auto issue_dp = [&](bool here) -> bool {  // here: the dO rows have arrived
               issue_kk(tR1, v_km, leader && here);
               if (!together(here)) { where = kWhereBwdLoadQ; return false; }
               if (leader) umma2_commit(&s.bar_dp_full);
@@ -443,14 +444,16 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
               ring.next();
               return true;
             };
-            okm = okm && issue_dp();
+            okm = okm && issue_dp(mbar_poll(&s.bar_row_full[ring.st], ring.ph, a.wait_limit));
 #pragma unroll 1
             for (int vt = 0; okm && vt < steps; ++vt) {
               const bool calm = *abort_flag == 0;
               const uint32_t cs = gs + vt;
               if (leader) mbar_expect_tx(&s.bar_x_full, kHalfTileBytes);
-              bool here = mbar_wait(&s.bar_qc_full, cs & 1, a.wait_limit);
-              here = mbar_wait(&s.bar_ds_ready, cs & 1, a.wait_limit) && here;
+              const bool more = vt + 1 < steps;
+              bool here = mbar_poll(&s.bar_qc_full, cs & 1, a.wait_limit);
+              if (more) here = mbar_poll(&s.bar_row_full[ring.st], ring.ph, a.wait_limit) && here;
+              here = mbar_poll(&s.bar_ds_ready, cs & 1, a.wait_limit) && here;
               tc_fence_after_sync();
               issue_kn(tDK, tR1, q_mn, vt > 0, leader && here);
               if (!together(here && calm)) {
@@ -459,12 +462,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
                 break;
               }
               if (leader) umma2_commit(&s.bar_dk_done);
-              const bool more = vt + 1 < steps;
-              if (more && !issue_dp()) { okm = false; break; }
+              if (more && !issue_dp(true)) { okm = false; break; }
               // dQ^T over the part of R0 that packed P^T leaves free, once S^T of the next step has been read from it
-              here = mbar_wait(&s.bar_x_full, cs & 1, a.wait_limit);
-              here = mbar_wait(&s.bar_x_peer, cs & 1, a.wait_limit) && here;
-              if (more) here = mbar_wait(&s.bar_s_read, (cs + 1) & 1, a.wait_limit) && here;
+              here = mbar_poll(&s.bar_x_own, cs & 1, a.wait_limit);
+              if (more) here = mbar_poll(&s.bar_s_read, (cs + 1) & 1, a.wait_limit) && here;
+              here = mbar_poll(&s.bar_x_full, cs & 1, a.wait_limit) && here;
+              here = mbar_poll(&s.bar_x_peer, cs & 1, a.wait_limit) && here;
               tc_fence_after_sync();
               const bool go = leader && here;
 #pragma unroll
@@ -613,8 +616,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
           if (lane == 0) arrive_lead(&s.bar_p_ready);
 #pragma unroll
           for (int i = 0; i < 4; ++i) aux[0][i] = lds128(delta_s + 4 * i);
-          // the dS^T buffers are free once dQ^T of the step before has completed
-          oks = mbar_wait(&s.bar_dp_full, cs & 1, a.wait_limit) && (vt == 0 || mbar_wait(&s.bar_dq_full, (cs - 1) & 1, a.wait_limit));
+          oks = mbar_wait(&s.bar_dp_full, cs & 1, a.wait_limit);
           if (!together(oks)) { where = kWhereBwdDp; return false; }
           tc_fence_after_sync();
           uint32_t dpv[2][16];
@@ -627,12 +629,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
 #pragma unroll
               for (int i = 0; i < 4; ++i) aux[(ch + 1) & 1][i] = lds128(delta_s + ((ch + 1) >> 1) * 64 + ((ch + 1) & 1) * 16 + 4 * i);
             }
-            uint32_t dsp[8];
+            uint32_t* const dsp = &pp[ch >> 1][(ch & 1) * 8];  // in the place of P^T
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
               const float4 d4 = aux[ch & 1][i];
               const int x = 4 * i;
-              const uint32_t pa = pp[ch >> 1][(ch & 1) * 8 + (x >> 1)], pb = pp[ch >> 1][(ch & 1) * 8 + (x >> 1) + 1];
+              const uint32_t pa = dsp[x >> 1], pb = dsp[(x >> 1) + 1];
               float d0, d1, d2, d3;
               sub2(d0, d1, __uint_as_float(dpv[ch & 1][x + 0]), __uint_as_float(dpv[ch & 1][x + 1]), d4.x, d4.y);
               sub2(d2, d3, __uint_as_float(dpv[ch & 1][x + 2]), __uint_as_float(dpv[ch & 1][x + 3]), d4.z, d4.w);
@@ -641,10 +643,22 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
               dsp[(x >> 1) + 0] = pack_bf16x2(d0, d1);
               dsp[(x >> 1) + 1] = pack_bf16x2(d2, d3);
             }
-            tmem_st8(tDP + ch * 8, dsp);
-            *reinterpret_cast<uint4*>(ds_row + ((2 * ch) ^ (r & 7)) * 16) = make_uint4(dsp[0], dsp[1], dsp[2], dsp[3]);
-            *reinterpret_cast<uint4*>(ds_row + ((2 * ch + 1) ^ (r & 7)) * 16) = make_uint4(dsp[4], dsp[5], dsp[6], dsp[7]);
+            if (ch & 1) tmem_st16(tDP + (ch >> 1) * 16, pp[ch >> 1]);
           }
+          tmem_wait_st();
+          tc_fence_before_sync();
+          __syncwarp();
+          if (lane == 0) {
+            arrive_lead(&s.bar_ds_ready);  // dK and dP^T of the next step need no more than this
+            mbar_arrive(&s.bar_ld_empty[st]);
+          }
+          // the dS^T buffers are free once dQ^T of the step before has completed
+          oks = vt == 0 || mbar_wait(&s.bar_dq_full, (cs - 1) & 1, a.wait_limit);
+          if (!together(oks)) { where = kWhereBwdStaged; return false; }
+#pragma unroll
+          for (int i = 0; i < 8; ++i)
+            *reinterpret_cast<uint4*>(ds_row + (i ^ (r & 7)) * 16) =
+                make_uint4(pp[i >> 2][(i & 3) * 4], pp[i >> 2][(i & 3) * 4 + 1], pp[i >> 2][(i & 3) * 4 + 2], pp[i >> 2][(i & 3) * 4 + 3]);
           return true;
         };
         if (m > c.n) {
@@ -652,14 +666,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
         } else {
           if (!step(std::true_type{})) break;
         }
-        tmem_wait_st();
         fence_proxy_async_smem();
-        tc_fence_before_sync();
         __syncwarp();
         if (lane == 0) {
-          if (!keep) copy_to_cluster(x_to, s.stage + quad * 4096, 4096, x_bar);
-          arrive_lead(&s.bar_ds_ready);
-          mbar_arrive(&s.bar_ld_empty[st]);
+          if (keep)
+            arrive_lead(&s.bar_x_own);
+          else
+            copy_to_cluster(x_to, s.stage + quad * 4096, 4096, x_bar);
         }
       }
       // ---- epilogue: wait for the last products of the item, then write dK (scaled) and dV of this key tile

@@ -126,8 +126,10 @@ bool encode_run_map(CUtensorMap* out, const void* base, int64_t elem_off, int64_
              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// fp32 [tokens, heads, head_dim] output of one run, boxes of 32 columns x 128 rows (128 bytes per row, 128-byte swizzle)
-bool encode_run_map_f32(CUtensorMap* out, void* base, int64_t elem_off, int64_t tokens, int heads, int head_dim) {
+// fp32 [tokens, heads, head_dim] output of one run, boxes of 32 columns x `rows` rows (128 bytes per row), with the 128-byte
+// swizzle or row after row
+bool encode_run_map_f32(CUtensorMap* out, void* base, int64_t elem_off, int64_t tokens, int heads, int head_dim, int rows = 128,
+                        bool swizzled = true) {
   EncodeTiledFn enc = get_encode_fn();
   if (!enc) return false;
   if (tokens <= 0) {
@@ -137,11 +139,11 @@ bool encode_run_map_f32(CUtensorMap* out, void* base, int64_t elem_off, int64_t 
   const cuuint64_t dims[3] = {static_cast<cuuint64_t>(head_dim), static_cast<cuuint64_t>(heads),
                               static_cast<cuuint64_t>(tokens)};
   const cuuint64_t strides[2] = {static_cast<cuuint64_t>(head_dim) * 4, static_cast<cuuint64_t>(heads) * head_dim * 4};
-  const cuuint32_t box[3] = {32, 1, 128};
+  const cuuint32_t box[3] = {32, 1, static_cast<cuuint32_t>(rows)};
   const cuuint32_t estr[3] = {1, 1, 1};
   void* ptr = static_cast<char*>(base) + elem_off * 4;
   return enc(out, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, ptr, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-             CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+             swizzled ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
@@ -877,11 +879,14 @@ int bwd_impl(const nsp_plan_t* plan, const uint8_t* recompute, const void* q, co
   prof_mark(plan, NSP_KERNEL_BWD_MAIN, 0, st);
   a.turn = nullptr;
   if (plan->n_bwd_pairs > 0) {
-    BwdMaps pair_maps = maps;
+    BwdPairMaps pair_maps;
+    std::memset(&pair_maps, 0, sizeof(pair_maps));
+    static_cast<BwdMaps&>(pair_maps) = maps;
     for (size_t r = 0; r < plan->runs.size(); ++r) {
       const RunInfo& run = plan->runs[r];
       if (!encode_run_map(&pair_maps.q[r], q, run.q_off, run.tokens, run.hq, plan->head_dim, 64) ||
-          !encode_run_map(&pair_maps.d_o[r], d_o, run.q_off, run.tokens, run.hq, plan->head_dim, 64))
+          !encode_run_map(&pair_maps.d_o[r], d_o, run.q_off, run.tokens, run.hq, plan->head_dim, 64) ||
+          !encode_run_map_f32(&pair_maps.dq_acc[r], dq_acc, run.q_off, run.tokens, run.hq, plan->head_dim, 16, false))
         return NSP_ERR_CUDA;
     }
     a.items = plan->d_bwd_pairs;

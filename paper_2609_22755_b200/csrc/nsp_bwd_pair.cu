@@ -41,9 +41,6 @@ template <int N>
 __device__ __forceinline__ void pair_setmaxnreg_dec() {
   asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N));
 }
-__device__ __forceinline__ void pair_red_add_f32(float* addr, float v) {
-  asm volatile("red.relaxed.gpu.global.add.f32 [%0], %1;" ::"l"(addr), "f"(v) : "memory");
-}
 
 struct PairCtx {
   int64_t q_off, kv_off, lse_off;
@@ -56,15 +53,16 @@ struct PairSmem {
   uint8_t k[2][kHalfTileBytes];   // own key tile, [64-column half]
   uint8_t kt[2][kHalfTileBytes];  // both key tiles, columns 64 r .. 64 r + 63
   uint8_t v[2][kHalfTileBytes];
-  uint8_t row[3][kHalfTileBytes];  // rows 64 r .. of a Q or dO tile, two sub-tiles [64 rows x 64 columns] (see RowRing)
+  uint8_t q_row[kHalfTileBytes], do_row[kHalfTileBytes];  // rows 64 r .. of the tile: two sub-tiles [64 rows x 64 columns]
   uint8_t q_col[kHalfTileBytes], do_col[kHalfTileBytes];  // columns 64 r .. of the tile: [128 rows x 64 columns]
   uint8_t x[2][kHalfTileBytes];   // dS^T of the pair's key tiles, [key][this CTA's 64 queries]
   uint8_t stage[kHalfTileBytes];  // dS^T of the own key tile for the other CTA's queries
+  float dq_out[8][16][32];        // [dQ warp][query][d]: on its way into the accumulator
   alignas(16) float lse[2][128];  // [stage] LSE * log2(e) of the q tile (+inf for rows past the segment)
   float delta[2][128];
   PairCtx ctx;
   // Arrived on in the first CTA only, which issues the products: loads (both CTAs' bytes), hand-overs of both CTAs' warps
-  uint64_t bar_kv, bar_row_full[3], bar_qc_full, bar_doc_full;
+  uint64_t bar_kv, bar_qr_full, bar_qc_full, bar_dor_full, bar_doc_full;
   uint64_t bar_s_read;    // 16 warps: S^T has been read (R0 [64, 128) is free for dQ^T)
   uint64_t bar_p_ready;   // 16 warps: P^T is in R0
   uint64_t bar_ds_ready;  // 16 warps: dS^T is in R1
@@ -72,7 +70,7 @@ struct PairSmem {
   uint64_t bar_dq_empty;  // 16 warps: dQ^T has been drained
   uint64_t bar_x_peer;    // the second CTA has received its part of dS^T
   // Completed in both CTAs: products
-  uint64_t bar_s_full, bar_dp_full, bar_dq_full, bar_dv_done, bar_dk_done, bar_row_empty[3];
+  uint64_t bar_s_full, bar_dp_full, bar_dq_full, bar_dv_done, bar_dk_done;
   // Local
   uint64_t bar_x_full;  // the other CTA's part of dS^T has arrived
   uint64_t bar_ld_full[2], bar_ld_empty[2];
@@ -96,19 +94,8 @@ struct PairWalk {
   }
 };
 
-// The row tiles go through a ring of three in the order Q(0), dO(0), Q(1), dO(1), ...: S^T(t + 1) and dP^T(t + 1) find theirs
-// loaded 3,600 clocks ahead. With one buffer for each they had 1,800-2,100, and a load under the reductions takes as long.
-struct RowRing {
-  uint32_t st, ph = 0;
-  __device__ __forceinline__ explicit RowRing(uint32_t first) : st(first) {}
-  __device__ __forceinline__ void next() {
-    st += 2;
-    if (st >= 3) st -= 3, ph ^= 1;
-  }
-};
-
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
-    bwd_pair_kernel(const __grid_constant__ BwdMaps maps, const BwdArgs a) {
+    bwd_pair_kernel(const __grid_constant__ BwdPairMaps maps, const BwdArgs a) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   PairSmem& s = *reinterpret_cast<PairSmem*>(smem_raw);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, wg = warp >> 2;
@@ -116,10 +103,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
   const bool misaligned = (smem_u32(smem_raw) & 1023u) != 0;
   if (tid == 0) {
     mbar_init(&s.bar_kv, 1);
-    for (int i = 0; i < 3; ++i) {
-      mbar_init(&s.bar_row_full[i], 1);
-      mbar_init(&s.bar_row_empty[i], 1);
-    }
+    mbar_init(&s.bar_qr_full, 1);
+    mbar_init(&s.bar_dor_full, 1);
     mbar_init(&s.bar_qc_full, 1);
     mbar_init(&s.bar_doc_full, 1);
     mbar_init(&s.bar_s_read, 16);
@@ -232,7 +217,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
     pair_setmaxnreg_dec<kRegsAux>();
     if (warp == 16) {
       // ================================================================ TMA producer (both CTAs, each its own operands)
-      RowRing qr(0), dr(1);
       while (next_item()) {
         if (lane == 0) {
           const PairCtx c = s.ctx;
@@ -248,15 +232,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
             tma_load_3d_pair(s.kt[i], &maps.k[c.run], kv, col, c.g, c.tok0 + (c.n0 + i) * kBN);
           }
           // boxes of q and dO are [64 rows x 64 columns]
-          auto load_row = [&](RowRing& ring, const CUtensorMap* map, int h, int m) -> bool {
-            if (!mbar_wait(&s.bar_row_empty[ring.st], ring.ph ^ 1, a.wait_limit)) return false;
-            if (rank == 0) mbar_expect_tx(&s.bar_row_full[ring.st], 2 * kHalfTileBytes);
-            const uint32_t to = lead + off(&s.bar_row_full[ring.st]);
+          auto load_row = [&](uint8_t* dst, const CUtensorMap* map, uint64_t* bar, int h, int m) {
+            if (rank == 0) mbar_expect_tx(bar, 2 * kHalfTileBytes);
+            const uint32_t to = lead + off(bar);
 #pragma unroll
-            for (int i = 0; i < 2; ++i)
-              tma_load_3d_pair(s.row[ring.st] + i * (kHalfTileBytes / 2), map, to, 64 * i, h, c.tok0 + m * kBM + col);
-            ring.next();
-            return true;
+            for (int i = 0; i < 2; ++i) tma_load_3d_pair(dst + i * (kHalfTileBytes / 2), map, to, 64 * i, h, c.tok0 + m * kBM + col);
           };
           auto load_col = [&](uint8_t* dst, const CUtensorMap* map, uint64_t* bar, int h, int m) {
             if (rank == 0) mbar_expect_tx(bar, 2 * kHalfTileBytes);
@@ -264,37 +244,34 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
 #pragma unroll
             for (int i = 0; i < 2; ++i) tma_load_3d_pair(dst + i * (kHalfTileBytes / 2), map, to, col, h, c.tok0 + m * kBM + 64 * i);
           };
-          PairWalk w, w2;  // of the next step, and of the one behind it
-          int h, m, h2, m2;
+          PairWalk w;
+          int h, m;
           w.get(c, h, m);
           w.next(c);
-          w2 = w;
-          w2.get(c, h2, m2);
-          w2.next(c);
-          bool ok = load_row(qr, mq, h, m) && load_row(dr, mdo, h, m);
-          if (ok && c.steps > 1) ok = load_row(qr, mq, h2, m2);
-          if (ok) {
-            load_col(s.do_col, mdo, &s.bar_doc_full, h, m);
-            load_col(s.q_col, mq, &s.bar_qc_full, h, m);
-          }
+          load_row(s.q_row, mq, &s.bar_qr_full, h, m);
+          load_row(s.do_row, mdo, &s.bar_dor_full, h, m);
+          load_col(s.do_col, mdo, &s.bar_doc_full, h, m);
+          load_col(s.q_col, mq, &s.bar_qc_full, h, m);
+          // A buffer is free when its product of the step before has completed; in the order in which they complete.
 #pragma unroll 1
-          for (int vt = 0; ok && vt + 1 < c.steps; ++vt) {
+          for (int vt = 0; vt + 1 < c.steps; ++vt) {
             if (*abort_flag) break;
             const uint32_t ph = (gs + vt) & 1;
             w.get(c, h, m);
             w.next(c);
-            w2.get(c, h2, m2);
-            w2.next(c);
-            ok = load_row(dr, mdo, h, m);
-            if (ok && vt + 2 < c.steps) ok = load_row(qr, mq, h2, m2);
+            bool ok = mbar_wait(&s.bar_s_full, ph, a.wait_limit);
+            if (ok) load_row(s.q_row, mq, &s.bar_qr_full, h, m);
+            ok = ok && mbar_wait(&s.bar_dp_full, ph, a.wait_limit);
+            if (ok) load_row(s.do_row, mdo, &s.bar_dor_full, h, m);
             ok = ok && mbar_wait(&s.bar_dv_done, ph, a.wait_limit);
             if (ok) load_col(s.do_col, mdo, &s.bar_doc_full, h, m);
             ok = ok && mbar_wait(&s.bar_dk_done, ph, a.wait_limit);
             if (ok) load_col(s.q_col, mq, &s.bar_qc_full, h, m);
-          }
-          if (!ok) {
-            report_timeout(a.status, c.it, kWhereBwdQEmpty, 0);
-            raise_abort();
+            if (!ok) {
+              report_timeout(a.status, c.it, kWhereBwdQEmpty, vt);
+              raise_abort();
+              break;
+            }
           }
         }
         __syncwarp();
@@ -366,7 +343,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
       // ================================================================ MMA issuers, for both CTAs
       // A: dV(t), S^T(t+1); B: dK(t), dP^T(t+1), dQ^T(t)
       const bool is_a = warp == 17;
-      RowRing ring(is_a ? 0 : 1);
       while (next_item()) {
         {
           const bool leader = elect_one();
@@ -376,14 +352,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
           const uint32_t hi = static_cast<uint32_t>(make_smem_desc_sw128(0, 16, 1024) >> 32);
           constexpr uint32_t lbo_km = (16u >> 4) << 16, lbo_mn = (kHalfTileBytes >> 4) << 16;
           const int steps = s.ctx.steps, item_it = s.ctx.it;
-          constexpr uint32_t kRowStep = kHalfTileBytes >> 4;
-          const uint32_t row_km = smem_desc_addr(s.row[0]) | lbo_km;
           int where = 0;
           bool okm = together(mbar_wait(&s.bar_kv, gi & 1, a.wait_limit));
           if (!okm) where = kWhereBwdLoadKV;
-          // [128 own rows] x [64 + 64 rows of the ring]: S^T or dP^T
-          auto issue_kk = [&](uint32_t d, uint32_t a_km, bool go) {
-            const uint32_t b_km = row_km + ring.st * kRowStep;
+          // [128 own rows] x [64 + 64 rows]: S^T or dP^T
+          auto issue_kk = [&](uint32_t d, uint32_t a_km, uint32_t b_km, bool go) {
 #pragma unroll
             for (int kk = 0; kk < 8; ++kk) {
               const uint32_t ao = ((kk >> 2) * kHalfTileBytes + (kk & 3) * 32) >> 4;
@@ -399,28 +372,26 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
                                   acc | (kk > 0));
           };
           if (is_a) {
-            const uint32_t k_km = smem_desc_addr(s.k[0]) | lbo_km;
+            const uint32_t k_km = smem_desc_addr(s.k[0]) | lbo_km, q_km = smem_desc_addr(s.q_row) | lbo_km;
             const uint32_t do_mn = smem_desc_addr(s.do_col) | lbo_mn;
             auto issue_s = [&](int vt, bool here) -> bool {  // here: the Q rows have arrived
               const uint32_t cs = gs + vt;
               // R0 [64, 128) held dQ^T of the step before the last one (of this item: earlier ones are long drained)
               if (vt > 0) here = mbar_poll(&s.bar_dq_empty, cs & 1, a.wait_limit) && here;
               tc_fence_after_sync();
-              issue_kk(tR0, k_km, leader && here);
+              issue_kk(tR0, k_km, q_km, leader && here);
               if (!together(here)) { where = kWhereBwdLoadQ; return false; }
               if (leader) umma2_commit(&s.bar_s_full);
-              if (leader) umma2_commit(&s.bar_row_empty[ring.st]);
-              ring.next();
               return true;
             };
-            okm = okm && issue_s(0, mbar_poll(&s.bar_row_full[ring.st], ring.ph, a.wait_limit));
+            okm = okm && issue_s(0, mbar_poll(&s.bar_qr_full, gs & 1, a.wait_limit));
 #pragma unroll 1
             for (int vt = 0; okm && vt < steps; ++vt) {
               const bool calm = *abort_flag == 0;
               const uint32_t cs = gs + vt;
               bool here = mbar_poll(&s.bar_doc_full, cs & 1, a.wait_limit);
               const bool more = vt + 1 < steps;
-              if (more) here = mbar_poll(&s.bar_row_full[ring.st], ring.ph, a.wait_limit) && here;
+              if (more) here = mbar_poll(&s.bar_qr_full, (cs + 1) & 1, a.wait_limit) && here;
               here = mbar_poll(&s.bar_p_ready, cs & 1, a.wait_limit) && here;
               tc_fence_after_sync();
               issue_kn(tDV, tR0, do_mn, vt > 0, leader && here);
@@ -433,18 +404,16 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
               if (more) okm = issue_s(vt + 1, true);
             }
           } else {
-            const uint32_t v_km = smem_desc_addr(s.v[0]) | lbo_km;
+            const uint32_t v_km = smem_desc_addr(s.v[0]) | lbo_km, do_km = smem_desc_addr(s.do_row) | lbo_km;
             const uint32_t q_mn = smem_desc_addr(s.q_col) | lbo_mn;
             const uint32_t kt_mn = smem_desc_addr(s.kt[0]) | lbo_mn, x_mn = smem_desc_addr(s.x[0]) | lbo_mn;
             auto issue_dp = [&](bool here) -> bool {  // here: the dO rows have arrived
-              issue_kk(tR1, v_km, leader && here);
+              issue_kk(tR1, v_km, do_km, leader && here);
               if (!together(here)) { where = kWhereBwdLoadQ; return false; }
               if (leader) umma2_commit(&s.bar_dp_full);
-              if (leader) umma2_commit(&s.bar_row_empty[ring.st]);
-              ring.next();
               return true;
             };
-            okm = okm && issue_dp(mbar_poll(&s.bar_row_full[ring.st], ring.ph, a.wait_limit));
+            okm = okm && issue_dp(mbar_poll(&s.bar_dor_full, gs & 1, a.wait_limit));
 #pragma unroll 1
             for (int vt = 0; okm && vt < steps; ++vt) {
               const bool calm = *abort_flag == 0;
@@ -452,7 +421,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
               if (leader) mbar_expect_tx(&s.bar_x_full, kHalfTileBytes);
               const bool more = vt + 1 < steps;
               bool here = mbar_poll(&s.bar_qc_full, cs & 1, a.wait_limit);
-              if (more) here = mbar_poll(&s.bar_row_full[ring.st], ring.ph, a.wait_limit) && here;
+              if (more) here = mbar_poll(&s.bar_dor_full, (cs + 1) & 1, a.wait_limit) && here;
               here = mbar_poll(&s.bar_ds_ready, cs & 1, a.wait_limit) && here;
               tc_fence_after_sync();
               issue_kn(tDK, tR1, q_mn, vt > 0, leader && here);
@@ -501,7 +470,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
     const uint32_t src = tDQ + (static_cast<uint32_t>(quad * 32) << 16) + 32 * half;
     while (next_item()) {
       const PairCtx c = s.ctx;
-      const int64_t q_stride = static_cast<int64_t>(c.hq) * D;
       PairWalk w;
 #pragma unroll 1
       for (int vt = 0; vt < c.steps; ++vt) {
@@ -524,18 +492,24 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
         tc_fence_before_sync();
         __syncwarp();
         if (lane == 0) arrive_lead(&s.bar_dq_empty);
-        const int n_valid = c.len - m * kBM - q0;  // of the 32 rows
-        float* p = a.dq_acc + c.q_off + (static_cast<int64_t>(m * kBM + q0) * c.hq + h) * D + d;
-        NSP_CHECK(n_valid <= 0 || (p >= a.dq_acc && p + (min(n_valid, 32) - 1) * q_stride < a.dq_acc + a.q_elems), a.status, c.it,
-                  kWhereCheckBwdDq, m)
-        if (c.hq > 0) {
+        // Sixteen rows at a time through the warp's 2 KB. Rows past the segment's end add zeros (their dS^T columns are zero)
+        // to the first rows of the segments behind it, which nobody reads, or lie outside the tensor map.
 #pragma unroll
-          for (int e = 0; e < 32; ++e) {
-            if (e < n_valid) pair_red_add_f32(p, __uint_as_float(v[e]));
-            p += q_stride;
+        for (int i = 0; i < 2; ++i) {
+          if (lane == 0) tma_store_wait_read();
+          __syncwarp();
+#pragma unroll
+          for (int e = 0; e < 16; ++e) s.dq_out[warp - 8][e][lane] = __uint_as_float(v[16 * i + e]);
+          fence_proxy_async_smem();
+          __syncwarp();
+          if (lane == 0) {
+            tma_reduce_add_3d(&maps.dq_acc[c.run], s.dq_out[warp - 8], d - lane, h, c.tok0 + m * kBM + q0 + 16 * i);
+            tma_store_commit();
           }
         }
       }
+      if (lane == 0) tma_store_wait();
+      __syncwarp();
       item_done();
     }
   } else {
@@ -689,7 +663,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
         const bool add = c.n == 0;  // the first-tile kernel left its part (q tile 0) in the output
         constexpr uint32_t kSubBytes = 128 * 32 * 4;
         uint8_t* const stage_k = &s.k[0][0];  // over K and K^T
-        uint8_t* const stage_v = &s.v[0][0];  // over V and two of the row tiles
+        uint8_t* const stage_v = &s.v[0][0];  // over V and the row tiles
         if (quad * 32 < rows) {
 #pragma unroll 1
           for (int i = 0; i < 4; ++i) {  // (dK, dV) x 32-column sub-tiles
@@ -808,7 +782,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
 
 }  // namespace
 
-cudaError_t launch_bwd_pair(const BwdMaps& maps, const BwdArgs& args, int num_sms, cudaStream_t st) {
+cudaError_t launch_bwd_pair(const BwdPairMaps& maps, const BwdArgs& args, int num_sms, cudaStream_t st) {
   if (args.n_items == 0) return cudaSuccess;
   cudaError_t e = cudaFuncSetAttribute(bwd_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(sizeof(PairSmem)));
   if (e != cudaSuccess) return e;

@@ -60,6 +60,12 @@ struct BwdMaps {
   CUtensorMap dk[NSP_MAX_RUNS], dv[NSP_MAX_RUNS];  // fp32 dK / dV outputs (tile stores of 32 columns x 128 rows); unset for bf16 outputs
 };
 
+// The pair kernel's: q and d_o with boxes of 64 rows, and the fp32 dQ accumulator (reductions of 32 columns x 16 rows).
+struct BwdPairMaps : BwdMaps {
+  CUtensorMap dq_acc[NSP_MAX_RUNS];
+};
+static_assert(sizeof(BwdPairMaps) + 256 <= 32764, "kernel parameters");
+
 // Device status record {code, item, where, aux}; the first writer wins (atomicCAS on the code in device memory) and
 // also copies its record into mapped pinned host memory, code last, so that the host sees a failure at its next API
 // call without synchronising.
@@ -240,8 +246,8 @@ cudaError_t launch_bwd_preprocess(const SegInfo* d_seg, int n_seg, const int64_t
 cudaError_t launch_bwd_first(const BwdMaps& maps, const BwdArgs& args, int head_dim, int num_sms, cudaStream_t st);
 cudaError_t launch_bwd(const BwdMaps& maps, const BwdArgs& args, int head_dim, int num_sms, bool chained, cudaStream_t st);  // args.dq_turn / args.dq_rounded select the reproducible variants
 // the long segments' share of the main kernel's work, on CTA pairs: items (segment, kv head, two key tiles), head dimension
-// 128; maps.q and maps.d_o have boxes of 64 rows
-cudaError_t launch_bwd_pair(const BwdMaps& maps, const BwdArgs& args, int num_sms, cudaStream_t st);
+// 128
+cudaError_t launch_bwd_pair(const BwdPairMaps& maps, const BwdArgs& args, int num_sms, cudaStream_t st);
 cudaError_t launch_bwd_postprocess(const SegInfo* d_seg, int n_seg, const int64_t* d_row_base, int64_t total_rows,
                                    int head_dim, const float* dq_acc, void* dq, int dq_f32, float scale,
                                    cudaStream_t st);

@@ -377,22 +377,22 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
             auto issue_s = [&](int vt, bool here) -> bool {  // here: the Q rows have arrived
               const uint32_t cs = gs + vt;
               // R0 [64, 128) held dQ^T of the step before the last one (of this item: earlier ones are long drained)
-              if (vt > 0) here = mbar_poll(&s.bar_dq_empty, cs & 1, a.wait_limit) && here;
+              if (vt > 0) here = mbar_wait(&s.bar_dq_empty, cs & 1, a.wait_limit) && here;
               tc_fence_after_sync();
               issue_kk(tR0, k_km, q_km, leader && here);
               if (!together(here)) { where = kWhereBwdLoadQ; return false; }
               if (leader) umma2_commit(&s.bar_s_full);
               return true;
             };
-            okm = okm && issue_s(0, mbar_poll(&s.bar_qr_full, gs & 1, a.wait_limit));
+            okm = okm && issue_s(0, mbar_wait(&s.bar_qr_full, gs & 1, a.wait_limit));
 #pragma unroll 1
             for (int vt = 0; okm && vt < steps; ++vt) {
               const bool calm = *abort_flag == 0;
               const uint32_t cs = gs + vt;
-              bool here = mbar_poll(&s.bar_doc_full, cs & 1, a.wait_limit);
               const bool more = vt + 1 < steps;
-              if (more) here = mbar_poll(&s.bar_qr_full, (cs + 1) & 1, a.wait_limit) && here;
-              here = mbar_poll(&s.bar_p_ready, cs & 1, a.wait_limit) && here;
+              bool here = more ? mbar_wait2(&s.bar_doc_full, cs & 1, &s.bar_qr_full, (cs + 1) & 1, a.wait_limit)
+                               : mbar_wait(&s.bar_doc_full, cs & 1, a.wait_limit);
+              here = mbar_wait(&s.bar_p_ready, cs & 1, a.wait_limit) && here;
               tc_fence_after_sync();
               issue_kn(tDV, tR0, do_mn, vt > 0, leader && here);
               if (!together(here && calm)) {
@@ -413,16 +413,16 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
               if (leader) umma2_commit(&s.bar_dp_full);
               return true;
             };
-            okm = okm && issue_dp(mbar_poll(&s.bar_dor_full, gs & 1, a.wait_limit));
+            okm = okm && issue_dp(mbar_wait(&s.bar_dor_full, gs & 1, a.wait_limit));
 #pragma unroll 1
             for (int vt = 0; okm && vt < steps; ++vt) {
               const bool calm = *abort_flag == 0;
               const uint32_t cs = gs + vt;
               if (leader) mbar_expect_tx(&s.bar_x_full, kHalfTileBytes);
               const bool more = vt + 1 < steps;
-              bool here = mbar_poll(&s.bar_qc_full, cs & 1, a.wait_limit);
-              if (more) here = mbar_poll(&s.bar_dor_full, (cs + 1) & 1, a.wait_limit) && here;
-              here = mbar_poll(&s.bar_ds_ready, cs & 1, a.wait_limit) && here;
+              bool here = more ? mbar_wait2(&s.bar_qc_full, cs & 1, &s.bar_dor_full, (cs + 1) & 1, a.wait_limit)
+                               : mbar_wait(&s.bar_qc_full, cs & 1, a.wait_limit);
+              here = mbar_wait(&s.bar_ds_ready, cs & 1, a.wait_limit) && here;
               tc_fence_after_sync();
               issue_kn(tDK, tR1, q_mn, vt > 0, leader && here);
               if (!together(here && calm)) {
@@ -433,10 +433,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
               if (leader) umma2_commit(&s.bar_dk_done);
               if (more && !issue_dp(true)) { okm = false; break; }
               // dQ^T over the part of R0 that packed P^T leaves free, once S^T of the next step has been read from it
-              here = mbar_poll(&s.bar_x_own, cs & 1, a.wait_limit);
-              if (more) here = mbar_poll(&s.bar_s_read, (cs + 1) & 1, a.wait_limit) && here;
-              here = mbar_poll(&s.bar_x_full, cs & 1, a.wait_limit) && here;
-              here = mbar_poll(&s.bar_x_peer, cs & 1, a.wait_limit) && here;
+              here = more ? mbar_wait2(&s.bar_x_own, cs & 1, &s.bar_s_read, (cs + 1) & 1, a.wait_limit)
+                          : mbar_wait(&s.bar_x_own, cs & 1, a.wait_limit);
+              here = mbar_wait2(&s.bar_x_full, cs & 1, &s.bar_x_peer, cs & 1, a.wait_limit) && here;
               tc_fence_after_sync();
               const bool go = leader && here;
 #pragma unroll
@@ -535,7 +534,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
         w.get(c, h, m);
         w.next(c);
         const bool calm = *abort_flag == 0;
-        oks = mbar_wait(&s.bar_ld_full[st], (cs >> 1) & 1, a.wait_limit) && mbar_wait(&s.bar_s_full, cs & 1, a.wait_limit);
+        oks = mbar_wait2(&s.bar_ld_full[st], (cs >> 1) & 1, &s.bar_s_full, cs & 1, a.wait_limit);
         if (!together(oks && calm)) {
           if (!together(oks)) where = kWhereBwdS;
           oks = false;
@@ -590,7 +589,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
           if (lane == 0) arrive_lead(&s.bar_p_ready);
 #pragma unroll
           for (int i = 0; i < 4; ++i) aux[0][i] = lds128(delta_s + 4 * i);
-          oks = mbar_wait(&s.bar_dp_full, cs & 1, a.wait_limit);
+          // the dS^T buffers are free once dQ^T of the step before has completed
+          oks = mbar_wait2(&s.bar_dp_full, cs & 1, &s.bar_dq_full, (cs - 1) & 1, a.wait_limit);
           if (!together(oks)) { where = kWhereBwdDp; return false; }
           tc_fence_after_sync();
           uint32_t dpv[2][16];
@@ -618,6 +618,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
               dsp[(x >> 1) + 1] = pack_bf16x2(d2, d3);
             }
             if (ch & 1) tmem_st16(tDP + (ch >> 1) * 16, pp[ch >> 1]);
+            *reinterpret_cast<uint4*>(ds_row + ((2 * ch) ^ (r & 7)) * 16) = make_uint4(dsp[0], dsp[1], dsp[2], dsp[3]);
+            *reinterpret_cast<uint4*>(ds_row + ((2 * ch + 1) ^ (r & 7)) * 16) = make_uint4(dsp[4], dsp[5], dsp[6], dsp[7]);
           }
           tmem_wait_st();
           tc_fence_before_sync();
@@ -626,13 +628,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
             arrive_lead(&s.bar_ds_ready);  // dK and dP^T of the next step need no more than this
             mbar_arrive(&s.bar_ld_empty[st]);
           }
-          // the dS^T buffers are free once dQ^T of the step before has completed
-          oks = vt == 0 || mbar_wait(&s.bar_dq_full, (cs - 1) & 1, a.wait_limit);
-          if (!together(oks)) { where = kWhereBwdStaged; return false; }
-#pragma unroll
-          for (int i = 0; i < 8; ++i)
-            *reinterpret_cast<uint4*>(ds_row + (i ^ (r & 7)) * 16) =
-                make_uint4(pp[i >> 2][(i & 3) * 4], pp[i >> 2][(i & 3) * 4 + 1], pp[i >> 2][(i & 3) * 4 + 2], pp[i >> 2][(i & 3) * 4 + 3]);
           return true;
         };
         if (m > c.n) {

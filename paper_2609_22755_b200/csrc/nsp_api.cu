@@ -197,7 +197,13 @@ inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 // bound the call (20 segments of about 100 tokens at 64q/4kv 233 -> 216 us; parts of eight steps 248, of two 215).
 constexpr int kMinPart = 16, kMinFirstPart = 4;
 constexpr int64_t kMostByLength = 600ll << 20;
-constexpr int kPairTiles = 16;
+// Backward items that run on CTA pairs: segments of at least kPairTiles key tiles and kPairSteps steps for the first of them. A
+// pair computes one tile more than it needs (the second key tile has nothing of the item's last q tile) and meets its partner
+// between items. Backward pass over about 131,072 tokens, ms, pairs / single CTAs: 32q/4kv in segments of 512 tokens (4
+// tiles) not paired, 1,024 4.56 / 4.55, 1,536 5.91 / 5.98, 2,048 7.22 / 7.36, 3,072 9.58 / 10.03, 4,096 12.2 / 12.6;
+// 64q/4kv in 4,096 24.0 / 25.3; one head per KV head (16q/16kv) 2,000 4.32 / 4.25, 3,000 5.16 / 5.17. Batches whose longest
+// item would bound the kernel are divided instead (divide_items), and small ones (small_bwd) run their kernels side by side.
+constexpr int kPairTiles = 16, kPairSteps = 32;
 struct WholeItem {
   int32_t seg, head, tile, steps;
 };
@@ -503,7 +509,7 @@ int nsp_plan_tiles(const int32_t* cu_seqlens, const int32_t* hq, const int32_t* 
         for (; paired < order.size(); ++paired) {
           const SegInfo& sg = p->seg[order[paired]];
           const int32_t Mt = (sg.len + bm - 1) / bm, G = sg.hq / sg.hkv;
-          if (Mt < kPairTiles) break;
+          if (Mt < kPairTiles || G * Mt < kPairSteps) break;
           for (int g = 0; g < sg.hkv; ++g)
             for (int32_t n = 0; n < Mt; n += 2) {
               pairs.push_back(nsp_tile_t{order[paired], g, n / 2, G * (Mt - std::max(n, 1))});

@@ -1,0 +1,65 @@
+"""Backward pass of long segments on CTA pairs: against the oracle and against the plan option whose dQ additions are ordered,
+which runs every segment on single CTAs."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+def _batch(lengths, hq, hkv):
+    import torch
+
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA device")
+    from paper_2609_22755_b200 import workloads as W
+
+    return W.custom(lengths, hq, hkv, seed=43)
+
+
+# The pair kernel takes segments of 16 key tiles (32 with one head per KV head) and more, of a batch that fills the chip.
+@pytest.mark.parametrize("lengths,hq,hkv,dkv_dtype", [
+    ([2048] * 20, 16, 4, "f32"),                             # whole tiles, an even number of them
+    ([2049] * 30, 8, 2, "f32"),                              # an odd number: the second CTA of the last pair has no keys
+    ([4100, 3969, 4097, 3968, 200, 40, 4200] * 3, 8, 8, "f32"),  # one head per KV head, ragged tiles, segments just below
+    ([2200, 1999, 1921, 1920, 129] * 3, 24, 8, "bf16"),      # bf16 gradients, odd groups, segments just below
+    ([4300, 3500, 100, 4299] * 4, 64, 1, "f32"),             # the start alignment of long items
+])
+def test_pairs_against_single_ctas(lengths, hq, hkv, dkv_dtype):
+    import parity_util as P
+
+    w = _batch(lengths, hq, hkv)
+    run = P.GpuRun(w, dq_dtype="f32", dkv_dtype=dkv_dtype)
+    single = P.GpuRun(w, tensors=run.host, dq_dtype="f32", dkv_dtype=dkv_dtype, deterministic=True)
+    got = []
+    for r in (run, single):
+        r.forward()
+        for _ in range(2):
+            for t in (r.dq, r.dk, r.dv):
+                t.fill_(float("nan"))
+            r.backward()
+        assert r.status()[0] == 0
+        got.append(r.results())
+    # The same products of the same operands; what differs is the order in which the tensor core adds and in which up to 32
+    # tiles are added to a row of dQ, one fp32 rounding each: 32 * 2^-24 of the largest partial sum. bf16 results: one step.
+    for n in ("dq", "dk", "dv"):
+        tol = 2.0 ** -8 if n != "dq" and dkv_dtype == "bf16" else 2e-5
+        assert np.max(np.abs(got[0][n] - got[1][n])) <= tol * np.max(np.abs(got[1][n])), n
+
+
+def test_pairs_against_the_oracle():
+    import parity_util as P
+    from paper_2609_22755_b200 import workloads as W
+
+    L, n, hq, hkv = 3073, 16, 8, 2
+    w = _batch([L] * n, hq, hkv)
+    run = P.GpuRun(w)
+    run.forward()
+    run.backward()
+    assert run.status()[0] == 0
+    res = run.results()
+    s = n - 1  # the last segment: behind its end lies the end of the tensors
+    one = W.custom([L], hq, hkv, seed=43)
+    q, kv, lse = (slice(s * L * h * x, (s + 1) * L * h * x) for h, x in ((hq, 128), (hkv, 128), (hq, 1)))
+    host = {k: run.host[k][kv if k in "kv" else q] for k in ("q", "k", "v", "do")}
+    cut = {k: res[k][{"lse": lse, "dk": kv, "dv": kv}.get(k, q)] for k in res}
+    P.compare_full(one, cut, P.oracle_full(one, host))

@@ -518,7 +518,9 @@ int nsp_plan_tiles(const int32_t* cu_seqlens, const int32_t* hq, const int32_t* 
             }
           p->n_bwd_paired += static_cast<int64_t>(sg.hkv) * Mt;
         }
-        if (longest * (p->num_sms / 2) > steps) {  // the longest item would bound the kernel
+        // Not where the longest item would bound the kernel, nor where other segments have more than a quarter of the steps:
+        // the two launches each have a tail.
+        if (longest * (p->num_sms / 2) > steps || 8 * steps < 3 * bwd_steps) {
           paired = 0;
           p->n_bwd_paired = 0;
           pairs.clear();

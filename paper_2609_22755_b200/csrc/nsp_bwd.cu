@@ -2,7 +2,7 @@
 //
 // Three launches:
 //   preprocess   delta[h, i] = sum_d dO[i,h,d] * O[i,h,d]                      (HBM-bound, one warp per row)
-//   main         key-stationary persistent kernel, see below
+//   main         key-stationary persistent kernel, see below; long segments run on CTA pairs instead (nsp_bwd_pair.cu)
 //   postprocess  dQ = scale * fp32 accumulator -> bf16 / fp32                   (HBM-bound)
 //
 // Main kernel. One CTA per SM (640 threads, five warpgroups with their own register budgets; 896 in seven at D = 64) pops items

@@ -78,7 +78,7 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, long l
     if (clock64() - t0 > limit) return false;
   }
 }
-// Two phases at once: the tests are in flight together. A test that finds its phase complete takes ~200 clocks on an SM whose
+// Two phases at once: the tests are in flight together. A test that finds its phase complete takes 110-140 clocks on an SM whose
 // tensor core and reductions keep shared memory busy, so waits one behind the other are what a chain of hand-overs consists of.
 __device__ __forceinline__ bool mbar_wait2(uint64_t* bar_a, uint32_t parity_a, uint64_t* bar_b, uint32_t parity_b, long long limit) {
   const long long t0 = clock64();

@@ -69,12 +69,12 @@ struct PairSmem {
   uint64_t bar_s_read;    // 16 warps: S^T has been read (R0 [64, 128) is free for dQ^T)
   uint64_t bar_p_ready;   // 16 warps: P^T is in R0
   uint64_t bar_ds_ready;  // 16 warps: dS^T is in R1
-  uint64_t bar_x_own;     // 8 warps: the parts of dS^T that stay in their CTA are in shared memory
   uint64_t bar_dq_empty;  // 16 warps: dQ^T has been drained
-  uint64_t bar_x_peer;    // the second CTA has received its part of dS^T
+  uint64_t bar_x_peer;    // the second CTA's dS^T buffers are complete (its own warps' part and the received one)
   // Completed in both CTAs: products
   uint64_t bar_s_full, bar_dp_full, bar_dq_full, bar_dv_done, bar_dk_done;
   // Local
+  uint64_t bar_x_own;   // 4 warps: the part of dS^T that stays in this CTA is in shared memory
   uint64_t bar_x_full;  // the other CTA's part of dS^T has arrived
   uint64_t bar_ld_full[2], bar_ld_empty[2];
   uint64_t bar_out;
@@ -113,7 +113,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
     mbar_init(&s.bar_s_read, 16);
     mbar_init(&s.bar_p_ready, 16);
     mbar_init(&s.bar_ds_ready, 16);
-    mbar_init(&s.bar_x_own, 8);
+    mbar_init(&s.bar_x_own, 4);
     mbar_init(&s.bar_dq_empty, 16);
     mbar_init(&s.bar_x_peer, 1);
     mbar_init(&s.bar_s_full, 1);
@@ -150,12 +150,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
   }
   uint32_t gs = 0, gi = 0;  // steps and items completed by this pair
   auto together = [&](bool here) -> bool { return __all_sync(0xffffffffu, here); };
-  // One lane of a warp whose part is done: to the first CTA's barrier
+  // One lane of a warp whose part in TMEM is done, to the first CTA's barrier
   auto arrive_lead = [&](uint64_t* bar) {
     if (rank == 0)
       mbar_arrive(bar);
     else
-      cluster_arrive(lead + off(bar));
+      cluster_arrive_relaxed(lead + off(bar));
   };
 
   // The first CTA's thread 0 pops for both. Every thread of both CTAs goes by the popped position alone, so both leave
@@ -323,7 +323,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
       }
     } else if (rank != 0) {
       // ================================================================ second CTA: no products to issue
-      // warp 19 passes on that this CTA has received its part of dS^T
+      // warp 19 passes on that this CTA's dS^T buffers are complete: a release at cluster scope that orders what its softmax
+      // warps stored and handed to this warp ahead of the first CTA's products
       while (next_item()) {
         if (warp == 19 && lane == 0) {
           const int steps = s.ctx.steps, it = s.ctx.it;
@@ -331,12 +332,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
           for (int vt = 0; vt < steps; ++vt) {
             if (*abort_flag) break;
             mbar_expect_tx(&s.bar_x_full, kHalfTileBytes);
-            if (!mbar_wait(&s.bar_x_full, (gs + vt) & 1, a.wait_limit)) {
+            if (!mbar_wait2(&s.bar_x_full, (gs + vt) & 1, &s.bar_x_own, (gs + vt) & 1, a.wait_limit)) {
               report_timeout(a.status, it, kWhereBwdStaged, vt);
               raise_abort();
               break;
             }
-            cluster_arrive(lead + off(&s.bar_x_peer));
+            cluster_arrive_release(lead + off(&s.bar_x_peer));
           }
         }
         __syncwarp();
@@ -356,7 +357,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
           constexpr uint32_t lbo_km = (16u >> 4) << 16, lbo_mn = (kHalfTileBytes >> 4) << 16;
           const int steps = s.ctx.steps, item_it = s.ctx.it;
           int where = 0;
-          bool okm = together(mbar_wait(&s.bar_kv, gi & 1, a.wait_limit));
+          bool okm = together(cluster_wait(&s.bar_kv, gi & 1, a.wait_limit));
           if (!okm) where = kWhereBwdLoadKV;
           // [128 own rows] x [64 + 64 rows]: S^T or dP^T
           auto issue_kk = [&](uint32_t d, uint32_t a_km, uint32_t b_km, bool go) {
@@ -380,22 +381,22 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
             auto issue_s = [&](int vt, bool here) -> bool {  // here: the Q rows have arrived
               const uint32_t cs = gs + vt;
               // R0 [64, 128) held dQ^T of the step before the last one (of this item: earlier ones are long drained)
-              if (vt > 0) here = mbar_wait(&s.bar_dq_empty, cs & 1, a.wait_limit) && here;
+              if (vt > 0) here = cluster_wait_tmem(&s.bar_dq_empty, cs & 1, a.wait_limit) && here;
               tc_fence_after_sync();
               issue_kk(tR0, k_km, q_km, leader && here);
               if (!together(here)) { where = kWhereBwdLoadQ; return false; }
               if (leader) umma2_commit(&s.bar_s_full);
               return true;
             };
-            okm = okm && issue_s(0, mbar_wait(&s.bar_qr_full, gs & 1, a.wait_limit));
+            okm = okm && issue_s(0, cluster_wait(&s.bar_qr_full, gs & 1, a.wait_limit));
 #pragma unroll 1
             for (int vt = 0; okm && vt < steps; ++vt) {
               const bool calm = *abort_flag == 0;
               const uint32_t cs = gs + vt;
               const bool more = vt + 1 < steps;
-              bool here = more ? mbar_wait2(&s.bar_doc_full, cs & 1, &s.bar_qr_full, (cs + 1) & 1, a.wait_limit)
-                               : mbar_wait(&s.bar_doc_full, cs & 1, a.wait_limit);
-              here = mbar_wait(&s.bar_p_ready, cs & 1, a.wait_limit) && here;
+              bool here = more ? cluster_wait2(&s.bar_doc_full, cs & 1, &s.bar_qr_full, (cs + 1) & 1, a.wait_limit)
+                               : cluster_wait(&s.bar_doc_full, cs & 1, a.wait_limit);
+              here = cluster_wait_tmem(&s.bar_p_ready, cs & 1, a.wait_limit) && here;
               tc_fence_after_sync();
               issue_kn(tDV, tR0, do_mn, vt > 0, leader && here);
               if (!together(here && calm)) {
@@ -416,16 +417,18 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
               if (leader) umma2_commit(&s.bar_dp_full);
               return true;
             };
-            okm = okm && issue_dp(mbar_wait(&s.bar_dor_full, gs & 1, a.wait_limit));
+            okm = okm && issue_dp(cluster_wait(&s.bar_dor_full, gs & 1, a.wait_limit));
 #pragma unroll 1
             for (int vt = 0; okm && vt < steps; ++vt) {
               const bool calm = *abort_flag == 0;
               const uint32_t cs = gs + vt;
               if (leader) mbar_expect_tx(&s.bar_x_full, kHalfTileBytes);
               const bool more = vt + 1 < steps;
-              bool here = more ? mbar_wait2(&s.bar_qc_full, cs & 1, &s.bar_dor_full, (cs + 1) & 1, a.wait_limit)
-                               : mbar_wait(&s.bar_qc_full, cs & 1, a.wait_limit);
-              here = mbar_wait(&s.bar_ds_ready, cs & 1, a.wait_limit) && here;
+              bool here = more ? cluster_wait2(&s.bar_qc_full, cs & 1, &s.bar_dor_full, (cs + 1) & 1, a.wait_limit)
+                               : cluster_wait(&s.bar_qc_full, cs & 1, a.wait_limit);
+              here = cluster_wait_tmem(&s.bar_ds_ready, cs & 1, a.wait_limit) && here;
+              // every phase is waited for once, so that none is taken for the one before (below: from the second step on)
+              if (vt == 0) here = cluster_wait_tmem(&s.bar_s_read, cs & 1, a.wait_limit) && here;
               tc_fence_after_sync();
               issue_kn(tDK, tR1, q_mn, vt > 0, leader && here);
               if (!together(here && calm)) {
@@ -436,9 +439,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
               if (leader) umma2_commit(&s.bar_dk_done);
               if (more && !issue_dp(true)) { okm = false; break; }
               // dQ^T over the part of R0 that packed P^T leaves free, once S^T of the next step has been read from it
-              here = more ? mbar_wait2(&s.bar_x_own, cs & 1, &s.bar_s_read, (cs + 1) & 1, a.wait_limit)
-                          : mbar_wait(&s.bar_x_own, cs & 1, a.wait_limit);
-              here = mbar_wait2(&s.bar_x_full, cs & 1, &s.bar_x_peer, cs & 1, a.wait_limit) && here;
+              here = wait_both([&] { return mbar_try_wait(&s.bar_x_own, cs & 1); },
+                               [&] { return !more || cluster_try_wait_relaxed(&s.bar_s_read, (cs + 1) & 1); }, a.wait_limit);
+              here = cluster_wait2(&s.bar_x_full, cs & 1, &s.bar_x_peer, cs & 1, a.wait_limit) && here;
               tc_fence_after_sync();
               const bool go = leader && here;
 #pragma unroll
@@ -495,8 +498,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
         __syncwarp();
         if (lane == 0) arrive_lead(&s.bar_dq_empty);
         // Added by TMA: as 32 reductions per thread they fill the memory queue that the softmax warps' waits and shared-memory
-        // accesses go through (65,536 tokens at 4q/1kv 10.4 -> 10.1 ms a backward pass). Sixteen rows at a time through the warp's 2 KB. Rows past the segment's end add zeros (their dS^T columns are zero)
-        // to the first rows of the segments behind it, which nobody reads, or lie outside the tensor map.
+        // accesses go through (65,536 tokens at 4q/1kv 10.4 -> 10.1 ms a backward pass). Sixteen rows at a time through the
+        // warp's 2 KB. Rows past the segment's end add zeros (their dS^T columns are zero) to the first rows of the segments
+        // behind it, which nobody reads, or lie outside the tensor map.
 #pragma unroll
         for (int i = 0; i < 2; ++i) {
           if (lane == 0) tma_store_wait_read();
@@ -643,7 +647,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
         __syncwarp();
         if (lane == 0) {
           if (keep)
-            arrive_lead(&s.bar_x_own);
+            mbar_arrive(&s.bar_x_own);
           else
             copy_to_cluster(x_to, s.stage + quad * 4096, 4096, x_bar);
         }

@@ -78,16 +78,29 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, long l
     if (clock64() - t0 > limit) return false;
   }
 }
-// Two phases at once: the tests are in flight together. A test that finds its phase complete takes 110-140 clocks on an SM whose
-// tensor core and reductions keep shared memory busy, so waits one behind the other are what a chain of hand-overs consists of.
-__device__ __forceinline__ bool mbar_wait2(uint64_t* bar_a, uint32_t parity_a, uint64_t* bar_b, uint32_t parity_b, long long limit) {
+template <typename Test>
+__device__ __forceinline__ bool wait_for(Test test, long long limit) {
   const long long t0 = clock64();
 #pragma unroll 1
   for (;;) {
-    const bool a = mbar_try_wait(bar_a, parity_a), b = mbar_try_wait(bar_b, parity_b);
+    if (test()) return true;
+    if (clock64() - t0 > limit) return false;
+  }
+}
+// Two phases at once: the tests are in flight together. A test that finds its phase complete takes 110-140 clocks on an SM whose
+// tensor core and reductions keep shared memory busy, so waits one behind the other are what a chain of hand-overs consists of.
+template <typename TestA, typename TestB>
+__device__ __forceinline__ bool wait_both(TestA test_a, TestB test_b, long long limit) {
+  const long long t0 = clock64();
+#pragma unroll 1
+  for (;;) {
+    const bool a = test_a(), b = test_b();
     if (a && b) return true;
     if (clock64() - t0 > limit) return false;
   }
+}
+__device__ __forceinline__ bool mbar_wait2(uint64_t* bar_a, uint32_t parity_a, uint64_t* bar_b, uint32_t parity_b, long long limit) {
+  return wait_both([&] { return mbar_try_wait(bar_a, parity_a); }, [&] { return mbar_try_wait(bar_b, parity_b); }, limit);
 }
 // One look: has the phase completed? (To say which of several waits failed, once one has.)
 __device__ __forceinline__ bool mbar_test(uint64_t* bar, uint32_t parity) {
@@ -295,11 +308,54 @@ __device__ __forceinline__ uint32_t cluster_addr(const void* p, uint32_t rank) {
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(p)), "r"(rank));
   return a;
 }
-// Released at CTA scope: what it hands over is TMEM contents (ordered by tcgen05 fences) and shared memory that only the
-// tensor core reads (ordered by a proxy fence). Released at cluster scope it held its warp up for ~1,000 clocks, four times a
-// step.
-__device__ __forceinline__ void cluster_arrive(uint32_t bar) {
-  asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
+// Arrivals on the other CTA's barriers, and waits on the barriers that the other CTA's threads or loads arrive on. An arrival and
+// a wait synchronise in the memory model only where their scope covers both threads, so all of them name cluster scope.
+// TMEM contents are handed over by the tcgen05 fences on either side: the relaxed forms do. What was written to shared
+// memory by ordinary stores needs a release. It is the fence restricted to shared memory: a plain
+// mbarrier.arrive.release.cluster takes ~1,000 clocks even in an idle warp (backward pass over 16 x 8,192 tokens at 32q/4kv
+// 25.5 ms, with the restricted fence 21.6; 64 x 2,048 8.1 / 6.7).
+__device__ __forceinline__ void cluster_arrive_relaxed(uint32_t bar) {
+  asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ void cluster_arrive_release(uint32_t bar) {
+  asm volatile(
+      "fence.release.sync_restrict::shared::cta.cluster;\n\t"
+      "mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];"
+      ::"r"(bar)
+      : "memory");
+}
+__device__ __forceinline__ bool cluster_try_wait_relaxed(uint64_t* bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.try_wait.parity.relaxed.cluster.shared::cta.b64 p, [%1], %2, %3;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok)
+      : "r"(smem_u32(bar)), "r"(parity), "r"(200000u)
+      : "memory");
+  return ok != 0;
+}
+__device__ __forceinline__ bool cluster_try_wait(uint64_t* bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2, %3;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok)
+      : "r"(smem_u32(bar)), "r"(parity), "r"(200000u)
+      : "memory");
+  return ok != 0;
+}
+// Bounded waits of these forms: TMEM only, and everything else (see mbar_wait, mbar_wait2).
+__device__ __forceinline__ bool cluster_wait_tmem(uint64_t* bar, uint32_t parity, long long limit) {
+  return wait_for([&] { return cluster_try_wait_relaxed(bar, parity); }, limit);
+}
+__device__ __forceinline__ bool cluster_wait(uint64_t* bar, uint32_t parity, long long limit) {
+  return wait_for([&] { return cluster_try_wait(bar, parity); }, limit);
+}
+__device__ __forceinline__ bool cluster_wait2(uint64_t* bar_a, uint32_t parity_a, uint64_t* bar_b, uint32_t parity_b,
+                                              long long limit) {
+  return wait_both([&] { return cluster_try_wait(bar_a, parity_a); }, [&] { return cluster_try_wait(bar_b, parity_b); }, limit);
 }
 __device__ __forceinline__ void cluster_store(uint32_t addr, int32_t v) {
   asm volatile("st.relaxed.cluster.shared::cluster.b32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");

@@ -318,12 +318,24 @@ int nsp_selftest_wait_timeout(const nsp_plan_t* plan, int64_t limit_clk, void* s
  * INVALID_ARG. */
 int nsp_plan_set_wait_limit(nsp_plan_t* plan, int64_t sm_clocks);
 
+/* Tile loads of the backward kernel on CTA pairs, for nsp_checked_withhold_pair_load. */
+enum {
+  NSP_WITHHOLD_V = 1,
+  NSP_WITHHOLD_Q_ROWS = 2,
+  NSP_WITHHOLD_DO_ROWS = 3,
+  NSP_WITHHOLD_DO_COLUMNS = 4,
+  NSP_WITHHOLD_Q_COLUMNS = 5
+};
+
 #ifdef NSP_CHECKED
 /* Checked build only (libnsp_checked.so, compiled with -DNSP_CHECKED: every index a kernel computes for a global
  * access is verified first, a failing one is recorded as NSP_ERR_DEVICE_ASSERT and the access skipped). Test switch for
  * the failure path: with enable != 0 the next forward launch leaves out one V tile load, so that the waits behind it
  * run out (use a small nsp_plan_set_wait_limit); nothing faults, the launch ends with NSP_ERR_DEVICE_TIMEOUT. */
 int nsp_checked_withhold_load(nsp_plan_t* plan, int enable);
+/* The same for the backward kernel that runs on pairs of thread blocks: later backward launches leave out one tile load of the
+ * second block, a tile of V or one of the fourth step (load = 0: none). UNSUPPORTED if the plan has no such items. */
+int nsp_checked_withhold_pair_load(nsp_plan_t* plan, int load);
 #endif
 
 /* Kernels of the path, for nsp_plan_kernel_ms. */

@@ -34,7 +34,7 @@ EXPORTS = [
     "nsp_selftest_wait_timeout", "nsp_a2a_gather_heads_to", "nsp_plan_set_wait_limit",
     "nsp_plan_step_host_ws_bytes", "nsp_attn_step_host", "nsp_trim",
 ]
-CHECKED_EXPORTS = ["nsp_checked_withhold_load"]  # libnsp_checked.so only
+CHECKED_EXPORTS = ["nsp_checked_withhold_load", "nsp_checked_withhold_pair_load"]  # libnsp_checked.so only
 NSP_COST_BUCKETS = 16
 NSP_STATIC_WS_BYTES = 32 * 1024 * 1024
 KERNEL_FWD, KERNEL_BWD_PRE, KERNEL_BWD_MAIN, KERNEL_BWD_POST, KERNEL_BWD_FIRST, KERNEL_FWD_FIRST = 0, 1, 2, 3, 4, 5
@@ -110,6 +110,8 @@ def lib() -> ctypes.CDLL:
         if hasattr(L, "nsp_checked_withhold_load"):
             L.nsp_checked_withhold_load.argtypes = [vp, ctypes.c_int]
             L.nsp_checked_withhold_load.restype = ctypes.c_int
+            L.nsp_checked_withhold_pair_load.argtypes = [vp, ctypes.c_int]
+            L.nsp_checked_withhold_pair_load.restype = ctypes.c_int
         L.nsp_selftest_wait_timeout.argtypes = [vp, ctypes.c_int64, vp]
         L.nsp_selftest_wait_timeout.restype = ctypes.c_int
         L.nsp_device_status.argtypes = [vp, i32p]
@@ -507,6 +509,15 @@ def nsp_checked_withhold_load(plan: Plan, enable: bool):
     rc = lib().nsp_checked_withhold_load(plan.handle, int(bool(enable)))
     if rc != NSP_OK:
         raise NspError(rc, "nsp_checked_withhold_load")
+
+
+def nsp_checked_withhold_pair_load(plan: Plan, load: int):
+    """Checked build only: later backward launches on CTA pairs leave out one tile load (1 .. 5, see nsp.h; 0: none)."""
+    if not hasattr(lib(), "nsp_checked_withhold_pair_load"):
+        raise NspError(NSP_ERR_UNSUPPORTED, "nsp_checked_withhold_pair_load (needs libnsp_checked.so)")
+    rc = lib().nsp_checked_withhold_pair_load(plan.handle, int(load))
+    if rc != NSP_OK:
+        raise NspError(rc, "nsp_checked_withhold_pair_load")
 
 
 def nsp_device_status(plan: Plan):

@@ -79,6 +79,7 @@ struct nsp_plan {
   int sticky = 0;
   long long wait_limit = NSP_WAIT_CYCLES_DEFAULT;  // SM clocks a device-side wait may take
   int withhold = 0;                                // checked build: failure-detection test switch
+  int withhold_pair = 0;                           // likewise, the pair kernel of the backward pass
   // optional per-kernel timing (CUDA events on the launching stream)
   bool profiling = false;
   cudaEvent_t ev[2 * NSP_KERNEL_COUNT] = {};
@@ -874,6 +875,7 @@ int bwd_impl(const nsp_plan_t* plan, const uint8_t* recompute, const void* q, co
   a.q_elems = plan->q_elems;
   a.kv_elems = plan->kv_elems;
   a.lse_elems = plan->lse_elems;
+  a.withhold = plan->withhold_pair;
   // first-tile kernel: q tile 0 of every segment (its dQ rows; its part of, or all of, dK / dV rows 0..127)
   const bool f_parts = a.dkv_f32 && plan->n_first_parts > 0;  // bf16 gradients are not added up piece by piece
   a.items = f_parts ? plan->d_bwd_first_parts : plan->d_bwd_first;
@@ -1111,6 +1113,12 @@ int nsp_plan_set_wait_limit(nsp_plan_t* plan, int64_t sm_clocks) {
 int nsp_checked_withhold_load(nsp_plan_t* plan, int enable) {
   if (!plan) return NSP_ERR_INVALID_ARG;
   plan->withhold = enable != 0;
+  return NSP_OK;
+}
+int nsp_checked_withhold_pair_load(nsp_plan_t* plan, int load) {
+  if (!plan || load < 0 || load > NSP_WITHHOLD_Q_COLUMNS) return NSP_ERR_INVALID_ARG;
+  if (load != 0 && plan->n_bwd_pairs == 0) return NSP_ERR_UNSUPPORTED;
+  plan->withhold_pair = load;
   return NSP_OK;
 }
 #endif

@@ -226,12 +226,20 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
           const CUtensorMap* mq = &maps.q[c.run];
           const CUtensorMap* mdo = &maps.d_o[c.run];
           const int col = 64 * static_cast<int>(rank);
+          // checked build, failure-detection test: one tile of the second CTA never arrives (K / V, or in the fourth step)
+          auto withheld = [&]([[maybe_unused]] int load, [[maybe_unused]] int vt) -> bool {
+#ifdef NSP_CHECKED
+            return a.withhold == load && rank == 1 && c.it == 0 && vt == 2;
+#else
+            return false;
+#endif
+          };
           if (rank == 0) mbar_expect_tx(&s.bar_kv, 2 * 6 * kHalfTileBytes);
           const uint32_t kv = lead + off(&s.bar_kv);
 #pragma unroll
           for (int i = 0; i < 2; ++i) {
             tma_load_3d_pair(s.k[i], &maps.k[c.run], kv, 64 * i, c.g, c.tok0 + c.n * kBN);
-            tma_load_3d_pair(s.v[i], &maps.v[c.run], kv, 64 * i, c.g, c.tok0 + c.n * kBN);
+            if (!withheld(NSP_WITHHOLD_V, 2)) tma_load_3d_pair(s.v[i], &maps.v[c.run], kv, 64 * i, c.g, c.tok0 + c.n * kBN);
             tma_load_3d_pair(s.kt[i], &maps.k[c.run], kv, col, c.g, c.tok0 + (c.n0 + i) * kBN);
           }
           // boxes of q and dO are [64 rows x 64 columns]
@@ -263,13 +271,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
             w.get(c, h, m);
             w.next(c);
             bool ok = mbar_wait(&s.bar_s_full, ph, a.wait_limit);
-            if (ok) load_row(s.q_row, mq, &s.bar_qr_full, h, m);
+            if (ok && !withheld(NSP_WITHHOLD_Q_ROWS, vt)) load_row(s.q_row, mq, &s.bar_qr_full, h, m);
             ok = ok && mbar_wait(&s.bar_dp_full, ph, a.wait_limit);
-            if (ok) load_row(s.do_row, mdo, &s.bar_dor_full, h, m);
+            if (ok && !withheld(NSP_WITHHOLD_DO_ROWS, vt)) load_row(s.do_row, mdo, &s.bar_dor_full, h, m);
             ok = ok && mbar_wait(&s.bar_dv_done, ph, a.wait_limit);
-            if (ok) load_col(s.do_col, mdo, &s.bar_doc_full, h, m);
+            if (ok && !withheld(NSP_WITHHOLD_DO_COLUMNS, vt)) load_col(s.do_col, mdo, &s.bar_doc_full, h, m);
             ok = ok && mbar_wait(&s.bar_dk_done, ph, a.wait_limit);
-            if (ok) load_col(s.q_col, mq, &s.bar_qc_full, h, m);
+            if (ok && !withheld(NSP_WITHHOLD_Q_COLUMNS, vt)) load_col(s.q_col, mq, &s.bar_qc_full, h, m);
             if (!ok) {
               report_timeout(a.status, c.it, kWhereBwdQEmpty, vt);
               raise_abort();
@@ -777,6 +785,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
     }
   }
 
+  // After a failed wait (both flags are set: the barriers of next_item lie in between) roles of either CTA have left loads,
+  // products and copies of dS^T to the other CTA under way, which nobody waits for any more: they end before either leaves.
+  if (*abort_flag) drain_products();
   __syncwarp();
   tc_fence_before_sync();
   cluster_sync();  // neither CTA leaves while the other may still reach its shared memory or issue products into its TMEM

@@ -181,6 +181,7 @@ struct BwdArgs {
   float scale_log2;
   long long wait_limit;  // SM clocks a device-side wait may take before it gives up
   int64_t q_elems, kv_elems, lse_elems;  // tensor sizes (checked build)
+  int32_t withhold;  // checked build only: the load the pair kernel leaves out (NSP_WITHHOLD_*), or 0
   int32_t* front;    // [n_items / kFrontBlock + 1] arrival counters, zeroed by the preprocess kernel (see next_item)
   int32_t* turn;     // null, or items are parts (see kMaxParts): one counter per divided item, zero between launches
   const RowInfo* rows;  // row tables of the packs (first-tile kernel)

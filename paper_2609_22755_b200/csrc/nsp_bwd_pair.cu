@@ -270,16 +270,17 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
             const uint32_t ph = (gs + vt) & 1;
             w.get(c, h, m);
             w.next(c);
+            int at = 0;
             bool ok = mbar_wait(&s.bar_s_full, ph, a.wait_limit);
             if (ok && !withheld(NSP_WITHHOLD_Q_ROWS, vt)) load_row(s.q_row, mq, &s.bar_qr_full, h, m);
-            ok = ok && mbar_wait(&s.bar_dp_full, ph, a.wait_limit);
+            ok = ok && (++at, mbar_wait(&s.bar_dp_full, ph, a.wait_limit));
             if (ok && !withheld(NSP_WITHHOLD_DO_ROWS, vt)) load_row(s.do_row, mdo, &s.bar_dor_full, h, m);
-            ok = ok && mbar_wait(&s.bar_dv_done, ph, a.wait_limit);
+            ok = ok && (++at, mbar_wait(&s.bar_dv_done, ph, a.wait_limit));
             if (ok && !withheld(NSP_WITHHOLD_DO_COLUMNS, vt)) load_col(s.do_col, mdo, &s.bar_doc_full, h, m);
-            ok = ok && mbar_wait(&s.bar_dk_done, ph, a.wait_limit);
+            ok = ok && (++at, mbar_wait(&s.bar_dk_done, ph, a.wait_limit));
             if (ok && !withheld(NSP_WITHHOLD_Q_COLUMNS, vt)) load_col(s.q_col, mq, &s.bar_qc_full, h, m);
             if (!ok) {
-              report_timeout(a.status, c.it, kWhereBwdQEmpty, vt);
+              report_timeout(a.status, c.it, kWhereBwdQEmpty, 100000 * at + vt);  // of S^T, dP^T, dV, dK
               raise_abort();
               break;
             }
@@ -341,7 +342,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
             if (*abort_flag) break;
             mbar_expect_tx(&s.bar_x_full, kHalfTileBytes);
             if (!mbar_wait2(&s.bar_x_full, (gs + vt) & 1, &s.bar_x_own, (gs + vt) & 1, a.wait_limit)) {
-              report_timeout(a.status, it, kWhereBwdStaged, vt);
+              report_timeout(a.status, it, mbar_test(&s.bar_x_full, (gs + vt) & 1) ? kWhereBwdStaged : kWhereBwdXFull, vt);
               raise_abort();
               break;
             }
@@ -367,6 +368,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
           int where = 0;
           bool okm = together(cluster_wait(&s.bar_kv, gi & 1, a.wait_limit));
           if (!okm) where = kWhereBwdLoadKV;
+          int vt = 0;
           // [128 own rows] x [64 + 64 rows]: S^T or dP^T
           auto issue_kk = [&](uint32_t d, uint32_t a_km, uint32_t b_km, bool go) {
 #pragma unroll
@@ -392,13 +394,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
               if (vt > 0) here = cluster_wait_tmem(&s.bar_dq_empty, cs & 1, a.wait_limit) && here;
               tc_fence_after_sync();
               issue_kk(tR0, k_km, q_km, leader && here);
-              if (!together(here)) { where = kWhereBwdLoadQ; return false; }
+              if (!together(here)) { where = vt > 0 ? kWhereBwdDqEmpty : kWhereBwdLoadQ; return false; }
               if (leader) umma2_commit(&s.bar_s_full);
               return true;
             };
             okm = okm && issue_s(0, cluster_wait(&s.bar_qr_full, gs & 1, a.wait_limit));
 #pragma unroll 1
-            for (int vt = 0; okm && vt < steps; ++vt) {
+            for (; okm && vt < steps; ++vt) {
               const bool calm = *abort_flag == 0;
               const uint32_t cs = gs + vt;
               const bool more = vt + 1 < steps;
@@ -413,7 +415,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
                 break;
               }
               if (leader) umma2_commit(&s.bar_dv_done);
-              if (more) okm = issue_s(vt + 1, true);
+              if (more && !issue_s(vt + 1, true)) { okm = false; break; }
             }
           } else {
             const uint32_t v_km = smem_desc_addr(s.v[0]) | lbo_km, do_km = smem_desc_addr(s.do_row) | lbo_km;
@@ -427,7 +429,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
             };
             okm = okm && issue_dp(cluster_wait(&s.bar_dor_full, gs & 1, a.wait_limit));
 #pragma unroll 1
-            for (int vt = 0; okm && vt < steps; ++vt) {
+            for (; okm && vt < steps; ++vt) {
               const bool calm = *abort_flag == 0;
               const uint32_t cs = gs + vt;
               if (leader) mbar_expect_tx(&s.bar_x_full, kHalfTileBytes);
@@ -464,6 +466,21 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
             }
           }
           if (!okm) {
+            // Which of the waits in front of the failed vote: the first whose phase is still missing, or the last of them.
+            // (Told apart inside the loops it cost 0.5 % of a pass.)
+            const uint32_t cs = gs + vt;
+            const bool more = vt + 1 < steps;
+            auto missing = [&](uint64_t* bar, uint32_t parity) -> bool { return !together(mbar_test(bar, parity & 1)); };
+            if (where == kWhereBwdPReady) {
+              if (missing(&s.bar_doc_full, cs) || (more && missing(&s.bar_qr_full, cs + 1))) where = kWhereBwdLoadQ;
+            } else if (where == kWhereBwdDsReady) {
+              if (missing(&s.bar_qc_full, cs) || (more && missing(&s.bar_dor_full, cs + 1))) where = kWhereBwdLoadQ;
+              else if (vt == 0 && missing(&s.bar_s_read, cs)) where = kWhereBwdSRead;
+            } else if (where == kWhereBwdStaged && !missing(&s.bar_x_own, cs)) {
+              where = more && missing(&s.bar_s_read, cs + 1) ? kWhereBwdSRead
+                      : missing(&s.bar_x_full, cs)           ? kWhereBwdXFull
+                                                             : kWhereBwdXPeer;
+            }
             if (leader && where != 0) report_timeout(a.status, item_it, where, is_a ? 0 : 1);
             drain_products();
             raise_abort();
@@ -541,10 +558,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
     while (next_item()) {
       const PairCtx c = s.ctx;
       bool oks = true;
-      int where = 0;
+      int where = 0, vt = 0;
       PairWalk w;
 #pragma unroll 1
-      for (int vt = 0; vt < c.steps; ++vt) {
+      for (; vt < c.steps; ++vt) {
         const uint32_t cs = gs + vt, st = cs & 1;
         int h, m;
         w.get(c, h, m);
@@ -666,7 +683,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
         oks = mbar_wait(&s.bar_dv_done, lastp, a.wait_limit) && mbar_wait(&s.bar_dk_done, lastp, a.wait_limit) &&
               mbar_wait(&s.bar_dq_full, lastp, a.wait_limit);
         oks = together(oks);
-        if (!oks) where = kWhereBwdDqFull;
+        if (!oks) where = kWhereBwdMma2;
       }
       const int rows = min(kBN, c.len - c.n * kBN);  // none for the second CTA where the segment has an odd number of key tiles
       if (oks) {
@@ -778,7 +795,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
           fence_proxy_async_smem();
         }
       } else if (where != 0 && lane == 0) {
-        report_timeout(a.status, c.it, where, 0);
+        // which of the two waits of a step, or of the three behind the last
+        const uint32_t cs = gs + vt;
+        if (where == kWhereBwdS && !mbar_test(&s.bar_ld_full[cs & 1], (cs >> 1) & 1)) where = kWhereBwdLdFull;
+        if (where == kWhereBwdDp && mbar_test(&s.bar_dp_full, cs & 1)) where = kWhereBwdDqFull;
+        if (where == kWhereBwdMma2 && !mbar_test(&s.bar_dq_full, (cs - 1) & 1)) where = kWhereBwdDqFull;
+        report_timeout(a.status, c.it, where, vt);
         raise_abort();
       }
       item_done();

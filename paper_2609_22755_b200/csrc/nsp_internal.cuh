@@ -98,6 +98,10 @@ enum DeviceWhere : int32_t {
   kWhereBwdItemBarrier = 25,
   kWhereBwdTmemBase = 26,
   kWhereBwdTurn = 27,  // the parts before this one (deterministic dQ: the key tiles) did not finish their additions
+  kWhereBwdLdFull = 28,  // CTA pairs: LSE / delta of the step
+  kWhereBwdSRead = 29,   // S^T of the next step has not been read
+  kWhereBwdXFull = 30,   // the other CTA's part of dS^T
+  kWhereBwdXPeer = 31,   // the second CTA's dS^T buffers
   kWhereCheckFwdO = 40,    // checked build: an index outside the tensor (O, LSE / delta, dQ, dK / dV, LSE read)
   kWhereCheckFwdLse = 41,
   kWhereCheckBwdDq = 42,

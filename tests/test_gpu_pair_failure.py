@@ -1,4 +1,5 @@
-"""A wait of the CTA-pair kernel that runs out: a child process on the checked build, one load left out (withheld_pair_load_case.py)."""
+"""A wait of the CTA-pair kernel that runs out: a child process on the checked build, one load left out
+(withheld_pair_load_case.py). The record names the wait."""
 import os
 import subprocess
 import sys
@@ -10,8 +11,17 @@ pytestmark = pytest.mark.gpu
 ROOT = Path(__file__).resolve().parent.parent
 
 
-@pytest.mark.parametrize("load", [1, 2, 3, 4, 5])  # V, Q rows, dO rows, dO columns, Q columns
-def test_both_ctas_unwind(load):
+LOAD_KV, LOAD_Q, S_FULL, DQ_FULL, LD_FULL = 11, 12, 13, 20, 28  # kWhereBwd*
+
+
+@pytest.mark.parametrize("load,wheres,issuer", [
+    (1, {LOAD_KV, S_FULL, DQ_FULL, LD_FULL}, None),  # V: every role's first wait begins with the item
+    (2, {LOAD_Q}, 0),  # Q rows: the issuer of S^T is the first to wait for them, a step ahead
+    (3, {LOAD_Q}, 1),  # dO rows
+    (4, {LOAD_Q}, 0),  # dO columns
+    (5, {LOAD_Q}, 1),  # Q columns
+])
+def test_both_ctas_unwind(load, wheres, issuer):
     import torch
 
     if not torch.cuda.is_available():
@@ -20,5 +30,6 @@ def test_both_ctas_unwind(load):
     r = subprocess.run([sys.executable, str(ROOT / "tests" / "withheld_pair_load_case.py"), str(load)], env=env,
                        capture_output=True, text=True, timeout=300)
     assert r.returncode == 0, r.stdout + r.stderr
-    code = int(r.stdout.split("status ")[1].split()[0])
-    assert code == 5  # NSP_ERR_DEVICE_TIMEOUT
+    code, item, where, aux = map(int, r.stdout.split("status ")[1].split())
+    assert (code, item) == (5, 0) and where in wheres, (code, item, where, aux)  # NSP_ERR_DEVICE_TIMEOUT
+    assert issuer is None or aux == issuer

@@ -427,7 +427,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
               if (leader) umma2_commit(&s.bar_dp_full);
               return true;
             };
-            okm = okm && issue_dp(cluster_wait(&s.bar_dor_full, gs & 1, a.wait_limit));
+            // Every phase of s_read is waited for, so that none is taken for the one before; the first one here, ahead of the dP^T
+            // without which the softmax warps do not get to the next step (behind dS^T of the first step the barrier may be two
+            // phases ahead, and the wait for it would not end).
+            const bool s_read = cluster_wait_tmem(&s.bar_s_read, gs & 1, a.wait_limit);
+            okm = okm && issue_dp(cluster_wait(&s.bar_dor_full, gs & 1, a.wait_limit) && s_read);
 #pragma unroll 1
             for (; okm && vt < steps; ++vt) {
               const bool calm = *abort_flag == 0;
@@ -437,8 +441,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
               bool here = more ? cluster_wait2(&s.bar_qc_full, cs & 1, &s.bar_dor_full, (cs + 1) & 1, a.wait_limit)
                                : cluster_wait(&s.bar_qc_full, cs & 1, a.wait_limit);
               here = cluster_wait_tmem(&s.bar_ds_ready, cs & 1, a.wait_limit) && here;
-              // every phase is waited for once, so that none is taken for the one before (below: from the second step on)
-              if (vt == 0) here = cluster_wait_tmem(&s.bar_s_read, cs & 1, a.wait_limit) && here;
               tc_fence_after_sync();
               issue_kn(tDK, tR1, q_mn, vt > 0, leader && here);
               if (!together(here && calm)) {
@@ -475,7 +477,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
               if (missing(&s.bar_doc_full, cs) || (more && missing(&s.bar_qr_full, cs + 1))) where = kWhereBwdLoadQ;
             } else if (where == kWhereBwdDsReady) {
               if (missing(&s.bar_qc_full, cs) || (more && missing(&s.bar_dor_full, cs + 1))) where = kWhereBwdLoadQ;
-              else if (vt == 0 && missing(&s.bar_s_read, cs)) where = kWhereBwdSRead;
+            } else if (where == kWhereBwdLoadQ && !is_a) {
+              if (!missing(&s.bar_dor_full, gs)) where = kWhereBwdSRead;
             } else if (where == kWhereBwdStaged && !missing(&s.bar_x_own, cs)) {
               where = more && missing(&s.bar_s_read, cs + 1) ? kWhereBwdSRead
                       : missing(&s.bar_x_full, cs)           ? kWhereBwdXFull

@@ -450,9 +450,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
               }
               if (leader) umma2_commit(&s.bar_dk_done);
               if (more && !issue_dp(true)) { okm = false; break; }
-              // dQ^T over the part of R0 that packed P^T leaves free, once S^T of the next step has been read from it
+              // dQ^T over the part of R0 that packed P^T leaves free, once S^T of the next step, which waits for the drain of the
+              // dQ^T before, has been read from it; behind the last S^T that drain itself is waited for
+              uint64_t* const free_bar = more ? &s.bar_s_read : &s.bar_dq_empty;
               here = wait_both([&] { return mbar_try_wait(&s.bar_x_own, cs & 1); },
-                               [&] { return !more || cluster_try_wait_relaxed(&s.bar_s_read, (cs + 1) & 1); }, a.wait_limit);
+                               [&] { return cluster_try_wait_relaxed(free_bar, (cs + 1) & 1); }, a.wait_limit);
               here = cluster_wait2(&s.bar_x_full, cs & 1, &s.bar_x_peer, cs & 1, a.wait_limit) && here;
               tc_fence_after_sync();
               const bool go = leader && here;
@@ -480,9 +482,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
             } else if (where == kWhereBwdLoadQ && !is_a) {
               if (!missing(&s.bar_dor_full, gs)) where = kWhereBwdSRead;
             } else if (where == kWhereBwdStaged && !missing(&s.bar_x_own, cs)) {
-              where = more && missing(&s.bar_s_read, cs + 1) ? kWhereBwdSRead
-                      : missing(&s.bar_x_full, cs)           ? kWhereBwdXFull
-                                                             : kWhereBwdXPeer;
+              where = missing(more ? &s.bar_s_read : &s.bar_dq_empty, cs + 1) ? (more ? kWhereBwdSRead : kWhereBwdDqEmpty)
+                      : missing(&s.bar_x_full, cs)                            ? kWhereBwdXFull
+                                                                              : kWhereBwdXPeer;
             }
             if (leader && where != 0) report_timeout(a.status, item_it, where, is_a ? 0 : 1);
             drain_products();

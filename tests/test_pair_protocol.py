@@ -335,7 +335,7 @@ def test_no_wait_is_missing():
     assert faults(300) == []
 
 
-@pytest.mark.parametrize("without", ["s_read ahead of dP"])
+@pytest.mark.parametrize("without", ["last drain", "s_read ahead of dP"])
 def test_the_model_sees_a_missing_wait(without):
     assert faults(300, without=[without])
 
@@ -345,6 +345,6 @@ def test_the_kernel_has_the_waits_of_the_model():
     b = text[text.index("const uint32_t v_km = smem_desc_addr"):text.index("if (!okm) {")]
     head, loop = b.split("#pragma unroll 1", 1)
     assert re.search(r"wait\w*\(&s\.bar_s_read, gs & 1.*issue_dp\(", head, re.S)  # ahead of the first dP^T
-    # in front of dQ^T: S^T of the next step has been read
-    dq = loop[loop.index("bar_x_own"):loop.index("umma2_ss_lh(tDQ")]
-    assert loop.count("bar_s_read") == dq.count("bar_s_read") == 1
+    # in front of dQ^T: S^T of the next step has been read, or, behind the last step's, dQ^T of the one before has been drained
+    dq = loop[loop.index("issue_dp(true)"):loop.index("umma2_ss_lh(tDQ")]
+    assert "bar_dq_empty" in dq and loop.count("bar_s_read") == dq.count("bar_s_read") == 1

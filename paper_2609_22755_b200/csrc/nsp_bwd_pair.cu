@@ -365,6 +365,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
           const uint32_t hi = static_cast<uint32_t>(make_smem_desc_sw128(0, 16, 1024) >> 32);
           constexpr uint32_t lbo_km = (16u >> 4) << 16, lbo_mn = (kHalfTileBytes >> 4) << 16;
           const int steps = s.ctx.steps, item_it = s.ctx.it;
+          // The steps of q tile n0, the last ones, lie before every key of the second CTA (with n0 = 0 that q tile belongs to the
+          // first-tile kernel). Its P^T and dS^T are zero there, but zero times a value that is not finite, of that q
+          // tile or of keys that may be the next segment's, is not: they are left out of its dV and dK and of dQ^T.
+          const int alone = s.ctx.n0 > 0 ? steps - s.ctx.G : steps;  // first of them
           int where = 0;
           bool okm = together(cluster_wait(&s.bar_kv, gi & 1, a.wait_limit));
           if (!okm) where = kWhereBwdLoadKV;
@@ -379,7 +383,15 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
             }
           };
           // packed P^T or dS^T: 16 queries = 8 columns; queries 16 kk .. belong to warpgroup (kk >> 1) & 1
-          auto issue_kn = [&](uint32_t d, uint32_t a_tmem, uint32_t b_mn, uint32_t acc, bool go) {
+          auto issue_kn = [&](uint32_t d, uint32_t a_tmem, uint32_t b_mn, int at, bool go) {
+            const uint32_t acc = at > 0;
+            if (at >= alone) {
+#pragma unroll 1
+              for (int kk = 0; kk < 8; ++kk)
+                if (go) umma2_ts_lh_first(d, a_tmem + ((kk >> 1) & 1) * 32 + (kk >> 2) * 16 + (kk & 1) * 8, b_mn + kk * 128, hi,
+                                          idesc_kn, acc | (kk > 0));
+              return;
+            }
 #pragma unroll
             for (int kk = 0; kk < 8; ++kk)
               if (go) umma2_ts_lh(d, a_tmem + ((kk >> 1) & 1) * 32 + (kk >> 2) * 16 + (kk & 1) * 8, b_mn + kk * 128, hi, idesc_kn,
@@ -408,7 +420,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
                                : cluster_wait(&s.bar_doc_full, cs & 1, a.wait_limit);
               here = cluster_wait_tmem(&s.bar_p_ready, cs & 1, a.wait_limit) && here;
               tc_fence_after_sync();
-              issue_kn(tDV, tR0, do_mn, vt > 0, leader && here);
+              issue_kn(tDV, tR0, do_mn, vt, leader && here);
               if (!together(here && calm)) {
                 if (!together(here)) where = kWhereBwdPReady;
                 okm = false;
@@ -442,7 +454,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
                                : cluster_wait(&s.bar_qc_full, cs & 1, a.wait_limit);
               here = cluster_wait_tmem(&s.bar_ds_ready, cs & 1, a.wait_limit) && here;
               tc_fence_after_sync();
-              issue_kn(tDK, tR1, q_mn, vt > 0, leader && here);
+              issue_kn(tDK, tR1, q_mn, vt, leader && here);
               if (!together(here && calm)) {
                 if (!together(here)) where = kWhereBwdDsReady;
                 okm = false;
@@ -459,8 +471,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
               tc_fence_after_sync();
               const bool go = leader && here;
 #pragma unroll
-              for (int kk = 0; kk < 16; ++kk)
-                if (go) umma2_ss_lh(tDQ, kt_mn + kk * 128, hi, x_mn + kk * 128, hi, idesc_nn, kk > 0);
+              for (int kk = 0; kk < 16; ++kk)  // sixteen keys each, the first CTA's key tile first
+                if (go && (kk < 8 || vt < alone)) umma2_ss_lh(tDQ, kt_mn + kk * 128, hi, x_mn + kk * 128, hi, idesc_nn, kk > 0);
               if (!together(here)) {
                 where = kWhereBwdStaged;
                 okm = false;

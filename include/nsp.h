@@ -117,8 +117,14 @@ int nsp_plan_tiles(const int32_t* cu_seqlens, const int32_t* hq, const int32_t* 
 int nsp_plan_sizes(const nsp_plan_t* plan, int64_t* q_elems, int64_t* kv_elems, int64_t* lse_elems,
                    size_t* fwd_ws_bytes, size_t* bwd_ws_bytes);
 
+/* How backward calls with dK / dV of dkv_dtype run the plan's items of the main kernels: n_pairs on pairs of thread blocks, each
+ * two neighbouring key tiles of a long segment, and n_left of the backward list on single ones. Either may be NULL.
+ * Host-only, no CUDA call. */
+int nsp_plan_pair_items(const nsp_plan_t* plan, int dkv_dtype, int64_t* n_pairs, int64_t* n_left);
+
 /* Copy a work list to the host (pass 0 = forward, 1 = backward: the lists defined above, bit-exact; pass 2 = the
- * backward items in the order the backward kernel actually walks them, a permutation of pass 1 that is just as
+ * backward items in the order in which single thread blocks walk them (those that run on pairs, see nsp_plan_pair_items, are its
+ * first, and are walked two key tiles at a time), a permutation of pass 1 that is just as
  * unique: the (segment, kv head) groups by segment length descending, then segment, then kv head ascending; inside a
  * group the key tiles ascending. Group-major order keeps the dQ accumulator rows of a q tile in L2 while all key tiles
  * of the group add to them. Writes min(cap, n) items, stores n in *n_items (host_out may be NULL to query). Waits

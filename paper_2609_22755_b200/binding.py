@@ -32,7 +32,7 @@ EXPORTS = [
     "nsp_attn_bwd_static", "nsp_recompute_mark", "nsp_plan_recompute_ws_bytes", "nsp_attn_bwd_recompute",
     "nsp_cost_table", "nsp_route_sp_tree", "nsp_a2a_gather_heads", "nsp_a2a_scatter_heads",
     "nsp_selftest_wait_timeout", "nsp_a2a_gather_heads_to", "nsp_plan_set_wait_limit",
-    "nsp_plan_step_host_ws_bytes", "nsp_attn_step_host", "nsp_trim",
+    "nsp_plan_step_host_ws_bytes", "nsp_attn_step_host", "nsp_trim", "nsp_plan_pair_items",
 ]
 CHECKED_EXPORTS = ["nsp_checked_withhold_load", "nsp_checked_withhold_pair_load"]  # libnsp_checked.so only
 NSP_COST_BUCKETS = 16
@@ -73,6 +73,8 @@ def lib() -> ctypes.CDLL:
         L.nsp_plan_sizes.restype = ctypes.c_int
         L.nsp_plan_get.argtypes = [vp, ctypes.c_int, vp, ctypes.c_int64, i64p]
         L.nsp_plan_get.restype = ctypes.c_int
+        L.nsp_plan_pair_items.argtypes = [vp, ctypes.c_int, i64p, i64p]
+        L.nsp_plan_pair_items.restype = ctypes.c_int
         L.nsp_attn_fwd.argtypes = [vp, vp, vp, vp, vp, vp, ctypes.c_float, vp, ctypes.c_size_t, vp]
         L.nsp_attn_fwd.restype = ctypes.c_int
         L.nsp_attn_bwd.argtypes = [vp, vp, vp, vp, vp, vp, vp, vp, vp, vp, ctypes.c_int, ctypes.c_int, ctypes.c_float,
@@ -273,6 +275,15 @@ def nsp_plan_get(plan: Plan, pass_: int) -> np.ndarray:
     if rc != NSP_OK:
         raise NspError(rc, "nsp_plan_get")
     return out[: n.value]
+
+
+def nsp_plan_pair_items(plan: Plan, dkv_dtype: int = NSP_F32):
+    """(items on pairs of thread blocks, items on single ones) of the backward main kernels with dK / dV of that type."""
+    pairs, left = ctypes.c_int64(), ctypes.c_int64()
+    rc = lib().nsp_plan_pair_items(plan.handle, int(dkv_dtype), ctypes.byref(pairs), ctypes.byref(left))
+    if rc != NSP_OK:
+        raise NspError(rc, "nsp_plan_pair_items")
+    return pairs.value, left.value
 
 
 def nsp_attn_fwd(plan: Plan, q, k, v, o, lse, softmax_scale, ws=None, stream=None):

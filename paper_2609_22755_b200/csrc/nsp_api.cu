@@ -52,6 +52,7 @@ struct nsp_plan {
   int64_t n_parts = 0, n_first_parts = 0;   // 0: not divided
   nsp_tile_t* d_bwd_pairs = nullptr;          // items of the pair kernel: two key tiles of a segment of at least kPairTiles
   int64_t n_bwd_pairs = 0, n_bwd_paired = 0;  // their number, and how many of d_bwd_exec's first items they stand for
+  bool pairs_bf16 = false;                    // with bf16 dK / dV too (see kPairRest)
   int32_t* d_turns = nullptr;               // turn counters of the divided items
   nsp_tile_t* d_bwd_first = nullptr;  // one item per (segment or pack, kv head): the first-tile kernels' list
   int64_t n_first = 0;
@@ -205,6 +206,13 @@ constexpr int64_t kMostByLength = 600ll << 20;
 // 64q/4kv in 4,096 24.0 / 25.3; one head per KV head (16q/16kv) 2,000 4.32 / 4.25, 3,000 5.16 / 5.17. Batches whose longest
 // item would bound the kernel are divided instead (divide_items), and small ones (small_bwd) run their kernels side by side.
 constexpr int kPairTiles = 16, kPairSteps = 32;
+// The items that are left run behind the pairs, and with bf16 gradients undivided: that launch then lasts at least as long as
+// its longest item. There nothing is paired unless this item is, times the SMs, at most 1 / kPairRest of the paired items'
+// steps (counted per key tile). Main kernels, us, pairs / single CTAs, at 32q/4kv and bf16 gradients, by that share: 16 segments of 2,048
+// tokens and one of 1,900 at 64q/4kv (23 %) 3,370 / 3,030, 14 of 2,048 and four of 1,900 (26 %) 1,672 / 1,549, 32 of 2,048 and one of
+// 1,900 (11 %) 3,180 / 3,030, 16 of 4,096 and one (6 %) 5,785 / 5,984, 64 of 2,048 and one (5.7 %) 6,220 / 6,149, 24 of 4,096 and one
+// (4 %) 8,492 / 8,704, 32 of 4,096 and 20 of 1,000 (1.5 %) 11,310 / 11,550, 16 of 8,192 and one (1.5 %) 20,500 / 21,800.
+constexpr int kPairRest = 20;
 struct WholeItem {
   int32_t seg, head, tile, steps;
 };
@@ -262,6 +270,11 @@ struct UsesArena {
   }
   ~UsesArena() { arena_used(plan->arena, st); }
 };
+
+// Do backward calls with dK / dV of that type run the plan's long segments on CTA pairs?
+bool runs_on_pairs(const nsp_plan* plan, int dkv_dtype) {
+  return plan->n_bwd_pairs > 0 && (dkv_dtype == NSP_F32 || plan->pairs_bf16);
+}
 
 // Record the start / stop event of kernel `id` when profiling is on.
 void prof_mark(const nsp_plan* plan, int id, int stop, cudaStream_t st) {
@@ -503,7 +516,7 @@ int nsp_plan_tiles(const int32_t* cu_seqlens, const int32_t* hq, const int32_t* 
     if (tiles * n_seg > kMostSumTerms) bases = plan_tile_bases(keys, order);
     if (!p->deterministic && !p->rounded_dq) {
       std::vector<WholeItem> main_items, first_items;
-      int64_t main_steps = 0, first_steps = 0;
+      int64_t main_steps = 0, first_steps = 0, pair_steps = 0, longest_left = 0;
       size_t paired = 0;  // segments, in the order of their lengths, whose items run on CTA pairs
       if (head_dim == 128 && !p->small_bwd) {
         int64_t steps = 0, longest = 0;
@@ -526,6 +539,7 @@ int nsp_plan_tiles(const int32_t* cu_seqlens, const int32_t* hq, const int32_t* 
           p->n_bwd_paired = 0;
           pairs.clear();
         }
+        pair_steps = steps;
       }
       for (size_t at = paired; at < order.size(); ++at) {
         const int s = order[at];
@@ -536,8 +550,10 @@ int nsp_plan_tiles(const int32_t* cu_seqlens, const int32_t* hq, const int32_t* 
             const int32_t steps = G * (Mt - std::max(n, 1));
             if (steps > 0) main_items.push_back(WholeItem{s, g, n, steps});
             main_steps += steps;
+            longest_left = std::max<int64_t>(longest_left, steps);
           }
       }
+      p->pairs_bf16 = !pairs.empty() && kPairRest * longest_left * p->num_sms <= 2 * pair_steps;
       for (const nsp_tile_t& t : bwd_first) {
         first_items.push_back(WholeItem{t.seg, t.head, 0, t.cost});
         first_steps += t.cost;
@@ -693,6 +709,14 @@ int nsp_plan_get(const nsp_plan_t* plan, int pass, nsp_tile_t* host_out, int64_t
   if (cudaMemcpy(host_out, src, sizeof(nsp_tile_t) * m, cudaMemcpyDeviceToHost) !=
       cudaSuccess)
     return NSP_ERR_CUDA;
+  return NSP_OK;
+}
+
+int nsp_plan_pair_items(const nsp_plan_t* plan, int dkv_dtype, int64_t* n_pairs, int64_t* n_left) {
+  if (!plan || (dkv_dtype != NSP_BF16 && dkv_dtype != NSP_F32)) return NSP_ERR_INVALID_ARG;
+  const bool paired = runs_on_pairs(plan, dkv_dtype);
+  if (n_pairs) *n_pairs = paired ? plan->n_bwd_pairs : 0;
+  if (n_left) *n_left = paired ? plan->n_bwd - plan->n_bwd_paired : plan->n_bwd;
   return NSP_OK;
 }
 
@@ -888,7 +912,8 @@ int bwd_impl(const nsp_plan_t* plan, const uint8_t* recompute, const void* q, co
   // main kernels: everything else, the long segments on CTA pairs
   prof_mark(plan, NSP_KERNEL_BWD_MAIN, 0, st);
   a.turn = nullptr;
-  if (plan->n_bwd_pairs > 0) {
+  const bool paired = runs_on_pairs(plan, dkv_dtype);
+  if (paired) {
     BwdPairMaps pair_maps;
     std::memset(&pair_maps, 0, sizeof(pair_maps));
     static_cast<BwdMaps&>(pair_maps) = maps;
@@ -907,8 +932,9 @@ int bwd_impl(const nsp_plan_t* plan, const uint8_t* recompute, const void* q, co
     a.front = plan->d_front;
   }
   const bool m_parts = a.dkv_f32 && plan->n_parts > 0;
-  a.items = m_parts ? plan->d_bwd_parts : plan->d_bwd_exec + plan->n_bwd_paired;
-  a.n_items = static_cast<int32_t>(m_parts ? plan->n_parts : plan->n_bwd - plan->n_bwd_paired);
+  const int64_t done = paired ? plan->n_bwd_paired : 0;
+  a.items = m_parts ? plan->d_bwd_parts : plan->d_bwd_exec + done;
+  a.n_items = static_cast<int32_t>(m_parts ? plan->n_parts : plan->n_bwd - done);
   a.turn = m_parts ? plan->d_turns : nullptr;
   a.counter = plan->d_counters + 1;
   if (multi && launch_bwd(maps, a, plan->head_dim, plan->num_sms, plan->small_bwd, st) != cudaSuccess) return NSP_ERR_CUDA;

@@ -21,7 +21,7 @@ def _batch(lengths, hq, hkv):
     ([2048] * 20, 16, 4, "f32"),                             # whole tiles, an even number of them
     ([2049] * 30, 8, 2, "f32"),                              # an odd number: the second CTA of the last pair has no keys
     ([4100, 3969, 4097, 3968, 200, 40, 4200] * 3, 8, 8, "f32"),  # one head per KV head, ragged tiles, segments just below
-    ([2200, 1999, 1921, 1920, 129] * 3, 24, 8, "bf16"),      # bf16 gradients, odd groups, segments just below
+    ([2200, 1999, 1921] * 14 + [1920, 129], 24, 8, "bf16"),  # bf16 gradients, odd groups, segments just below
     ([4300, 3500, 100, 4299] * 4, 64, 1, "f32"),             # the start alignment of long items
 ])
 def test_pairs_against_single_ctas(lengths, hq, hkv, dkv_dtype):
@@ -63,3 +63,22 @@ def test_pairs_against_the_oracle():
     host = {k: run.host[k][kv if k in "kv" else q] for k in ("q", "k", "v", "do")}
     cut = {k: res[k][{"lse": lse, "dk": kv, "dv": kv}.get(k, q)] for k in res}
     P.compare_full(one, cut, P.oracle_full(one, host))
+
+
+# With bf16 gradients the items that are left are not divided: a long one beside few pairs keeps the whole batch on single CTAs.
+@pytest.mark.parametrize("lengths,hq,hkv,paired_bf16", [
+    ([2048] * 14 + [1900] * 4, 32, 4, False),
+    ([4096] * 8 + [1900], 32, 4, False),
+    ([2048] * 96 + [1900], 32, 4, True),
+    ([2048] * 20, 16, 4, True),  # nothing is left
+])
+def test_long_items_behind_the_pairs(lengths, hq, hkv, paired_bf16):
+    from paper_2609_22755_b200 import binding as B
+
+    w = _batch(lengths, hq, hkv)
+    plan = B.nsp_plan_tiles(w.cu_seqlens, w.hq, w.hkv, w.head_dim)
+    tiles = np.array([-(-x // 128) for x in lengths])
+    pairs = int((-(-tiles // 2) * (tiles >= 16)).sum()) * hkv
+    left = int((tiles * (tiles < 16)).sum()) * hkv
+    assert B.nsp_plan_pair_items(plan, B.NSP_F32) == (pairs, left)
+    assert B.nsp_plan_pair_items(plan, B.NSP_BF16) == ((pairs, left) if paired_bf16 else (0, int(tiles.sum()) * hkv))

@@ -196,7 +196,10 @@ inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 // 694, 737. Smaller parts than kMinPart steps cost more than they give: 1,511 tokens of three head structures, parts of
 // 24 / 16 / 12 / 8 / 4 steps: 101, 85, 88, 109, 125 us (whole: 114). The first-tile kernel's items have one step per q
 // head of twice that length and run beside the main kernel: divided they are worth it where they, not the main kernel,
-// bound the call (20 segments of about 100 tokens at 64q/4kv 233 -> 216 us; parts of eight steps 248, of two 215).
+// bound the call (20 segments of about 100 tokens at 64q/4kv 233 -> 216 us; parts of eight steps 248, of two 215). The pair
+// kernel does not start beside them: there they are divided where the parts fit one wave (first-tile kernel, us, whole /
+// parts: 8 segments of 2,048 tokens at 64q/4kv 103 / 65, 16 of 8,192 at 32q/4kv 85 / 65; in two or more waves 32 of
+// 4,096 90 / 112, 64 of 2,048 156 / 195, 64 of 2,048 at 64q/4kv 285 / 310).
 constexpr int kMinPart = 16, kMinFirstPart = 4;
 constexpr int64_t kMostByLength = 600ll << 20;
 // Backward items that run on CTA pairs: segments of at least kPairTiles key tiles and kPairSteps steps for the first of them. A
@@ -562,6 +565,7 @@ int nsp_plan_tiles(const int32_t* cu_seqlens, const int32_t* hq, const int32_t* 
                            q_off * 4 <= kMostByLength, &n_turns);
       first_parts = divide_items(first_items, std::max<int64_t>(kMinFirstPart, (first_steps + main_steps) / (2 * p->num_sms)), true,
                                  &n_turns);
+      if (!pairs.empty() && static_cast<int64_t>(first_parts.size()) > p->num_sms) first_parts.clear();
     }
     p->n_bwd_pairs = static_cast<int64_t>(pairs.size());
     p->n_parts = static_cast<int64_t>(parts.size());

@@ -82,3 +82,24 @@ def test_long_items_behind_the_pairs(lengths, hq, hkv, paired_bf16):
     left = int((tiles * (tiles < 16)).sum()) * hkv
     assert B.nsp_plan_pair_items(plan, B.NSP_F32) == (pairs, left)
     assert B.nsp_plan_pair_items(plan, B.NSP_BF16) == ((pairs, left) if paired_bf16 else (0, int(tiles.sum()) * hkv))
+
+
+def test_first_tile_kernel_beside_pairs():
+    """Its items are not divided into more parts than one wave takes (as such parts 32 segments of 4,096 tokens took 112 us, whole 90)."""
+    import parity_util as P
+    from paper_2609_22755_b200 import binding as B
+
+    w = _batch([4096] * 32, 32, 4)
+    host, best = None, []
+    for deterministic in (False, True):  # the ordered plan divides nothing
+        run = P.GpuRun(w, tensors=host, deterministic=deterministic)
+        host = run.host
+        run.forward()
+        B.nsp_plan_set_profiling(run.plan, True)
+        times = []
+        for _ in range(8):
+            run.backward()
+            times.append(B.nsp_plan_kernel_ms(run.plan, B.KERNEL_BWD_FIRST))
+        best.append(min(times))
+        del run
+    assert best[0] <= 1.12 * best[1], best

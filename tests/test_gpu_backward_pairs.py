@@ -16,6 +16,14 @@ def _batch(lengths, hq, hkv):
     return W.custom(lengths, hq, hkv, seed=43)
 
 
+def _pairs(lengths, hq, hkv):
+    """Items of the pair kernel where the rule takes every segment that is long enough: two key tiles each, per KV head."""
+    hq, hkv = (np.broadcast_to(h, len(lengths)) for h in (hq, hkv))
+    tiles = np.array([-(-x // 128) for x in lengths])
+    long = (tiles >= 16) & (hq // hkv * tiles >= 32)
+    return int(((tiles + 1) // 2 * hkv * long).sum()), int((tiles * hkv * ~long).sum())
+
+
 # The pair kernel takes segments of 16 key tiles (32 with one head per KV head) and more, of a batch that fills the chip.
 @pytest.mark.parametrize("lengths,hq,hkv,dkv_dtype", [
     ([2048] * 20, 16, 4, "f32"),                             # whole tiles, an even number of them
@@ -23,13 +31,20 @@ def _batch(lengths, hq, hkv):
     ([4100, 3969, 4097, 3968, 200, 40, 4200] * 3, 8, 8, "f32"),  # one head per KV head, ragged tiles, segments just below
     ([2200, 1999, 1921] * 14 + [1920, 129], 24, 8, "bf16"),  # bf16 gradients, odd groups, segments just below
     ([4300, 3500, 100, 4299] * 4, 64, 1, "f32"),             # the start alignment of long items
+    ([4096] * 8 + [1900, 1500, 1300], 32, 4, "f32"),         # the items that are left are divided
+    ([2050, 2048] * 8 + [4000] * 6 + [300], [16] * 16 + [8] * 7, [4] * 16 + [1] * 7, "f32"),  # two runs
 ])
 def test_pairs_against_single_ctas(lengths, hq, hkv, dkv_dtype):
     import parity_util as P
+    from paper_2609_22755_b200 import binding as B
 
     w = _batch(lengths, hq, hkv)
     run = P.GpuRun(w, dq_dtype="f32", dkv_dtype=dkv_dtype)
     single = P.GpuRun(w, tensors=run.host, dq_dtype="f32", dkv_dtype=dkv_dtype, deterministic=True)
+    dtype = B.NSP_F32 if dkv_dtype == "f32" else B.NSP_BF16
+    n_pairs, n_left = _pairs(lengths, hq, hkv)
+    assert n_pairs > 0 and B.nsp_plan_pair_items(run.plan, dtype) == (n_pairs, n_left)
+    assert B.nsp_plan_pair_items(single.plan, dtype)[0] == 0
     got = []
     for r in (run, single):
         r.forward()
@@ -39,20 +54,52 @@ def test_pairs_against_single_ctas(lengths, hq, hkv, dkv_dtype):
             r.backward()
         assert r.status()[0] == 0
         got.append(r.results())
+    _compare(*got, dkv_dtype)
+
+
+def _compare(pairs, single, dkv_dtype):
     # The same products of the same operands; what differs is the order in which the tensor core adds and in which up to 32
     # tiles are added to a row of dQ, one fp32 rounding each: 32 * 2^-24 of the largest partial sum. bf16 results: one step.
     for n in ("dq", "dk", "dv"):
         tol = 2.0 ** -8 if n != "dq" and dkv_dtype == "bf16" else 2e-5
-        assert np.max(np.abs(got[0][n] - got[1][n])) <= tol * np.max(np.abs(got[1][n])), n
+        assert np.max(np.abs(pairs[n] - single[n])) <= tol * np.max(np.abs(single[n])), n
+
+
+def test_pairs_with_recomputed_segments():
+    import parity_util as P
+    import torch
+    from paper_2609_22755_b200 import binding as B
+
+    w = _batch([2049, 2048, 2300, 1000] * 6, 16, 4)
+    flags = np.arange(24, dtype=np.uint8) % 3 == 0  # paired segments and others
+    host, got = None, []
+    for deterministic in (False, True):
+        run = P.GpuRun(w, tensors=host, dq_dtype="f32", deterministic=deterministic)
+        host = run.host
+        assert (B.nsp_plan_pair_items(run.plan)[0] > 0) == (not deterministic)
+        run.forward()
+        cu = w.cu_seqlens
+        for s in np.flatnonzero(flags):  # neither O nor LSE of a marked segment is read
+            run.o[int(cu[s]) * 16 * 128:int(cu[s + 1]) * 16 * 128] = float("nan")
+            run.lse[int(cu[s]) * 16:int(cu[s + 1]) * 16] = float("nan")
+        ws = torch.empty(B.nsp_plan_recompute_ws_bytes(run.plan), dtype=torch.uint8, device=run.dev)
+        B.nsp_attn_bwd_recompute(run.plan, flags.astype(np.uint8), run.q, run.k, run.v, run.o, run.do, run.lse, run.dq, run.dk,
+                                 run.dv, w.softmax_scale, ws)
+        assert run.status()[0] == 0
+        got.append(run.results())
+    assert all(np.isfinite(got[0][n]).all() for n in ("dq", "dk", "dv"))
+    _compare(*got, "f32")
 
 
 def test_pairs_against_the_oracle():
     import parity_util as P
+    from paper_2609_22755_b200 import binding as B
     from paper_2609_22755_b200 import workloads as W
 
     L, n, hq, hkv = 3073, 16, 8, 2
     w = _batch([L] * n, hq, hkv)
     run = P.GpuRun(w)
+    assert B.nsp_plan_pair_items(run.plan) == _pairs([L] * n, hq, hkv)
     run.forward()
     run.backward()
     assert run.status()[0] == 0
@@ -77,11 +124,10 @@ def test_long_items_behind_the_pairs(lengths, hq, hkv, paired_bf16):
 
     w = _batch(lengths, hq, hkv)
     plan = B.nsp_plan_tiles(w.cu_seqlens, w.hq, w.hkv, w.head_dim)
-    tiles = np.array([-(-x // 128) for x in lengths])
-    pairs = int((-(-tiles // 2) * (tiles >= 16)).sum()) * hkv
-    left = int((tiles * (tiles < 16)).sum()) * hkv
+    pairs, left = _pairs(lengths, hq, hkv)
     assert B.nsp_plan_pair_items(plan, B.NSP_F32) == (pairs, left)
-    assert B.nsp_plan_pair_items(plan, B.NSP_BF16) == ((pairs, left) if paired_bf16 else (0, int(tiles.sum()) * hkv))
+    everything = sum(-(-x // 128) for x in lengths) * hkv
+    assert B.nsp_plan_pair_items(plan, B.NSP_BF16) == ((pairs, left) if paired_bf16 else (0, everything))
 
 
 def test_first_tile_kernel_beside_pairs():

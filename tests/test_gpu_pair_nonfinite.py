@@ -35,6 +35,7 @@ def test_reach_of_nonfinite_values(name, token, value):
     got = []
     for deterministic in (False, True):  # the ordered additions run every segment on single CTAs
         run = P.GpuRun(w, tensors=clean, dq_dtype="f32", deterministic=deterministic)
+        assert (run.B.nsp_plan_pair_items(run.plan)[0] > 0) == (not deterministic)
         run.forward()  # O and LSE of finite inputs
         for n in ("q", "k", "v", "do"):
             getattr(run, n).copy_(host[n])

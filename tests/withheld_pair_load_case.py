@@ -21,6 +21,7 @@ host = W.make_tensors(w)
 
 def healthy():
     run = P.GpuRun(w, tensors=host, dq_dtype="f32")
+    assert B.nsp_plan_pair_items(run.plan)[0] > 0
     run.forward()
     run.backward()
     assert run.status() == (0, 0, 0, 0), run.status()

@@ -1,7 +1,7 @@
-"""The hand-overs of the CTA-pair kernel (csrc/nsp_bwd_pair.cu) as a model on the CPU: its roles, barriers and buffers, run under random and
-lopsided delays. Two kinds of fault are looked for. A wait goes by the parity of a phase alone, so a barrier that is two phases
-ahead of a waiter holds it for good, and one that is a phase behind lets it through; and every buffer and TMEM region has to hold the step
-that its reader means, from the start of the read to its end. A missing wait shows up here without a GPU."""
+"""The hand-overs of the CTA-pair kernel (csrc/nsp_bwd_pair.cu) as a model on the CPU: its roles, barriers and buffers, run under
+random and lopsided delays. Two kinds of fault are looked for. A wait goes by the parity of a phase alone, so a barrier that is
+two phases ahead of a waiter holds it for good, and one that is a phase behind lets it through; and every buffer and TMEM region has
+to hold the step that its reader means, from the start of the read to its end. A missing wait shows up here without a GPU."""
 import heapq
 import random
 import re
@@ -55,7 +55,7 @@ class Sim:
         self.items, self.without = items, set(without)
         # every run has its own idea of which activities are slow
         self.slow, self.waiting = {}, []
-        count = {"qr": 2, "dor": 2, "doc": 2, "qc": 2, "s_read": 16, "p_ready": 16, "ds_ready": 16, "dq_empty": 16, "x_peer": 1}
+        count = {"qr": 2, "dor": 2, "doc": 2, "qc": 2, "s_read": 16, "p_ready": 16, "ds_ready": 16, "dq_empty": 16, "x_peer": 2}
         self.bar = {n: Barrier(self, n, c) for n, c in count.items()}  # qr ..: one load of each CTA
         for r in (0, 1):
             for n, c in {"s_full": 1, "dp_full": 1, "dq_full": 1, "dv_done": 1, "dk_done": 1, "x_own": 4, "x_full": 4, "ld_full0": 1,
@@ -189,12 +189,12 @@ class Sim:
                 self.bar["ld_full%d" % (cs & 1), r].arrive()
             gs += steps
 
-    def relay(self):
+    def relay(self, part):
         gs = 0
         for steps in self.items:
             yield "meet", 0
             for cs in range(gs, gs + steps):
-                yield self.wait((("x_full", 1), cs), (("x_own", 1), cs))
+                yield self.wait(((part, 1), cs))
                 yield "work", "relay"
                 self.remote(1, "x_peer")
             gs += steps
@@ -304,7 +304,7 @@ class Sim:
             yield "work", "epilogue"
 
     def run(self):
-        roles = [("A", self.issuer_a()), ("B", self.issuer_b()), ("relay", self.relay())]
+        roles = [("A", self.issuer_a()), ("B", self.issuer_b()), ("relay17", self.relay("x_own")), ("relay19", self.relay("x_full"))]
         for r in (0, 1):
             roles += [("producer%d" % r, self.producer(r)), ("loader%d" % r, self.loader(r))]
             roles += [("softmax%d.%d" % (r, w), self.softmax(r, w)) for w in range(8)]

@@ -146,6 +146,8 @@ int nsp_attn_fwd(const nsp_plan_t* plan, const void* q, const void* k, const voi
  * dk/dv hold the sum over the hq/hkv query heads that share a KV head on THIS GPU (with a replicated KV head
  * at high degree the cross-GPU sum belongs to the epilogue collective, outside this library).
  * ws: at least bwd_ws_bytes, 256-byte aligned; contents undefined afterwards.
+ * Inputs are meant to be finite. Masked scores of a 128 x 128 tile enter the products as zeros, so a value that is not finite can
+ * reach results of any row of its tiles, and behind a segment's ragged end rows of the last tile of the segment before.
  * Errors: as nsp_attn_fwd.
  */
 int nsp_attn_bwd(const nsp_plan_t* plan, const void* q, const void* k, const void* v, const void* o, const void* d_o,

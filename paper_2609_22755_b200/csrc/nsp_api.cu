@@ -202,11 +202,13 @@ inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 // 4,096 90 / 112, 64 of 2,048 156 / 195, 64 of 2,048 at 64q/4kv 285 / 310).
 constexpr int kMinPart = 16, kMinFirstPart = 4;
 constexpr int64_t kMostByLength = 600ll << 20;
-// Backward items that run on CTA pairs: segments of at least kPairTiles key tiles and kPairSteps steps for the first of them. A
+// Backward items that run on CTA pairs: segments of at least kPairTiles key tiles and kPairSteps steps for the first of them,
+// taken from the longest down to the first that has fewer (a batch whose longest has too few steps is left alone). A
 // pair computes one tile more than it needs (the second key tile has nothing of the item's last q tile) and meets its partner
-// between items. Backward pass over about 131,072 tokens, ms, pairs / single CTAs: 32q/4kv in segments of 512 tokens (4
-// tiles) not paired, 1,024 4.56 / 4.55, 1,536 5.91 / 5.98, 2,048 7.22 / 7.36, 3,072 9.58 / 10.03, 4,096 12.2 / 12.6;
-// 64q/4kv in 4,096 24.0 / 25.3; one head per KV head (16q/16kv) 2,000 4.32 / 4.25, 3,000 5.16 / 5.17. Batches whose longest
+// between items. Backward pass over about 131,072 tokens, ms, pairs / single CTAs: 32q/4kv in segments of 1,024 tokens (8
+// tiles) 4.25 / 4.22, 1,536 5.55 / 5.71 (main kernels alone 4.74 / 4.71), 2,048 6.68 / 6.71 (5.88 / 6.07), 3,072 9.56 /
+// 9.81, 4,096 12.2 / 12.6; 64q/4kv in 1,024 8.9 / 8.9, 2,048 14.0 / 14.4, 4,096 24.4 / 25.7; one head per KV head (16q/16kv)
+// 2,000 4.10 / 3.84, 3,000 5.32 / 5.10, 4,000 6.50 / 6.69. Batches whose longest
 // item would bound the kernel are divided instead (divide_items), and small ones (small_bwd) run their kernels side by side.
 constexpr int kPairTiles = 16, kPairSteps = 32;
 // The items that are left run behind the pairs, and with bf16 gradients undivided: that launch then lasts at least as long as
@@ -536,7 +538,8 @@ int nsp_plan_tiles(const int32_t* cu_seqlens, const int32_t* hq, const int32_t* 
           p->n_bwd_paired += static_cast<int64_t>(sg.hkv) * Mt;
         }
         // Not where the longest item would bound the kernel, nor where other segments have more than a quarter of the steps:
-        // the two launches each have a tail.
+        // the two launches each have a tail. Backward pass, ms, pairs / single CTAs: 131,072 tokens around 432 at 32q/4kv, its
+        // segments of 2,048 tokens and more on pairs, 6.15 / 6.01; 65,536 around 1,024 (nearly all steps) 12.3 / 13.05.
         if (longest * (p->num_sms / 2) > steps || 8 * steps < 3 * bwd_steps) {
           paired = 0;
           p->n_bwd_paired = 0;

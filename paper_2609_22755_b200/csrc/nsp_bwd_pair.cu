@@ -12,9 +12,12 @@
 //                                 queries (this CTA's query set)                                         M = 128, K = 256
 // For dQ^T each CTA needs the other's dS^T of its own query set: 16 KB of bf16 per step and direction through distributed
 // shared memory (one bulk copy per softmax warp, under the next step).
-// What bounds a step (3,910 clocks; the single-CTA kernel's takes 4,340): the loop of exchange, dQ^T, its drain and the S^T behind
-// it, with 2,560 clocks of tensor pipe and ~2,900 of shared-memory traffic under it. Whole steps under the 1,000 W cap, single CTAs /
-// pairs: sixteen segments of 8,192 tokens at 32q/4kv 32.6 / 30.8 ms, 393,216 tokens at 4q/1kv beside a tail 541 / 505 ms.
+// A step takes 3,880 active clocks, 2,570 of them of tensor pipe (ncu, 65,536 tokens at 4q/1kv beside a tail; 4,060 on single CTAs).
+// What bounds it are two loops of hand-overs. One step long: dS^T 830, fence 390, copy and relay ~1,500, dQ^T ~1,000, then the dS^T
+// buffers are free for the next step's: ~3,700. Two steps long, because S^T(t + 2) goes over dQ^T(t): fence, copy and relay,
+// dQ^T, its drain ~800, S^T ~900, its reading 240, exponentials 1,080, dS^T: ~6,700, half of that per step. (Parts by
+// clock stamps, 16 x 8,192 tokens.) Whole steps under the 1,000 W cap, single CTAs / pairs: sixteen segments of 8,192 tokens at
+// 32q/4kv 33.0 / 31.2 ms, 393,216 tokens at 4q/1kv beside a tail 538.6 / 504.4.
 // Query sets: softmax warpgroup w has the queries 32 w .. 32 w + 31 and 64 + 32 w .. of a tile, so that packed P^T and dS^T of
 // both warpgroups go to [0, 64) of their region over columns the same thread has read, and CTA r's query set is the one of
 // warpgroup r.
